@@ -35,9 +35,11 @@
 // segment's worst-case slot of the workspace; a one-CTA scan then lays out
 // the header and length table and a gather moves every code into place.
 // Decompression: a one-CTA scan checks the header and table and finds every
-// segment's start; then one thread per segment decodes its tokens, copying
-// a match's bits from the output it has written (a source that overlaps the
-// bits being produced repeats with the match distance as its period).
+// segment's start; then a CTA of two warps decodes each segment 32 tokens at
+// a time, the first warp finding the tokens and reading their fields, the
+// second copying a match's bits from the output it has written (a source
+// that overlaps the bits being produced repeats with the match distance as
+// its period).  Very many segments are decoded by a thread each instead.
 #include <cstdint>
 
 #include "api_trace.h"
@@ -55,11 +57,18 @@ constexpr uint32_t kRingMaxWindow = 16384;  // the shared-memory window ring
 // dynamic shared memory of the largest ring (W = 16384: 1024 words, twice, per warp)
 constexpr size_t kMaxRingSmem = (size_t)kLzWarps * 2 * 1024 * 4;
 constexpr uint64_t kMaxSegment = 1ull << 24;
-constexpr int kLzDecThreads = 32;              // decompress: one warp per CTA, a segment per thread
-constexpr uint32_t kDecRing = 128;             // output words kept per thread (a power of two)
-constexpr uint32_t kDecRingMaxWindow = 2048;   // windows whose words fit the ring with 4 to spare
-constexpr uint32_t kLzInCells = 8;             // decompress: 16-byte cells of code staged per thread
+constexpr int kThrBlock = 32;             // thread-per-segment decompress: one warp per CTA
+constexpr uint32_t kThrRing = 128;        // output words kept per thread (a power of two)
+constexpr uint32_t kThrMaxWindow = 2048;  // windows whose words fit that ring with 4 to spare
+constexpr uint32_t kLzInCells = 8;        // 16-byte cells of code staged per thread
 constexpr uint32_t kLzInFlight = kLzInCells - 1;  // copies left in flight when a word is read
+constexpr uint32_t kPathNone = 0, kPathWarps = 1, kPathThreads = 2;  // k_lzss_dlayout's choice
+constexpr uint32_t kDecRing = 256;   // decompress: output words kept per warp (a power of two)
+constexpr uint32_t kDecAhead = 66;   // 31 words not stored yet, 33 a batch of 32 tokens may fill, one begun
+constexpr uint32_t kDecHistory = kDecRing - kDecAhead - 4;  // stored words that stay readable
+constexpr uint32_t kCodeRing = 256;  // code words staged per warp (a power of two)
+constexpr uint32_t kWalkBits = 64;   // code bits per lane and find_tokens
+constexpr uint32_t kTokList = 2048;  // 31 tokens left and the kWalkBits * 32 / 2 of one find_tokens
 
 struct LzParams {
     uint32_t W, lmin, lmax, blk, dict;
@@ -370,6 +379,34 @@ __global__ void __launch_bounds__(kLzBlock)
     }
 }
 
+// Exclusive sum of `own` over the CTA's kScanBlock threads; the total of all in
+// `total`.  `part` holds 32 values.
+__device__ __forceinline__ unsigned long long block_scan(unsigned long long own,
+                                                         unsigned long long *part,
+                                                         unsigned long long &total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long incl = own;
+    for (int k = 1; k < 32; k <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, k);
+        if (lane >= k)
+            incl += y;
+    }
+    __syncthreads();  // part's last readers
+    if (lane == 31)
+        part[warp] = incl;
+    __syncthreads();
+    unsigned long long p = part[lane];
+    for (int k = 1; k < 32; k <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, p, k);
+        if (lane >= k)
+            p += y;
+    }
+    total = __shfl_sync(0xffffffffu, p, 31);
+    const unsigned long long before = __shfl_sync(0xffffffffu, p, warp ? warp - 1 : 0);
+    return (warp ? before : 0) + incl - own;
+}
+
 // Header, length table and segment starts of the container; the size into
 // *out_bytes, HUFF_ERR_CAPACITY when it exceeds `cap`.
 __global__ void __launch_bounds__(kScanBlock)
@@ -377,30 +414,22 @@ __global__ void __launch_bounds__(kScanBlock)
                   uint64_t *__restrict__ start, uint8_t *__restrict__ out, uint64_t cap,
                   unsigned long long *out_bytes, int32_t *status)
 {
-    __shared__ unsigned long long s_part[kScanBlock];
+    __shared__ unsigned long long s_part[32];
     if (chain_failed(status))
         return;
     const int tid = threadIdx.x;
     const uint64_t count = n ? (n + seg - 1) / seg : 0;
     const uint64_t head = al16(kLzHead + 4 * count);
-    const uint64_t per = (count + kScanBlock - 1) / kScanBlock;
-    const uint64_t b0 = tid * per, b1 = b0 + per < count ? b0 + per : count;
-    unsigned long long own = 0;
-    for (uint64_t i = b0; i < b1; ++i)
-        own += al16((bits[i] + 7) / 8);
-    s_part[tid] = own;
-    __syncthreads();
-    unsigned long long before = 0;
-    for (int t = 0; t < tid; ++t)
-        before += s_part[t];
-    for (uint64_t i = b0; i < b1; ++i) {
-        start[i] = head + before;
-        before += al16((bits[i] + 7) / 8);
-    }
-    __syncthreads();
     unsigned long long total = head;
-    for (int t = 0; t < kScanBlock; ++t)
-        total += s_part[t];
+    for (uint64_t i0 = 0; i0 < count; i0 += kScanBlock) {
+        const uint64_t i = i0 + tid;
+        unsigned long long sum;
+        const unsigned long long at =
+            block_scan(i < count ? al16(((uint64_t)bits[i] + 7) / 8) : 0, s_part, sum);
+        if (i < count)
+            start[i] = total + at;
+        total += sum;
+    }
     if (tid == 0) {
         *out_bytes = total;
         if (total > cap)
@@ -462,22 +491,34 @@ __global__ void k_lzss_gather(uint64_t n, uint64_t seg, LzParams P, const uint8_
 }
 
 // ---------------------------------------------------------------- decompress
+// Whether a thread per segment decodes faster than a CTA of two warps per
+// segment: its tokens cost a quarter of the instructions (32 segments share
+// each one), but every segment is one chain of ~700 cycles a token, so it
+// takes very many segments to fill the chip.  1024/12/24/8, stored prefix, the
+// bitstream stand-in, threads against warps: 16384 segments 1.10 / 0.67 ms
+// (64 MiB), 65536 segments 0.74 / 0.79 (64 MiB), 2.28 / 2.52 (256 MiB), 7.1 /
+// 9.3 (1 GiB), 262144 segments 0.96 / 1.34 (64 MiB); so from 320 segments per
+// SM (48640) on.  Its branch-free step wants the stored prefix, a window that
+// fits the thread's ring and literals that fit a token's first word.
+__device__ __forceinline__ bool threads_better(uint64_t count, uint32_t W, uint32_t blk,
+                                               uint32_t dict, uint32_t sms)
+{
+    return count >= 320ull * sms && W >= 32 && W <= kThrMaxWindow && dict == 2 && blk <= 31;
+}
+
 // Header and table checks, segment starts (scan), *d_n; statuses as the
 // oracle's: CORRUPT for an inconsistent header or table, CAPACITY for n >
-// cap.  ok[0] = 1 when the segments may be decoded.
+// cap.  *path: the decoder to run, kPathNone when the segments may not be
+// decoded.
 __global__ void __launch_bounds__(kScanBlock)
     k_lzss_dlayout(const uint8_t *__restrict__ c, uint64_t bytes, uint64_t cap,
                    uint64_t *__restrict__ start, uint64_t max_count,
-                   unsigned long long *d_n, int32_t *status, uint32_t *ok)
+                   unsigned long long *d_n, int32_t *status, uint32_t *path, uint32_t sms)
 {
-    __shared__ unsigned long long s_part[kScanBlock];
-    __shared__ int s_bad;
+    __shared__ unsigned long long s_part[32];
     const int tid = threadIdx.x;
-    if (tid == 0) {
-        *ok = 0;
-        s_bad = 0;
-    }
-    __syncthreads();
+    if (tid == 0)
+        *path = kPathNone;
     if (chain_failed(status))
         return;
     if (bytes < kLzHead) {
@@ -500,40 +541,453 @@ __global__ void __launch_bounds__(kScanBlock)
     }
     const uint8_t *tab = c + kLzHead;
     const uint64_t head = al16(kLzHead + 4 * count);
-    const uint64_t per = (count + kScanBlock - 1) / kScanBlock;
-    const uint64_t b0 = tid * per, b1 = b0 + per < count ? b0 + per : count;
-    unsigned long long own = 0;
-    for (uint64_t i = b0; i < b1; ++i) {
-        const uint32_t nb = *reinterpret_cast<const uint32_t *>(tab + 4 * i);
-        own += al16(((uint64_t)nb + 7) / 8);
-    }
-    s_part[tid] = own;
-    __syncthreads();
-    unsigned long long before = 0, total = head;
-    for (int t = 0; t < kScanBlock; ++t) {
-        if (t < tid)
-            before += s_part[t];
-        total += s_part[t];
-    }
-    for (uint64_t i = b0; i < b1; ++i) {
-        start[i] = head + before;
-        before += al16(((uint64_t)*reinterpret_cast<const uint32_t *>(tab + 4 * i) + 7) / 8);
+    unsigned long long total = head;
+    for (uint64_t i0 = 0; i0 < count; i0 += kScanBlock) {
+        const uint64_t i = i0 + tid;
+        unsigned long long sum;
+        const uint64_t nb = i < count ? *reinterpret_cast<const uint32_t *>(tab + 4 * i) : 0u;
+        const unsigned long long at = block_scan(al16((nb + 7) / 8), s_part, sum);
+        if (i < count)
+            start[i] = total + at;
+        total += sum;
     }
     if (tid == 0) {
         if (total != bytes) {
             set_status(status, HUFF_ERR_CORRUPT_STREAM);
-            s_bad = 1;
         } else {
             *d_n = n;
-            if (n > cap) {
+            if (n > cap)
                 set_status(status, HUFF_ERR_CAPACITY);
-                s_bad = 1;
-            }
+            else
+                *path = threads_better(count, f[0], f[3], f[4], sms) ? kPathThreads : kPathWarps;
         }
     }
-    __syncthreads();
-    if (tid == 0 && !s_bad)
-        *ok = 1;
+}
+
+// Store output word q (MSB-first bytes) of an m-byte segment output.
+__device__ __forceinline__ void store_out_word(uint8_t *y, uint32_t m, uint32_t q, uint32_t w)
+{
+    const uint32_t b = 4 * q;
+    if (b + 4 <= m) {
+        __stcg(reinterpret_cast<uint32_t *>(y) + q, bswap32(w));
+    } else {
+        for (uint32_t k = 0; k < 4; ++k)
+            if (b + k < m)
+                y[b + k] = (uint8_t)(w >> (24 - 8 * k));
+    }
+}
+
+// Shared memory of one decoding CTA: a front warp and a copy warp, the first
+// one batch of tokens ahead of the second.
+struct alignas(16) DecShared {
+    uint32_t out[kDecRing];    // copy warp: output word q at q mod kDecRing
+    uint32_t code[kCodeRing];  // front warp: code word q at q mod kCodeRing
+    uint16_t list[kTokList];   // front warp: token starts not decoded yet (position << 1 | flag)
+    uint16_t exits[(kWalkBits + 33) * 32];  // front warp: [offset][lane], see find_tokens
+    struct Batch {  // 32 tokens: place in the output, kTok* fields, distance or literal bits
+        uint32_t o[32], info[32], x[32];
+    } batch[2];
+};
+// a token's fields in Batch::info above its length (bits 0..5)
+constexpr uint32_t kTokRef = 64, kTokValid = 128, kTokEnd = 256;
+
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v) : "memory");
+}
+// named barriers of the two warps: 1, 2 a batch is full, 3, 4 it is read
+// (ids as immediates: with an id in a register the kernel reserves all 16
+// barriers, which leaves four CTAs per SM resident)
+__device__ __forceinline__ void full_sync(uint32_t turn)
+{
+    if (turn & 1)
+        asm volatile("bar.sync 2, 64;" ::: "memory");
+    else
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+}
+__device__ __forceinline__ void full_arrive(uint32_t turn)
+{
+    if (turn & 1)
+        asm volatile("bar.arrive 2, 64;" ::: "memory");
+    else
+        asm volatile("bar.arrive 1, 64;" ::: "memory");
+}
+__device__ __forceinline__ void read_sync(uint32_t turn)
+{
+    if (turn & 1)
+        asm volatile("bar.sync 4, 64;" ::: "memory");
+    else
+        asm volatile("bar.sync 3, 64;" ::: "memory");
+}
+__device__ __forceinline__ void read_arrive(uint32_t turn)
+{
+    if (turn & 1)
+        asm volatile("bar.arrive 4, 64;" ::: "memory");
+    else
+        asm volatile("bar.arrive 3, 64;" ::: "memory");
+}
+
+// The segment a CTA decodes.
+struct SegIn {
+    const uint32_t *w;  // the code's words (16-byte aligned, padded to a 16-byte boundary)
+    uint32_t nw;        // their number; words past them read as zero
+    uint32_t code_bits;
+    uint8_t *y;         // the output, 16-byte aligned
+    uint32_t m, nbits;  // its bytes and bits
+    uint32_t raw;       // bits stored as they are before the tokens
+    __device__ __forceinline__ uint32_t load(uint32_t i) const
+    {
+        return i < nw ? bswap32(__ldg(w + i)) : 0u;
+    }
+};
+
+// The front warp's state.
+struct Front {
+    uint32_t bpos;        // code bits whose tokens are listed
+    uint32_t loaded;      // code words staged
+    uint32_t pre0, pre1;  // the next 64 code words, two per lane
+    uint32_t head, avail; // the list's first token and its length
+};
+
+// exits[e] of one lane's kWalkBits bits (hi:lo), from the last offset back;
+// G offsets at a time: no token is shorter than G bits, so the loads of a
+// group do not depend on its own stores.
+template <int G>
+__device__ __forceinline__ void fill_exits(uint32_t col, uint32_t hi, uint32_t lo, uint32_t len_ref,
+                                           uint32_t len_lit)
+{
+    const uint32_t cr = col + 64 * len_ref, cl = col + 64 * len_lit;
+#pragma unroll
+    for (int g = (int)kWalkBits - G; g >= 0; g -= G) {
+        uint32_t v[G];
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+            const int p = g + j;
+            const bool ref = ((p < 32 ? hi : lo) & (0x80000000u >> (p & 31))) != 0;
+            v[j] = lds_u16((ref ? cr : cl) + 64 * p);
+        }
+#pragma unroll
+        for (int j = 0; j < G; ++j)
+            sts_u16(col + 64 * (g + j), v[j] + 0x100u);
+    }
+}
+
+// List the starts of the tokens in the next kWalkBits * 32 code bits.  A
+// token's length depends on its flag alone, so where a walk leaves a stretch
+// of code is a function of where it enters.  Lane l takes the kWalkBits bits
+// from bit kWalkBits * l on and fills, for every offset e, exits[e][l]: the
+// offset in lane l + 1's bits at which a walk entering at e leaves, and the
+// tokens it passes << 8 (exits[e] = exits[e + the length of the token at e]
+// plus one token; offsets past the stretch map to themselves).  Then one
+// chain of 32 loads gives every lane its true entry and its tokens' place in
+// the list, and each lane walks only its own few tokens: a walk of all the
+// tokens by itself costs one warp ~150 cycles a token.
+__device__ __forceinline__ void find_tokens(const SegIn &sg, Front &fr, DecShared &sh,
+                                            uint32_t len_ref, uint32_t len_lit, int lane)
+{
+    // the stretch, the longest token's rest past it and a word of slack
+    while (fr.loaded < (fr.bpos >> 5) + kWalkBits + 4) {
+        sh.code[(fr.loaded + lane) & (kCodeRing - 1)] = fr.pre0;
+        sh.code[(fr.loaded + 32 + lane) & (kCodeRing - 1)] = fr.pre1;
+        fr.loaded += 64;
+        fr.pre0 = sg.load(fr.loaded + lane);
+        fr.pre1 = sg.load(fr.loaded + 32 + lane);
+    }
+    __syncwarp();
+    const uint32_t at = (fr.bpos & 31u) + kWalkBits * (uint32_t)lane;
+    const uint32_t q = (fr.bpos >> 5) + (at >> 5);
+    const uint32_t w0 = sh.code[q & (kCodeRing - 1)], w1 = sh.code[(q + 1) & (kCodeRing - 1)],
+                   w2 = sh.code[(q + 2) & (kCodeRing - 1)];
+    uint32_t hi = __funnelshift_l(w1, w0, at & 31u), lo = __funnelshift_l(w2, w1, at & 31u);
+    const uint32_t tab = smem_u32(sh.exits);
+    if (len_ref >= 8 && len_lit >= 8)
+        fill_exits<8>(tab + 2 * lane, hi, lo, len_ref, len_lit);
+    else
+        fill_exits<2>(tab + 2 * lane, hi, lo, len_ref, len_lit);
+    __syncwarp();
+    uint32_t e = 0, acc = 0, mine = 0;  // acc, mine: tokens so far << 8 | entry
+#pragma unroll
+    for (int l = 0; l < 32; ++l) {
+        mine = lane == l ? acc : mine;
+        const uint32_t v = lds_u16(tab + e * 64 + 2 * l);
+        e = v & 0xffu;
+        acc = (acc & ~0xffu) + v;
+    }
+    uint32_t p = mine & 0xffu, i = fr.head + fr.avail + (mine >> 8);
+    const uint32_t base = (fr.bpos + kWalkBits * (uint32_t)lane) << 1;
+    const uint64_t b = (((uint64_t)hi << 32) | lo) << p;
+    hi = (uint32_t)(b >> 32);
+    lo = (uint32_t)b;
+    while (p < kWalkBits) {
+        const uint32_t flag = hi >> 31, step = flag ? len_ref : len_lit;
+        sh.list[i & (kTokList - 1)] = (uint16_t)(base + 2 * p + flag);
+        ++i;
+        p += step;
+        hi = __funnelshift_l(lo, hi, 1);
+        lo <<= 1;
+        hi = __funnelshift_lc(lo, hi, step - 1);  // step <= 33
+        lo = __funnelshift_lc(0u, lo, step - 1);
+    }
+    fr.avail += acc >> 8;
+    fr.bpos += 32 * kWalkBits + e;
+    __syncwarp();
+}
+
+// Front warp: the segment's tokens, 32 per batch, to the copy warp.  `turn`
+// counts the batches of the CTA.  False (warp-uniform) if the code is corrupt.
+__device__ __forceinline__ bool read_segment(const SegIn &sg, DecShared &sh, const LzParams &P,
+                                             int lane, uint32_t &turn)
+{
+    uint32_t opos = sg.raw, cpos = sg.raw;
+    bool good = sg.raw <= sg.code_bits, ended = false;
+    Front fr;
+    fr.bpos = cpos;
+    fr.loaded = cpos >> 5;
+    fr.pre0 = sg.load(fr.loaded + lane);
+    fr.pre1 = sg.load(fr.loaded + 32 + lane);
+    fr.head = fr.avail = 0;
+    const uint32_t len_ref = 1 + P.ob + P.lb, len_lit = 1 + P.blk;
+    while (!ended) {
+        uint32_t o = 0, info = kTokEnd, x = 0;
+        if (good && opos < sg.nbits) {
+            if (fr.avail < 32)
+                find_tokens(sg, fr, sh, len_ref, len_lit, lane);
+            const uint32_t tok = sh.list[(fr.head + lane) & (kTokList - 1)];
+            const bool ref = tok & 1u;
+            const uint32_t dc = ((tok >> 1) - cpos) & 0x7fffu;
+            const uint32_t at = (cpos & 31u) + dc + 1;
+            const uint32_t q = (cpos >> 5) + (at >> 5);
+            const uint32_t body = __funnelshift_l(sh.code[(q + 1) & (kCodeRing - 1)],
+                                                  sh.code[q & (kCodeRing - 1)], at & 31u);
+            const uint32_t d = (body >> (32 - P.ob)) + 1;
+            uint32_t len = ref ? (P.lb ? (body << P.ob) >> (32 - P.lb) : 0u) + P.lmin : P.blk;
+            o = len;
+#pragma unroll
+            for (int k = 1; k < 32; k <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, o, k);
+                if (lane >= k)
+                    o += y;
+            }
+            o += opos - len;
+            const bool valid = o < sg.nbits;
+            const uint32_t room = sg.nbits - o, left = sg.code_bits - cpos;
+            if (!ref && valid && len > room)
+                len = room;
+            const uint32_t used = ref ? len_ref : 1 + len;
+            const bool bad = valid && (dc + used > left || (ref && (len > P.lmax || len > room ||
+                                                                    (P.dict == 2 && d > o))));
+            good = !__any_sync(0xffffffffu, bad);
+            if (good) {
+                const int last = 31 - __clz(__ballot_sync(0xffffffffu, valid));
+                opos = __shfl_sync(0xffffffffu, o + len, last);
+                cpos += __shfl_sync(0xffffffffu, dc + used, last);
+                fr.head += last + 1;
+                fr.avail -= last + 1;
+                info = valid ? len | (ref ? kTokRef : 0u) | kTokValid : 0u;
+                if (opos >= sg.nbits)
+                    info |= kTokEnd;
+                x = ref ? d : body;
+            }
+        }
+        ended = !good || opos >= sg.nbits;
+        if (turn >= 2)
+            read_sync(turn);
+        DecShared::Batch &bt = sh.batch[turn & 1];
+        bt.o[lane] = o;
+        bt.info[lane] = info;
+        bt.x[lane] = x;
+        __threadfence_block();
+        full_arrive(turn);
+        ++turn;
+    }
+    return good && cpos == sg.code_bits;
+}
+
+// Copy warp's view of the output.
+struct Back {
+    const uint32_t *ring;
+    const uint8_t *y;
+    uint32_t flushed;  // output words stored
+    // output word q: the dictionary before the segment (q < 0), the ring, or,
+    // for windows wider than the ring's history, the output already stored
+    __device__ __forceinline__ uint32_t word_at(int32_t q, const LzParams &P) const
+    {
+        if (q < 0)
+            return P.W >= 32 ? dict_word((uint32_t)(q + (int32_t)(P.W / 32)))
+                             : dict_word(0) >> (32 - P.W);
+        if (q + (int32_t)kDecHistory >= (int32_t)flushed)
+            return ring[(uint32_t)q & (kDecRing - 1)];
+        return bswap32(__ldcg(reinterpret_cast<const uint32_t *>(y) + q));
+    }
+    // the 32 bits at output bit s; near: they are in the ring
+    __device__ __forceinline__ uint32_t bits_at(int32_t s, const LzParams &P, bool near) const
+    {
+        const int32_t q = s >> 5;  // floor
+        uint32_t a, b;
+        if (near) {
+            a = ring[(uint32_t)q & (kDecRing - 1)];
+            b = ring[(uint32_t)(q + 1) & (kDecRing - 1)];
+        } else {
+            a = word_at(q, P);
+            b = word_at(q + 1, P);
+        }
+        return __funnelshift_l(b, a, (uint32_t)s & 31u);
+    }
+};
+
+// Copy warp: write the segment's tokens as they come, 32 at a time.
+// A literal is ready at once, a match once the bits it reads lie before the
+// first token still waiting (rounds, at most 32; 1.2 on average on the
+// bitstream stand-in).  Consecutive matches of one distance d -- the form a
+// zero run or any longer repeat takes -- would wait on one another; each
+// instead reads the period of d bits before the first of them, at its own
+// phase, so the whole run is ready together.  Every 32 completed words leave
+// with one coalesced store, and as many words ahead are cleared.
+__device__ __forceinline__ void write_segment(const SegIn &sg, DecShared &sh, const LzParams &P,
+                                              int lane, uint32_t &turn)
+{
+    uint32_t first = 0;  // the word being filled
+    for (uint32_t q = (uint32_t)lane; q < (sg.raw >> 5); q += 32) {
+        const uint32_t v = sg.load(q);
+        sh.out[q & (kDecRing - 1)] = v;
+        store_out_word(sg.y, sg.m, q, v);
+    }
+    if (sg.raw & 31u)
+        first = sg.load(sg.raw >> 5) & ~(0xffffffffu >> (sg.raw & 31u));
+    __syncwarp();
+    // the word being filled and the words a batch may reach past it
+    Back bk;
+    bk.ring = sh.out;
+    bk.y = sg.y;
+    bk.flushed = sg.raw >> 5;
+    for (uint32_t j = (uint32_t)lane; j <= kDecAhead; j += 32)
+        sh.out[(bk.flushed + j) & (kDecRing - 1)] = j == 0 ? first : 0u;
+    uint32_t opos = sg.raw;
+    for (bool more = true; more;) {
+        full_sync(turn);
+        const DecShared::Batch &bt = sh.batch[turn & 1];
+        const uint32_t o = bt.o[lane], info = bt.info[lane], x = bt.x[lane];
+        read_arrive(turn);
+        ++turn;
+        const uint32_t len = info & 63u;
+        const bool ref = (info & kTokRef) != 0;
+        more = !(info & kTokEnd);  // the same in every lane
+        uint32_t pend = __ballot_sync(0xffffffffu, (info & kTokValid) != 0);
+        if (pend == 0)
+            break;
+        const uint32_t refs = __ballot_sync(0xffffffffu, ref);
+        const int last = 31 - __clz(pend);
+        const uint32_t d = x;  // of a match
+        const uint32_t pd = __shfl_up_sync(0xffffffffu, x, 1);
+        const bool cont = lane > 0 && ((refs >> lane) & (refs >> (lane - 1)) & 1u) && pd == d;
+        const uint32_t heads = refs & ~__ballot_sync(0xffffffffu, cont);
+        const uint32_t hl = heads & (0xffffffffu >> (31 - lane));
+        const uint32_t o_r = __shfl_sync(0xffffffffu, o, hl ? 31 - __clz(hl) : 0);
+        uint32_t phase = o - o_r;
+        if (ref && phase >= d)
+            phase %= d;
+        // bits from the source up to the run's start, and where the reads end
+        const uint32_t avail = d - phase;
+        const bool wrap = ref && avail < len;  // the period starts again (avail < 32)
+        const int32_t src = (int32_t)(o_r - avail), again = (int32_t)(o_r - d);
+        const int32_t need = !ref ? INT32_MIN : (int32_t)(wrap ? o_r : o_r - avail + len);
+        // the lowest word read: past the dictionary and in the ring?
+        const int32_t low = (wrap ? again : src) >> 5;
+        const bool near = !__any_sync(
+            0xffffffffu, ref && (low < 0 || low + (int32_t)kDecHistory < (int32_t)bk.flushed));
+        int32_t front = (int32_t)opos;  // the first token waiting
+        for (;;) {
+            const bool go = ((pend >> lane) & 1u) && need <= front;
+            if (go) {
+                uint32_t v = x;
+                if (ref) {
+                    v = bk.bits_at(src, P, near);
+                    if (wrap) {
+                        v = (v & ~(0xffffffffu >> avail)) | (bk.bits_at(again, P, near) >> avail);
+                        if (d < len) {
+                            v &= ~(0xffffffffu >> d);
+                            for (uint32_t s = d; s < len; s <<= 1)
+                                v |= v >> s;
+                        }
+                    }
+                }
+                v &= ~__funnelshift_rc(0xffffffffu, 0u, len);
+                const uint32_t sft = o & 31u;
+                const uint32_t hi = v >> sft, lo = __funnelshift_l(0u, v, 32u - sft);
+                if (hi)
+                    atomicOr(sh.out + ((o >> 5) & (kDecRing - 1)), hi);
+                if (sft && lo)
+                    atomicOr(sh.out + (((o >> 5) + 1) & (kDecRing - 1)), lo);
+            }
+            pend &= ~__ballot_sync(0xffffffffu, go);
+            __syncwarp();
+            if (!pend)
+                break;
+            front = (int32_t)__shfl_sync(0xffffffffu, o, __ffs(pend) - 1);
+        }
+        opos = __shfl_sync(0xffffffffu, o + len, last);
+        if ((opos >> 5) - bk.flushed >= 32) {
+            const uint32_t j = bk.flushed + lane;
+            __stcg(reinterpret_cast<uint32_t *>(sg.y) + j, bswap32(sh.out[j & (kDecRing - 1)]));
+            sh.out[(j + kDecAhead + 1) & (kDecRing - 1)] = 0u;
+            bk.flushed += 32;
+            __syncwarp();
+        }
+    }
+    for (uint32_t j = bk.flushed + lane; 32 * j < opos; j += 32)
+        store_out_word(sg.y, sg.m, j, sh.out[j & (kDecRing - 1)]);
+    __syncwarp();
+}
+
+// One CTA of two warps per segment.  Bound by the latency of the two warps'
+// steps at a thousand segments (64 MiB in 64 KiB segments: 7 CTAs per SM) and
+// by instruction issue from about 4000 on.  64 MiB of the bitstream stand-in
+// with 1024/12/24/8: 11.9 -> 0.90 ms in 64 KiB segments, 3.35 -> 0.69 ms in
+// 16 KiB segments (before: a thread per segment); one warp doing both parts
+// took 1.19 ms, and 3.1 ms with a walk over the token flags in registers.
+__global__ void __launch_bounds__(64) k_lzss_decode(const uint8_t *__restrict__ c,
+                                                    const uint64_t *__restrict__ start,
+                                                    uint8_t *__restrict__ out, int32_t *status,
+                                                    const uint32_t *path)
+{
+    __shared__ DecShared sh;
+    if (*path != kPathWarps)
+        return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t n = *reinterpret_cast<const uint64_t *>(c);
+    const uint64_t seg = *reinterpret_cast<const uint64_t *>(c + 8);
+    const uint32_t *f = reinterpret_cast<const uint32_t *>(c + 16);
+    const LzParams P = make_params(f[0], f[1], f[2], f[3], f[4]);
+    const uint64_t count = *reinterpret_cast<const uint64_t *>(c + 40);
+    if (warp == 0)
+        for (uint32_t e = 0; e < 33; ++e)  // a walk past its stretch has left it
+            sh.exits[(kWalkBits + e) * 32 + lane] = (uint16_t)e;
+    uint32_t turn = 0;
+    for (uint64_t s = blockIdx.x; s < count; s += gridDim.x) {
+        SegIn sg;
+        sg.m = (uint32_t)(s + 1 < count ? seg : n - s * seg);
+        sg.nbits = 8 * sg.m;
+        sg.code_bits = *reinterpret_cast<const uint32_t *>(c + kLzHead + 4 * s);
+        sg.w = reinterpret_cast<const uint32_t *>(c + start[s]);
+        sg.nw = (uint32_t)(al16(((uint64_t)sg.code_bits + 7) / 8) / 4);
+        sg.y = out + s * seg;
+        sg.raw = P.dict == 2 ? (sg.nbits < P.W ? sg.nbits : P.W) : 0u;
+        if (warp == 0) {
+            if (!read_segment(sg, sh, P, lane, turn) && lane == 0)
+                set_status(status, HUFF_ERR_CORRUPT_STREAM);
+        } else {
+            write_segment(sg, sh, P, lane, turn);
+        }
+    }
+    if (warp == 0)  // the copy warp's last two reads
+        for (uint32_t t = turn < 2 ? 0 : turn - 2; t < turn; ++t)
+            read_sync(t);
 }
 
 // MSB-first bit reader over a segment's code: a 64-bit buffer refilled from
@@ -582,68 +1036,24 @@ struct CodeReader {
     }
 };
 
-// Store output word q (MSB-first bytes) of an m-byte segment output.
-__device__ __forceinline__ void store_out_word(uint8_t *y, uint64_t m, uint64_t q, uint32_t w)
-{
-    const uint64_t b = 4 * q;
-    if (b + 4 <= m) {
-        reinterpret_cast<uint32_t *>(y)[q] = bswap32(w);
-    } else {
-        for (int k = 0; k < 4; ++k)
-            if (b + k < m)
-                y[b + k] = (uint8_t)(w >> (24 - 8 * k));
-    }
-}
-
-// The bits a thread has produced so far, read back: completed words from
-// the output (or, with a ring, from the thread's ring of recent words in
-// shared memory), the pending word from its register; positions before the
-// segment from the counting-numbers dictionary.  With a ring, completed
-// words are written out four at a time with one 16-byte store.
-template <bool kRing>
+// The bits a thread has produced so far, read back from the thread's ring of
+// recent words in shared memory; the word being filled is in a register.
+// Completed words are written out four at a time with one 16-byte store.
 struct OutBits {
     uint8_t *y;      // the segment's output (16-byte aligned)
     uint32_t m;      // its bytes (at most 16 MiB)
-    uint32_t W;
-    uint32_t *ring;  // kRing: kDecRing words, word q at q mod kDecRing
+    uint32_t *ring;  // kThrRing words, word q at q mod kThrRing
     uint32_t pend;   // bits of the word being filled, left-aligned
     uint32_t npend;  // their count
     uint32_t pos;    // bits produced (< 2^27)
-    __device__ __forceinline__ uint32_t word_at(int32_t q) const  // output word q (may be < 0)
+    __device__ __forceinline__ uint32_t word_at(uint32_t q) const
     {
-        if (q < 0) {  // the dictionary: virtual word q + W/32 (W >= 32 here)
-            return dict_word((uint32_t)(q + (int32_t)(W / 32)));
-        }
-        if ((uint32_t)q == (pos >> 5))
-            return pend;
-        if ((uint32_t)q > (pos >> 5))
-            return 0u;
-        if (kRing)
-            return ring[(uint32_t)q & (kDecRing - 1)];
-        return bswap32(__ldcg(reinterpret_cast<const uint32_t *>(y) + q));
+        return q == (pos >> 5) ? pend : q > (pos >> 5) ? 0u : ring[q & (kThrRing - 1)];
     }
-    // the 32 bits at output bit s (s may be negative: the dictionary)
-    __device__ __forceinline__ uint32_t bits_at(int32_t s) const
+    // the 32 bits at output bit s
+    __device__ __forceinline__ uint32_t bits_at(uint32_t s) const
     {
-        if (W < 32 && s < 0) {  // narrow dictionary, bit by bit
-            uint32_t out = 0;
-            for (int i = 0; i < 32; ++i) {
-                const int32_t t = s + i;
-                uint32_t b;
-                if (t < 0) {
-                    const uint32_t j = (uint32_t)(t + (int32_t)W);
-                    b = (((uint32_t)(j >> 3) & 255) >> (7 - (j & 7))) & 1;
-                } else {
-                    b = (word_at(t >> 5) >> (31 - (t & 31))) & 1;
-                }
-                out = (out << 1) | b;
-            }
-            return out;
-        }
-        const int32_t q = s >> 5;  // floor
-        const uint32_t sh = (uint32_t)(s & 31);
-        const uint32_t a = word_at(q), b = word_at(q + 1);
-        return sh ? __funnelshift_l(b, a, sh) : a;
+        return __funnelshift_l(word_at((s >> 5) + 1), word_at(s >> 5), s & 31u);
     }
     // append the top k (1..32) bits of v
     __device__ __forceinline__ void put(uint32_t v, uint32_t k)
@@ -663,33 +1073,25 @@ struct OutBits {
     }
     __device__ __forceinline__ void complete(uint32_t q, uint32_t w) const
     {
-        if (!kRing) {
-            if (4 * q + 4 <= m)
-                __stcg(reinterpret_cast<uint32_t *>(y) + q, bswap32(w));
-            else
-                store_out_word(y, m, q, w);
-            return;
-        }
-        ring[(uint32_t)q & (kDecRing - 1)] = w;
+        ring[q & (kThrRing - 1)] = w;
         if ((q & 3) == 3) {  // a whole 16-byte group
             const uint32_t g = q >> 2;
             if (16 * g + 16 <= m) {
-                const uint32_t r = (uint32_t)(q - 3) & (kDecRing - 1);
+                const uint32_t r = (q - 3) & (kThrRing - 1);
                 *reinterpret_cast<uint4 *>(y + 16 * g) =
                     make_uint4(bswap32(ring[r]), bswap32(ring[r + 1]), bswap32(ring[r + 2]),
                                bswap32(ring[r + 3]));
             } else {
                 for (uint32_t j = q - 3; j <= q; ++j)
-                    store_out_word(y, m, j, ring[(uint32_t)j & (kDecRing - 1)]);
+                    store_out_word(y, m, j, ring[j & (kThrRing - 1)]);
             }
         }
     }
     __device__ __forceinline__ void finish() const
     {
         const uint32_t q = pos >> 5;  // the word being filled
-        if (kRing)  // completed words of the last, unfinished group
-            for (uint32_t j = q & ~3u; j < q; ++j)
-                store_out_word(y, m, j, ring[(uint32_t)j & (kDecRing - 1)]);
+        for (uint32_t j = q & ~3u; j < q; ++j)  // completed words of the last, unfinished group
+            store_out_word(y, m, j, ring[j & (kThrRing - 1)]);
         if (npend)
             store_out_word(y, m, q, pend);
     }
@@ -720,7 +1122,7 @@ struct CodeRing {
     __device__ __forceinline__ void top_up(const uint32_t *w, uint32_t word)
     {
         while (fetched < (word >> 2) + kLzInCells && fetched < ncells) {
-            lz_cp_async16(col + (fetched & (kLzInCells - 1)) * (kLzDecThreads * 16), w + 4 * fetched);
+            lz_cp_async16(col + (fetched & (kLzInCells - 1)) * (kThrBlock * 16), w + 4 * fetched);
             lz_cp_commit();
             ++fetched;
         }
@@ -736,7 +1138,7 @@ struct CodeRing {
             lz_cp_wait<0>();
         else
             lz_cp_wait<kLzInFlight>();
-        return lds(col + ((word >> 2) & (kLzInCells - 1)) * (kLzDecThreads * 16) + (word & 3u) * 4);
+        return lds(col + ((word >> 2) & (kLzInCells - 1)) * (kThrBlock * 16) + (word & 3u) * 4);
     }
 };
 
@@ -749,7 +1151,7 @@ struct CodeRing {
 // diverge: both the match and the literal are formed and the token
 // selects.  False (and the caller's status) only for a length field above
 // the longest match.
-__device__ __forceinline__ bool decode_fast(CodeReader &rd, OutBits<true> &ob, const LzParams &P,
+__device__ __forceinline__ bool decode_fast(CodeReader &rd, OutBits &ob, const LzParams &P,
                                             uint32_t nbits, uint32_t in_col)
 {
     CodeRing rg;
@@ -774,7 +1176,7 @@ __device__ __forceinline__ bool decode_fast(CodeReader &rd, OutBits<true> &ob, c
         // the output and the ring; read whether or not the token is a match)
         const uint32_t src = ob.pos - d;
         const uint32_t q = src >> 5, cur = ob.pos >> 5;
-        const uint32_t wa = ob.ring[q & (kDecRing - 1)], wb = ob.ring[(q + 1) & (kDecRing - 1)];
+        const uint32_t wa = ob.ring[q & (kThrRing - 1)], wb = ob.ring[(q + 1) & (kThrRing - 1)];
         const uint32_t a = q == cur ? ob.pend : wa;
         const uint32_t b = q + 1 == cur ? ob.pend : (q + 1 > cur ? 0u : wb);
         uint32_t v = __funnelshift_l(b, a, src & 31u);
@@ -809,23 +1211,18 @@ __device__ __forceinline__ bool decode_fast(CodeReader &rd, OutBits<true> &ob, c
 }
 
 // Decode one segment's tokens; false if the code is corrupt.
-template <bool kRing>
-__device__ __forceinline__ bool decode_segment(CodeReader &rd, OutBits<kRing> &ob, const LzParams &P,
-                                               uint32_t nbits, uint32_t in_col = 0)
+__device__ __forceinline__ bool decode_segment(CodeReader &rd, OutBits &ob, const LzParams &P,
+                                               uint32_t nbits, uint32_t in_col)
 {
-    if (P.dict == 2) {
-        const uint32_t raw = nbits < P.W ? nbits : P.W;
-        while (ob.pos < raw) {
-            const uint32_t k = raw - ob.pos < 32 ? (uint32_t)(raw - ob.pos) : 32u;
-            if (rd.pos + k > rd.nbits)
-                return false;
-            ob.put(rd.get(k) << (32 - k), k);
-        }
-    }
-    if constexpr (kRing) {
-        if (P.dict == 2 && P.blk <= 31 && !decode_fast(rd, ob, P, nbits, in_col))
+    const uint32_t raw = nbits < P.W ? nbits : P.W;
+    while (ob.pos < raw) {
+        const uint32_t k = raw - ob.pos < 32 ? raw - ob.pos : 32u;
+        if (rd.pos + k > rd.nbits)
             return false;
+        ob.put(rd.get(k) << (32 - k), k);
     }
+    if (!decode_fast(rd, ob, P, nbits, in_col))
+        return false;
     while (ob.pos < nbits) {
         if (rd.pos >= rd.nbits)
             return false;
@@ -835,9 +1232,9 @@ __device__ __forceinline__ bool decode_segment(CodeReader &rd, OutBits<kRing> &o
                 return false;
             const uint32_t d = rd.get(P.ob) + 1;
             const uint32_t len = rd.get(P.lb) + P.lmin;
-            if (len > P.lmax || len > r || (P.dict == 2 && d > ob.pos))
+            if (len > P.lmax || len > r || d > ob.pos)
                 return false;
-            uint32_t v = ob.bits_at((int32_t)ob.pos - (int32_t)d);
+            uint32_t v = ob.bits_at(ob.pos - d);
             if (d < len) {  // the source runs into these bits: period d
                 v &= ~(0xffffffffu >> d);
                 for (uint32_t sh = d; sh < len; sh <<= 1)
@@ -854,20 +1251,16 @@ __device__ __forceinline__ bool decode_segment(CodeReader &rd, OutBits<kRing> &o
     return rd.pos == rd.nbits;
 }
 
-// One thread per segment.  Windows of up to kDecRingMaxWindow bits keep the
-// thread's recent output words in a shared-memory ring (the matches' source
-// words are read there, not back through L2, and output leaves in 16-byte
-// stores); wider windows read their sources back from the output.
-__global__ void __launch_bounds__(kLzDecThreads) k_lzss_decode(const uint8_t *__restrict__ c,
-                                                               const uint64_t *__restrict__ start,
-                                                               uint8_t *__restrict__ out,
-                                                               int32_t *status, const uint32_t *ok)
+// One thread per segment, for very many segments (see threads_better).
+__global__ void __launch_bounds__(kThrBlock)
+    k_lzss_decode_threads(const uint8_t *__restrict__ c, const uint64_t *__restrict__ start,
+                          uint8_t *__restrict__ out, int32_t *status, const uint32_t *path)
 {
-    // ring of thread t at t * (kDecRing + 1): the odd stride spreads the
+    // ring of thread t at t * (kThrRing + 1): the odd stride spreads the
     // threads' equal ring positions over the banks
-    __shared__ uint32_t rings[kLzDecThreads * (kDecRing + 1)];
-    __shared__ __align__(16) uint4 in_ring[kLzInCells * kLzDecThreads];  // [cell][thread]
-    if (!*ok || chain_failed(status))
+    __shared__ uint32_t rings[kThrBlock * (kThrRing + 1)];
+    __shared__ __align__(16) uint4 in_ring[kLzInCells * kThrBlock];  // [cell][thread]
+    if (*path != kPathThreads)
         return;
     const uint32_t in_col = smem_u32(in_ring) + threadIdx.x * 16;
     const uint64_t n = *reinterpret_cast<const uint64_t *>(c);
@@ -875,39 +1268,21 @@ __global__ void __launch_bounds__(kLzDecThreads) k_lzss_decode(const uint8_t *__
     const uint32_t *f = reinterpret_cast<const uint32_t *>(c + 16);
     const LzParams P = make_params(f[0], f[1], f[2], f[3], f[4]);
     const uint64_t count = *reinterpret_cast<const uint64_t *>(c + 40);
-    const bool use_ring = P.W >= 32 && P.W <= kDecRingMaxWindow;
     for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s < count;
          s += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t m = s + 1 < count ? seg : n - s * seg;
         CodeReader rd;
         rd.init(c + start[s], *reinterpret_cast<const uint32_t *>(c + kLzHead + 4 * s));
-        bool good;
-        if (use_ring) {
-            OutBits<true> ob;
-            ob.y = out + s * seg;
-            ob.m = (uint32_t)m;
-            ob.W = P.W;
-            ob.ring = rings + threadIdx.x * (kDecRing + 1);
-            ob.pend = 0;
-            ob.npend = 0;
-            ob.pos = 0;
-            good = decode_segment(rd, ob, P, (uint32_t)(8 * m), in_col);
-            if (good)
-                ob.finish();
-        } else {
-            OutBits<false> ob;
-            ob.y = out + s * seg;
-            ob.m = (uint32_t)m;
-            ob.W = P.W;
-            ob.ring = nullptr;
-            ob.pend = 0;
-            ob.npend = 0;
-            ob.pos = 0;
-            good = decode_segment(rd, ob, P, (uint32_t)(8 * m));
-            if (good)
-                ob.finish();
-        }
-        if (!good)
+        OutBits ob;
+        ob.y = out + s * seg;
+        ob.m = (uint32_t)m;
+        ob.ring = rings + threadIdx.x * (kThrRing + 1);
+        ob.pend = 0;
+        ob.npend = 0;
+        ob.pos = 0;
+        if (decode_segment(rd, ob, P, (uint32_t)(8 * m), in_col))
+            ob.finish();
+        else
             set_status(status, HUFF_ERR_CORRUPT_STREAM);
     }
 }
@@ -1022,22 +1397,23 @@ huff_status_t huff_lzss_decompress(const uint8_t *d_in, uint64_t in_bytes, uint8
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     k_lzss_set<<<1, 1, 0, s>>>(d_status, reinterpret_cast<unsigned long long *>(d_n), 0);
     const uint64_t max_count = in_bytes > kLzHead ? (in_bytes - kLzHead) / 4 : 0;
-    uint32_t *ok = static_cast<uint32_t *>(d_ws);
-    uint64_t *start = reinterpret_cast<uint64_t *>(static_cast<uint8_t *>(d_ws) + 16);
-    k_lzss_dlayout<<<1, kScanBlock, 0, s>>>(d_in, in_bytes, out_cap, start, max_count,
-                                            reinterpret_cast<unsigned long long *>(d_n), d_status,
-                                            ok);
     const int sms = device_sm_count();
     if (sms < 1)
         return HUFF_ERR_CUDA;
-    // one thread per segment; the count is only known on the device, so
-    // bound the grid by the table size
-    uint64_t grid = (max_count + kLzDecThreads - 1) / kLzDecThreads;
+    uint32_t *path = static_cast<uint32_t *>(d_ws);
+    uint64_t *start = reinterpret_cast<uint64_t *>(static_cast<uint8_t *>(d_ws) + 16);
+    k_lzss_dlayout<<<1, kScanBlock, 0, s>>>(d_in, in_bytes, out_cap, start, max_count,
+                                            reinterpret_cast<unsigned long long *>(d_n), d_status,
+                                            path, (uint32_t)sms);
+    // the count is only known on the device, so bound the grids by the table
+    // size; the decoder that k_lzss_dlayout did not choose returns at once
+    uint64_t grid = max_count;
     if (grid > (uint64_t)sms * 32)
         grid = (uint64_t)sms * 32;
     if (grid < 1)
         grid = 1;
-    k_lzss_decode<<<(unsigned)grid, kLzDecThreads, 0, s>>>(d_in, start, d_out, d_status, ok);
+    k_lzss_decode<<<(unsigned)grid, 64, 0, s>>>(d_in, start, d_out, d_status, path);
+    k_lzss_decode_threads<<<(unsigned)grid, kThrBlock, 0, s>>>(d_in, start, d_out, d_status, path);
     return cudaGetLastError() == cudaSuccess ? HUFF_OK : HUFF_ERR_CUDA;
 }
 
