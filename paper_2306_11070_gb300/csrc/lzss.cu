@@ -20,18 +20,11 @@
 //    segment's code packed MSB first into bytes from a 16-byte boundary,
 //    zero padded to the next one.
 //
-// Compression: one warp per segment.  For each token the 32 lanes search
-// the window together: lane j tries distances j + 1, j + 33, j + 65, ...;
-// their sources all start at the same bit offset within a word, so each
-// candidate costs one window word, a funnel shift, an XOR with the 32
-// look-ahead bits (its bits past the longest allowed match forced to 1, so
-// the count of leading zeros is already capped) and a count of leading
-// zeros; one warp max over (length, -distance) keys picks the token, and a
-// match shorter than Lmin then reads as a literal.  For windows of 64 to
-// 16384 bits the words come from a per-warp ring in shared memory, filled 32
-// words at a time as the position advances and stored twice (at i and
-// i + R), so a token's candidates read one straight run of words, no wrap.  Every lane keeps the same
-// 64-bit output accumulator and lane 0 stores the completed words into the
+// Compression: one warp per segment.  For each token the 32 lanes search the
+// window together: for windows of 64 to 16384 bits all distances bit-parallel
+// (a lane's 32-bit mask holds 32 sources) from a ring in shared memory, other
+// windows a distance at a time through L1.  Every lane keeps the same 64-bit
+// output accumulator and lane 0 stores the completed words into the
 // segment's worst-case slot of the workspace; a one-CTA scan then lays out
 // the header and length table and a gather moves every code into place.
 // Decompression: a one-CTA scan checks the header and table and finds every
@@ -54,8 +47,6 @@ constexpr int kLzBlock = 32 * kLzWarps;
 constexpr int kScanBlock = 1024;
 constexpr uint32_t kMaxWindow = 65536;
 constexpr uint32_t kRingMaxWindow = 16384;  // the shared-memory window ring
-// dynamic shared memory of the largest ring (W = 16384: 1024 words, twice, per warp)
-constexpr size_t kMaxRingSmem = (size_t)kLzWarps * 2 * 1024 * 4;
 constexpr uint64_t kMaxSegment = 1ull << 24;
 constexpr int kThrBlock = 32;             // thread-per-segment decompress: one warp per CTA
 constexpr uint32_t kThrRing = 128;        // output words kept per thread (a power of two)
@@ -211,12 +202,14 @@ struct WarpBits {
     }
 };
 
-// Ring words per warp (R, a power of two): the window's W/32 words, the
-// look-ahead's two and a batch of 32 loaded at once.  Stored twice.
+// Ring words per warp (R, a power of two): the window's W/32 words, 34 ahead
+// of the position and a batch of 128 loaded at once.  Stored twice, at i and
+// i + R, so that neighbouring words are read at neighbouring addresses.
+constexpr uint32_t kRingBatch = 128;
 __host__ __device__ __forceinline__ uint32_t ring_words(uint32_t W)
 {
     uint32_t r = 64;
-    while (r < W / 32 + 36)
+    while (r < W / 32 + 36 + kRingBatch)
         r <<= 1;
     return r;
 }
@@ -225,44 +218,260 @@ __host__ __device__ __forceinline__ bool ring_ok(const LzParams &P)
     return P.W >= 64 && P.W <= kRingMaxWindow;
 }
 
-// 2^16 from the constant bank: search_run forms its key by one multiply-add
-// on the FMA pipe (a visible power of two would become a shift and an add on
-// the ALU pipe, which the candidate loop already fills)
-static __constant__ uint32_t kKeyScale = 65536u;
-
-// The best key over this lane's candidates from a straight run of window
-// words: w points at the word after the one where candidate 0's source
-// begins; candidate k's source begins k words lower.
-// key = (capped match length << 16) - 32 k; the caller adds 65535 - lane.
-template <int NK>
-__device__ __forceinline__ int32_t search_run(const uint32_t *w, uint32_t nk, uint32_t sh, uint32_t X,
-                                              uint32_t cap)
+// The longest match of lo..maxlen bits over 1024 distances at once, the
+// smallest distance among equally long ones.  Lane j holds 32 sources, the
+// The longest match of lo..maxlen bits over 1024 distances at once, the
+// smallest distance among equally long ones.  Lane j holds 32 sources, the
+// bits a:b (64 bits of the window from bit P - 32 j - 32 of position P); bit
+// 31 - i of a mask stands for the source that starts i bits on.  After t
+// steps a mask's bits are the sources that agree with the first t bits of the
+// look-ahead X: step t ands it with the window shifted by t, complemented
+// where X's bit is 0.  About four instructions a step for 1024 candidates,
+// against six for 32 when each candidate is shifted into place and compared
+// by itself.  One vote after the first 4 G0 steps (G0 = Lmin / 4, straight-line)
+// ends most searches; else every lane finishes its steps and a warp maximum
+// picks the match.  Returns its length << 10 | (1023 - (d - 1)) with d counted
+// within the 1024, 0 for none of lo..maxlen bits.
+__device__ __forceinline__ uint32_t sign_byte3(uint32_t v)  // the top bit, 32 times
 {
-    int32_t best = INT32_MIN;
-    uint32_t hiw = w[0];
-    if (NK > 0) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, 0xbbbb;" : "=r"(r) : "r"(v));
+    return r;
+}
+__device__ __forceinline__ uint32_t sign_byte2(uint32_t v)  // bit 23
+{
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, 0xaaaa;" : "=r"(r) : "r"(v));
+    return r;
+}
+__device__ __forceinline__ uint32_t sign_byte1(uint32_t v)  // bit 15
+{
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, 0x9999;" : "=r"(r) : "r"(v));
+    return r;
+}
+__device__ __forceinline__ uint32_t sign_byte0(uint32_t v)  // bit 7
+{
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, 0x8888;" : "=r"(r) : "r"(v));
+    return r;
+}
+template <int G0>
+__device__ __forceinline__ uint32_t search_masks(uint32_t a, uint32_t b, uint32_t m, uint32_t X,
+                                                 uint32_t lo, uint32_t maxlen, int lane)
+{
+    uint32_t nx[8];  // ~X shifted by 0..7: their bytes' top bits are its bits
 #pragma unroll
-        for (int k = 0; k < NK; ++k) {
-            const uint32_t low = w[-(k + 1)];
-            const uint32_t src = __funnelshift_l(hiw, low, sh);
-            hiw = low;
-            const int32_t key = (int32_t)imad((uint32_t)__clz((src ^ X) | cap), kKeyScale,
-                                              (uint32_t)(-32 * k));
-            best = key > best ? key : best;
-        }
-    } else {
-        for (uint32_t k = 0; k < nk; ++k) {
-            const uint32_t low = w[-(int)(k + 1)];
-            const uint32_t src = __funnelshift_l(hiw, low, sh);
-            hiw = low;
-            const int32_t key = (int32_t)imad((uint32_t)__clz((src ^ X) | cap), kKeyScale,
-                                              0u - 32u * k);
-            best = key > best ? key : best;
+    for (int i = 0; i < 8; ++i)
+        nx[i] = ~X << i;
+    auto step = [&](int t, uint32_t c) {
+        const uint32_t v = nx[t & 7];
+        const uint32_t no = t < 8    ? sign_byte3(v)
+                            : t < 16 ? sign_byte2(v)
+                            : t < 24 ? sign_byte1(v)
+                                     : sign_byte0(v);
+        return c & (__funnelshift_l(b, a, t) ^ no);
+    };
+#pragma unroll
+    for (int t = 0; t < 4 * G0; ++t)
+        m = step(t, m);
+    if (G0 > 0 && !__any_sync(0xffffffffu, m != 0))
+        return 0;
+    uint32_t len = m ? 4 * G0 : 0, best = m;
+#pragma unroll
+    for (int t = 4 * G0; t < 32; ++t) {
+        if ((t & 3) == 0 && (uint32_t)t >= maxlen)
+            break;
+        m = step(t, m);
+        if (m && (uint32_t)t < maxlen) {
+            best = m;
+            len = t + 1;
         }
     }
-    return best;
+    const uint32_t key =
+        len >= lo && len <= maxlen ? len << 10 | (1024u - 32u * lane - __ffs(best)) : 0u;
+    return __reduce_max_sync(0xffffffffu, key);
 }
 
+// Output bits of one warp, the same in every lane: the pending n < 32 bits
+// left-aligned in `top`, zeros below; lane 0 stores each completed word.
+struct WarpOut {
+    uint32_t top, n, word;
+    uint32_t *out;
+    // the top k (1..32) bits of v, zeros below them
+    __device__ __forceinline__ void put(uint32_t v, uint32_t k, int lane)
+    {
+        const uint32_t t = top | (v >> n);
+        const uint32_t rest = __funnelshift_lc(0u, v, 32u - n);  // 0 at n = 0
+        n += k;
+        if (n >= 32) {
+            if (lane == 0)
+                out[word] = bswap32(t);
+            ++word;
+            n -= 32;
+            top = rest;
+        } else {
+            top = t;
+        }
+    }
+};
+
+// Windows of 64..16384 bits: one warp per segment, the window in a ring in
+// shared memory.  Bound by the latency of one token's steps (a warp alone
+// issues about every 4.5 cycles; at 64 KiB segments an SM holds 7) and, from
+// some 4000 segments on, by instruction issue.  64 MiB of the bitstream
+// stand-in with 1024/12/24/8: 19.1 -> 4.4 ms in 64 KiB segments, 13.1 -> 2.4
+// ms in 16 KiB, 10.4 -> 1.9 ms in 4 KiB (before: one candidate a lane and
+// step); W = 4096 in 16 KiB segments 40.9 -> 4.6 ms.  With Lmin's steps not
+// straight-line (a run-time bound on each) it took 7.0 ms.  Where the bits ahead repeat the bit
+// before them (a zero run), distance 1 gives the longest match there is and
+// no distance is smaller: all the tokens of the run that the ring shows (up
+// to 1024 bits) are written at once, as the repeating words they form.
+template <int G0>
+__global__ void __launch_bounds__(32)
+    k_lzss_compress_ring(const uint8_t *__restrict__ in, uint64_t n, uint64_t seg, LzParams P,
+                         uint8_t *__restrict__ slots, uint32_t *__restrict__ bits_out,
+                         const int32_t *status)
+{
+    if (chain_failed(status))
+        return;
+    extern __shared__ uint32_t ring[];
+    const int lane = threadIdx.x;
+    const uint64_t count = n ? (n + seg - 1) / seg : 0;
+    const uint64_t sbytes = slot_bytes(seg, P);
+    const uint32_t R = ring_words(P.W), dwords = P.W / 32, passes = (P.W + 1023) / 1024;
+    const uint32_t len_ref = 1 + P.ob + P.lb, run_bits = 32 - P.lmax;
+    const uint32_t lit_mask = P.blk < 31 ? ~(0x7fffffffu >> P.blk) : ~0u;  // of a literal's token
+    // the token of a run: distance 1, the longest length; and its repetition
+    uint64_t run_rep = (uint64_t)(0x80000000u | ((P.lmax - P.lmin) << (32 - len_ref))) << 32;
+    for (uint32_t k = len_ref; k < 64; k <<= 1)
+        run_rep |= run_rep >> k;
+    // x / len_ref and x / lmax as x * inv >> 20: exact up to 2^20 / 32
+    const uint32_t inv_ref = ((1u << 20) + len_ref - 1) / len_ref;
+    const uint32_t inv_max = ((1u << 20) + P.lmax - 1) / P.lmax;
+    for (uint64_t s = blockIdx.x; s < count; s += gridDim.x) {
+        const uint8_t *x = in + s * seg;
+        const uint32_t m = (uint32_t)(s + 1 < count ? seg : n - s * seg);
+        const uint32_t nbits = 8 * m;
+        WarpOut out;
+        out.top = out.n = out.word = 0;
+        out.out = reinterpret_cast<uint32_t *>(slots + s * sbytes);
+        uint32_t p = 0;
+        if (P.dict == 2) {  // the first W bits as they are
+            const uint32_t raw = nbits < P.W ? nbits : P.W;
+            for (uint32_t q = lane; q < raw / 32; q += 32)
+                out.out[q] = bswap32(seg_word(x, m, q));
+            out.word = raw / 32;
+            out.n = raw & 31u;
+            out.top = out.n ? seg_word(x, m, raw / 32) & ~(0xffffffffu >> out.n) : 0u;
+            p = raw;
+        }
+        // ring: words [hw - R, hw) of "dictionary ++ segment" (bit v = W + p);
+        // pre: the next batch, loaded ahead
+        uint32_t hw = p >> 5;
+        uint32_t pre[kRingBatch / 32];
+#pragma unroll
+        for (int k = 0; k < (int)kRingBatch / 32; ++k)
+            pre[k] = vword(x, m, dwords, hw + 32 * k + lane);
+        while (p < nbits) {
+            const uint32_t v = P.W + p, q = v >> 5, sh = v & 31u;
+            if (hw < q + 34) {
+                do {
+#pragma unroll
+                    for (int k = 0; k < (int)kRingBatch / 32; ++k) {
+                        const uint32_t i = (hw + 32 * k + lane) & (R - 1);
+                        ring[i] = pre[k];
+                        ring[i + R] = pre[k];
+                        pre[k] = vword(x, m, dwords, hw + kRingBatch + 32 * k + lane);
+                    }
+                    hw += kRingBatch;
+                } while (hw < q + 34);
+                __syncwarp();
+            }
+            const uint32_t r = nbits - p;
+            const uint32_t *const cur = ring + (q & (R - 1));
+            const uint32_t *const win = ring + ((q - lane - 1) & (R - 1));
+            const uint32_t c0 = cur[0], X = __funnelshift_l(cur[1], c0, sh);  // the look-ahead bits
+            const uint32_t w0 = win[0], w1 = win[1], w2 = win[2];
+            // all ones or zeros, as the bit before the position
+            const uint32_t prev = 0u - (__funnelshift_l(c0, cur[R - 1], sh) & 1u);
+            if (((X ^ prev) >> run_bits) == 0 && r >= P.lmax) {
+                const uint32_t *const z = ring + ((q + lane) & (R - 1));
+                const uint32_t diff = __funnelshift_l(z[1], z[0], sh) ^ prev;
+                const uint32_t stop = __ballot_sync(0xffffffffu, diff != 0);
+                const int f = stop ? __ffs(stop) - 1 : 31;
+                uint32_t run = 32 * f + __shfl_sync(0xffffffffu, (uint32_t)__clz(diff), f);
+                run = run < r ? run : r;
+                const uint32_t k = run * inv_max >> 20;  // tokens, 1..1024
+                p += k * P.lmax;
+                const uint32_t total = out.n + k * len_ref, full = total >> 5;
+                for (uint32_t i = lane; i <= full; i += 32) {
+                    // word i of the pending bits and the repeated token
+                    const uint32_t o = 32 * i - out.n;
+                    uint32_t w = (uint32_t)(run_rep << (o - (o * inv_ref >> 20) * len_ref) >> 32);
+                    if (i == 0)
+                        w = out.top | (uint32_t)(run_rep >> 32 >> out.n);
+                    if (i < full)
+                        out.out[out.word + i] = bswap32(w);
+                    else
+                        out.top = w;
+                }
+                out.top = __shfl_sync(0xffffffffu, out.top, full & 31u);
+                out.word += full;
+                out.n = total & 31u;
+                out.top &= ~__funnelshift_rc(0xffffffffu, 0u, out.n);
+                continue;
+            }
+            const uint32_t maxlen = r < P.lmax ? r : P.lmax;
+            uint32_t len = 0, dm1 = 0;
+            if (maxlen >= P.lmin) {
+                uint32_t key = search_masks<G0>(__funnelshift_l(w1, w0, sh), __funnelshift_l(w2, w1, sh),
+                                            lane < (int)dwords ? 0xffffffffu : 0u, X, P.lmin, maxlen,
+                                            lane);
+                if (key) {
+                    len = key >> 10;
+                    dm1 = 1023 - (key & 1023u);
+                }
+                for (uint32_t k = 1; k < passes && len < maxlen; ++k) {
+                    const uint32_t *const w = ring + ((q - 32 * k - lane - 1) & (R - 1));
+                    key = search_masks<G0>(__funnelshift_l(w[1], w[0], sh),
+                                       __funnelshift_l(w[2], w[1], sh), 0xffffffffu, X,
+                                       len ? len + 1 : P.lmin, maxlen, lane);
+                    if (key) {  // longer than any nearer one
+                        len = key >> 10;
+                        dm1 = 1024 * k + 1023 - (key & 1023u);
+                    }
+                }
+            }
+            if (len) {  // a match: 1, d - 1, l - Lmin
+                out.put(0x80000000u | (dm1 << (31 - P.ob)) |
+                            (P.lb ? (len - P.lmin) << (32 - len_ref) : 0u),
+                        len_ref, lane);
+                p += len;
+            } else if (r >= P.blk && P.blk < 32) {  // a literal: 0, the next B bits
+                out.put((X >> 1) & lit_mask, P.blk + 1, lane);
+                p += P.blk;
+            } else {  // a literal of min(B, r) bits
+                const uint32_t k = r < P.blk ? r : P.blk;
+                out.put(0u, 1, lane);
+                out.put(X & ~__funnelshift_rc(0xffffffffu, 0u, k), k, lane);
+                p += k;
+            }
+        }
+        if (lane == 0) {  // the last word and zeros up to the slot's 16-byte boundary
+            uint32_t w = out.word;
+            if (out.n)
+                out.out[w++] = bswap32(out.top);
+            while (w & 3u)
+                out.out[w++] = 0u;
+            bits_out[s] = out.word * 32 + out.n;
+        }
+        __syncwarp();
+    }
+}
+
+// Every other window: the words through L1, each lane trying its own distances
+// one by one.
 __global__ void __launch_bounds__(kLzBlock)
     k_lzss_compress(const uint8_t *__restrict__ in, uint64_t n, uint64_t seg, LzParams P,
                     uint8_t *__restrict__ slots, uint32_t *__restrict__ bits_out,
@@ -270,13 +479,9 @@ __global__ void __launch_bounds__(kLzBlock)
 {
     if (chain_failed(status))
         return;
-    extern __shared__ uint32_t lz_ring[];
     const int lane = threadIdx.x & 31;
     const uint64_t count = n ? (n + seg - 1) / seg : 0;
     const uint64_t sbytes = slot_bytes(seg, P);
-    const bool use_ring = ring_ok(P);
-    const uint32_t R = ring_words(P.W);
-    uint32_t *ring = lz_ring + (threadIdx.x >> 5) * 2 * R;  // used only when use_ring
     const uint64_t nwarps = (uint64_t)gridDim.x * kLzWarps;
     for (uint64_t s = (uint64_t)blockIdx.x * kLzWarps + (threadIdx.x >> 5); s < count; s += nwarps) {
         const uint8_t *x = in + s * seg;
@@ -299,40 +504,12 @@ __global__ void __launch_bounds__(kLzBlock)
         const uint64_t vbase = P.W;  // virtual bit of the segment's bit 0
         const uint32_t dwords = P.W >= 32 ? P.W / 32 : 0;
         const uint32_t nk = P.W >= 32 ? P.W / 32 : 1;  // candidates per lane
-        // ring: words [hw - R, hw) of the virtual string are held (twice)
-        uint64_t hw = vbase + p >= P.W + 64 ? ((vbase + p - P.W) >> 5) - 2 : 0;
         while (p < nbits) {
             const uint64_t r = nbits - p;
             const uint32_t maxlen = r < P.lmax ? (uint32_t)r : P.lmax;
-            uint32_t X;  // the 32 look-ahead bits
-            if (use_ring) {
-                const uint64_t need = ((vbase + p) >> 5) + 2;
-                while (hw < need) {  // warp-uniform: 32 words at a time
-                    const uint32_t v = vword(x, m, dwords, hw + lane);
-                    const uint32_t i = (uint32_t)(hw + lane) & (R - 1);
-                    ring[i] = v;
-                    ring[i + R] = v;
-                    hw += 32;
-                    __syncwarp();
-                }
-                const uint64_t q = (vbase + p) >> 5;
-                X = __funnelshift_l(ring[(uint32_t)(q + 1) & (R - 1)], ring[(uint32_t)q & (R - 1)],
-                                    (uint32_t)((vbase + p) & 31));
-            } else {
-                X = vbits(x, m, P.W, vbase + p);
-            }
+            const uint32_t X = vbits(x, m, P.W, vbase + p);  // the 32 look-ahead bits
             uint32_t key = 0;
-            if (maxlen >= P.lmin && use_ring && (P.dict == 1 || p >= P.W)) {
-                // every distance 1..W is allowed: the ring's straight run
-                const uint64_t v0 = vbase + p - (uint64_t)lane - 1;
-                const uint32_t *w = ring + ((uint32_t)((v0 >> 5) + 1) & (R - 1)) + R;
-                const uint32_t cap = maxlen >= 32 ? 0u : 0x80000000u >> maxlen;
-                const int32_t best = nk == 32 ? search_run<32>(w, nk, (uint32_t)(v0 & 31), X, cap)
-                                              : search_run<0>(w, nk, (uint32_t)(v0 & 31), X, cap);
-                key = __reduce_max_sync(0xffffffffu, (uint32_t)(best + (int32_t)(65535 - lane)));
-                if ((key >> 16) < P.lmin)
-                    key = 0;
-            } else if (maxlen >= P.lmin) {
+            if (maxlen >= P.lmin) {
                 // lane's sources: virtual bit v_k = vbase + p - (lane + 1) - 32 k
                 const uint64_t v0 = vbase + p - (uint64_t)lane - 1;
                 if (P.W >= 32) {
@@ -1356,17 +1533,29 @@ huff_status_t huff_lzss_compress(const uint8_t *d_in, uint64_t n, uint64_t segme
     if (sms < 1)
         return HUFF_ERR_CUDA;
     if (count) {
-        const size_t smem = ring_ok(P) ? (size_t)kLzWarps * 2 * ring_words(P.W) * 4 : 0;
-        static KernelSetup setup;
-        int per_sm = 0;
-        if (kernel_setup(setup, (const void *)k_lzss_compress, kLzBlock, kMaxRingSmem, &per_sm) !=
-            cudaSuccess)
-            return HUFF_ERR_CUDA;
-        uint64_t grid = (count + kLzWarps - 1) / kLzWarps;
-        if (grid > (uint64_t)sms * 64)
-            grid = (uint64_t)sms * 64;
-        k_lzss_compress<<<(unsigned)grid, kLzBlock, smem, s>>>(d_in, n, segment_bytes, P, slots, bits,
-                                                               d_status);
+        if (ring_ok(P)) {
+            const size_t smem = 2 * (size_t)ring_words(P.W) * 4;  // at most 8 KB
+            const uint64_t grid = count < (uint64_t)sms * 64 ? count : (uint64_t)sms * 64;
+            auto run = [&](auto kernel) {
+                kernel<<<(unsigned)grid, 32, smem, s>>>(d_in, n, segment_bytes, P, slots, bits,
+                                                        d_status);
+            };
+            switch (P.lmin / 4) {
+            case 0: run(k_lzss_compress_ring<0>); break;
+            case 1: run(k_lzss_compress_ring<1>); break;
+            case 2: run(k_lzss_compress_ring<2>); break;
+            case 3: run(k_lzss_compress_ring<3>); break;
+            case 4: run(k_lzss_compress_ring<4>); break;
+            case 5: run(k_lzss_compress_ring<5>); break;
+            default: run(k_lzss_compress_ring<6>); break;
+            }
+        } else {
+            uint64_t grid = (count + kLzWarps - 1) / kLzWarps;
+            if (grid > (uint64_t)sms * 64)
+                grid = (uint64_t)sms * 64;
+            k_lzss_compress<<<(unsigned)grid, kLzBlock, 0, s>>>(d_in, n, segment_bytes, P, slots,
+                                                                bits, d_status);
+        }
     }
     k_lzss_layout<<<1, kScanBlock, 0, s>>>(n, segment_bytes, P, bits, start, d_out, out_cap,
                                            reinterpret_cast<unsigned long long *>(d_out_bytes),
