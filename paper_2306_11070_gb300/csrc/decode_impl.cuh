@@ -45,6 +45,7 @@ struct Tables {
     const uint32_t *start;
     const uint8_t *sorted;
     uint32_t max_len;
+    uint32_t fixed_len;  // the length all codes have, 0 if they differ
     __device__ __forceinline__ uint32_t entry(uint32_t idx) const { return lut[idx * copies]; }
 };
 
@@ -58,6 +59,7 @@ struct DecodeShared {
     uint32_t count[kMaxCodeLen + 1];
     uint32_t first[kMaxCodeLen + 1];
     uint32_t start[kMaxCodeLen + 1];
+    uint8_t group[8][kMaxCodeLen + 1];  // symbols of each length among 32 byte values
     unsigned long long s_kraft;
     int s_max, s_nsym, s_bad;
 };
@@ -432,61 +434,43 @@ __device__ __forceinline__ void count_codes(const Tables &T, const uint8_t *pay,
     e = pos;
 }
 
-// Codeword boundaries seen in the first kSyncBits bits of a sub-segment's
-// count (bit d set: a codeword starts d bits after the cut), kept in four
-// named registers (the word is picked by selects, never by an array index,
-// which would put the map in local memory).  256 bits: a Huffman decode
-// started off the true path almost always rejoins it within that distance,
-// so the settle walk below rarely has to recount a whole sub-segment.
-constexpr uint32_t kSyncBits = 256;
-struct SyncMap {
-    uint64_t w0, w1, w2, w3;
-    __device__ __forceinline__ void clear()
-    {
-        w0 = 1;  // the cut itself
-        w1 = w2 = w3 = 0;
-    }
-    __device__ __forceinline__ void set(uint32_t d)
-    {
-        const uint64_t b = 1ull << (d & 63);
-        const uint32_t j = d >> 6;
-        w0 |= j == 0 ? b : 0;
-        w1 |= j == 1 ? b : 0;
-        w2 |= j == 2 ? b : 0;
-        w3 |= j == 3 ? b : 0;
-    }
-    __device__ __forceinline__ uint64_t word(uint32_t j) const
-    {
-        return j == 0 ? w0 : j == 1 ? w1 : j == 2 ? w2 : w3;
-    }
-    __device__ __forceinline__ bool test(uint32_t d) const { return (word(d >> 6) >> (d & 63)) & 1; }
-    // boundaries before d (d < kSyncBits)
-    __device__ __forceinline__ uint32_t below(uint32_t d) const
-    {
-        const uint32_t j = d >> 6;
-        return (j > 0 ? __popcll(w0) : 0) + (j > 1 ? __popcll(w1) : 0) + (j > 2 ? __popcll(w2) : 0) +
-               __popcll(word(j) & ((1ull << (d & 63)) - 1));
-    }
-};
+// Boundaries of a sub-segment's counted path, kept while it is counted: the
+// start of each of the first 24 pairs of lookups (on text the first 430 bits
+// or so), then of every window (a sub-segment of a few thousand bits to its
+// end, so the walk below hardly ever recounts one: with only a map of the
+// first 256 bits, one text sub-segment in a few hundred did, and a warp waits
+// for its slowest lane).  Entries are bits from the cut << 16 | 8 x codewords
+// before, in the lane's column of the output ring, which is free until the
+// decoding pass; the cut itself is not listed.
+constexpr uint32_t kPairMarks = 24, kMarks = kOutRing;
 
-// Sub-segment [g, stop) was counted from g (cnt1 codewords, exit e1, early
-// boundaries bmap).  Given its true entry point, walk the true path one
-// codeword at a time until it lands on one of the recorded boundaries: from
+// Sub-segment [g, stop) was counted from g (cnt1 codewords, exit e1, `marks`
+// boundaries listed in column `col`).  Given its true entry point, walk the
+// true path one codeword at a time until it lands on a listed boundary: from
 // there both paths are the same codeword sequence, so only the codewords
-// before the meeting point change.  If they do not meet within the recorded
-// kSyncBits bits, recount from the entry point.
+// before the meeting point change.  If they do not meet up to the last one,
+// count on to the end.
 __device__ __forceinline__ void settle_segment(const Tables &T, const uint8_t *pay, uint64_t nw,
                                                uint64_t cbase, uint32_t g, uint32_t stop,
-                                               uint32_t entry, const SyncMap &bmap, uint32_t cnt1,
-                                               uint32_t e1, uint32_t &cnt, uint32_t &e)
+                                               uint32_t entry, uint32_t col, uint32_t marks,
+                                               uint32_t cnt1, uint32_t e1, uint32_t &cnt, uint32_t &e)
 {
-    uint32_t pos = entry, steps = 0;
+    if (entry == g) {
+        cnt = cnt1;
+        e = e1;
+        return;
+    }
+    uint32_t pos = entry, steps = 0, i = 0;
+    uint32_t mark = marks ? lds(col) : 0u;
     Reader rd;
     bool started = false;
     for (;;) {
-        const uint32_t d = pos - g;
-        if (d < kSyncBits && bmap.test(d)) {  // met: same path from here on
-            cnt = steps + cnt1 - bmap.below(d);
+        while (i < marks && (mark >> 16) < pos - g) {
+            ++i;
+            mark = i < marks ? lds(col + i * 128) : 0u;
+        }
+        if (i < marks && (mark >> 16) == pos - g) {  // met: same path from here on
+            cnt = steps + cnt1 - ((mark & 0xffffu) >> 3);
             e = e1;
             return;
         }
@@ -495,7 +479,7 @@ __device__ __forceinline__ void settle_segment(const Tables &T, const uint8_t *p
             e = pos;
             return;
         }
-        if (d >= kSyncBits)
+        if (i >= marks)
             break;
         if (!started) {
             rd.init(pay, nw, cbase + pos);
@@ -504,7 +488,7 @@ __device__ __forceinline__ void settle_segment(const Tables &T, const uint8_t *p
         rd.refill();
         const uint32_t idx = (uint32_t)(rd.buf >> (64 - kLutBits));
         uint32_t L = T.len0[idx];  // first code only: every boundary matters
-        if (T.entry(idx) == 0) {
+        if (L == 0) {
             uint32_t sym;
             if (!long_code(T, (uint32_t)(rd.buf >> 32), L, sym))
                 L = 1;
@@ -513,7 +497,8 @@ __device__ __forceinline__ void settle_segment(const Tables &T, const uint8_t *p
         ++steps;
         rd.consume(L);
     }
-    count_codes(T, pay, nw, cbase, entry, stop, cnt, e);
+    count_codes(T, pay, nw, cbase, pos, stop, cnt, e);
+    cnt += steps;
 }
 
 // Validate the stream header and build the decode tables of one stream in
@@ -555,26 +540,57 @@ __device__ __forceinline__ bool prepare(const uint8_t *stream_in, uint64_t bytes
         return false;
     }
 
-    // ---- lengths: range, longest, sh.count, Kraft sum ----
-    if (tid <= (int)kMaxCodeLen)
-        sh.count[tid] = 0;
-    if (tid == 0) {
-        sh.s_kraft = 0;
-        sh.s_max = 0;
-        sh.s_nsym = 0;
+    // ---- lengths: range, and how many byte values of each 32 have each ----
+    static_assert(NT % 32 == 0 && NT >= 64, "whole warps");
+    for (int i = tid; i < (int)sizeof(sh.group) / 4; i += NT)
+        reinterpret_cast<uint32_t *>(sh.group)[i] = 0;
+    if (tid == 0)
         sh.s_bad = 0;
+    sync();
+    uint32_t own_len[(256 + NT - 1) / NT], own_rank[(256 + NT - 1) / NT];
+#pragma unroll
+    for (int i = 0; i < (256 + NT - 1) / NT; ++i) {
+        const int b = tid + i * NT;
+        if (b < 256) {  // whole warps
+            const uint32_t L = stream[b];
+            const uint32_t same = __match_any_sync(kFull, L);
+            own_len[i] = L;
+            own_rank[i] = __popc(same & ((1u << (tid & 31)) - 1u));
+            if (L > kMaxCodeLen)
+                sh.s_bad = 1;
+            else if (own_rank[i] == 0)
+                sh.group[b >> 5][L] = (uint8_t)__popc(same);
+        }
     }
     sync();
-    for (int b = tid; b < 256; b += NT) {
-        const uint32_t L = stream[b];
-        sh.len_s[b] = (uint8_t)L;
-        if (L > kMaxCodeLen) {
-            sh.s_bad = 1;
-        } else if (L) {
-            atomicMax(&sh.s_max, (int)L);
-            atomicAdd(&sh.s_nsym, 1);
-            atomicAdd(&sh.s_kraft, 1ull << (32 - L));
-            atomicAdd(&sh.count[L], 1u);
+    // one warp, lane L - 1 for length L: counts, the Kraft sum, first codes (the
+    // RFC 1951 recurrence in closed form) and starts in symbol order
+    if (tid < 32) {
+        const uint32_t L = (uint32_t)tid + 1;
+        uint32_t cnt = 0;
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+            cnt += sh.group[g][L];
+        const uint64_t part = (uint64_t)cnt << (32 - L);
+        uint64_t kraft = part;
+        uint32_t syms = cnt;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint64_t y = __shfl_up_sync(kFull, (unsigned long long)kraft, d);
+            const uint32_t z = __shfl_up_sync(kFull, syms, d);
+            if (tid >= d) {
+                kraft += y;
+                syms += z;
+            }
+        }
+        sh.count[L] = cnt;
+        sh.first[L] = (uint32_t)((kraft - part) >> (32 - L));
+        sh.start[L] = syms - cnt;
+        const uint32_t used = __ballot_sync(kFull, cnt != 0);
+        if (tid == 31) {
+            sh.s_kraft = kraft;
+            sh.s_nsym = (int)syms;
+            sh.s_max = 32 - __clz(used);
         }
     }
     sync();
@@ -598,38 +614,36 @@ __device__ __forceinline__ bool prepare(const uint8_t *stream_in, uint64_t bytes
     if (n == 0)
         return false;
 
-    // ---- canonical tables (RFC 1951 next_code recurrence) ----
-    if (tid == 0) {
-        uint32_t code = 0, idx = 0;
-        for (uint32_t L = 1; L <= kMaxCodeLen; ++L) {
-            code = (code + sh.count[L - 1]) << 1;
-            sh.first[L] = code;
-            sh.start[L] = idx;
-            idx += sh.count[L];
-        }
-    }
-    sync();
-    for (int b = tid; b < 256; b += NT) {
-        const uint32_t L = sh.len_s[b];
-        if (L) {
-            uint32_t r = 0;
-            for (int j = 0; j < b; ++j)
-                r += sh.len_s[j] == L;
+    // ---- symbols in code order ----
+#pragma unroll
+    for (int i = 0; i < (256 + NT - 1) / NT; ++i) {
+        const int b = tid + i * NT;
+        if (b < 256 && own_len[i]) {
+            const uint32_t L = own_len[i];
+            uint32_t r = own_rank[i];
+            for (int g = 0; g < (b >> 5); ++g)
+                r += sh.group[g][L];
             sh.sorted[sh.start[L] + r] = (uint8_t)b;
         }
     }
     sync();
-    // pass 1: the first code of every 12-bit window, sym | L << 8 (0: none)
-    const uint32_t lut_len = max_len < (uint32_t)kLutBits ? max_len : (uint32_t)kLutBits;
+    // pass 1: the first code of every 12-bit window, sym | L << 8 (0: none).
+    // The windows whose first code has length L are those from bound[L - 1] up
+    // to bound[L]; all bounds are in registers, so a window costs a dozen
+    // compares and one dependent chain of loads.
+    uint32_t bound[kLutBits];
+#pragma unroll
+    for (int L = 1; L <= kLutBits; ++L)
+        bound[L - 1] = (sh.first[L] + sh.count[L]) << (kLutBits - L);
+#pragma unroll 4
     for (int v = tid; v < kLutSize; v += NT) {
+        uint32_t L = 1;
+#pragma unroll
+        for (int k = 0; k < kLutBits; ++k)
+            L += (uint32_t)v >= bound[k];
         uint32_t ent = 0;
-        for (uint32_t L = 1; L <= lut_len; ++L) {
-            const uint32_t c = (uint32_t)v >> (kLutBits - L);
-            if (sh.count[L] && c - sh.first[L] < sh.count[L]) {
-                ent = sh.sorted[sh.start[L] + c - sh.first[L]] | (L << 8);
-                break;
-            }
-        }
+        if (L <= (uint32_t)kLutBits)
+            ent = sh.sorted[sh.start[L] + ((uint32_t)v >> (kLutBits - L)) - sh.first[L]] | (L << 8);
         scratch[v] = (uint16_t)ent;
     }
     sync();
@@ -677,6 +691,7 @@ __device__ __forceinline__ bool prepare(const uint8_t *stream_in, uint64_t bytes
     si.T.start = sh.start;
     si.T.sorted = sh.sorted;
     si.T.max_len = max_len;
+    si.T.fixed_len = sh.count[max_len] == (uint32_t)nsym ? max_len : 0u;
     return true;
 }
 
@@ -773,102 +788,107 @@ __device__ __forceinline__ bool decode_task_s(const StreamInfo &si, uint32_t S_a
             lim = (uint32_t)(limit - cbase < 32ull * m ? limit - cbase : 32ull * m + 32);
             g = (uint32_t)(span * k / S);
             stop = (uint32_t)(span * (k + 1) / S);
+            if (T.fixed_len > 1) {  // such codes never resynchronise: cut between them
+                g -= g % T.fixed_len;
+                if (k + 1 < S)
+                    stop -= stop % T.fixed_len;
+            }
         }
     }
     const bool work = valid && !bad;
     const uint32_t *pw = reinterpret_cast<const uint32_t *>(pay);
     const uint32_t b0 = (uint32_t)(cbase & 31);  // chunk bit 0 within word w0
 
-    // 1. count each sub-segment but the last from its cut point
-    uint32_t cnt1 = 0, e1 = g;
-    SyncMap bmap;
-    bmap.clear();
+    // 1. count each sub-segment but the last from its cut point, listing
+    //    boundaries (see kPairMarks)
+    uint32_t cnt1 = 0, e1 = g, marks = 0;
     if (S > 1) {  // uniform: every lane of the warp takes this branch
         BitsT<C> rs = {};
-        bool act = work && k + 1 < S && g < stop;
+        const bool counted = work && k + 1 < S && g < stop;
+        bool act = counted;
         if (act)
             rs.init(in_s, pw, pay_words, cbase >> 5, b0 + g);
+        const uint32_t from = b0 + g;
         uint32_t pos = g;
-        // 1a. code by code through the first kSyncBits bits, recording the
-        //     boundaries
-        bool head = act;
-        while (__any_sync(kFull, head)) {
-            if (head) {
+        uint32_t cnt8 = 0;  // 8 x codes
+        for (uint32_t w = 0; __any_sync(kFull, act); ++w) {
+            // windows of pairs of lookups without checks: long ones while
+            // every lane has the room, then short ones; a lane too close to
+            // its end takes single codes.  A window reads at most one long
+            // code and its lookups of <= 12 bits each.
+            const uint32_t room = stop - pos;
+            uint32_t pairs = 4;
+            if (w >= kPairMarks / 4) {
+                if (__all_sync(kFull, !act || room >= 32 + kLutBits * kWindow))
+                    pairs = kWindow / 2;
+                else if (__all_sync(kFull, !act || room >= 32 + kLutBits * 24))
+                    pairs = 12;
+            }
+            if (act && room >= 32 + kLutBits * 2 * pairs) {
                 rs.refill();
-                uint32_t L = len0_at(len0, rs.bh);
-                if (L == 0) {
-                    uint32_t sym;
+                if (lut_ld(lut_l, stride, rs.bh) == 0) {  // a long code (rare)
+                    uint32_t L, sym;
                     if (!long_code(T, rs.bh, L, sym))
                         L = 1;
+                    rs.consume(L);
+                    cnt8 += 8;
                 }
-                rs.consume(L);
-                rs.refill();
-                pos += L;
-                ++cnt1;
-                if (pos - g < kSyncBits)
-                    bmap.set(pos - g);
-                head = pos - g < kSyncBits && pos < stop;
-                act = pos < stop;
-            }
-        }
-        // 1b. windows of table lookups, several codes per lookup
-        uint32_t cnt8 = 0;  // 8 x codes
-        while (__any_sync(kFull, act)) {
-            // an unchecked window reads at most one long code plus kWindow
-            // table lookups of <= 12 bits
-            const bool easy = stop - pos >= 32 + kLutBits * kWindow;
-            if (__all_sync(kFull, easy || !act)) {
-                if (act) {
-                    rs.refill();
-                    if (lut_ld(lut_l, stride, rs.bh) == 0) {  // a long code (rare)
-                        uint32_t L, sym;
-                        if (!long_code(T, rs.bh, L, sym))
-                            L = 1;
-                        rs.consume(L);
-                        rs.refill();
-                        cnt8 += 8;
-                    }
-                }
+                const bool list = w < kPairMarks / 4;
+#pragma unroll 1
+                for (uint32_t j = 0; j < pairs; j += 4) {
 #pragma unroll
-                for (int j = 0; j < kWindow; ++j) {
-                    if (act) {
-                        if ((j & 1) == 0 && j > 0)
-                            rs.refill();  // two lookups use at most 24 of >= 32 bits
+                    for (int i = 0; i < 4; ++i) {
+                        rs.refill();  // two lookups use at most 24 of >= 32 bits
+                        if (list)
+                            sts(out_s + (marks + i) * 128, (rs.bitpos() - from) << 16 | cnt8);
                         // a long code's entry is all zero: the lane stays on
                         // it for the rest of the window
-                        const uint32_t ent = lut_ld(lut_l, stride, rs.bh);
+                        uint32_t ent = lut_ld(lut_l, stride, rs.bh);
                         rs.consume_t(ent);
-                        cnt8 += (ent >> 8) & 24u;
+                        cnt8 = __dp4a(ent, 0x100u, cnt8);  // its second byte, 8 x codes
+                        ent = lut_ld(lut_l, stride, rs.bh);
+                        rs.consume_t(ent);
+                        cnt8 = __dp4a(ent, 0x100u, cnt8);  // its second byte, 8 x codes
                     }
                 }
-            } else {
+                marks += list ? 4 : 0;
+            } else if (act) {
+                // near the end: one lookup at a time, both codes of an entry
+                // while the second starts before the end
 #pragma unroll 1
-                for (int j = 0; j < kCheckedWindow; ++j) {
-                    if (act) {
-                        rs.refill();
-                        uint32_t L = len0_at(len0, rs.bh);  // one code at a time
-                        if (L == 0) {
-                            uint32_t sym;
-                            if (!long_code(T, rs.bh, L, sym))
-                                L = 1;
-                        }
-                        rs.consume(L);
-                        cnt8 += 8;
-                        act = rs.bitpos() - b0 < stop;
+                for (int j = 0; j < kCheckedWindow && pos < stop; ++j) {
+                    rs.refill();
+                    const uint32_t ent = lut_ld(lut_l, stride, rs.bh);
+                    uint32_t L = len0_at(len0, rs.bh);
+                    const bool two = pos + ent_len(ent) < stop;
+                    cnt8 += two ? (ent >> 8) & 24u : 8u;
+                    L = two ? ent_len(ent) : L;
+                    if (ent == 0) {
+                        uint32_t sym;
+                        if (!long_code(T, rs.bh, L, sym))
+                            L = 1;
+                        cnt8 += two ? 8u : 0u;
                     }
+                    rs.consume(L);
+                    pos += L;
                 }
             }
             if (act) {
                 pos = rs.bitpos() - b0;
                 act = pos < stop;
             }
-            if (act)
+            if (act) {
+                if (w + 1 >= kPairMarks / 4 && marks < kMarks) {
+                    sts(out_s + marks * 128, (pos - g) << 16 | cnt8);
+                    ++marks;
+                }
                 rs.top_up();
+            }
             cp_async_wait<kInFlight>();
         }
         cp_async_wait<0>();  // the ring is reused below
-        if (work && k + 1 < S && g < stop) {
-            cnt1 += cnt8 >> 3;
+        if (counted) {
+            cnt1 = cnt8 >> 3;
             e1 = rs.bitpos() - b0;
         }
     }
@@ -887,8 +907,8 @@ __device__ __forceinline__ bool decode_task_s(const StreamInfo &si, uint32_t S_a
             used = pe;
             entry = pe;
             if (k + 1 < S)
-                settle_segment(T, pay, pay_words, cbase, g, stop, entry, bmap, cnt1, e1, cnt,
-                               e);
+                settle_segment(T, pay, pay_words, cbase, g, stop, entry, out_s, marks, cnt1, e1,
+                               cnt, e);
         }
         first = false;
     }
@@ -919,15 +939,23 @@ __device__ __forceinline__ bool decode_task_s(const StreamInfo &si, uint32_t S_a
         if (act)
             rs.init(in_s, pw, pay_words, cbase >> 5, b0 + entry);
         while (__any_sync(kFull, act)) {
-            // far from the segment's end a window needs no per-code checks:
-            // at most 2 * kWindow symbols and kWindow x 12 bits, plus one
-            // long code.  The unchecked window runs only when every lane of
-            // the warp is in that state, so it needs no per-lane predicate
-            // either.
-            const bool easy = act && qend - q >= 1 + kMaxPerLookup * kWindow &&
-                              lim - pos >= 32 + kLutBits * kWindow;
+            // far from the segment's end a window needs no per-code checks: at
+            // most two symbols and 12 bits per lookup, plus one long code.
+            // The longest window every lane has room for runs; a lane with
+            // room for the shortest only runs that, one without takes single
+            // codes.
+            const uint32_t qroom = qend - q, broom = lim - pos;
+            auto room = [&](uint32_t lookups) {
+                return qroom >= 1 + kMaxPerLookup * lookups && broom >= 32 + kLutBits * lookups;
+            };
+            uint32_t halves = 1, pairs = 16;
+            if (__all_sync(kFull, !act || room(kWindow))) {
+                halves = kWindow / 32;
+            } else if (kWindow == 32 || !__all_sync(kFull, !act || room(32))) {
+                pairs = 4;
+            }
             uint32_t q0 = q, row0 = ow.row(), p0 = ow.pending();
-            if (__all_sync(kFull, easy)) {
+            if (act && room(2 * pairs)) {
                 rs.refill();
                 if (lut_ld(lut_l, stride, rs.bh) == 0) {  // a long code (rare)
                     uint32_t L = 0, sym = 0;
@@ -952,19 +980,22 @@ __device__ __forceinline__ bool decode_task_s(const StreamInfo &si, uint32_t S_a
                 // word at most, within the ring bound).
                 uint32_t ent = lut_ld(lut_l, stride, rs.bh);
 #pragma unroll 1
-                for (int half = 0; half < kWindow / 32; ++half) {
-#pragma unroll 4
-                    for (int p = 0; p < 16; ++p) {
-                        rs.consume_t(ent);
-                        const uint32_t ent1 = lut_ld(lut_l, stride, rs.bh);
-                        ow.merge(ent);
-                        rs.consume_t(ent1);
-                        rs.refill();
-                        ent = lut_ld(lut_l, stride, rs.bh);
-                        ow.merge(ent1);
-                        ow.store();
+                for (uint32_t half = 0; half < halves; ++half) {
+#pragma unroll 1
+                    for (uint32_t p = 0; p < pairs; p += 4) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            rs.consume_t(ent);
+                            const uint32_t ent1 = lut_ld(lut_l, stride, rs.bh);
+                            ow.merge(ent);
+                            rs.consume_t(ent1);
+                            rs.refill();
+                            ent = lut_ld(lut_l, stride, rs.bh);
+                            ow.merge(ent1);
+                            ow.store();
+                        }
                     }
-                    if (half + 1 < kWindow / 32) {
+                    if (half + 1 < halves) {
                         // a 64-lookup window flushes after its first 32 lookups
                         // (at most 65 bytes and 17 rows so far), so the output
                         // ring never holds more than one half's bytes
@@ -981,42 +1012,37 @@ __device__ __forceinline__ bool decode_task_s(const StreamInfo &si, uint32_t S_a
                         p0 = ow.pending();
                     }
                 }
-            } else {
+            } else if (act) {
 #pragma unroll 1
-                for (int j = 0; j < kCheckedWindow; ++j) {
-                    if (act) {
-                        rs.refill();
-                        const uint32_t ent = lut_ld(lut_l, stride, rs.bh);
-                        uint32_t L, ns, y;
-                        if (ent == 0) {
-                            uint32_t sym = 0;
-                            L = 0;
-                            if (!long_code(T, rs.bh, L, sym))
-                                bad = true;
-                            ns = 1;
-                            y = (sym << 24) | (8u << 8);
-                        } else {
-                            L = ent_len(ent);
-                            ns = ent_count(ent);
-                            y = ent;
-                            if (q + ns > qend || pos + L > lim) {  // first code only
-                                L = len0_at(len0, rs.bh);
-                                ns = 1;
-                                y = (ent & 0xff000000u) | (8u << 8);
-                            }
-                        }
-                        if (pos + L > lim)
+                for (int j = 0; j < kCheckedWindow && act; ++j) {
+                    rs.refill();
+                    uint32_t ent = lut_ld(lut_l, stride, rs.bh);
+                    uint32_t L = len0_at(len0, rs.bh);
+                    // the entry whole, or its first code only
+                    const uint32_t l2 = ent_len(ent), ns = ent_count(ent);
+                    const bool whole = q + ns <= qend && pos + l2 <= lim;
+                    uint32_t y = whole ? ent : (ent & 0xff000000u) | (8u << 8);
+                    uint32_t got = whole ? ns : 1u;
+                    L = whole ? l2 : L;
+                    if (ent == 0) {
+                        uint32_t sym = 0;
+                        L = 0;
+                        if (!long_code(T, rs.bh, L, sym))
                             bad = true;
-                        if (!bad) {
-                            rs.consume(L);
-                            ow.merge(y);
-                            ow.store();
-                            q += ns;
-                            pos += L;
-                        }
-                        act = !bad && q < qend;
+                        got = 1;
+                        y = (sym << 24) | (8u << 8);
                     }
+                    bad |= pos + L > lim;
+                    if (bad)
+                        break;
+                    rs.consume(L);
+                    ow.merge(y);
+                    ow.store();
+                    q += got;
+                    pos += L;
+                    act = q < qend;
                 }
+                act = act && !bad;
             }
             // bytes queued in this window: whole rows stored plus the change
             // in pending bytes (a window moves fewer than kOutRing rows)
