@@ -6,8 +6,10 @@
 // doubling.  Every position i carries a rank RK[i] = the first sorted slot
 // of its group (the rotations that agree on the prefix compared so far);
 // slots of block b are [b * block, b * block + m_b), so ranks are global.
-//   round 0: sort all positions by (block, first 4 bytes of the rotation);
-//   round r: with h = 4 * 2^(r-1), the still-unresolved positions (groups of
+//   round 0: sort all positions by (block, first q bytes of the rotation),
+//            the bytes as digits of a number in base sigma, the number of byte
+//            values that occur (q = 11 on text; see first_key);
+//   round r: with h = q * 2^(r-1), the still-unresolved positions (groups of
 //            more than one) are sorted by (group, RK[i + h within the block])
 //            and their groups split where that second rank changes;
 // until no group has two members or the compared prefix covers the longest
@@ -28,6 +30,8 @@
 // re-walks its stretch writing the bytes in place.  A periodic block's walk
 // returns to the primary row after one period c; the rest of the block
 // repeats it.
+#include <cmath>
+
 #include "api_trace.h"
 #include "sort_impl.cuh"
 
@@ -67,22 +71,51 @@ __device__ __forceinline__ void block_span(uint32_t i, uint32_t block, uint32_t 
 }
 
 // ---- forward --------------------------------------------------------------
-// round 0 keys: (block id, big-endian first 4 bytes of the rotation)
-__global__ void k_bwt_init(const uint8_t *x, uint32_t n, uint32_t block, uint64_t *key,
-                           uint32_t *val, uint32_t *act)
+// Round 0's key: q bytes as base-sigma digits below the block id.
+struct FirstKey {
+    uint32_t q, sigma;
+    uint32_t bits;      // of the digits' number
+    uint8_t code[256];  // a byte value's digit
+};
+constexpr uint32_t kInitTile = 2048;
+constexpr uint32_t kMaxFirst = 16;  // most bytes in a first key
+
+// round 0 keys: (block id, the digits of the rotation's first q bytes)
+__global__ void __launch_bounds__(kEw) k_bwt_init(const uint8_t *x, uint32_t n, uint32_t block,
+                                                  const __grid_constant__ FirstKey f, uint64_t *key,
+                                                  uint32_t *val)
 {
-    for (uint32_t i = blockIdx.x * kEw + threadIdx.x; i < n; i += gridDim.x * kEw) {
-        uint32_t s, m;
-        block_span(i, block, n, s, m);
-        const uint32_t r = i - s;
-        uint32_t k = 0;
-#pragma unroll
-        for (uint32_t t = 0; t < 4; ++t)
-            k = (k << 8) | x[s + (uint32_t)(((uint64_t)r + t) % m)];
-        key[i] = ((uint64_t)(i / block) << 32) | k;
-        val[i] = i;
-        act[i] = i;
+    __shared__ uint8_t code[256], tile[kInitTile + kMaxFirst];
+    static_assert(kEw == 256, "a thread per byte value");
+    code[threadIdx.x] = f.code[threadIdx.x];
+    for (uint64_t t0 = (uint64_t)blockIdx.x * kInitTile; t0 < n; t0 += (uint64_t)gridDim.x * kInitTile) {
+        __syncthreads();
+        for (uint32_t j = threadIdx.x; j < kInitTile + kMaxFirst; j += kEw)
+            tile[j] = t0 + j < n ? code[x[t0 + j]] : 0;
+        __syncthreads();
+        for (uint32_t j = threadIdx.x; j < kInitTile && t0 + j < n; j += kEw) {
+            const uint32_t i = (uint32_t)t0 + j;
+            uint32_t s, m;
+            block_span(i, block, n, s, m);
+            uint64_t k = 0;
+            if (i - s + f.q <= m) {
+                for (uint32_t t = 0; t < f.q; ++t)
+                    k = k * f.sigma + tile[j + t];
+            } else {  // the rotation goes on at the block's start
+                for (uint32_t t = 0; t < f.q; ++t)
+                    k = k * f.sigma + code[x[s + (uint32_t)(((uint64_t)(i - s) + t) % m)]];
+            }
+            key[i] = f.bits < 64 ? ((uint64_t)(i / block) << f.bits) | k : k;
+            val[i] = i;
+        }
     }
+}
+
+// the counts of the bytes before the first 16-byte boundary
+__global__ void k_count_head(const uint8_t *x, uint32_t count, unsigned long long *hist)
+{
+    if (threadIdx.x < count)
+        atomicAdd(hist + x[threadIdx.x], 1ull);
 }
 
 // round r keys: (group, rank of the rotation h bytes on, relative to the
@@ -407,7 +440,7 @@ __device__ __forceinline__ void rf_stage(const uint64_t *key, const uint32_t *ac
     }
     for (uint32_t t = threadIdx.x; t < kRfTile; t += kRfThreads) {
         const uint64_t k = t0 + t;
-        sact[rf_pad(t)] = k < count ? act[k] : 0u;
+        sact[rf_pad(t)] = k < count ? (act ? act[k] : (uint32_t)k) : 0u;
         if (val)
             sval[rf_pad(t)] = k < count ? val[k] : 0u;
     }
@@ -672,9 +705,11 @@ cudaError_t refine(FwdWs &w, const uint64_t *ks, const uint32_t *vs, uint32_t co
         (e = kernel_setup(setup_apply, (const void *)k_refine_apply, kRfThreads, kRfApplySmem,
                           &per_sm)) != cudaSuccess)
         return e;
-    k_refine_tiles<<<tiles, kRfThreads, kRfTilesSmem, s>>>(ks, w.act, count, gbits, ph, pf, pm);
+    // the first list is every slot in order
+    const uint32_t *act = gbits < 64 ? w.act : nullptr;
+    k_refine_tiles<<<tiles, kRfThreads, kRfTilesSmem, s>>>(ks, act, count, gbits, ph, pf, pm);
     k_refine_parts<<<1, kRfThreads, 0, s>>>(ph, pf, pm, tiles, w.scal);
-    k_refine_apply<<<tiles, kRfThreads, kRfApplySmem, s>>>(ks, vs, w.act, count, gbits, ph, pf, pm,
+    k_refine_apply<<<tiles, kRfThreads, kRfApplySmem, s>>>(ks, vs, act, count, gbits, ph, pf, pm,
                                                            w.sa, w.rk, w.act2, w.grp2);
     uint32_t h[2];
     if ((e = cudaGetLastError()) != cudaSuccess ||
@@ -690,6 +725,50 @@ cudaError_t refine(FwdWs &w, const uint64_t *ks, const uint32_t *vs, uint32_t co
     w.grp = w.grp2;
     w.grp2 = t;
     return cudaSuccess;
+}
+
+// The first key of an input with these byte counts: as many bytes as make most
+// rotations of a block of m bytes differ, then as many more as the last pass
+// has room for.  On the synthetic text (34 byte values, order-0 entropy 4.3
+// bits, 1 MiB blocks) 96% of the positions are left in groups after 4 bytes,
+// 42% after 8 and a quarter after 11, and a position left costs as much as
+// about eight passes over it, so text wants 2.4 log2 m bits of order-0 entropy;
+// bytes close to random differ after 1.5 log2 m.  Forward transform of 64 MiB
+// in 1 MiB blocks against keys of four bytes always (and a radix pass that
+// ranked with match.any): text 13.1 -> 8.2 ms, Zipf bytes 8.8 -> 7.0, uniform
+// bytes 7.0 -> 4.9, the bitstream stand-in 47.3 -> 45.5.
+FirstKey first_key(const unsigned long long *hist, uint64_t n, uint64_t blocks, uint64_t m)
+{
+    FirstKey f;
+    f.sigma = 0;
+    double entropy = 0;
+    for (int b = 0; b < 256; ++b) {
+        f.code[b] = (uint8_t)f.sigma;
+        if (hist[b]) {
+            ++f.sigma;
+            const double p = (double)hist[b] / (double)n;
+            entropy -= p * std::log2(p);
+        }
+    }
+    if (f.sigma < 2)
+        f.sigma = 2;
+    const uint32_t room = 64 - bit_width(blocks - 1);
+    const double want = (entropy > 7.5 ? 1.5 : 2.4) * bit_width(m - 1);
+    f.q = f.bits = 0;
+    for (uint64_t v = 1; f.q < kMaxFirst;) {  // v = sigma^q
+        if (v > ~0ull / f.sigma)
+            break;
+        v *= f.sigma;
+        const uint32_t bits = bit_width(v - 1);
+        if (bits > room)
+            break;
+        const uint32_t used = 64 - room;
+        if (f.q >= 4 && f.q * entropy >= want && (bits + used + 7) / 8 > (f.bits + used + 7) / 8)
+            break;  // enough, and one more byte would take another pass
+        ++f.q;
+        f.bits = bits;
+    }
+    return f;
 }
 
 // ---- inverse --------------------------------------------------------------
@@ -941,15 +1020,28 @@ huff_status_t huff_bwt_forward(const uint8_t *d_in, uint64_t n, uint32_t block, 
     FwdWs w = fwd_layout(static_cast<uint8_t *>(d_ws), n);
     const uint64_t blocks = (n + block - 1) / block;
     const uint64_t mmax = n < block ? n : block;
-    k_bwt_init<<<ew_grid(n), kEw, 0, s>>>(d_in, N, block, w.k0, w.v0, w.act);
+    // byte counts (in the workspace's first 2 KiB, not in use yet)
+    auto *hist = static_cast<unsigned long long *>(d_ws);
+    const uint32_t lead = (uint32_t)(0u - reinterpret_cast<uintptr_t>(d_in)) & 15u;
+    const uint32_t head = lead < N ? lead : N;
+    unsigned long long h_hist[256];
+    if (launch_histogram(d_in + head, n - head, hist, nullptr, s) != cudaSuccess)
+        return HUFF_ERR_CUDA;
+    if (head)
+        k_count_head<<<1, 32, 0, s>>>(d_in, head, hist);
+    if (cudaMemcpyAsync(h_hist, hist, sizeof(h_hist), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return HUFF_ERR_CUDA;
+    const FirstKey f = first_key(h_hist, n, blocks, mmax);
+    k_bwt_init<<<ew_grid((n + 7) / 8), kEw, 0, s>>>(d_in, N, block, f, w.k0, w.v0);
     uint64_t *ks;
     uint32_t *vs;
-    if (sort_keys(w, N, 32 + bit_width(blocks - 1), s, ks, vs) != cudaSuccess)
+    if (sort_keys(w, N, f.bits + bit_width(blocks - 1), s, ks, vs) != cudaSuccess)
         return HUFF_ERR_CUDA;
     uint32_t n_act = 0, groups = 0;
     if (refine(w, ks, vs, N, 64, s, n_act, groups) != cudaSuccess)
         return HUFF_ERR_CUDA;
-    for (uint64_t h = 4; n_act > 0 && h < mmax; h *= 2) {
+    for (uint64_t h = f.q; n_act > 0 && h < mmax; h *= 2) {
         const uint32_t lo_bits = bit_width(mmax - 1);
         k_bwt_round_keys<<<ew_grid(n_act), kEw, 0, s>>>(w.sa, w.rk, w.act, w.grp, n_act, N, block, h,
                                                         lo_bits, w.k0, w.v0);

@@ -1,0 +1,41 @@
+"""The block-sorting transform's first keys: alphabets of one byte value to
+all 256, blocks shorter than a key, rotations that wrap inside it, and inputs
+that do not start on a 16-byte boundary; and radix tiles that are not full."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+import paper_2306_11070_gb300 as hg
+from paper_2306_11070_gb300 import build as nvbuild
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    nvbuild.build()
+    hg.lib()
+
+
+def _input(sigma, n):
+    if sigma == "text":
+        return synth.text(n, n)
+    vals = np.linspace(0, 255, sigma).astype(np.uint8)
+    return vals[synth.uniform(n, n).astype(np.int64) * sigma // 256]
+
+
+@pytest.mark.parametrize("sigma", [1, 2, 3, 17, 256, "text"])
+@pytest.mark.parametrize("block", [1, 7, 16, 300, 4096, 5000, 20000])
+def test_first_keys_against_oracle(sigma, block):
+    for n, off in ((9, 3), (15, 0), (4096, 0), (12289, 1), (20000, 15)):
+        x = _input(sigma, n)
+        d = torch.zeros(n + 16, dtype=torch.uint8, device="cuda")[off:off + n]
+        d.copy_(torch.from_numpy(x))
+        ref_last, ref_prim = oracle.bwt(x, block)
+        last, prim, st = hg.huff_bwt_forward(d, block)
+        torch.cuda.synchronize()
+        assert int(st.item()) == 0
+        assert np.array_equal(last.cpu().numpy(), ref_last), (n, off)
+        assert np.array_equal(prim.cpu().numpy().astype(np.uint32), ref_prim), (n, off)
