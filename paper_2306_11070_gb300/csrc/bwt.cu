@@ -22,14 +22,15 @@
 // of the larger groups go through the global radix passes.
 //
 // Inverse: LF[p] = the slot of row p's last byte in a stable sort of the
-// last column by (block, byte); the block is the walk p -> LF[p] from the
-// primary row, emitted backwards.  The walk is cut at sample rows (every
-// 64th row and the primary rows): each sample walks to the next sample and
-// records the distance, list ranking by pointer jumping over the samples
-// gives each sample's distance from the primary row, and every sample then
-// re-walks its stretch writing the bytes in place.  A periodic block's walk
-// returns to the primary row after one period c; the rest of the block
-// repeats it.
+// last column by (block, byte), which is the byte's first slot in the block
+// plus the rank of row p among the block's rows with that byte: counted per
+// tile and scanned, so LF is written in row order.  The block is the walk
+// p -> LF[p] from the primary row, emitted backwards.  The walk is cut at
+// sample rows (every 64th row and the primary rows): each sample walks to the
+// next sample, keeping the bytes it passes, list ranking by pointer jumping
+// over the samples gives each sample's distance from the primary row, and its
+// bytes are copied to their place.  A periodic block's walk returns to the
+// primary row after one period c; the rest of the block repeats it.
 #include <cmath>
 
 #include "api_trace.h"
@@ -41,7 +42,16 @@ namespace {
 using namespace srt;
 
 constexpr int kEw = 256;               // threads of the elementwise kernels
-constexpr uint32_t kSampleGap = 64;    // rows between regular samples
+// Rows between regular samples of the inverse: 32 for blocks whose samples
+// are ranked in one CTA's shared memory (k_rank), 64 for others.  The longest
+// of the walks, ln(samples) gaps, and the cached part of LF that the walks in
+// flight read both shrink with the gap: 64 MiB of text in 1 MiB blocks, walk
+// 0.72 -> 0.57 ms.
+constexpr uint32_t kRankMin = 4096, kRankMax = 1u << 20;  // such blocks, bytes
+__host__ __device__ __forceinline__ uint32_t sample_gap(uint64_t most)
+{
+    return most >= kRankMin && most <= kRankMax ? 32u : 64u;
+}
 constexpr uint32_t kNil = 0xffffffffu;
 
 unsigned ew_grid(uint64_t count)
@@ -781,10 +791,131 @@ __global__ void k_lf_keys(const uint8_t *last, uint32_t n, uint32_t block, uint6
     }
 }
 
-__global__ void k_lf_scatter(const uint32_t *vs, uint32_t n, uint32_t *lf)
+// A row's LF within its block and its byte in one word, so that a step of a
+// walk is one load: 32 bits for blocks of up to 16 MiB, else 64.
+template <class T>
+__device__ __forceinline__ T lf_word(uint32_t lf, uint32_t byte)
+{
+    return (T)lf << 8 | byte;
+}
+constexpr uint32_t kMaxBlock32 = 1u << 24;
+
+// blocks of less than a tile: from the sorted (block, byte) keys
+__global__ void k_lf_scatter(const uint64_t *ks, const uint32_t *vs, uint32_t n, uint32_t block,
+                             uint32_t *lf)
 {
     for (uint32_t q = blockIdx.x * kEw + threadIdx.x; q < n; q += gridDim.x * kEw)
-        lf[vs[q]] = q;
+        lf[vs[q]] = lf_word<uint32_t>(q % block, (uint32_t)ks[q] & 255u);
+}
+
+// Other blocks: tiles of 4096 rows that do not cross blocks, `per` of them to a
+// block; byte counts at [(block * 256 + byte) * per + tile], whose exclusive
+// sum is a tile's first slot for each byte.
+constexpr int kLfThreads = 512;
+constexpr int kLfItems = 8;
+constexpr int kLfWarps = kLfThreads / 32;
+constexpr uint32_t kLfTile = kLfThreads * kLfItems;
+
+// a warp's rows of the tile in order, 32 at a time
+__device__ __forceinline__ void lf_tile(uint32_t n, uint32_t block, uint32_t per, uint32_t &s,
+                                        uint32_t &t, uint32_t &row, uint32_t &left)
+{
+    const uint32_t b = blockIdx.x / per;
+    t = blockIdx.x - b * per;
+    s = b * block;
+    const uint32_t m = n - s < block ? n - s : block;
+    row = t * kLfTile + (threadIdx.x >> 5) * (kLfItems * 32);  // within the block
+    left = row < m ? (m - row < kLfItems * 32 ? m - row : kLfItems * 32) : 0u;
+}
+
+// same_digit for a transformed column: where a warp's 32 rows hold few runs
+// they hold few distinct bytes, which match.any takes one by one faster than
+// eight ballots
+__device__ __forceinline__ uint32_t same_byte(uint32_t d, bool ok)
+{
+    const uint32_t key = ok ? d : 256u;
+    const uint32_t before = __shfl_up_sync(0xffffffffu, key, 1);
+    if (__popc(__ballot_sync(0xffffffffu, key != before)) <= 6)
+        return __match_any_sync(0xffffffffu, key);
+    return same_digit(d, ok);
+}
+
+__global__ void __launch_bounds__(kLfThreads) k_lf_count(const uint8_t *last, uint32_t n,
+                                                         uint32_t block, uint32_t per,
+                                                         uint32_t *hist)
+{
+    __shared__ uint32_t c[256];
+    if (threadIdx.x < 256)
+        c[threadIdx.x] = 0;
+    __syncthreads();
+    uint32_t s, t, row, left;
+    lf_tile(n, block, per, s, t, row, left);
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t d[kLfItems];
+#pragma unroll
+    for (int j = 0; j < kLfItems; ++j)
+        d[j] = j * 32 + lane < left ? last[s + row + j * 32 + lane] : 0u;
+#pragma unroll
+    for (int j = 0; j < kLfItems; ++j) {
+        // the last row of each run adds the run (a transformed column is runs)
+        const bool ok = j * 32 + lane < left;
+        const uint32_t key = ok ? d[j] : 256u;
+        const uint32_t after = __shfl_down_sync(0xffffffffu, key, 1);
+        const bool end = lane == 31 || after != key;
+        const uint32_t before = __ballot_sync(0xffffffffu, end) & lanemask_lt();
+        if (ok && end)
+            atomicAdd(&c[d[j]], lane + 1 - (before ? 32 - __clz(before) : 0));
+    }
+    __syncthreads();
+    if (threadIdx.x < 256)
+        hist[((uint64_t)(blockIdx.x / per) * 256 + threadIdx.x) * per + t] = c[threadIdx.x];
+}
+
+template <class T>
+__global__ void __launch_bounds__(kLfThreads) k_lf_rank(const uint8_t *last, uint32_t n,
+                                                        uint32_t block, uint32_t per,
+                                                        const uint32_t *offs, T *lf)
+{
+    __shared__ uint32_t cnts[kLfWarps][256];
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t s, t, row, left;
+    lf_tile(n, block, per, s, t, row, left);
+    uint32_t *const cnt = cnts[w];
+    uint32_t d[kLfItems], rank[kLfItems];
+#pragma unroll
+    for (int j = 0; j < kLfItems; ++j)
+        d[j] = j * 32 + lane < left ? last[s + row + j * 32 + lane] : 0u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        cnt[j * 32 + lane] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < kLfItems; ++j) {
+        const bool ok = j * 32 + lane < left;
+        const uint32_t mask = same_byte(d[j], ok);
+        rank[j] = cnt[d[j]] + __popc(mask & lanemask_lt());
+        __syncwarp();
+        if (ok && lane == (uint32_t)__ffs(mask) - 1)
+            cnt[d[j]] += __popc(mask);
+        __syncwarp();
+    }
+    __syncthreads();
+    // per byte: the tile's first slot in the block, then the warps before
+    if (threadIdx.x < 256) {
+        uint32_t run =
+            offs[((uint64_t)(blockIdx.x / per) * 256 + threadIdx.x) * per + t] - s;
+#pragma unroll
+        for (int ww = 0; ww < kLfWarps; ++ww) {
+            const uint32_t x = cnts[ww][threadIdx.x];
+            cnts[ww][threadIdx.x] = run;
+            run += x;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kLfItems; ++j)
+        if (j * 32 + lane < left)
+            lf[s + row + j * 32 + lane] = lf_word<T>(cnt[d[j]] + rank[j], d[j]);
 }
 
 __global__ void k_check_primary(const uint32_t *primary, uint32_t n, uint32_t block,
@@ -799,59 +930,67 @@ __global__ void k_check_primary(const uint32_t *primary, uint32_t n, uint32_t bl
 }
 
 struct Samples {
-    uint32_t n, block, regular;  // regular samples: rows 0, 64, 128, ...
-    const uint32_t *primary;
-    // sample id of row p, or kNil: a primary row is its block's extra
-    // sample (regular + block), even when it is also a multiple of 64
-    __device__ __forceinline__ uint32_t id_of(uint32_t p) const
-    {
-        const uint32_t b = p / block;
-        if (p - b * block == primary[b])
-            return regular + b;
-        return (p % kSampleGap) == 0 ? p / kSampleGap : kNil;
-    }
+    uint32_t n, block, regular, gap;  // regular samples: rows 0, gap, 2 gap, ...
+    const uint32_t *primary;  // a primary row is its block's extra sample (id regular + block)
     // row of sample id, or kNil for a regular sample that is a primary row
     __device__ __forceinline__ uint32_t row_of(uint32_t id) const
     {
         if (id >= regular)
             return (id - regular) * block + primary[id - regular];
-        const uint32_t p = id * kSampleGap;
+        const uint32_t p = id * gap;
         const uint32_t b = p / block;
         return p - b * block == primary[b] ? kNil : p;
     }
 };
 
-// every sample walks to the next sample: link and length; the link into a
-// block's primary sample is cut (kNil), which turns the primary's cycle into
-// a list headed by the primary
-__global__ void k_walk_link(const uint32_t *lf, Samples S, uint32_t count, uint32_t *nxt,
-                            uint32_t *len, int32_t *status)
+// The inverse of 64 MiB of text in 1 MiB blocks takes 1.21 ms (4.32 ms with LF
+// from two radix passes and a scatter, bytes read in a second walk and global
+// pointer jumping): LF 0.38, walk 0.57, rank 0.06, emit 0.13.  The walk is bound
+// by its random reads of LF, 64 M sectors of L2 (half of them in it).
+//
+// Every sample walks to the next sample: link, length and the first `cap`
+// bytes on the way (kept[id * cap]).  The link into a block's primary sample
+// is cut (kNil), which turns the primary's cycle into a list headed by the
+// primary.
+template <class T>
+__global__ void k_walk(const T *lf, Samples S, uint32_t count, uint32_t cap, uint32_t *nxt,
+                       uint32_t *len, uint8_t *kept, int32_t *status)
 {
     if (chain_failed(status))
         return;
     for (uint32_t id = blockIdx.x * kEw + threadIdx.x; id < count; id += gridDim.x * kEw) {
         const uint32_t p0 = S.row_of(id);
-        if (p0 == kNil) {
-            nxt[id] = kNil;
-            len[id] = 0;
-            continue;
+        uint32_t t = 0, to = kNil;
+        if (p0 != kNil) {
+            const uint32_t b = p0 / S.block, s = b * S.block;
+            const uint32_t m = S.n - s < S.block ? S.n - s : S.block;
+            const uint32_t prim = S.primary[b];
+            uint64_t acc = 0;
+            uint2 *const out = reinterpret_cast<uint2 *>(kept + (uint64_t)id * cap);
+            uint32_t r = p0 - s;
+            bool more = true;
+            do {  // ends on p0 at the latest: LF is a permutation of the block
+                const T v = lf[s + r];
+                r = (uint32_t)(v >> 8);
+                acc |= (uint64_t)((uint32_t)v & 255u) << (8 * (t & 7u));
+                ++t;
+                more = r != prim && ((s + r) & (S.gap - 1)) != 0 && t < m;
+                if ((t & 7u) == 0 || !more) {
+                    if (t <= cap)  // a multiple of 8
+                        out[(t - 1) >> 3] = make_uint2((uint32_t)acc, (uint32_t)(acc >> 32));
+                    acc = 0;
+                }
+            } while (more);
+            if (r != prim) {
+                to = (s + r) / S.gap;
+                if (((s + r) & (S.gap - 1)) != 0) {  // cannot happen for a sorted column
+                    set_status(status, HUFF_ERR_CORRUPT_STREAM);
+                    to = kNil;
+                    t = 0;
+                }
+            }
         }
-        uint32_t s, m;
-        block_span(p0, S.block, S.n, s, m);
-        uint32_t p = p0, t = 0, c;
-        do {  // ends on p0 at the latest: LF is a permutation of the block
-            p = lf[p];
-            ++t;
-            c = p < S.n ? S.id_of(p) : kNil;
-        } while (c == kNil && t < m && p < S.n);
-        if (c == kNil) {  // not a permutation: cannot happen for a sorted column
-            set_status(status, HUFF_ERR_CORRUPT_STREAM);
-            nxt[id] = kNil;
-            len[id] = 0;
-            continue;
-        }
-        const uint32_t b = p0 / S.block;
-        nxt[id] = c == S.regular + b ? kNil : c;
+        nxt[id] = to;
         len[id] = t;
     }
 }
@@ -875,48 +1014,169 @@ __global__ void k_jump(const uint32_t *nx_in, const uint32_t *sum_in, uint32_t c
     }
 }
 
-// samples on their block's primary list write their stretch: the primary's
-// sum is the cycle length c, a sample's distance from the primary is
-// c - its own sum
-__global__ void k_walk_emit(const uint32_t *lf, const uint8_t *last, Samples S, uint32_t count,
-                            const uint32_t *len, const uint32_t *nx, const uint32_t *sum,
-                            uint8_t *out, int32_t *status)
+// The same for one block per CTA, in shared memory: sum[id] = stretch lengths
+// from id to the end of its list, nx_out[id] = kNil where the list ends (all of
+// them, but for lists that close in a cycle, which keep a link).  Up to
+// kRankThreads - 1 evenly spaced samples and the primary split the lists; each
+// walks its piece (about 32 links at 1 MiB, a chain of shared loads), pointer
+// jumping ranks the pieces, and each walks its piece again to hand out the
+// sums (and to mark its samples as ended).  A block's one list that ends is
+// headed by the primary, so its pieces hold all of it.  For 64 blocks of 1 MiB 64
+// us, against 209 us in 16 launches of global jumps at half the samples.
+constexpr int kRankThreads = 1024;
+constexpr uint32_t kRankCap = kRankMax / 32 + 3;  // samples of a block
+constexpr uint32_t kRankEnd = 0xffffu;            // no link
+struct RankShared {
+    uint32_t len[kRankCap];  // a stretch's length, then its sum
+    uint16_t nxt[kRankCap];
+    uint32_t sum[2][kRankThreads];  // of the pieces
+    uint16_t to[2][kRankThreads];   // the splitter a piece ends at
+};
+
+__global__ void __launch_bounds__(kRankThreads) k_rank(const uint32_t *nxt, const uint32_t *len,
+                                                       Samples S, uint32_t *nx_out, uint32_t *sum_out,
+                                                       const int32_t *status)
+{
+    extern __shared__ __align__(16) unsigned char rank_sm[];
+    RankShared &sh = *reinterpret_cast<RankShared *>(rank_sm);
+    if (chain_failed(status))
+        return;
+    const uint32_t tid = threadIdx.x, b = blockIdx.x;
+    const uint32_t s = b * S.block, m = S.n - s < S.block ? S.n - s : S.block;
+    // the block's regular samples, then its primary's
+    const uint32_t first = (s + S.gap - 1) / S.gap;
+    const uint32_t regs = (s + m + S.gap - 1) / S.gap - first, count = regs + 1;
+    for (uint32_t i = tid; i < count; i += kRankThreads) {
+        const uint32_t id = i < regs ? first + i : S.regular + b;
+        const uint32_t to = nxt[id];
+        sh.len[i] = len[id];
+        sh.nxt[i] = (uint16_t)(to == kNil ? kRankEnd : to - first);  // a primary is never linked to
+    }
+    __syncthreads();
+    // splitters: the samples step, 2 step, ... and the primary (the last piece)
+    uint32_t step = 32;
+    while (regs && (regs - 1) / step + 1 > (uint32_t)kRankThreads)
+        step <<= 1;
+    const uint32_t pieces = (regs ? (regs - 1) / step : 0u) + 1;
+    const uint32_t own = tid + 1 < pieces ? (tid + 1) * step : regs;
+    auto split = [&](uint32_t i) { return i == regs || (i && (i & (step - 1)) == 0); };
+    uint32_t total = 0, at = own;
+    if (tid < pieces) {
+        uint32_t left = count;
+        do {
+            total += sh.len[at];
+            at = sh.nxt[at];
+        } while (at != kRankEnd && !split(at) && --left);
+        sh.sum[0][tid] = total;
+        sh.to[0][tid] = (uint16_t)(at == kRankEnd ? kRankEnd : at == regs ? pieces - 1 : at / step - 1);
+    }
+    __syncthreads();
+    uint32_t cur = 0;
+    for (uint32_t d = 1; d < pieces; d <<= 1, cur ^= 1) {
+        if (tid < pieces) {
+            const uint32_t t = sh.to[cur][tid];
+            sh.sum[cur ^ 1][tid] = sh.sum[cur][tid] + (t != kRankEnd ? sh.sum[cur][t] : 0u);
+            sh.to[cur ^ 1][tid] = t != kRankEnd ? sh.to[cur][t] : (uint16_t)kRankEnd;
+        }
+        __syncthreads();
+    }
+    // sums handed out along each piece of a list that ends
+    if (tid < pieces && sh.to[cur][tid] == kRankEnd) {
+        uint32_t rest = sh.sum[cur][tid], i = own;
+        do {
+            const uint32_t l = sh.len[i], j = sh.nxt[i];
+            sh.len[i] = rest;
+            rest -= l;
+            sh.nxt[i] = (uint16_t)kRankEnd;
+            i = j;
+        } while (i != kRankEnd && !split(i));
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < count; i += kRankThreads) {
+        const uint32_t id = i < regs ? first + i : S.regular + b;
+        nx_out[id] = sh.nxt[i] == kRankEnd ? kNil : 0u;
+        sum_out[id] = sh.len[i];
+    }
+}
+
+// Samples on their block's primary list put their bytes in place, last first:
+// the primary's sum is the cycle length c, a sample's distance from the
+// primary is c - its own sum.  A warp takes 32 samples, a lane each for their
+// numbers and all lanes for each one's bytes; a stretch longer than `cap` is
+// walked again.
+template <class T>
+__global__ void k_emit(const T *lf, Samples S, uint32_t count, uint32_t cap, const uint32_t *len,
+                       const uint32_t *nx, const uint32_t *sum, const uint8_t *kept, uint8_t *out,
+                       int32_t *status)
 {
     if (chain_failed(status))
         return;
-    for (uint32_t id = blockIdx.x * kEw + threadIdx.x; id < count; id += gridDim.x * kEw) {
-        const uint32_t L = len[id];
-        if (L == 0 || nx[id] != kNil)
-            continue;  // not a sample, or not on the primary's cycle
-        uint32_t p = S.row_of(id);
-        uint32_t s, m;
-        block_span(p, S.block, S.n, s, m);
-        const uint32_t c = sum[S.regular + p / S.block];
-        const uint32_t d = c - sum[id];
-        if (c > m || d + L > c) {
-            set_status(status, HUFF_ERR_CORRUPT_STREAM);
-            continue;
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint32_t i0 = (blockIdx.x * kEw + threadIdx.x) & ~31u; i0 < count; i0 += gridDim.x * kEw) {
+        const uint32_t id = i0 + lane;
+        uint32_t L = id < count ? len[id] : 0u;
+        if (L && nx[id] != kNil)
+            L = 0;  // not on the primary's cycle
+        uint32_t end = 0;  // the place of the first byte
+        if (L) {
+            const uint32_t p = S.row_of(id);
+            uint32_t s, m;
+            block_span(p, S.block, S.n, s, m);
+            const uint32_t c = sum[S.regular + p / S.block];
+            const uint32_t d = c - sum[id];
+            if (c > m || d + L > c) {
+                set_status(status, HUFF_ERR_CORRUPT_STREAM);
+                L = 0;
+            } else {
+                end = s + m - 1 - d;
+                if (L > cap) {
+                    uint32_t r = p - s;
+                    for (uint32_t t = 0; t < L; ++t) {
+                        const T v = lf[s + r];
+                        if (t >= cap)
+                            out[end - t] = (uint8_t)v;
+                        r = (uint32_t)(v >> 8);
+                    }
+                    L = cap;
+                }
+            }
         }
-        for (uint32_t t = 0; t < L && p < S.n; ++t) {
-            out[s + m - 1 - (d + t)] = last[p];
-            p = lf[p];
+        __syncwarp();
+        for (int j = 0; j < 32; j += 4) {  // four at a time: their loads in flight together
+            uint32_t Lj[4], ej[4], a[4], b[4];
+            const uint8_t *src[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                Lj[q] = __shfl_sync(0xffffffffu, L, j + q);
+                ej[q] = __shfl_sync(0xffffffffu, end, j + q);
+                src[q] = kept + (uint64_t)(i0 + j + q) * cap + lane;
+                a[q] = lane < Lj[q] ? src[q][0] : 0u;
+                b[q] = lane + 32 < Lj[q] ? src[q][32] : 0u;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (lane < Lj[q])
+                    out[ej[q] - lane] = (uint8_t)a[q];
+                if (lane + 32 < Lj[q])
+                    out[ej[q] - lane - 32] = (uint8_t)b[q];
+                for (uint32_t t = 64; t + lane < Lj[q]; t += 32)
+                    out[ej[q] - lane - t] = src[q][t];
+            }
         }
     }
 }
 
 // a block whose walk closed after c < m rows repeats its last c bytes
-__global__ void k_periodic_fill(uint8_t *out, uint32_t n, uint32_t block, uint32_t regular,
-                                const uint32_t *sum, const int32_t *status)
+__global__ void k_periodic_fill(uint8_t *out, uint32_t n, uint32_t block, uint32_t blocks,
+                                uint32_t regular, const uint32_t *sum, const int32_t *status)
 {
     if (chain_failed(status))
         return;
-    for (uint32_t q = blockIdx.x * kEw + threadIdx.x; q < n; q += gridDim.x * kEw) {
-        uint32_t s, m;
-        block_span(q, block, n, s, m);
-        const uint32_t c = sum[regular + q / block];
-        const uint32_t t = s + m - 1 - q;  // walk step of q
-        if (c < m && t >= c)
-            out[q] = out[s + m - 1 - t % c];
+    for (uint32_t b = blockIdx.x; b < blocks; b += gridDim.x) {
+        const uint32_t s = b * block, m = n - s < block ? n - s : block;
+        const uint32_t c = sum[regular + b];
+        for (uint32_t t = c + threadIdx.x; t < m; t += kEw)  // walk steps past the cycle
+            out[s + m - 1 - t] = out[s + m - 1 - t % c];
     }
 }
 
@@ -930,7 +1190,8 @@ struct InvWs {
 
 uint32_t sample_count(uint64_t n, uint32_t block)
 {
-    return (uint32_t)((n + kSampleGap - 1) / kSampleGap + (n + block - 1) / block);
+    const uint32_t gap = sample_gap(n < block ? n : block);
+    return (uint32_t)((n + gap - 1) / gap + (n + block - 1) / block);
 }
 
 InvWs inv_layout(uint8_t *base, uint64_t n, uint32_t block)
@@ -951,6 +1212,87 @@ InvWs inv_layout(uint8_t *base, uint64_t n, uint32_t block)
     w.radix = carve<uint8_t>(base, off, radix_scratch_bytes(n));
     w.bytes = off;
     return w;
+}
+
+// The inverse after the primary rows are checked, with LF words in `lf` (w.lf,
+// or w.k1 where they are 64 bits wide).  The bytes kept by the walks, at most
+// `cap` a sample (a multiple of 8 no larger than a block needs), lie from w.k0
+// on: S * cap bytes for the S samples, with a gap of 32 at most 16 n + 512
+// blocks of 4 KiB and more, with 64 at most 9 n + 1 KiB (24 n from w.k0 to the
+// end of w.v1), with 64-bit words 4 n + 256 blocks (8 n from w.k0 to w.k1).
+constexpr uint32_t kKept = 512;
+
+template <class T>
+bool invert(InvWs &w, const uint8_t *last, uint32_t n, uint32_t block, uint32_t blocks,
+            const uint32_t *d_primary, uint8_t *d_out, int32_t *d_status, T *lf, uint32_t cap,
+            cudaStream_t s)
+{
+    const uint32_t most = n < block ? n : block;  // of a block
+    if (most >= kLfTile) {
+        const uint32_t per = div_up(most, kLfTile);
+        const uint64_t tiles = (uint64_t)blocks * per;
+        uint32_t *hist = reinterpret_cast<uint32_t *>(w.k0);  // 1 KiB per tile: at most n / 2 and a block's
+        k_lf_count<<<(unsigned)tiles, kLfThreads, 0, s>>>(last, n, block, per, hist);
+        if (scan_u32(hist, hist, (uint32_t)(256 * tiles), false, w.v0, nullptr, s) != cudaSuccess)
+            return false;
+        k_lf_rank<T><<<(unsigned)tiles, kLfThreads, 0, s>>>(last, n, block, per, hist, lf);
+    } else {
+        k_lf_keys<<<ew_grid(n), kEw, 0, s>>>(last, n, block, w.k0, w.v0);
+        bool flip = false;
+        if (radix_sort_bits(w.k0, w.v0, w.k1, w.v1, n, 0, 8 + bit_width(blocks - 1), w.radix, s,
+                            flip) != cudaSuccess)
+            return false;
+        k_lf_scatter<<<ew_grid(n), kEw, 0, s>>>(flip ? w.k1 : w.k0, flip ? w.v1 : w.v0, n, block,
+                                                w.lf);  // (blocks this short have 32-bit words)
+    }
+    if (cap > ((most + 7) & ~7u))
+        cap = (most + 7) & ~7u;
+    uint8_t *const kept = reinterpret_cast<uint8_t *>(w.k0);
+    Samples S;
+    S.n = n;
+    S.block = block;
+    S.gap = sample_gap(most);
+    S.regular = (uint32_t)(((uint64_t)n + S.gap - 1) / S.gap);
+    S.primary = d_primary;
+    const uint32_t count = sample_count(n, block);
+    k_walk<T><<<ew_grid(count), kEw, 0, s>>>(lf, S, count, cap, w.nxt, w.len, kept, d_status);
+    uint32_t *nx = w.nxt, *sm = w.len;
+    if (S.gap == 32) {
+        static KernelSetup setup;
+        int per_sm = 0;
+        if (kernel_setup(setup, (const void *)k_rank, kRankThreads, sizeof(RankShared), &per_sm) !=
+            cudaSuccess)
+            return false;
+        k_rank<<<blocks, kRankThreads, sizeof(RankShared), s>>>(w.nxt, w.len, S, w.nx2, w.sum,
+                                                                d_status);
+        nx = w.nx2;
+        sm = w.sum;
+    } else {
+        // the longest list is one block's samples
+        const uint64_t per_block = (uint64_t)most / S.gap + 2;
+        const uint32_t rounds = bit_width(per_block) + 1;
+        uint32_t *nx_o = w.nx2, *sm_o = w.sum;
+        for (uint32_t r = 0; r < rounds; ++r) {
+            k_jump<<<ew_grid(count), kEw, 0, s>>>(nx, sm, count, nx_o, sm_o, d_status);
+            if (r == 0) {  // len stays; later steps ping-pong between sum and sum2
+                nx = nx_o;
+                sm = sm_o;
+                nx_o = w.nxt;
+                sm_o = w.sum2;
+            } else {
+                uint32_t *t = nx;
+                nx = nx_o;
+                nx_o = t;
+                t = sm;
+                sm = sm_o;
+                sm_o = t;
+            }
+        }
+    }
+    k_emit<T><<<ew_grid(count), kEw, 0, s>>>(lf, S, count, cap, w.len, nx, sm, kept, d_out, d_status);
+    k_periodic_fill<<<ew_grid((uint64_t)blocks * kEw), kEw, 0, s>>>(d_out, n, block, blocks, S.regular,
+                                                                    sm, d_status);
+    return true;
 }
 
 bool bwt_args_ok(uint64_t n, uint32_t block)
@@ -1071,42 +1413,13 @@ huff_status_t huff_bwt_inverse(const uint8_t *d_last, uint64_t n, uint32_t block
     InvWs w = inv_layout(static_cast<uint8_t *>(d_ws), n, block);
     const uint32_t blocks = (uint32_t)((n + block - 1) / block);
     k_check_primary<<<ew_grid(blocks), kEw, 0, s>>>(d_primary, N, block, blocks, d_status);
-    k_lf_keys<<<ew_grid(n), kEw, 0, s>>>(d_last, N, block, w.k0, w.v0);
-    bool flip = false;
-    if (radix_sort_bits(w.k0, w.v0, w.k1, w.v1, N, 0, 8 + bit_width(blocks - 1), w.radix, s, flip) !=
-        cudaSuccess)
+    const bool wide = block > kMaxBlock32 && n > kMaxBlock32;
+    const bool ok = wide ? invert(w, d_last, N, block, blocks, d_primary, d_out, d_status,
+                                  reinterpret_cast<uint64_t *>(w.k1), kKept / 2, s)
+                         : invert(w, d_last, N, block, blocks, d_primary, d_out, d_status, w.lf, kKept,
+                                  s);
+    if (!ok)
         return HUFF_ERR_CUDA;
-    k_lf_scatter<<<ew_grid(n), kEw, 0, s>>>(flip ? w.v1 : w.v0, N, w.lf);
-    Samples S;
-    S.n = N;
-    S.block = block;
-    S.regular = (uint32_t)((n + kSampleGap - 1) / kSampleGap);
-    S.primary = d_primary;
-    const uint32_t count = sample_count(n, block);
-    k_walk_link<<<ew_grid(count), kEw, 0, s>>>(w.lf, S, count, w.nxt, w.len, d_status);
-    // the longest list is one block's samples
-    const uint64_t per_block = (uint64_t)((n < block ? n : block) + kSampleGap - 1) / kSampleGap + 1;
-    const uint32_t rounds = bit_width(per_block) + 1;
-    uint32_t *nx = w.nxt, *sm = w.len, *nx_o = w.nx2, *sm_o = w.sum;
-    for (uint32_t r = 0; r < rounds; ++r) {
-        k_jump<<<ew_grid(count), kEw, 0, s>>>(nx, sm, count, nx_o, sm_o, d_status);
-        if (r == 0) {  // len stays; later steps ping-pong between sum and sum2
-            nx = nx_o;
-            sm = sm_o;
-            nx_o = w.nxt;
-            sm_o = w.sum2;
-        } else {
-            uint32_t *t = nx;
-            nx = nx_o;
-            nx_o = t;
-            t = sm;
-            sm = sm_o;
-            sm_o = t;
-        }
-    }
-    k_walk_emit<<<ew_grid(count), kEw, 0, s>>>(w.lf, d_last, S, count, w.len, nx, sm, d_out,
-                                              d_status);
-    k_periodic_fill<<<ew_grid(n), kEw, 0, s>>>(d_out, N, block, S.regular, sm, d_status);
     return cudaGetLastError() == cudaSuccess ? HUFF_OK : HUFF_ERR_CUDA;
 }
 

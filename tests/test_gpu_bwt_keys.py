@@ -39,3 +39,40 @@ def test_first_keys_against_oracle(sigma, block):
         assert int(st.item()) == 0
         assert np.array_equal(last.cpu().numpy(), ref_last), (n, off)
         assert np.array_equal(prim.cpu().numpy().astype(np.uint32), ref_prim), (n, off)
+
+
+# LF by tiles (blocks from 4 KiB) and by sorting (below), samples every 32 rows
+# ranked in shared memory (4 KiB..1 MiB) or every 64 by global jumps, walks of
+# a few rows to a whole block (periodic and constant blocks), blocks that do
+# not start at a sample
+@pytest.mark.parametrize("block", [4095, 4096, 4097, 8192, 33333, 1 << 20, (1 << 20) + 1])
+@pytest.mark.parametrize("kind", ["text", "constant", "periodic", "almost"])
+def test_inverse_against_input(block, kind):
+    n = 2 * block + 4100
+    x = {"text": lambda: synth.text(n, 3), "constant": lambda: np.full(n, 7, np.uint8),
+         "periodic": lambda: np.resize(np.frombuffer(b"abcab", np.uint8), n),
+         "almost": lambda: np.resize(np.frombuffer(b"abcab", np.uint8), n)}[kind]().copy()
+    if kind == "almost":
+        x[::block] = ord("z")  # one byte breaks each block's period
+    if n <= 70000:
+        last, prim = oracle.bwt(x, block)
+        L = torch.from_numpy(last).cuda()
+        P = torch.from_numpy(prim.astype(np.int32)).cuda()
+    else:  # (the oracle sorts a periodic block slowly)
+        L, P, st = hg.huff_bwt_forward(torch.from_numpy(x).cuda(), block)
+        assert int(st.item()) == 0
+    back, st = hg.huff_bwt_inverse(L, block, P)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    assert np.array_equal(back.cpu().numpy(), x)
+
+
+def test_blocks_beyond_16_mib():
+    """LF words of 64 bits."""
+    block = (1 << 24) + 33
+    x = torch.from_numpy(synth.text(block + 5000, 9)).cuda()
+    L, P, st = hg.huff_bwt_forward(x, block)
+    assert int(st.item()) == 0
+    back, st = hg.huff_bwt_inverse(L, block, P)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and torch.equal(back, x)
