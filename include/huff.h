@@ -243,7 +243,9 @@ typedef struct huff_batch_params {
     uint32_t decode_lanes;  /* decompress: lanes to spread a buffer over
                                (1..65536): its chunks are split into the
                                smallest power of two S <= 32 of sub-segments
-                               with chunks x S >= decode_lanes            */
+                               with chunks x S >= decode_lanes.  A batch with
+                               chunks for half the launch's lanes splits a
+                               buffer only as far as that saves idle lanes  */
     uint32_t use_graph;     /* capture the launch in a CUDA graph (1) or not  */
     uint32_t barrier_extra; /* test hook, 0 in use: nonzero makes the launch's
                                grid barriers wait for that many CTAs more than
@@ -296,7 +298,8 @@ huff_status_t huff_batch_info(const huff_batch_plan_t *plan, huff_batch_params_t
  * per segment); callers that must not allocate while they run keep a
  * persistent plan over the segments with huff_batch_plan / huff_batch_run.
  * Decompression spreads each segment over enough lanes that the whole
- * container fills about one wave of decoders (256 lanes per SM). */
+ * container fills about one wave of decoders (256 lanes per SM), 128 at
+ * least. */
 uint64_t huff_segmented_max_size(uint64_t n, uint64_t segment_bytes, uint32_t chunk_symbols);
 /* Device scratch of huff_segmented_compress: the streams in worst-case
  * slots, then per-segment sizes and statuses. */

@@ -18,8 +18,9 @@ constexpr int kHalfWarps = kBatchWarps / 2;
 constexpr int kUnitsPerItem = kHalfWarps;  // encode: one unit per warp of a half
 constexpr int kTasksPerItem = kHalfWarps;  // decode: one task per warp of a half
 
-// control words (device): barrier arrivals and generation, then tickets
-enum { kCtlArrive = 0, kCtlGen = 1, kCtlTicket0 = 2, kCtlWords = 8 };
+// control words (device): barrier arrivals and generation, then three tickets
+// and the lanes a buffer's decoding is spread over
+enum { kCtlArrive = 0, kCtlGen = 1, kCtlTicket0 = 2, kCtlLanes = 5, kCtlWords = 8 };
 
 struct BatchBuf {
     const uint8_t *in;

@@ -310,10 +310,13 @@ huff_status_t huff_segmented_decompress(const uint8_t *d_in, uint64_t in_bytes, 
     huff_batch_default_params(&prm);
     prm.use_graph = 0;
     // spread each segment over enough lanes that the whole container fills
-    // about one wave of decoders (256 lanes per SM, the single-stream rule)
+    // about one wave of decoders (256 lanes per SM, the single-stream rule),
+    // but over the 128 of an item's four warps at least: 64 MiB in 64 KiB
+    // segments 0.67 -> 0.60 ms (text) and 1.17 -> 0.85 ms (move-to-front
+    // coded) against 64 lanes
     {
         const uint64_t want = ((uint64_t)device_sm_count() * 256 + count - 1) / count;
-        uint32_t lanes = 32;
+        uint32_t lanes = 128;
         while (lanes < want && lanes < 65536)
             lanes <<= 1;
         prm.decode_lanes = lanes;

@@ -76,3 +76,30 @@ def test_cut_short_payloads_report_corruption():
                 x.size, dtype=torch.uint8, device="cuda"))
             torch.cuda.synchronize()
             assert int(st.item()) == ost, (kind, cut)
+
+
+@pytest.mark.parametrize("chunks", [1, 19, 33, 64, 100])
+def test_batches_that_fill_the_chip(chunks):
+    """Enough chunks that a buffer is split by what it costs, not by the lanes
+    asked for; the sizes differ, so the largest go first."""
+    cs = 4096  # (small chunks: the rule counts chunks)
+    lanes = torch.cuda.get_device_properties(0).multi_processor_count * 2 * 256
+    sizes = [cs * chunks - (37 * i) % cs for i in range(lanes // 2 // chunks + 200)]
+    sizes[7] = 1
+    x = torch.from_numpy(synth.text(2 * cs * chunks, 3)).cuda()
+    ins = [x[16 * (i % 50):16 * (i % 50) + n] for i, n in enumerate(sizes)]
+    prm = hg.huff_batch_default_params()
+    prm.chunk_symbols = cs
+    outs = [torch.zeros(hg.huff_max_stream_size(n, cs), dtype=torch.uint8, device="cuda")
+            for n in sizes]
+    plan = hg.BatchPlan(ins, outs, hg.HUFF_BATCH_COMPRESS, prm)
+    plan.run()
+    got = plan.out_bytes.tolist()
+    assert not any(plan.status.tolist())
+    back = [torch.zeros(n, dtype=torch.uint8, device="cuda") for n in sizes]
+    plan = hg.BatchPlan([o[:g] for o, g in zip(outs, got)], back, hg.HUFF_BATCH_DECOMPRESS)
+    plan.run()
+    assert not any(plan.status.tolist()) and plan.out_bytes.tolist() == sizes
+    assert all(torch.equal(a, b) for a, b in zip(ins, back))
+    one = oracle.compress(ins[-1].cpu().numpy(), cs)[1]
+    assert np.array_equal(outs[-1][:got[-1]].cpu().numpy(), one)
