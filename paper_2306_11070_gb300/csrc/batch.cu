@@ -738,6 +738,31 @@ huff_status_t batch_check(const huff_batch_desc_t *descs, uint32_t count, huff_o
     return HUFF_OK;
 }
 
+huff_status_t batch_once(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
+                         const huff_batch_params_t &prm, void *scratch, uint64_t scratch_bytes,
+                         std::vector<uint8_t> &host, cudaStream_t s, bool &ran)
+{
+    ran = false;
+    const huff_status_t st = batch_check(descs, count, op, prm);
+    if (st != HUFF_OK)
+        return st;
+    BatchLayout L;
+    batch_layout(descs, count, op, L);
+    if (!scratch || L.bytes > scratch_bytes)
+        return HUFF_OK;
+    const int per_sm = batch_occupancy(op);
+    if (per_sm < 1)
+        return HUFF_ERR_CUDA;
+    host.resize(L.upload_bytes);
+    if (batch_upload(L, scratch, host.data(), s) != cudaSuccess)
+        return HUFF_ERR_CUDA;
+    const BatchArgs args = batch_args(L, scratch, prm.chunk_symbols, prm.decode_lanes);
+    if (batch_launch(op, args, (unsigned)(device_sm_count() * per_sm), s) != cudaSuccess)
+        return HUFF_ERR_CUDA;
+    ran = true;
+    return HUFF_OK;
+}
+
 }  // namespace huff
 
 using namespace huff;

@@ -68,7 +68,26 @@ BatchArgs batch_args(const BatchLayout &L, void *d_block, uint32_t cs, uint32_t 
 cudaError_t batch_upload(const BatchLayout &L, void *d_block, uint8_t *host, cudaStream_t s);
 int batch_occupancy(huff_op_t op);
 cudaError_t batch_launch(huff_op_t op, const BatchArgs &args, unsigned grid, cudaStream_t s);
+// Run a batch once without a plan, its device block in `scratch` (16-byte
+// aligned); `ran` is false when the block does not fit there.  `host` is read
+// by the upload until the stream has passed it.
+huff_status_t batch_once(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
+                         const huff_batch_params_t &prm, void *scratch, uint64_t scratch_bytes,
+                         std::vector<uint8_t> &host, cudaStream_t s, bool &ran);
 huff_status_t batch_check(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
                           const huff_batch_params_t &prm);
+
+// huff_segmented_compress / huff_segmented_decompress for a caller with device
+// memory to spare: the batch's block (and decompression's per-segment words)
+// go into scratch[0, scratch_bytes) where they fit, so that nothing is
+// allocated.
+huff_status_t segmented_compress(const uint8_t *d_in, uint64_t n, uint64_t segment_bytes,
+                                 uint32_t chunk_symbols, uint8_t *d_out, uint64_t out_cap,
+                                 uint64_t *d_out_bytes, void *d_ws, uint64_t ws_bytes,
+                                 int32_t *d_status, cudaStream_t s, void *scratch,
+                                 uint64_t scratch_bytes);
+huff_status_t segmented_decompress(const uint8_t *d_in, uint64_t in_bytes, uint8_t *d_out,
+                                   uint64_t out_cap, uint64_t *d_n, int32_t *d_status,
+                                   cudaStream_t s, void *scratch, uint64_t scratch_bytes);
 
 }  // namespace huff

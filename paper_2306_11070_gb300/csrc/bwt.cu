@@ -34,6 +34,7 @@
 #include <cmath>
 
 #include "api_trace.h"
+#include "batch_internal.cuh"
 #include "sort_impl.cuh"
 
 namespace huff {
@@ -1473,9 +1474,14 @@ huff_status_t huff_m3_compress(const uint8_t *d_in, uint64_t n, uint32_t block,
     k_m3_header<<<1, 256, 0, s>>>(d_out, n, block, (uint32_t)count, stages, head);
     if (cudaGetLastError() != cudaSuccess)
         return HUFF_ERR_CUDA;
-    st = huff_segmented_compress(last, n, segment_bytes, chunk_symbols, d_out + head,
-                                 out_cap - head, d_out_bytes, rest, ws_bytes - (uint64_t)(rest - ws),
-                                 d_status, stream);
+    // the transform's workspace is free again: what the coder's leaves of it
+    // holds the batch's block, so that nothing is allocated
+    const uint64_t seg_ws =
+        (huff_segmented_workspace_size(n, segment_bytes, chunk_symbols) + 255) & ~255ull;
+    st = segmented_compress(last, n, segment_bytes, chunk_symbols, d_out + head, out_cap - head,
+                            d_out_bytes, rest, rest_bytes, d_status, s,
+                            seg_ws < rest_bytes ? rest + seg_ws : nullptr,
+                            seg_ws < rest_bytes ? rest_bytes - seg_ws : 0);
     if (st != HUFF_OK)
         return st;
     k_add_u64<<<1, 1, 0, s>>>(reinterpret_cast<unsigned long long *>(d_out_bytes), head, d_status);
@@ -1540,8 +1546,9 @@ huff_status_t huff_m3_decompress(const uint8_t *d_in, uint64_t in_bytes, uint8_t
     uint8_t *ws = static_cast<uint8_t *>(d_ws);
     uint8_t *last = ws;
     uint8_t *rest = ws + ((n + 255) & ~255ull);
-    huff_status_t st = huff_segmented_decompress(d_in + head, in_bytes - head, last, n, d_n,
-                                                 d_status, stream);
+    const uint64_t rest_bytes = ws_bytes - (uint64_t)(rest - ws);
+    huff_status_t st = segmented_decompress(d_in + head, in_bytes - head, last, n, d_n, d_status, s,
+                                            rest, rest_bytes);
     if (st != HUFF_OK)
         return st;
     // the segmented container must hold exactly n bytes
@@ -1560,7 +1567,6 @@ huff_status_t huff_m3_decompress(const uint8_t *d_in, uint64_t in_bytes, uint8_t
             return HUFF_ERR_CUDA;
         return HUFF_OK;
     }
-    const uint64_t rest_bytes = ws_bytes - (uint64_t)(rest - ws);
     if (stages & HUFF_M3_MTF) {
         st = huff_mtf_inverse(last, n, block, last, rest, rest_bytes, stream);
         if (st != HUFF_OK)

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "api_trace.h"
+#include "batch_internal.cuh"
 #include "huff_internal.cuh"
 
 namespace huff {
@@ -169,41 +170,18 @@ huff_status_t put_status(int32_t *d_status, int32_t v, cudaStream_t s)
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace
-}  // namespace huff
 
-using namespace huff;
-
-extern "C" {
-
-uint64_t huff_segmented_max_size(uint64_t n, uint64_t segment_bytes, uint32_t chunk_symbols)
+huff_status_t segmented_compress(const uint8_t *d_in, uint64_t n, uint64_t segment_bytes,
+                                 uint32_t chunk_symbols, uint8_t *d_out, uint64_t out_cap,
+                                 uint64_t *d_out_bytes, void *d_ws, uint64_t ws_bytes,
+                                 int32_t *d_status, cudaStream_t s, void *scratch,
+                                 uint64_t scratch_bytes)
 {
-    SegLayout L;
-    if (!seg_layout(n, segment_bytes, chunk_symbols, L))
-        return 0;
-    uint64_t total = L.header;
-    for (uint64_t i = 0; i < L.count; ++i)
-        total += al16(huff_max_stream_size(i + 1 < L.count ? segment_bytes : L.last, chunk_symbols));
-    return total;
-}
-
-uint64_t huff_segmented_workspace_size(uint64_t n, uint64_t segment_bytes, uint32_t chunk_symbols)
-{
-    SegLayout L;
-    return seg_layout(n, segment_bytes, chunk_symbols, L) ? L.ws_bytes : 0;
-}
-
-huff_status_t huff_segmented_compress(const uint8_t *d_in, uint64_t n, uint64_t segment_bytes,
-                                      uint32_t chunk_symbols, uint8_t *d_out, uint64_t out_cap,
-                                      uint64_t *d_out_bytes, void *d_ws, uint64_t ws_bytes,
-                                      int32_t *d_status, huff_stream_t stream)
-{
-    HUFF_API_RANGE("huff_segmented_compress");
     SegLayout L;
     if (!seg_layout(n, segment_bytes, chunk_symbols, L) || !d_out || !d_out_bytes || !d_status ||
         (n && !d_in) || !d_ws || ws_bytes < L.ws_bytes || out_cap < L.header ||
         (d_in && !aligned16(d_in)) || !aligned16(d_out) || !aligned16(d_ws))
         return HUFF_ERR_INVALID_ARG;
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     uint8_t *ws = static_cast<uint8_t *>(d_ws);
     uint64_t *sizes = reinterpret_cast<uint64_t *>(ws + L.sizes_off);
     int32_t *sts = reinterpret_cast<int32_t *>(ws + L.status_off);
@@ -223,14 +201,19 @@ huff_status_t huff_segmented_compress(const uint8_t *d_in, uint64_t n, uint64_t 
         huff_batch_default_params(&prm);
         prm.chunk_symbols = chunk_symbols;
         prm.use_graph = 0;  // one run
-        huff_batch_plan_t *plan = nullptr;
         if (L.count > 0xffffffffull)
             return HUFF_ERR_INVALID_ARG;
-        huff_status_t st = huff_batch_plan(descs.data(), (uint32_t)L.count, HUFF_BATCH_COMPRESS,
-                                           &prm, &plan);
-        if (st == HUFF_OK)
-            st = huff_batch_run(plan, stream);
-        if (st == HUFF_OK && cudaStreamSynchronize(s) != cudaSuccess)
+        bool ran = false;
+        std::vector<uint8_t> host;
+        huff_batch_plan_t *plan = nullptr;
+        huff_status_t st = batch_once(descs.data(), (uint32_t)L.count, HUFF_BATCH_COMPRESS, prm,
+                                      scratch, scratch_bytes, host, s, ran);
+        if (st == HUFF_OK && !ran) {
+            st = huff_batch_plan(descs.data(), (uint32_t)L.count, HUFF_BATCH_COMPRESS, &prm, &plan);
+            if (st == HUFF_OK)
+                st = huff_batch_run(plan, reinterpret_cast<huff_stream_t>(s));
+        }
+        if (cudaStreamSynchronize(s) != cudaSuccess && st == HUFF_OK)
             st = HUFF_ERR_CUDA;
         huff_batch_destroy(plan);
         if (st != HUFF_OK)
@@ -250,14 +233,12 @@ huff_status_t huff_segmented_compress(const uint8_t *d_in, uint64_t n, uint64_t 
     return HUFF_OK;
 }
 
-huff_status_t huff_segmented_decompress(const uint8_t *d_in, uint64_t in_bytes, uint8_t *d_out,
-                                        uint64_t out_cap, uint64_t *d_n, int32_t *d_status,
-                                        huff_stream_t stream)
+huff_status_t segmented_decompress(const uint8_t *d_in, uint64_t in_bytes, uint8_t *d_out,
+                                   uint64_t out_cap, uint64_t *d_n, int32_t *d_status,
+                                   cudaStream_t s, void *scratch, uint64_t scratch_bytes)
 {
-    HUFF_API_RANGE("huff_segmented_decompress");
     if (!d_in || !d_n || !d_status || !aligned16(d_in) || (out_cap && !d_out))
         return HUFF_ERR_INVALID_ARG;
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess)
         return HUFF_ERR_CUDA;
     if (in_bytes < 32)
@@ -292,11 +273,15 @@ huff_status_t huff_segmented_decompress(const uint8_t *d_in, uint64_t in_bytes, 
         return put_status(d_status, HUFF_ERR_CORRUPT_STREAM, s);
     if (!aligned16(d_out))
         return HUFF_ERR_INVALID_ARG;
-    uint8_t *scratch = nullptr;
-    if (cudaMalloc(&scratch, 12 * count + 16) != cudaSuccess)
+    // sizes and statuses of the segments, then the batch's block
+    const uint64_t words = (12 * count + 15) & ~15ull;
+    const bool spare = scratch && words < scratch_bytes;
+    uint8_t *own = nullptr;
+    if (!spare && cudaMalloc(&own, words) != cudaSuccess)
         return HUFF_ERR_CUDA;
-    uint64_t *got = reinterpret_cast<uint64_t *>(scratch);
-    int32_t *sts = reinterpret_cast<int32_t *>(scratch + 8 * count);
+    uint8_t *const mem = spare ? static_cast<uint8_t *>(scratch) : own;
+    uint64_t *got = reinterpret_cast<uint64_t *>(mem);
+    int32_t *sts = reinterpret_cast<int32_t *>(mem + 8 * count);
     std::vector<huff_batch_desc_t> descs(count);
     for (uint64_t i = 0; i < count; ++i) {
         descs[i].d_in = d_in + start[i];
@@ -322,14 +307,20 @@ huff_status_t huff_segmented_decompress(const uint8_t *d_in, uint64_t in_bytes, 
         prm.decode_lanes = lanes;
     }
     huff_batch_plan_t *plan = nullptr;
-    huff_status_t st = huff_batch_plan(descs.data(), (uint32_t)count, HUFF_BATCH_DECOMPRESS, &prm,
-                                       &plan);
+    bool ran = false;
+    std::vector<uint8_t> host;
+    huff_status_t st = batch_once(descs.data(), (uint32_t)count, HUFF_BATCH_DECOMPRESS, prm,
+                                  spare ? mem + words : nullptr, spare ? scratch_bytes - words : 0,
+                                  host, s, ran);
+    if (st == HUFF_OK && !ran) {
+        st = huff_batch_plan(descs.data(), (uint32_t)count, HUFF_BATCH_DECOMPRESS, &prm, &plan);
+        if (st == HUFF_OK)
+            st = huff_batch_run(plan, reinterpret_cast<huff_stream_t>(s));
+    }
     if (st == HUFF_ERR_INVALID_ARG) {  // descriptors taken from a malformed table
-        cudaFree(scratch);
+        cudaFree(own);
         return put_status(d_status, HUFF_ERR_CORRUPT_STREAM, s);
     }
-    if (st == HUFF_OK)
-        st = huff_batch_run(plan, stream);
     if (st == HUFF_OK) {
         k_seg_check<<<1, kSegBlock, 0, s>>>(got, sts, count, n, seg, d_status);
         if (cudaGetLastError() != cudaSuccess)
@@ -338,8 +329,51 @@ huff_status_t huff_segmented_decompress(const uint8_t *d_in, uint64_t in_bytes, 
     if (cudaStreamSynchronize(s) != cudaSuccess && st == HUFF_OK)
         st = HUFF_ERR_CUDA;
     huff_batch_destroy(plan);
-    cudaFree(scratch);
+    cudaFree(own);
     return st;
+}
+
+}  // namespace huff
+
+using namespace huff;
+
+extern "C" {
+
+uint64_t huff_segmented_max_size(uint64_t n, uint64_t segment_bytes, uint32_t chunk_symbols)
+{
+    SegLayout L;
+    if (!seg_layout(n, segment_bytes, chunk_symbols, L))
+        return 0;
+    uint64_t total = L.header;
+    for (uint64_t i = 0; i < L.count; ++i)
+        total += al16(huff_max_stream_size(i + 1 < L.count ? segment_bytes : L.last, chunk_symbols));
+    return total;
+}
+
+uint64_t huff_segmented_workspace_size(uint64_t n, uint64_t segment_bytes, uint32_t chunk_symbols)
+{
+    SegLayout L;
+    return seg_layout(n, segment_bytes, chunk_symbols, L) ? L.ws_bytes : 0;
+}
+
+huff_status_t huff_segmented_compress(const uint8_t *d_in, uint64_t n, uint64_t segment_bytes,
+                                      uint32_t chunk_symbols, uint8_t *d_out, uint64_t out_cap,
+                                      uint64_t *d_out_bytes, void *d_ws, uint64_t ws_bytes,
+                                      int32_t *d_status, huff_stream_t stream)
+{
+    HUFF_API_RANGE("huff_segmented_compress");
+    return segmented_compress(d_in, n, segment_bytes, chunk_symbols, d_out, out_cap, d_out_bytes,
+                              d_ws, ws_bytes, d_status, reinterpret_cast<cudaStream_t>(stream),
+                              nullptr, 0);
+}
+
+huff_status_t huff_segmented_decompress(const uint8_t *d_in, uint64_t in_bytes, uint8_t *d_out,
+                                        uint64_t out_cap, uint64_t *d_n, int32_t *d_status,
+                                        huff_stream_t stream)
+{
+    HUFF_API_RANGE("huff_segmented_decompress");
+    return segmented_decompress(d_in, in_bytes, d_out, out_cap, d_n, d_status,
+                                reinterpret_cast<cudaStream_t>(stream), nullptr, 0);
 }
 
 }  // extern "C"
