@@ -34,6 +34,7 @@
 // that overlaps the bits being produced repeats with the match distance as
 // its period).  Very many segments are decoded by a thread each instead.
 #include <cstdint>
+#include <type_traits>
 
 #include "api_trace.h"
 #include "huff_internal.cuh"
@@ -316,64 +317,67 @@ struct WarpOut {
     }
 };
 
-// Windows of 64..16384 bits: one warp per segment, the window in a ring in
-// shared memory.  Bound by the latency of one token's steps (a warp alone
-// issues about every 4.5 cycles; at 64 KiB segments an SM holds 7) and, from
-// some 4000 segments on, by instruction issue.  64 MiB of the bitstream
-// stand-in with 1024/12/24/8: 19.1 -> 4.4 ms in 64 KiB segments, 13.1 -> 2.4
-// ms in 16 KiB, 10.4 -> 1.9 ms in 4 KiB (before: one candidate a lane and
-// step); W = 4096 in 16 KiB segments 40.9 -> 4.6 ms.  With Lmin's steps not
-// straight-line (a run-time bound on each) it took 7.0 ms.  Where the bits ahead repeat the bit
-// before them (a zero run), distance 1 gives the longest match there is and
-// no distance is smaller: all the tokens of the run that the ring shows (up
-// to 1024 bits) are written at once, as the repeating words they form.
-template <int G0>
-__global__ void __launch_bounds__(32)
-    k_lzss_compress_ring(const uint8_t *__restrict__ in, uint64_t n, uint64_t seg, LzParams P,
-                         uint8_t *__restrict__ slots, uint32_t *__restrict__ bits_out,
-                         const int32_t *status)
-{
-    if (chain_failed(status))
-        return;
-    extern __shared__ uint32_t ring[];
-    const int lane = threadIdx.x;
-    const uint64_t count = n ? (n + seg - 1) / seg : 0;
-    const uint64_t sbytes = slot_bytes(seg, P);
-    const uint32_t R = ring_words(P.W), dwords = P.W / 32, passes = (P.W + 1023) / 1024;
-    const uint32_t len_ref = 1 + P.ob + P.lb, run_bits = 32 - P.lmax;
-    const uint32_t lit_mask = P.blk < 31 ? ~(0x7fffffffu >> P.blk) : ~0u;  // of a literal's token
-    // the token of a run: distance 1, the longest length; and its repetition
-    uint64_t run_rep = (uint64_t)(0x80000000u | ((P.lmax - P.lmin) << (32 - len_ref))) << 32;
-    for (uint32_t k = len_ref; k < 64; k <<= 1)
-        run_rep |= run_rep >> k;
-    // x / len_ref and x / lmax as x * inv >> 20: exact up to 2^20 / 32
-    const uint32_t inv_ref = ((1u << 20) + len_ref - 1) / len_ref;
-    const uint32_t inv_max = ((1u << 20) + P.lmax - 1) / P.lmax;
-    for (uint64_t s = blockIdx.x; s < count; s += gridDim.x) {
-        const uint8_t *x = in + s * seg;
-        const uint32_t m = (uint32_t)(s + 1 < count ? seg : n - s * seg);
-        const uint32_t nbits = 8 * m;
-        WarpOut out;
-        out.top = out.n = out.word = 0;
-        out.out = reinterpret_cast<uint32_t *>(slots + s * sbytes);
-        uint32_t p = 0;
-        if (P.dict == 2) {  // the first W bits as they are
-            const uint32_t raw = nbits < P.W ? nbits : P.W;
-            for (uint32_t q = lane; q < raw / 32; q += 32)
-                out.out[q] = bswap32(seg_word(x, m, q));
-            out.word = raw / 32;
-            out.n = raw & 31u;
-            out.top = out.n ? seg_word(x, m, raw / 32) & ~(0xffffffffu >> out.n) : 0u;
-            p = raw;
-        }
+// One warp's coder for windows of 64..16384 bits, the window in a ring in shared
+// memory.  A token depends on its position alone (the window holds the data
+// itself), so coding may begin anywhere in a segment.  Where the bits ahead
+// repeat the bit before them (a zero run), distance 1 gives the longest match
+// there is and no distance is smaller: all the tokens of the run that the
+// ring shows (up to 1024 bits) are written at once, as the repeating words
+// they form.
+struct Coder {
+    LzParams P;
+    uint32_t *ring;
+    uint32_t R, dwords, passes, len_ref, lit_mask;
+    uint64_t run_rep;  // the token of a run (distance 1, the longest length), repeated
+    uint32_t inv_ref, inv_max;  // x / len_ref, x / lmax as x * inv >> 20: exact up to 2^20 / 32
+    const uint8_t *x;  // the segment
+    uint32_t m, nbits;
+    __device__ __forceinline__ void init(const LzParams &P_, uint32_t *ring_)
+    {
+        P = P_;
+        ring = ring_;
+        R = ring_words(P.W);
+        dwords = P.W / 32;
+        passes = (P.W + 1023) / 1024;
+        len_ref = 1 + P.ob + P.lb;
+        lit_mask = P.blk < 31 ? ~(0x7fffffffu >> P.blk) : ~0u;
+        run_rep = (uint64_t)(0x80000000u | ((P.lmax - P.lmin) << (32 - len_ref))) << 32;
+        for (uint32_t k = len_ref; k < 64; k <<= 1)
+            run_rep |= run_rep >> k;
+        inv_ref = ((1u << 20) + len_ref - 1) / len_ref;
+        inv_max = ((1u << 20) + P.lmax - 1) / P.lmax;
+    }
+    // bits stored as they are before the first token
+    __device__ __forceinline__ uint32_t raw() const
+    {
+        return P.dict != 2 ? 0u : nbits < P.W ? nbits : P.W;
+    }
+    __device__ __forceinline__ void put_raw(WarpOut &out, int lane) const
+    {
+        const uint32_t p = raw();
+        for (uint32_t q = lane; q < p / 32; q += 32)
+            out.out[q] = bswap32(seg_word(x, m, q));
+        out.word = p / 32;
+        out.n = p & 31u;
+        out.top = out.n ? seg_word(x, m, p / 32) & ~(0xffffffffu >> out.n) : 0u;
+    }
+    // Code from bit p up to the first token that ends at or past `stop`, whose
+    // end is returned; before(p) is asked ahead of every token (of a run, its
+    // first) and ends the coding when true.
+    template <int G0, class F>
+    __device__ __forceinline__ uint32_t code(uint32_t p, uint32_t stop, WarpOut &out, int lane,
+                                             F before) const
+    {
+        const uint32_t run_bits = 32 - P.lmax;
         // ring: words [hw - R, hw) of "dictionary ++ segment" (bit v = W + p);
         // pre: the next batch, loaded ahead
+        __syncwarp();
         uint32_t hw = p >> 5;
         uint32_t pre[kRingBatch / 32];
 #pragma unroll
         for (int k = 0; k < (int)kRingBatch / 32; ++k)
             pre[k] = vword(x, m, dwords, hw + 32 * k + lane);
-        while (p < nbits) {
+        while (p < stop && !before(p)) {
             const uint32_t v = P.W + p, q = v >> 5, sh = v & 31u;
             if (hw < q + 34) {
                 do {
@@ -398,8 +402,8 @@ __global__ void __launch_bounds__(32)
             if (((X ^ prev) >> run_bits) == 0 && r >= P.lmax) {
                 const uint32_t *const z = ring + ((q + lane) & (R - 1));
                 const uint32_t diff = __funnelshift_l(z[1], z[0], sh) ^ prev;
-                const uint32_t stop = __ballot_sync(0xffffffffu, diff != 0);
-                const int f = stop ? __ffs(stop) - 1 : 31;
+                const uint32_t other = __ballot_sync(0xffffffffu, diff != 0);
+                const int f = other ? __ffs(other) - 1 : 31;
                 uint32_t run = 32 * f + __shfl_sync(0xffffffffu, (uint32_t)__clz(diff), f);
                 run = run < r ? run : r;
                 const uint32_t k = run * inv_max >> 20;  // tokens, 1..1024
@@ -425,9 +429,10 @@ __global__ void __launch_bounds__(32)
             const uint32_t maxlen = r < P.lmax ? r : P.lmax;
             uint32_t len = 0, dm1 = 0;
             if (maxlen >= P.lmin) {
-                uint32_t key = search_masks<G0>(__funnelshift_l(w1, w0, sh), __funnelshift_l(w2, w1, sh),
-                                            lane < (int)dwords ? 0xffffffffu : 0u, X, P.lmin, maxlen,
-                                            lane);
+                uint32_t key = search_masks<G0>(__funnelshift_l(w1, w0, sh),
+                                                __funnelshift_l(w2, w1, sh),
+                                                lane < (int)dwords ? 0xffffffffu : 0u, X, P.lmin,
+                                                maxlen, lane);
                 if (key) {
                     len = key >> 10;
                     dm1 = 1023 - (key & 1023u);
@@ -435,8 +440,8 @@ __global__ void __launch_bounds__(32)
                 for (uint32_t k = 1; k < passes && len < maxlen; ++k) {
                     const uint32_t *const w = ring + ((q - 32 * k - lane - 1) & (R - 1));
                     key = search_masks<G0>(__funnelshift_l(w[1], w[0], sh),
-                                       __funnelshift_l(w[2], w[1], sh), 0xffffffffu, X,
-                                       len ? len + 1 : P.lmin, maxlen, lane);
+                                           __funnelshift_l(w[2], w[1], sh), 0xffffffffu, X,
+                                           len ? len + 1 : P.lmin, maxlen, lane);
                     if (key) {  // longer than any nearer one
                         len = key >> 10;
                         dm1 = 1024 * k + 1023 - (key & 1023u);
@@ -458,6 +463,39 @@ __global__ void __launch_bounds__(32)
                 p += k;
             }
         }
+        return p;
+    }
+};
+
+// Windows of 64..16384 bits, one warp per segment.  Bound by the latency of one
+// token's steps (a warp alone issues about every 4.5 cycles) and, from some
+// 8000 warps on, by instruction issue.  64 MiB of the bitstream stand-in with
+// 1024/12/24/8: 13.1 -> 2.4 ms in 16 KiB segments, 10.4 -> 1.9 ms in 4 KiB
+// (before: one candidate a lane and step); W = 4096 in 16 KiB segments 40.9 ->
+// 4.6 ms.  With Lmin's steps not straight-line (a run-time bound on each) it
+// took half as long again.
+template <int G0>
+__global__ void __launch_bounds__(32)
+    k_lzss_compress_ring(const uint8_t *__restrict__ in, uint64_t n, uint64_t seg, LzParams P,
+                         uint8_t *__restrict__ slots, uint32_t *__restrict__ bits_out,
+                         const int32_t *status)
+{
+    if (chain_failed(status))
+        return;
+    extern __shared__ uint32_t ring[];
+    const int lane = threadIdx.x;
+    const uint64_t count = n ? (n + seg - 1) / seg : 0;
+    const uint64_t sbytes = slot_bytes(seg, P);
+    Coder cd;
+    cd.init(P, ring);
+    for (uint64_t s = blockIdx.x; s < count; s += gridDim.x) {
+        cd.x = in + s * seg;
+        cd.m = (uint32_t)(s + 1 < count ? seg : n - s * seg);
+        cd.nbits = 8 * cd.m;
+        WarpOut out;
+        out.out = reinterpret_cast<uint32_t *>(slots + s * sbytes);
+        cd.put_raw(out, lane);
+        cd.code<G0>(cd.raw(), cd.nbits, out, lane, [](uint32_t) { return false; });
         if (lane == 0) {  // the last word and zeros up to the slot's 16-byte boundary
             uint32_t w = out.word;
             if (out.n)
@@ -466,7 +504,213 @@ __global__ void __launch_bounds__(32)
                 out.out[w++] = 0u;
             bits_out[s] = out.word * 32 + out.n;
         }
-        __syncwarp();
+    }
+}
+
+// Few segments leave most of the chip idle, so a segment is coded in `parts` by
+// a warp each.  A part begins at its cut whether or not a token does; since a
+// token depends on its position alone, its code is right from the first of
+// its tokens that begins where one of the segment's tokens does (chains of
+// tokens from two starts meet after some tens of them, not counting runs).
+// k_lzss_parts codes the parts, noting kMarks places where a token begins, the
+// first kDense and then one in kSparse; k_lzss_join,
+// a warp per segment, takes the parts in order: from where the one before
+// ended it codes on until it meets a noted token (or, if it meets none, to the
+// part's end); k_lzss_gather_parts puts the pieces together bit by bit.
+// In a segment's slot, part k from byte k * stride on: {end, code bits, marks,
+// 0}, the code, the bits before the meeting point, the marks
+// {position, code bits before}.  Part 0 is right as it is; its marks' place
+// holds the pieces {first bit in the slot, bits}, 2 per part.
+constexpr uint32_t kMarks = 128, kDense = 96, kSparse = 16, kMaxParts = 8;
+constexpr uint32_t kMinPart = 4096;  // bytes
+struct PartsLayout {
+    uint32_t parts;               // of a segment
+    uint32_t code, head, stride;  // bytes of a part's code, its head, a part
+};
+
+__device__ __forceinline__ uint32_t part_cut(const Coder &cd, uint32_t parts, uint32_t k)
+{
+    const uint32_t raw = cd.raw();
+    return raw + (uint32_t)((uint64_t)(cd.nbits - raw) * k / parts);
+}
+
+template <int G0>
+__global__ void __launch_bounds__(32)
+    k_lzss_parts(const uint8_t *__restrict__ in, uint64_t n, uint64_t seg, LzParams P, PartsLayout L,
+                 uint8_t *__restrict__ slots, const int32_t *status)
+{
+    if (chain_failed(status))
+        return;
+    extern __shared__ uint32_t ring[];
+    const int lane = threadIdx.x;
+    const uint64_t count = n ? (n + seg - 1) / seg : 0;
+    const uint64_t sbytes = slot_bytes(seg, P);
+    Coder cd;
+    cd.init(P, ring);
+    for (uint64_t i = blockIdx.x; i < count * L.parts; i += gridDim.x) {
+        const uint64_t s = i / L.parts;
+        const uint32_t k = (uint32_t)(i - s * L.parts);
+        cd.x = in + s * seg;
+        cd.m = (uint32_t)(s + 1 < count ? seg : n - s * seg);
+        cd.nbits = 8 * cd.m;
+        uint8_t *const part = slots + s * sbytes + (uint64_t)k * L.stride;
+        uint2 *const marks = reinterpret_cast<uint2 *>(part + 16 + L.code + L.head);
+        WarpOut out;
+        out.out = reinterpret_cast<uint32_t *>(part + 16);
+        out.top = out.n = out.word = 0;
+        if (k == 0)
+            cd.put_raw(out, lane);
+        uint32_t nm = k == 0 ? kMarks : 0, skip = 0;
+        const uint32_t end = cd.code<G0>(part_cut(cd, L.parts, k), part_cut(cd, L.parts, k + 1), out,
+                                         lane, [&](uint32_t p) {
+                                             if (nm < kMarks && skip-- == 0) {
+                                                 if (lane == 0)
+                                                     marks[nm] = make_uint2(p, 32 * out.word + out.n);
+                                                 skip = ++nm < kDense ? 0 : kSparse - 1;
+                                             }
+                                             return false;
+                                         });
+        if (lane == 0) {
+            if (out.n)
+                out.out[out.word] = bswap32(out.top);
+            *reinterpret_cast<uint4 *>(part) =
+                make_uint4(end, 32 * out.word + out.n, k == 0 ? 0u : nm, 0u);
+        }
+    }
+}
+
+template <int G0>
+__global__ void __launch_bounds__(32)
+    k_lzss_join(const uint8_t *__restrict__ in, uint64_t n, uint64_t seg, LzParams P, PartsLayout L,
+                uint8_t *__restrict__ slots, uint32_t *__restrict__ bits_out, const int32_t *status)
+{
+    if (chain_failed(status))
+        return;
+    extern __shared__ uint32_t ring[];
+    const int lane = threadIdx.x;
+    const uint64_t count = n ? (n + seg - 1) / seg : 0;
+    const uint64_t sbytes = slot_bytes(seg, P);
+    Coder cd;
+    cd.init(P, ring);
+    // bits of a head that a step may begin at: a run's tokens still fit
+    const uint32_t head_bits = 8 * L.head - 1024 / P.lmax * cd.len_ref - 96;
+    for (uint64_t s = blockIdx.x; s < count; s += gridDim.x) {
+        cd.x = in + s * seg;
+        cd.m = (uint32_t)(s + 1 < count ? seg : n - s * seg);
+        cd.nbits = 8 * cd.m;
+        uint8_t *const slot = slots + s * sbytes;
+        uint2 *const pieces = reinterpret_cast<uint2 *>(slot + 16 + L.code + L.head);
+        const uint4 first = *reinterpret_cast<const uint4 *>(slot);
+        uint32_t p = first.x, total = first.y;
+        if (lane < 2)
+            pieces[lane] = lane ? make_uint2(0, 0) : make_uint2(8 * 16, first.y);
+        for (uint32_t k = 1; k < L.parts; ++k) {
+            const uint32_t stop = part_cut(cd, L.parts, k + 1);
+            const uint32_t at = k * L.stride;  // bytes
+            uint2 head = make_uint2(0, 0), tail = make_uint2(0, 0);
+            if (p < stop) {
+                const uint4 part = *reinterpret_cast<const uint4 *>(slot + at);
+                const uint2 *const marks =
+                    reinterpret_cast<const uint2 *>(slot + at + 16 + L.code + L.head);
+                WarpOut out;
+                out.out = reinterpret_cast<uint32_t *>(slot + at + 16 + L.code);
+                out.top = out.n = out.word = 0;
+                uint32_t base = 0;  // lane's mark: base + lane
+                uint2 mark = lane < part.z ? marks[lane] : make_uint2(0xffffffffu, 0);
+                bool met = false, lost = false;
+                const uint32_t end = cd.code<G0>(p, stop, out, lane, [&](uint32_t at_bit) {
+                    uint32_t hit;
+                    for (;;) {
+                        hit = __ballot_sync(0xffffffffu, mark.x == at_bit);
+                        if (hit || __any_sync(0xffffffffu, mark.x > at_bit))
+                            break;
+                        base += 32;
+                        if (base >= part.z)
+                            break;
+                        mark = base + lane < part.z ? marks[base + lane] : make_uint2(0xffffffffu, 0);
+                    }
+                    met = hit != 0;
+                    lost = !met && (base >= part.z || 32 * out.word + out.n > head_bits);
+                    if (met)
+                        tail.x = __shfl_sync(0xffffffffu, mark.y, __ffs(hit) - 1);
+                    return met || lost;
+                });
+                if (lost) {  // the whole part again, over its code
+                    out.out = reinterpret_cast<uint32_t *>(slot + at + 16);
+                    out.top = out.n = out.word = 0;
+                    p = cd.code<G0>(p, stop, out, lane, [](uint32_t) { return false; });
+                    head = make_uint2(8 * (at + 16), 32 * out.word + out.n);
+                } else {
+                    head = make_uint2(8 * (at + 16 + L.code), 32 * out.word + out.n);
+                    p = met ? part.x : end;
+                    if (met)
+                        tail = make_uint2(8 * (at + 16) + tail.x, part.y - tail.x);
+                }
+                if (lane == 0 && out.n)
+                    out.out[out.word] = bswap32(out.top);
+            }
+            if (lane < 2)
+                pieces[2 * k + lane] = lane ? tail : head;
+            total += head.y + tail.y;
+        }
+        if (lane == 0)
+            bits_out[s] = total;
+    }
+}
+
+// Every segment's pieces to its place, zero padded to the 16-byte boundary.
+__global__ void __launch_bounds__(256)
+    k_lzss_gather_parts(uint64_t n, uint64_t seg, LzParams P, PartsLayout L,
+                        const uint8_t *__restrict__ slots, const uint32_t *__restrict__ bits,
+                        const uint64_t *__restrict__ start, uint8_t *__restrict__ out, uint64_t cap,
+                        const int32_t *status)
+{
+    __shared__ uint2 piece[2 * kMaxParts];       // first bit in the slot, first bit of the code
+    __shared__ uint32_t first[2 * kMaxParts + 1];
+    if (chain_failed(status))
+        return;
+    const uint64_t count = n ? (n + seg - 1) / seg : 0;
+    const uint64_t sbytes = slot_bytes(seg, P);
+    for (uint64_t s = blockIdx.x; s < count; s += gridDim.x) {
+        const uint8_t *const slot = slots + s * sbytes;
+        const uint32_t total = bits[s], words = (uint32_t)(al16(((uint64_t)total + 7) / 8) / 4);
+        if (start[s] + 4ull * words > cap)
+            continue;
+        __syncthreads();
+        if (threadIdx.x < 2 * L.parts)
+            piece[threadIdx.x] =
+                reinterpret_cast<const uint2 *>(slot + 16 + L.code + L.head)[threadIdx.x];
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint32_t at = 0;
+            for (uint32_t i = 0; i < 2 * L.parts; ++i) {
+                first[i] = at;
+                at += piece[i].y;
+            }
+            first[2 * L.parts] = at;
+        }
+        __syncthreads();
+        uint32_t *const dst = reinterpret_cast<uint32_t *>(out + start[s]);
+        const uint32_t *const src = reinterpret_cast<const uint32_t *>(slot);
+        uint32_t i = 0;
+        for (uint32_t j = threadIdx.x; j < words; j += blockDim.x) {
+            uint32_t w = 0, got = 0;  // bits of the word so far
+            const uint32_t at = 32 * j;
+            while (i + 1 < 2 * L.parts && first[i + 1] <= at)
+                ++i;
+            for (uint32_t q = i; q < 2 * L.parts && got < 32; ++q) {
+                const uint32_t from = at + got, to = first[q + 1];
+                if (from >= to)
+                    continue;
+                const uint32_t b = piece[q].x + (from - first[q]), a = b >> 5;
+                const uint32_t v = __funnelshift_l(bswap32(__ldcg(src + a + 1)), bswap32(__ldcg(src + a)),
+                                                   b & 31u);
+                const uint32_t take = to - from < 32 - got ? to - from : 32 - got;
+                w |= (v & ~__funnelshift_rc(0xffffffffu, 0u, take)) >> got;
+                got += take;
+            }
+            dst[j] = bswap32(w);
+        }
     }
 }
 
@@ -1471,6 +1715,45 @@ __global__ void k_lzss_set(int32_t *status, unsigned long long *p, uint64_t v)
         *p = v;
 }
 
+// Parts of a segment: 8 where that makes up to 15 warps per SM, 4 or 2 up to 27
+// (more parts mean more joins one after the other, and a full chip gains
+// nothing), of 4 KiB at least, if the slots hold them.  64 KiB segments with
+// 1024/12/24/8, one warp a segment against parts: 64 segments 3.60 / 1.10 ms (8
+// parts), 256: 3.80 / 1.57, 512: 3.82 / 2.03 (4 parts; 8: 2.18), 1024: 4.40 /
+// 2.99 (4; 8: 3.14); 4096 segments of 16 KiB 2.38 / 2.80 (2 parts), so none.
+PartsLayout parts_of(uint64_t n, uint64_t seg, uint64_t count, const LzParams &P, uint64_t sms)
+{
+    PartsLayout L = {1, 0, 0, 0};
+    if (!ring_ok(P) || P.lmax < 8 || n == 0)
+        return L;
+    const uint64_t ref = 1 + P.ob + P.lb, lit = 1 + P.blk;
+    for (uint64_t k = kMaxParts; k > 1; k >>= 1) {
+        if (seg / k < kMinPart || count * k > (k > 4 ? 15 : 27) * sms)
+            continue;
+        // a part's bits, the last step's past its end, each at the rate of the
+        // kind of token that grows it most
+        const uint64_t bits = 8 * seg / k + 1 + 1024 + 64;
+        const uint64_t code = (ref * P.blk > lit * P.lmin ? (bits * ref + P.lmin - 1) / P.lmin
+                                                          : (bits * lit + P.blk - 1) / P.blk) +
+                              2 * (ref > lit ? ref : lit) + P.W;
+        const uint64_t bytes = al16(code / 8 + 16);
+        // the rest of the slot for the bits before the meeting points: few
+        // tokens but for the runs among them (28 K bits at most in 500 parts of
+        // the stand-in)
+        const uint64_t stride = (slot_bytes(seg, P) - 32) / k & ~15ull;
+        const uint64_t fixed = 16 + bytes + 8 * kMarks;
+        if (stride < fixed + bytes / 4 + 512 || 8 * k * stride >> 32)
+            continue;  // (bit positions in a slot are 32 bits wide)
+        const uint64_t head = stride - fixed;
+        L.parts = (uint32_t)k;
+        L.code = (uint32_t)bytes;
+        L.head = (uint32_t)head;
+        L.stride = (uint32_t)stride;
+        return L;
+    }
+    return L;
+}
+
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 bool host_params(const huff_lzss_params_t *p, LzParams &P)
@@ -1532,22 +1815,33 @@ huff_status_t huff_lzss_compress(const uint8_t *d_in, uint64_t n, uint64_t segme
     const int sms = device_sm_count();
     if (sms < 1)
         return HUFF_ERR_CUDA;
+    const PartsLayout L = parts_of(n, segment_bytes, count, P, (uint64_t)sms);
     if (count) {
         if (ring_ok(P)) {
             const size_t smem = 2 * (size_t)ring_words(P.W) * 4;  // at most 8 KB
-            const uint64_t grid = count < (uint64_t)sms * 64 ? count : (uint64_t)sms * 64;
-            auto run = [&](auto kernel) {
-                kernel<<<(unsigned)grid, 32, smem, s>>>(d_in, n, segment_bytes, P, slots, bits,
-                                                        d_status);
+            const auto grid = [&](uint64_t warps) {
+                return (unsigned)(warps < (uint64_t)sms * 64 ? warps : (uint64_t)sms * 64);
+            };
+            auto run = [&](auto g0) {
+                constexpr int G0 = decltype(g0)::value;
+                if (L.parts > 1) {
+                    k_lzss_parts<G0><<<grid(count * L.parts), 32, smem, s>>>(
+                        d_in, n, segment_bytes, P, L, slots, d_status);
+                    k_lzss_join<G0><<<grid(count), 32, smem, s>>>(d_in, n, segment_bytes, P, L, slots,
+                                                                  bits, d_status);
+                } else {
+                    k_lzss_compress_ring<G0><<<grid(count), 32, smem, s>>>(d_in, n, segment_bytes, P,
+                                                                           slots, bits, d_status);
+                }
             };
             switch (P.lmin / 4) {
-            case 0: run(k_lzss_compress_ring<0>); break;
-            case 1: run(k_lzss_compress_ring<1>); break;
-            case 2: run(k_lzss_compress_ring<2>); break;
-            case 3: run(k_lzss_compress_ring<3>); break;
-            case 4: run(k_lzss_compress_ring<4>); break;
-            case 5: run(k_lzss_compress_ring<5>); break;
-            default: run(k_lzss_compress_ring<6>); break;
+            case 0: run(std::integral_constant<int, 0>()); break;
+            case 1: run(std::integral_constant<int, 1>()); break;
+            case 2: run(std::integral_constant<int, 2>()); break;
+            case 3: run(std::integral_constant<int, 3>()); break;
+            case 4: run(std::integral_constant<int, 4>()); break;
+            case 5: run(std::integral_constant<int, 5>()); break;
+            default: run(std::integral_constant<int, 6>()); break;
             }
         } else {
             uint64_t grid = (count + kLzWarps - 1) / kLzWarps;
@@ -1562,8 +1856,12 @@ huff_status_t huff_lzss_compress(const uint8_t *d_in, uint64_t n, uint64_t segme
                                            d_status);
     if (count) {
         const uint64_t grid = count < (uint64_t)sms * 16 ? count : (uint64_t)sms * 16;
-        k_lzss_gather<<<(unsigned)grid, 128, 0, s>>>(n, segment_bytes, P, slots, bits, start, d_out,
-                                                     out_cap, d_status);
+        if (L.parts > 1)
+            k_lzss_gather_parts<<<(unsigned)grid, 256, 0, s>>>(n, segment_bytes, P, L, slots, bits,
+                                                               start, d_out, out_cap, d_status);
+        else
+            k_lzss_gather<<<(unsigned)grid, 128, 0, s>>>(n, segment_bytes, P, slots, bits, start,
+                                                         d_out, out_cap, d_status);
     }
     return cudaGetLastError() == cudaSuccess ? HUFF_OK : HUFF_ERR_CUDA;
 }

@@ -75,3 +75,27 @@ def test_batch_edges_against_oracle(params, n):
         assert ost == oracle.OK
         y, got, s = _decode(torch.from_numpy(ref).cuda(), n)
         assert s == 0 and got == n and np.array_equal(y.cpu().numpy(), x)
+
+
+def _period(n, k, seed):
+    return np.resize(np.random.default_rng(seed).integers(0, 256, k).astype(np.uint8), n)
+
+
+# segments of 8 KiB and more coded in parts whose token chains must meet: quickly
+# (bitstream, random), at the end of a run, or never (constant data, a period
+# that matches are cut from), and parts that a run covers whole
+@pytest.mark.parametrize("params", [(256, 12, 24, 8, 2), (64, 9, 32, 16, 1), (512, 16, 16, 7, 2),
+                                    (128, 2, 8, 3, 2)])
+@pytest.mark.parametrize("seg", [16384, 32768, 65536])
+def test_segments_in_parts_against_oracle(params, seg):
+    n = seg + 9001
+    runs = synth.bitstream(n, 3)
+    runs[seg // 5:seg // 2] = 0
+    runs[seg // 2:seg // 2 + 3000] = 0xFF
+    for x in (runs, synth.uniform(n, 2), np.zeros(n, np.uint8), _period(n, 5, 1),
+              _period(n, 61, 2)):
+        ost, ref = oracle.lzss_segmented_compress(x, seg, params)
+        assert ost == oracle.OK
+        c, st = hg.huff_lzss_compress(torch.from_numpy(x).cuda(), seg, params)
+        torch.cuda.synchronize()
+        assert int(st.item()) == 0 and np.array_equal(c.cpu().numpy(), ref)
