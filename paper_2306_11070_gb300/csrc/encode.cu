@@ -8,23 +8,16 @@
 //    ever waits on another.  Each warp encodes whole units by itself in 16
 //    steps of 1024 symbols; the loop has no CTA barrier at all.
 //  - A step: every lane loads its 32 bytes (two 16-byte loads, issued one
-//    step ahead), looks up the 32 table entries and keeps them in registers,
-//    sums them (the low 10 bits of a sum of entries are the sum of their
-//    lengths), a warp scan of the sums gives every lane its bit position,
-//    the lanes pack their codes into the warp's word buffer in shared
-//    memory, and the warp writes the whole words with coalesced stores.  The
-//    partial last word is carried in a register into the next step.
-//  - Packing: two funnel shifts per code into a 64-bit register; every
-//    floor(32 / longest) codes at most one word completes, and a plain store
-//    writes the last completed word (see pack32 for why every word ends with
-//    the right value without atomics); after a warp barrier each lane ORs
-//    its last partial word into the next lane's first word.
-//  - Code table in shared memory, replicated per lane ([byte][lane]), so
-//    the 32 lookups of a warp never collide in a bank.  Entry =
-//    (code << (32 - len)) | len for codes up to 22 bits: the funnel shifts
-//    take the length from the entry's low 5 bits.  Longer codes (up to 32
-//    bits) use split code / length tables, 16 symbols per lane and a 64-bit
-//    accumulator.
+//    step ahead), gathers their codes into groups by multiply-add from a
+//    table in shared memory that is replicated per lane, so that the 32
+//    lookups of a warp never collide in a bank (see encode_impl.cuh), a warp
+//    scan of the lanes' bit counts gives every lane its bit position, the
+//    lanes pack their groups into the warp's word buffer in shared memory,
+//    and the warp writes the whole words with coalesced stores.  The partial
+//    last word is carried in a register into the next step.
+//  - What bounds it: on text the shared-memory data pipe is 73% busy while a
+//    unit runs (two wavefronts per 32 lookups, about 1.5 for the packed
+//    words) and 59% of the issue slots are taken.
 //  - The word a unit shares with the unit before it is completed by the later
 //    unit: it re-codes the last <= 31 bits of its predecessor from the 32
 //    input bytes before it, so no warp waits for another's output and the
@@ -36,13 +29,14 @@ namespace {
 
 using namespace enc;
 
-// One CTA of 16 warps per SM: one copy of the 32 KiB code table per SM; a
-// step keeps 32 table entries per lane in registers (~120 per thread), so
-// 16 warps are what fit without spills.
+// One CTA of 16 warps per SM: one copy of the 64 KiB code table per SM, and
+// 16 warps are what fit without spills (18 or 20 warps of 96 registers: 1 GiB
+// takes 1070 and 1030 us instead of 839).
 constexpr int kEncBlock = 512;
 constexpr int kEncWarps = kEncBlock / 32;
-// the (code, 2^len) table is the larger of the two table layouts
-constexpr int kEncSmemBytes = (kTbl2Words + kEncWarps * kWarpObuf) * 4;
+// the table, the padding before it, and the buffers if the gap is too small
+constexpr int kEncObufBytes = kEncWarps * kMadObuf * 4;
+constexpr int kEncSmemBytes = 65536 + kTbl2Words * 4 + kEncObufBytes;
 
 struct EncodeArgs {
     const uint8_t *in;
@@ -56,58 +50,93 @@ struct EncodeArgs {
     int32_t *status;
 };
 
-__global__ void __launch_bounds__(kEncBlock, 1) k_encode(EncodeArgs a)
+// This warp's part of the CTA's dynamic shared memory, and the code table:
+// [256][32] (code, 2^len) pairs, or 2 x [256][16] for 32-bit codes.  The table
+// lies at a 64 KiB boundary of the shared window, so that the address of a
+// byte's entry is one byte permutation of the data word and the lane's column
+// (a multiply-add per symbol fewer); the warps' buffers take the gap before
+// it.
+struct Smem {
+    uint32_t *tbl, *wob;
+};
+
+__device__ __forceinline__ Smem carve(uint4 *smem_raw)
+{
+    const uint32_t pad = (0u - smem_u32(smem_raw)) & 0xffffu;
+    unsigned char *raw = reinterpret_cast<unsigned char *>(smem_raw);
+    Smem m;
+    m.tbl = reinterpret_cast<uint32_t *>(raw + pad);
+    m.wob = reinterpret_cast<uint32_t *>(raw + (pad >= (uint32_t)kEncObufBytes ? 0u : pad + kTbl2Words * 4)) +
+            (threadIdx.x >> 5) * kMadObuf;
+    return m;
+}
+
+// Units go to the CTAs first and to their warps second: a last wave that does
+// not fill the chip leaves every SM with a few busy warps instead of some SMs
+// with none, and a few units get an SM each (1 MiB: the call takes 62 us
+// instead of 77).
+#define FOR_UNITS(u, J)                                                                      \
+    for (uint64_t u = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; u < (J).units; \
+         u += (uint64_t)gridDim.x * kEncWarps)
+
+// Codes of 11 to 31 bits, in groups of G that nearly always fit.  Functions of
+// their own, as is encode_long: inlined into the kernel they would make it
+// spill (1 GiB of text: the call takes 1010 us instead of 839).
+template <int G>
+__device__ __noinline__ void encode_try(const EncodeArgs &a)
 {
     extern __shared__ uint4 smem_raw[];
-    // [256][32] (code, 2^len) pairs, or 2 x [256][16] for codes over 22 bits
-    uint32_t *tbl = reinterpret_cast<uint32_t *>(smem_raw);
-    uint32_t *wob = tbl + kTbl2Words + (threadIdx.x >> 5) * kWarpObuf;  // this warp's buffer
-
-    if (chain_failed(a.status))
-        return;
+    const Smem m = carve(smem_raw);
     const Job J = make_job(a.in, a.n, a.cs, a.unit_off, a.out, a.out_cap);
-    const uint32_t max_len = a.cb->max_len;
-    const bool fast = max_len <= (uint32_t)kFastMaxLen;
-    if (fast && mad_group(max_len) >= 3)
-        return;  // k_encode_mad codes this stream
-    const int group = emit_group(max_len);
-    if (blockIdx.x == 0)
-        write_header(J, a.cb, a.out_bytes, a.status);
-    build_table(a.cb, tbl, fast);
-    __syncthreads();  // the only CTA barrier: the table is ready
-
-    const uint64_t nwarps = (uint64_t)gridDim.x * kEncWarps;
     bool overflow = false;
-    for (uint64_t u = (uint64_t)blockIdx.x * kEncWarps + (threadIdx.x >> 5); u < J.units; u += nwarps)
-        overflow |= encode_unit(J, u, tbl, fast, group, wob);
+    FOR_UNITS(u, J)
+        overflow |= encode_unit_mad<G, 1, 1>(J, u, m.tbl, m.wob);
     if (overflow)
         set_status(a.status, HUFF_ERR_CAPACITY);
 }
 
-// The same for codes of at most 10 bits, gathered by multiply-add (see
-// encode_impl.cuh); the two kernels are launched back to back and the one
-// that does not apply returns at once.
-__global__ void __launch_bounds__(kEncBlock, 1) k_encode_mad(EncodeArgs a)
+__device__ __noinline__ void encode_long(const EncodeArgs &a)
 {
     extern __shared__ uint4 smem_raw[];
-    uint32_t *tbl2 = reinterpret_cast<uint32_t *>(smem_raw);  // [256][32] (code, 2^len)
-    uint32_t *wob = tbl2 + kTbl2Words + (threadIdx.x >> 5) * kWarpObuf;
+    const Smem m = carve(smem_raw);
+    const Job J = make_job(a.in, a.n, a.cs, a.unit_off, a.out, a.out_cap);
+    bool overflow = false;
+    FOR_UNITS(u, J)
+        overflow |= encode_unit_long(J, u, m.tbl, m.wob);
+    if (overflow)
+        set_status(a.status, HUFF_ERR_CAPACITY);
+}
 
+// One kernel for all code lengths: the host does not know them, and a second
+// launch that only finds out that it does not apply costs 2 us or more.
+__global__ void __launch_bounds__(kEncBlock, 1) k_encode(const __grid_constant__ EncodeArgs a)
+{
+    extern __shared__ uint4 smem_raw[];
     if (chain_failed(a.status))
         return;
     const uint32_t max_len = a.cb->max_len;
-    const int mgroup = mad_group(max_len);
-    if (!(max_len <= (uint32_t)kFastMaxLen && mgroup >= 3))
-        return;
+    const Smem m = carve(smem_raw);
     const Job J = make_job(a.in, a.n, a.cs, a.unit_off, a.out, a.out_cap);
     if (blockIdx.x == 0)
         write_header(J, a.cb, a.out_bytes, a.status);
-    build_table2(a.cb, tbl2);
-    __syncthreads();
-    const uint64_t nwarps = (uint64_t)gridDim.x * kEncWarps;
+    const int group = max_len <= kMadMaxLen ? mad_group(max_len) : 0;
+    if (group)
+        build_table2(a.cb, m.tbl);
+    else
+        build_table(a.cb, m.tbl, false);
+    __syncthreads();  // the only CTA barrier: the table is ready
+    if (group < 3) {
+        if (!group)
+            encode_long(a);
+        else if (few_bits(J))
+            encode_try<4>(a);
+        else
+            encode_try<3>(a);
+        return;
+    }
     bool overflow = false;
-    for (uint64_t u = (uint64_t)blockIdx.x * kEncWarps + (threadIdx.x >> 5); u < J.units; u += nwarps)
-        overflow |= encode_unit_mad_g(J, u, tbl2, mgroup, wob);
+    FOR_UNITS(u, J)
+        overflow |= encode_unit_mad_g(J, u, m.tbl, group, m.wob);
     if (overflow)
         set_status(a.status, HUFF_ERR_CAPACITY);
 }
@@ -127,11 +156,9 @@ cudaError_t launch_encode(const uint8_t *d_in, uint64_t n, const huff_codebook_t
                           void *d_ws, const uint16_t *d_unit_hist, int32_t *d_status,
                           cudaStream_t s)
 {
-    static KernelSetup setup, setup_mad;
-    int per_sm = 0, per_sm_mad = 0;
+    static KernelSetup setup;
+    int per_sm = 0;
     cudaError_t err = kernel_setup(setup, (const void *)k_encode, kEncBlock, kEncSmemBytes, &per_sm);
-    if (err == cudaSuccess)
-        err = kernel_setup(setup_mad, (const void *)k_encode_mad, kEncBlock, kEncSmemBytes, &per_sm_mad);
     if (err != cudaSuccess)
         return err;
     const int sms = device_sm_count();
@@ -159,12 +186,10 @@ cudaError_t launch_encode(const uint8_t *d_in, uint64_t n, const huff_codebook_t
     a.out_bytes = d_out_bytes;
     a.status = d_status;
     uint64_t grid = (uint64_t)sms * per_sm;
-    const uint64_t want = (units + kEncWarps - 1) / kEncWarps;
-    if (grid > want)
-        grid = want;
+    if (grid > units)
+        grid = units;
     if (grid < 1)
         grid = 1;
-    k_encode_mad<<<(unsigned)grid, kEncBlock, kEncSmemBytes, s>>>(a);
     k_encode<<<(unsigned)grid, kEncBlock, kEncSmemBytes, s>>>(a);
     return cudaGetLastError();
 }

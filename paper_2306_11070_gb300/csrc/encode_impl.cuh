@@ -128,9 +128,10 @@ __device__ __forceinline__ void build_table(const huff_codebook_t *cb, uint32_t 
 
 // Zero this warp's buffer (kWarpObuf words at wob); every step leaves the
 // words it used zero again, so this runs once per unit.
+template <int kWords = kWarpObuf>
 __device__ __forceinline__ void clear_buffer(uint32_t *wob, int lane)
 {
-    for (int j = lane; j < kWarpObuf; j += 32)
+    for (int j = lane; j < kWords; j += 32)
         wob[j] = 0u;
     __syncwarp();
 }
@@ -277,7 +278,7 @@ template <int SPT, int STEP>
 __device__ __forceinline__ void step_chunks(const Job &J, const UnitState &st, uint64_t sb, int lane,
                                             uint32_t pos, uint32_t mid16)
 {
-    if (!J.table_fits)
+    if (!J.table_fits || (J.cs >= (uint32_t)STEP && st.lead >= (uint32_t)STEP))
         return;
     uint64_t *offs = reinterpret_cast<uint64_t *>(J.out + kHeaderBytes);
 #pragma unroll
@@ -347,9 +348,10 @@ __device__ __forceinline__ bool step_output(const Job &J, UnitState &st, bool la
 }
 
 // One 1024-symbol step of the fast encoder (codes of at most 22 bits, G =
-// floor(32 / longest)).  kInner: the step lies inside the input, the unit
-// is not the last one and its words fit the output, so the step needs none
-// of the bound checks; its 32 input bytes per lane (w) were loaded ahead.
+// floor(32 / longest)).  kInner: the step lies inside the input and the
+// unit's words fit the output, so the step needs none of the bound checks; its
+// 32 input bytes per lane (w) were loaded ahead.  It returns true, with
+// nothing done, if a lane has fewer than 32 bits (bytes without a code).
 template <int G, bool kInner>
 __device__ __forceinline__ bool fast_step(const Job &J, UnitState &st, int step, int lane,
                                           uint32_t tcol_s, uint32_t wob_s, uint32_t *wob,
@@ -383,6 +385,8 @@ __device__ __forceinline__ bool fast_step(const Job &J, UnitState &st, int step,
             mid16 = s & kSumMask;
     }
     const uint32_t bits = s & kSumMask;
+    if (kInner && !__all_sync(0xffffffffu, bits >= (uint32_t)kFastSyms))
+        return true;  // plain stores need whole words (see pack32)
     uint32_t pos, step_bits;
     scan_bits(bits, lane, pos, step_bits);
     const uint32_t p0 = (uint32_t)(st.gbit & 31) + pos;
@@ -430,6 +434,19 @@ __device__ __forceinline__ void load32(const uint8_t *p, uint32_t (&w)[8])
     w[7] = b.w;
 }
 
+// The steps of unit u that need no bound checks: those that lie inside the
+// input, if the unit's words (a last partial word included) fit the output.
+// Only what is left of the last unit takes the checked step, with its byte
+// loads and shared ORs; checking that whole unit made one warp run 60 us at
+// 64 MiB where the others took 41.
+__device__ __forceinline__ int full_steps(const Job &J, uint64_t u)
+{
+    if (((J.unit_off[u + 1] + 31) >> 5) > J.cap_words)
+        return 0;
+    const uint64_t left = (J.n - u * kUnitSymbols) / kFastStep;
+    return left < (uint64_t)kFastSteps ? (int)left : kFastSteps;
+}
+
 // Encode unit u of job J with the calling warp, codes of at most 22 bits.
 // wob is the warp's buffer of kWarpObuf words (word 0 is the guard), tbl the
 // CTA's table.  Returns true if a payload word fell outside the output
@@ -441,26 +458,28 @@ __device__ __forceinline__ bool encode_unit_fast(const Job &J, uint64_t u, const
     const int lane = threadIdx.x & 31;
     const uint32_t tcol_s = smem_u32(tbl + lane), wob_s = smem_u32(wob + 1);
     UnitState st = unit_start(J, u, tbl, true, lane);
-    const bool inner = st.base + kUnitSymbols < J.n && (J.unit_off[u + 1] >> 5) < J.cap_words;
-    if (!inner)
-        clear_buffer(wob, lane);
+    const int full = full_steps(J, u);
     bool overflow = false;
-    if (inner) {  // warp-uniform
+    int step = 0;
+    if (full) {  // warp-uniform
         const uint8_t *p = J.in + st.base + lane * kFastSyms;
         uint32_t w[8];
         load32(p, w);
-        for (int step = 0; step < kFastSteps; ++step) {
+        for (; step < full; ++step) {
             uint32_t nx[8];
-            if (step + 1 < kFastSteps)
+            if (step + 1 < full)
                 load32(p + (step + 1) * kFastStep, nx);  // one step ahead
-            fast_step<G, true>(J, st, step, lane, tcol_s, wob_s, wob + 1, w);
+            if (fast_step<G, true>(J, st, step, lane, tcol_s, wob_s, wob + 1, w))
+                break;
 #pragma unroll
             for (int j = 0; j < 8; ++j)
                 w[j] = nx[j];
         }
-    } else {
+    }
+    if (step < kFastSteps && st.base + (uint64_t)step * kFastStep < J.n) {
+        clear_buffer(wob, lane);
         const uint32_t none[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int step = 0; step < kFastSteps; ++step) {
+        for (; step < kFastSteps; ++step) {
             if (st.base + (uint64_t)step * kFastStep >= J.n)
                 break;  // warp-uniform
             overflow |= fast_step<G, false>(J, st, step, lane, tcol_s, wob_s, wob + 1, none);
@@ -474,25 +493,44 @@ __device__ __forceinline__ bool encode_unit_fast(const Job &J, uint64_t u, const
 // which bounds it.  Here a group of codes is gathered on the FMA pipe: the
 // table holds (code, 2^len) per byte and lane, and a = a * 2^len + code
 // appends a code to the group's bits; a starts at 1, so its leading one
-// marks the group's length (a group has at most 31 bits).  Only the group
-// then pays the funnel shifts into the 64-bit window and the emit check:
-// per code one byte extract, one table load (8 bytes) and one IMAD, per
-// group a leading-one search and three funnel shifts.  The groups of a lane
-// are cut at its 16th symbol too, where a chunk may start.  Same stream,
-// bit for bit.
+// marks the group's length (a group has at most 31 bits).  Per code that is
+// one byte permutation (which is the table address), one table load (8 bytes)
+// and one IMAD; only the group pays for its length, its place and the store.
+// The groups of a lane are cut at its 16th symbol too, where a chunk may
+// start.  Same stream, bit for bit.
+//  - Longest code of at most 10 bits: groups of floor(31 / longest) codes, at
+//    least 3, always fit.
+//  - Longer codes are rare wherever there are any: the groups take 4 codes
+//    where the average is at most 4 bits, else 3, and a multiply-add whose
+//    high word is not zero shows the group that does not fit; its step and the
+//    rest of the unit then go code by code.  On geometric bytes (longest 25 to
+//    29 bits, average 2) 64 MiB take 114 us instead of 211 and 1 GiB 911
+//    instead of 2127.  The same guess for codes of at most 10 bits (4 for 3)
+//    gained 2 to 4% on text and lost as much on Zipf bytes, where every unit
+//    has a group that does not fit: not done.
 constexpr int kTbl2Words = 256 * 32 * 2;  // [byte][lane] (code, 2^len), 64 KiB
+constexpr uint32_t kMadMaxLen = 31;       // the marker takes a bit
+// warp buffer: a guard word, then a step of 1024 codes after < 32 carried bits
+constexpr int kMadObuf = 1 + kFastStep * (int)kMadMaxLen / 32 + 15;
 
+// Built by 512 threads, two per byte: each reads its byte's length and code
+// once and fills half a row with eight 16-byte stores, rotated by the byte so
+// that a warp's stores spread over all eight 16-byte bank groups.
 __device__ __forceinline__ void build_table2(const huff_codebook_t *cb, uint32_t *tbl2)
 {
-    for (int i = threadIdx.x; i < 256 * 32; i += blockDim.x) {
-        const int b = i >> 5;
-        const uint32_t L = cb->len[b];
-        tbl2[2 * i] = L ? cb->code[b] : 0u;
-        tbl2[2 * i + 1] = 1u << L;  // 2^0 = 1 for a byte without a code: no bits
-    }
+    const int b = threadIdx.x >> 1;
+    if (b >= 256)
+        return;
+    const uint32_t L = cb->len[b];
+    const uint32_t c = L ? cb->code[b] : 0u;
+    const uint32_t p = 1u << L;  // 2^0 = 1 for a byte without a code: no bits
+    uint4 *row = reinterpret_cast<uint4 *>(tbl2 + b * 64) + (threadIdx.x & 1) * 8;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        row[(j + b) & 7] = make_uint4(c, p, c, p);
 }
 
-// Codes per group: floor(31 / longest), as a template (31: the marker bit).
+// Codes per group that always fit: floor(31 / longest) (31: the marker bit).
 __device__ __forceinline__ int mad_group(uint32_t max_len)
 {
     const uint32_t gq = max_len ? 31u / max_len : 16u;
@@ -532,26 +570,36 @@ __device__ __forceinline__ UnitState unit_start2(const Job &J, uint64_t u, const
     return st;
 }
 
-// One 1024-symbol step (codes of at most 22 bits; G codes per group).
-template <int G, bool kInner>
-__device__ __forceinline__ bool mad_step(const Job &J, UnitState &st, int step, int lane,
-                                         uint32_t tcol_s, uint32_t wob_s, uint32_t *wob,
-                                         const uint32_t (&w)[8])
+// st.shared of v at address a where w1 != w0.
+__device__ __forceinline__ void sts_if_ne(uint32_t w1, uint32_t w0, uint32_t a, uint32_t v)
 {
-    constexpr int NH = (16 + G - 1) / G;  // groups per 16 symbols
-    constexpr int NG = 2 * NH;
-    const uint64_t sb = st.base + (uint64_t)step * kFastStep;
-    int m = kFastSyms;
-    uint32_t tw[8];
-    if (kInner) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            tw[j] = w[j];
-    } else {
-        m = step_input_tail<kFastSyms>(J, sb, lane, tw);
-    }
-    uint32_t acc[NG], lg[NG];
-    uint32_t bits = 0, mid16 = 0;
+    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %0, %1;\n@p st.shared.u32 [%2], %3;\n}" ::"r"(w1),
+                 "r"(w0), "r"(a), "r"(v)
+                 : "memory");
+}
+
+// The 32 codes of a lane as groups of at most G codes (16 symbols, where a
+// chunk may start, end a group).
+template <int G>
+struct Groups {
+    static constexpr int NH = (16 + G - 1) / G;  // groups per 16 symbols
+    static constexpr int NG = 2 * NH;
+    uint32_t acc[NG];  // marker and bits
+    uint32_t len[NG];
+    uint32_t bits, mid16;  // of all 32 symbols and of the first 16
+};
+
+// Gather the codes of the lane's first m symbols.  A group's first kFirst
+// codes have at most 31 bits together, whatever they are; a multiply-add of
+// a later one whose high word is not zero has overflowed (the result, which
+// the caller then throws away, is nonzero).
+template <int G, int kFirst, bool kAll>
+__device__ __forceinline__ uint32_t mad_gather(Groups<G> &q, const uint32_t (&w)[8], int m,
+                                               uint32_t tcol_s)
+{
+    constexpr int NH = Groups<G>::NH, NG = Groups<G>::NG;
+    uint32_t over = 0;
+    q.bits = 0;
 #pragma unroll
     for (int g = 0; g < NG; ++g) {
         const int k0 = (g / NH) * 16 + (g % NH) * G;
@@ -559,52 +607,69 @@ __device__ __forceinline__ bool mad_step(const Job &J, UnitState &st, int step, 
 #pragma unroll
         for (int j = 0; j < G; ++j) {
             const int k = k0 + j;
-            if ((g % NH) * G + j < 16 && (kInner || k < m)) {
+            if ((g % NH) * G + j < 16 && (kAll || k < m)) {
                 uint2 x;
                 asm("ld.shared.v2.u32 {%0, %1}, [%2];"
                     : "=r"(x.x), "=r"(x.y)
-                    : "r"(imad(byte_of(tw, k), kc[k128] * 2u, tcol_s)));
-                a = a * x.y + x.x;
+                    : "r"(__byte_perm(w[k >> 2], tcol_s, 0x7604u | (uint32_t)(k & 3) << 4)));
+                if (j >= kFirst) {
+                    const uint64_t t = (uint64_t)a * x.y + x.x;
+                    over |= (uint32_t)(t >> 32);
+                    a = (uint32_t)t;
+                } else {
+                    a = a * x.y + x.x;
+                }
             }
         }
-        acc[g] = a;
-        lg[g] = 31u - __clz(a);
-        bits += lg[g];
+        q.acc[g] = a;
+        q.len[g] = 31u - __clz(a);
+        q.bits += q.len[g];
         if (g == NH - 1)
-            mid16 = bits;
+            q.mid16 = q.bits;
     }
+    return over;
+}
+
+// Pack and write the gathered step at symbol sb; kInner as for fast_step (the
+// caller has made sure that every lane has 32 bits).
+template <int G, bool kInner>
+__device__ __forceinline__ bool mad_pack(const Job &J, UnitState &st, uint64_t sb, int lane,
+                                         const Groups<G> &q, uint32_t wob_s, uint32_t *wob)
+{
     uint32_t pos, step_bits;
-    scan_bits(bits, lane, pos, step_bits);
+    scan_bits(q.bits, lane, pos, step_bits);
     const uint32_t p0 = (uint32_t)(st.gbit & 31) + pos;
-    step_chunks<kFastSyms, kFastStep>(J, st, sb, lane, pos, mid16);
+    step_chunks<kFastSyms, kFastStep>(J, st, sb, lane, pos, q.mid16);
     if (!kInner) {
         sts_if(lane == 0, wob_s, st.carry);  // word 0 starts with the carried bits
         __syncwarp();
     }
-    // groups into the 64-bit window hi:lo, the last completed word out after
-    // each group (see pack32 for why plain stores are enough when every
-    // lane has 32 codes)
-    // A group that crosses no word boundary would store the same word again:
-    // only groups that cross one store (about one group in 2.4 on text),
-    // which keeps the warp-buffer stores off the L1 data pipe.
-    uint32_t hi = 0u, lo = 0u, E = p0;
+    // lom + 1 holds the lane's last 32 bits.  A group of L bits x (a = 2^L + x)
+    // that takes the lane's end from E to E1 over a word boundary completes
+    // the word (lom + 1) << d | x >> r, with r = E1 mod 32 bits left over and
+    // d = L - r = -E mod 32; the marker's 2^d is the 2^d that lom lacks (see
+    // pack32 for why plain stores are enough when every lane has 32 bits).
+    // A group that crosses no boundary stores nothing (about one group in two
+    // crosses on text), which keeps the warp-buffer stores off the L1 data
+    // pipe; a predicated store, because some lane of 32 nearly always
+    // crosses.
+    uint32_t lom = ~0u, E = p0, nE = 0u - p0, wi = p0 >> 5;
 #pragma unroll
-    for (int g = 0; g < NG; ++g) {
-        const uint32_t L = lg[g];
-        const uint32_t top = __funnelshift_lc(0u, acc[g], 32u - L);  // the group's bits, high-aligned
-        hi = __funnelshift_l(lo, hi, L);
-        lo = __funnelshift_l(top, lo, L);
-        const uint32_t E0 = E;
+    for (int g = 0; g < Groups<G>::NG; ++g) {
+        const uint32_t L = q.len[g];
+        const uint32_t v0 = __funnelshift_l(0u, lom, nE);  // lom << (-E mod 32)
         E = imad(L, kc[kOne], E);
-        if ((E ^ E0) >> 5) {  // a word was completed
-            const uint32_t ad = imad(E >> 5, kc[kFour], wob_s - 4), v = __funnelshift_r(lo, hi, E);
-            if (kInner)
-                sts(ad, v);
-            else
-                red_or(ad, v);
-        }
+        nE -= L;
+        const uint32_t v = v0 + __funnelshift_r(q.acc[g], 0u, E);
+        const uint32_t w1 = E >> 5, ad = imad(w1, kc[kFour], wob_s - 4);
+        if (kInner)
+            sts_if_ne(w1, wi, ad, v);
+        else if (w1 != wi)
+            red_or(ad, v);
+        wi = w1;
+        lom = (lom << L) + q.acc[g] - 1u;
     }
-    const uint32_t part = __funnelshift_lc(0u, lo, 32u - (E & 31u));
+    const uint32_t part = __funnelshift_lc(0u, lom + 1u, 32u - (E & 31u));
     if (kInner) {
         __syncwarp();
         const uint32_t pa = imad(E >> 5, kc[kFour], wob_s);
@@ -625,51 +690,90 @@ __device__ __forceinline__ bool mad_step(const Job &J, UnitState &st, int step, 
     return overflow;
 }
 
-template <int G>
+// Steps [step, full) of a unit without bound checks; returns the first step
+// that cannot be done so (a group overflows, or a lane has fewer than 32 bits
+// because of bytes without a code), or full.
+template <int G, int kFirst>
+__device__ __forceinline__ int mad_steps(const Job &J, UnitState &st, int step, int full, int lane,
+                                         uint32_t tcol_s, uint32_t wob_s, uint32_t *wob)
+{
+    const uint8_t *p = J.in + st.base + lane * kFastSyms;
+    uint32_t w[8];
+    load32(p + step * kFastStep, w);
+    for (; step < full; ++step) {
+        uint32_t nx[8];
+        if (step + 1 < full)
+            load32(p + (step + 1) * kFastStep, nx);  // one step ahead
+        Groups<G> q;
+        const uint32_t over = mad_gather<G, kFirst, true>(q, w, kFastSyms, tcol_s);
+        if (!__all_sync(0xffffffffu, q.bits >= (uint32_t)kFastSyms && over == 0u))
+            break;
+        mad_pack<G, true>(J, st, st.base + (uint64_t)step * kFastStep, lane, q, wob_s, wob);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            w[j] = nx[j];
+    }
+    return step;
+}
+
+// The steps of a unit from `step` on in groups of S codes, which always fit:
+// the whole ones, then the checked rest.
+template <int S>
+__device__ __noinline__ bool mad_rest(const Job J, UnitState st, int step, int full, int lane,
+                                      uint32_t tcol_s, uint32_t wob_s, uint32_t *wob)
+{
+    bool overflow = false;
+    if (step < full)
+        step = mad_steps<S, S>(J, st, step, full, lane, tcol_s, wob_s, wob);
+    if (step < kFastSteps && st.base + (uint64_t)step * kFastStep < J.n) {
+        clear_buffer<kMadObuf>(wob - 1, lane);
+        for (; step < kFastSteps; ++step) {
+            const uint64_t sb = st.base + (uint64_t)step * kFastStep;
+            if (sb >= J.n)
+                break;  // warp-uniform
+            uint32_t w[8];
+            const int m = step_input_tail<kFastSyms>(J, sb, lane, w);
+            Groups<S> q;
+            mad_gather<S, S, false>(q, w, m, tcol_s);
+            overflow |= mad_pack<S, false>(J, st, sb, lane, q, wob_s, wob);
+        }
+    }
+    return overflow;
+}
+
+// Unit u in groups of G codes, of which kFirst always fit; the steps with a
+// group that does not fit, and all after them, in groups of S.
+template <int G, int kFirst, int S>
 __device__ __forceinline__ bool encode_unit_mad(const Job &J, uint64_t u, const uint32_t *tbl2,
                                                 uint32_t *wob)
 {
     const int lane = threadIdx.x & 31;
     const uint32_t tcol_s = smem_u32(tbl2 + 2 * lane), wob_s = smem_u32(wob + 1);
     UnitState st = unit_start2(J, u, tbl2, lane);
-    const bool inner = st.base + kUnitSymbols < J.n && (J.unit_off[u + 1] >> 5) < J.cap_words;
-    if (!inner)
-        clear_buffer(wob, lane);
-    bool overflow = false;
-    if (inner) {  // warp-uniform
-        const uint8_t *p = J.in + st.base + lane * kFastSyms;
-        uint32_t w[8];
-        load32(p, w);
-        for (int step = 0; step < kFastSteps; ++step) {
-            uint32_t nx[8];
-            if (step + 1 < kFastSteps)
-                load32(p + (step + 1) * kFastStep, nx);  // one step ahead
-            mad_step<G, true>(J, st, step, lane, tcol_s, wob_s, wob + 1, w);
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                w[j] = nx[j];
-        }
-    } else {
-        const uint32_t none[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int step = 0; step < kFastSteps; ++step) {
-            if (st.base + (uint64_t)step * kFastStep >= J.n)
-                break;  // warp-uniform
-            overflow |= mad_step<G, false>(J, st, step, lane, tcol_s, wob_s, wob + 1, none);
-        }
-    }
-    return overflow;
+    const int full = full_steps(J, u);
+    int step = 0;
+    if (full)  // warp-uniform
+        step = mad_steps<G, kFirst>(J, st, 0, full, lane, tcol_s, wob_s, wob + 1);
+    if (step < kFastSteps && st.base + (uint64_t)step * kFastStep < J.n)
+        return mad_rest<S>(J, st, step, full, lane, tcol_s, wob_s, wob + 1);
+    return false;
 }
 
-// group: mad_group of the longest code, at least 3 (longer codes keep the
-// funnel-shift path, where a group of one or two codes saves nothing)
+// At most 4 bits per code on average?
+__device__ __forceinline__ bool few_bits(const Job &J)
+{
+    return J.units && J.unit_off[J.units] <= 4 * J.n;
+}
+
+// group: mad_group of the longest code, at least 3
 __device__ __forceinline__ bool encode_unit_mad_g(const Job &J, uint64_t u, const uint32_t *tbl2,
                                                   int group, uint32_t *wob)
 {
     switch (group) {
-    case 16: return encode_unit_mad<16>(J, u, tbl2, wob);
-    case 8: return encode_unit_mad<8>(J, u, tbl2, wob);
-    case 4: return encode_unit_mad<4>(J, u, tbl2, wob);
-    default: return encode_unit_mad<3>(J, u, tbl2, wob);
+    case 16: return encode_unit_mad<16, 16, 16>(J, u, tbl2, wob);
+    case 8: return encode_unit_mad<8, 8, 8>(J, u, tbl2, wob);
+    case 4: return encode_unit_mad<4, 4, 4>(J, u, tbl2, wob);
+    default: return encode_unit_mad<3, 3, 3>(J, u, tbl2, wob);
     }
 }
 

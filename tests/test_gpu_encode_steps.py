@@ -1,0 +1,92 @@
+"""The encoder's steps where they can go wrong: every longest code length at
+which the grouping of codes changes, groups that do not fit, inputs that end
+just before, at and after a step or a unit, outputs that just hold the stream or
+just do not, and bytes without a code.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2306_11070_gb300 as hg
+from paper_2306_11070_gb300 import build as nvbuild
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    nvbuild.build()
+    hg.lib()
+
+
+SIZES = (1, 31, 1023, 1024, 1025, 3000, 16383, 16384, 16385, 17408, 50000)
+CHUNK = 4096
+
+
+def _codebook(lengths):
+    raw = np.zeros(hg.CODEBOOK_BYTES, np.uint8)
+    raw[:256] = lengths
+    raw[256:1280] = oracle.canonical_codes(lengths).astype("<u4").view(np.uint8)
+    raw[1280:1284] = np.array([np.count_nonzero(lengths)], "<u4").view(np.uint8)
+    raw[1284:1288] = np.array([lengths.max()], "<u4").view(np.uint8)
+    return torch.from_numpy(raw).cuda()
+
+
+def _encode(x, cb, cap):
+    d = torch.from_numpy(x).cuda()
+    out = torch.zeros(max(cap, 16), dtype=torch.uint8, device="cuda")
+    nbytes = torch.zeros(1, dtype=torch.int64, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(hg.huff_workspace_size(x.size, CHUNK), dtype=torch.uint8, device="cuda")
+    rc = hg.lib().huff_encode(d.data_ptr(), x.size, cb.data_ptr(), CHUNK, out.data_ptr(), cap,
+                              nbytes.data_ptr(), ws.data_ptr(), ws.numel(), status.data_ptr(), None)
+    torch.cuda.synchronize()
+    assert rc == 0
+    return int(status), int(nbytes), out.cpu().numpy()
+
+
+@pytest.mark.parametrize("longest", [1, 2, 3, 7, 8, 10, 11, 15, 16, 22, 23, 31, 32])
+@pytest.mark.parametrize("skewed", [False, True])
+def test_lengths_sizes_and_capacities(longest, skewed):
+    lengths = np.zeros(256, np.uint8)
+    lengths[: longest + 1] = list(range(1, longest + 1)) + [longest]
+    cb = _codebook(lengths)
+    rng = np.random.default_rng(longest)
+    for n in SIZES:
+        # skewed: as rare as the codes are long; else long codes in every group
+        x = rng.geometric(0.5, n) - 1 if skewed else rng.integers(0, longest + 1, n)
+        x = np.minimum(x, longest).astype(np.uint8)
+        x[-1] = longest  # a long last code
+        ost, ref, size = oracle.encode(x, lengths, CHUNK, 400 + 8 * n)
+        assert ost == oracle.OK
+        for cap in (size, size + 64):
+            st, nbytes, out = _encode(x, cb, cap)
+            assert (st, nbytes) == (0, size), (n, cap)
+            assert np.array_equal(out[:size], ref[:size]), (n, cap)
+        st, nbytes, _ = _encode(x, cb, size - 4)
+        assert (st, nbytes) == (hg.HUFF_ERR_CAPACITY, size), n
+
+
+@pytest.mark.parametrize("longest", [4, 8, 16])
+def test_bytes_without_a_code_add_no_bits(longest):
+    lengths = np.zeros(256, np.uint8)
+    lengths[: longest + 1] = list(range(1, longest + 1)) + [longest]
+    cb = _codebook(lengths)
+    rng = np.random.default_rng(longest)
+    for n in SIZES:
+        if n > 16384:
+            continue
+        x = np.full(n, 200, np.uint8)  # no code
+        some = rng.random(n) < rng.choice([0.0, 0.01, 0.3])
+        x[some] = rng.integers(0, longest + 1, int(some.sum()))
+        cap = 400 + 8 * n
+        st, nbytes, out = _encode(x, cb, cap)
+        kept = x[x != 200]
+        words = np.zeros(0, np.uint8)
+        if kept.size:
+            _, ref, size = oracle.encode(kept, lengths, CHUNK, 400 + 8 * n)
+            words = ref[272 + 8 * -(-kept.size // CHUNK) : size]
+        head = 272 + 8 * -(-n // CHUNK)
+        assert (st, nbytes) == (0, head + words.size), n
+        assert np.array_equal(out[head : head + words.size], words), n
