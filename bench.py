@@ -693,9 +693,9 @@ def run_ours(args):
     stream = torch.cuda.current_stream()
     # five events per timed step bracket the four calls (kernels on this stream)
     evs = [[torch.cuda.Event(enable_timing=True) for _ in range(5)] for _ in range(args.steps)]
-    # k_histogram, k_build_codebook, k_unit_bits_hist, k_scan_tile_sums,
-    # k_scan_apply, k_encode, k_decode
-    launches_per_step = 7
+    # k_clear, k_histogram, k_build_codebook, k_unit_bits_hist,
+    # k_scan_tile_sums, k_scan_apply, k_encode, k_decode
+    launches_per_step = 8
 
     def step(ev=None):
         if ev:

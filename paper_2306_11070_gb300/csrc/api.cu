@@ -234,9 +234,7 @@ huff_status_t huff_compress(const uint8_t *d_in, uint64_t n, uint32_t chunk_symb
     huff_codebook_t *cb = reinterpret_cast<huff_codebook_t *>(ws + kWsCodebookOffset);
     uint16_t *unit_hist = reinterpret_cast<uint16_t *>(ws + kWsUnitHistOffset);
     uint8_t *enc_ws = ws + kWsUnitHistOffset + unit_hist_bytes(n);
-    if (cudaMemsetAsync(d_status, 0, sizeof(int32_t), s) != cudaSuccess)
-        return HUFF_ERR_CUDA;
-    if (launch_histogram(d_in, n, hist, unit_hist, s) != cudaSuccess)
+    if (launch_histogram(d_in, n, hist, unit_hist, s, d_status) != cudaSuccess)
         return HUFF_ERR_CUDA;
     if (launch_build_codebook(hist, cb, d_status, s) != cudaSuccess)
         return HUFF_ERR_CUDA;

@@ -21,10 +21,12 @@ namespace {
 constexpr int kCbBlock = 256;
 
 __global__ void __launch_bounds__(kCbBlock)
-    k_build_codebook(const unsigned long long *__restrict__ hist, huff_codebook_t *__restrict__ cb,
+    k_build_codebook(const unsigned long long *hist, huff_codebook_t *cb,
                      int32_t *status, int limit, int limited)
 {
     __shared__ cbk::CodebookShared sh;
+    chain_wait();
+    chain_next();
     cbk::build_codebook(hist, cb, status, sh, limit, limited != 0);
 }
 
@@ -34,9 +36,8 @@ cudaError_t launch_build_codebook(const unsigned long long *d_hist, huff_codeboo
                                   int32_t *d_status, cudaStream_t s, uint32_t limit)
 {
     const bool limited = limit != 0;
-    k_build_codebook<<<1, kCbBlock, 0, s>>>(d_hist, d_cb, d_status,
-                                            limited ? (int)limit : (int)kMaxCodeLen, limited);
-    return cudaGetLastError();
+    return launch_chained(k_build_codebook, 1, kCbBlock, 0, s, d_hist, d_cb, d_status,
+                          limited ? (int)limit : (int)kMaxCodeLen, (int)limited);
 }
 
 }  // namespace huff

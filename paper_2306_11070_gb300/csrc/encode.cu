@@ -112,18 +112,22 @@ __device__ __noinline__ void encode_long(const EncodeArgs &a)
 __global__ void __launch_bounds__(kEncBlock, 1) k_encode(const __grid_constant__ EncodeArgs a)
 {
     extern __shared__ uint4 smem_raw[];
-    if (chain_failed(a.status))
-        return;
-    const uint32_t max_len = a.cb->max_len;
+    // the offsets' scan is the kernel before this one and lets it start once
+    // the kernels before the scan are complete, the codebook's among them: the
+    // table is built while the scan runs
     const Smem m = carve(smem_raw);
-    const Job J = make_job(a.in, a.n, a.cs, a.unit_off, a.out, a.out_cap);
-    if (blockIdx.x == 0)
-        write_header(J, a.cb, a.out_bytes, a.status);
+    const uint32_t max_len = a.cb->max_len;
     const int group = max_len <= kMadMaxLen ? mad_group(max_len) : 0;
     if (group)
         build_table2(a.cb, m.tbl);
     else
         build_table(a.cb, m.tbl, false);
+    chain_wait();
+    if (chain_failed(a.status))
+        return;
+    const Job J = make_job(a.in, a.n, a.cs, a.unit_off, a.out, a.out_cap);
+    if (blockIdx.x == 0)
+        write_header(J, a.cb, a.out_bytes, a.status);
     __syncthreads();  // the only CTA barrier: the table is ready
     if (group < 3) {
         if (!group)
@@ -190,8 +194,7 @@ cudaError_t launch_encode(const uint8_t *d_in, uint64_t n, const huff_codebook_t
         grid = units;
     if (grid < 1)
         grid = 1;
-    k_encode<<<(unsigned)grid, kEncBlock, kEncSmemBytes, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_encode, grid, kEncBlock, kEncSmemBytes, s, a);
 }
 
 }  // namespace huff

@@ -23,11 +23,23 @@ using namespace hst;
 
 constexpr int kHistBlock = kThreads;
 
+// Clears the totals (and the chain's status).  A kernel instead of memory sets,
+// because the histogram can be launched behind it and needs the totals only
+// at its end.
+__global__ void __launch_bounds__(256) k_clear(unsigned long long *hist, int32_t *status)
+{
+    chain_next();
+    hist[threadIdx.x] = 0;
+    if (status && threadIdx.x == 0)
+        *status = 0;
+}
+
 __global__ void __launch_bounds__(kHistBlock)
     k_histogram(const uint8_t *__restrict__ in, uint64_t n, unsigned long long *__restrict__ hist,
                 uint16_t *__restrict__ unit_hist)
 {
     __shared__ __align__(16) uint32_t cnt[256 * 32];
+    chain_next();
     const int tid = threadIdx.x, lane = tid & 31;
     for (int i = tid; i < 256 * 32; i += kHistBlock)
         cnt[i] = 0;
@@ -55,6 +67,7 @@ __global__ void __launch_bounds__(kHistBlock)
     }
     __syncthreads();
     const uint32_t s = fold_bin(cnt, tid);
+    chain_wait();  // the totals are cleared
     if (s)
         atomicAdd(hist + tid, (unsigned long long)s);
 }
@@ -62,9 +75,10 @@ __global__ void __launch_bounds__(kHistBlock)
 }  // namespace
 
 cudaError_t launch_histogram(const uint8_t *d_in, uint64_t n, unsigned long long *d_hist,
-                             uint16_t *d_unit_hist, cudaStream_t s)
+                             uint16_t *d_unit_hist, cudaStream_t s, int32_t *d_status)
 {
-    cudaError_t err = cudaMemsetAsync(d_hist, 0, 256 * sizeof(unsigned long long), s);
+    k_clear<<<1, 256, 0, s>>>(d_hist, d_status);
+    cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess || n == 0)
         return err;
     static KernelSetup setup;
@@ -78,8 +92,7 @@ cudaError_t launch_histogram(const uint8_t *d_in, uint64_t n, unsigned long long
     const uint64_t units = (n + kUnitSymbols - 1) / kUnitSymbols;
     const uint64_t cap = (uint64_t)sms * per_sm;
     const uint64_t grid = units < cap ? units : cap;
-    k_histogram<<<(unsigned)grid, kHistBlock, 0, s>>>(d_in, n, d_hist, d_unit_hist);
-    return cudaGetLastError();
+    return launch_chained(k_histogram, grid, kHistBlock, 0, s, d_in, n, d_hist, d_unit_hist);
 }
 
 }  // namespace huff

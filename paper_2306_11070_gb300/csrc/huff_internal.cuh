@@ -144,6 +144,45 @@ struct KernelSetup {
 cudaError_t kernel_setup(KernelSetup &ks, const void *func, int block, size_t dyn_smem,
                          int *per_sm);
 
+// ---- overlapped launches ----------------------------------------------------
+// Short kernels that follow one another in a stream: the next one is launched
+// while the one before it still runs, and waits for its end and its writes in
+// chain_wait(), so that a launch's latency (1 to 2 us) passes beside the work
+// instead of after it (64 MiB compress, six kernels: 89 -> 75 us, with the two
+// memory sets and the scan's first kernel gone).  Every thread of a kernel
+// launched so calls chain_wait()
+// on every path, before it touches what an earlier kernel writes or reads;
+// therefore, once a kernel is past its own wait, all kernels before its
+// predecessor are complete too.  chain_next() lets the next kernel start.  What
+// such a kernel reads of its predecessors has no __restrict__: a load through
+// the read-only path could be moved above the wait.
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+__device__ __forceinline__ void chain_next()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), uint64_t grid, int block, size_t smem,
+                                  cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 }  // namespace huff
 
 // Kernel launchers (one per translation unit); each returns a cudaError_t.
@@ -153,8 +192,9 @@ namespace huff {
 // optional per-unit histograms).  16 KiB; u16 counts cannot overflow.
 constexpr uint32_t kUnitSymbols = 16384;
 
+// d_status, if given, is cleared too
 cudaError_t launch_histogram(const uint8_t *d_in, uint64_t n, unsigned long long *d_hist,
-                             uint16_t *d_unit_hist, cudaStream_t s);
+                             uint16_t *d_unit_hist, cudaStream_t s, int32_t *d_status = nullptr);
 // limit 0: plain Huffman (codes over 32 bits are an error); 1..32: codes of
 // at most `limit` bits (package-merge where the Huffman code exceeds it)
 cudaError_t launch_build_codebook(const unsigned long long *d_hist, huff_codebook_t *d_cb,

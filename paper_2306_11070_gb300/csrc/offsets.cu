@@ -22,11 +22,13 @@ constexpr int kDotBlock = 256;
 constexpr int kCountBlock = 256;
 
 __global__ void __launch_bounds__(kDotBlock)
-    k_unit_bits_hist(const uint16_t *__restrict__ unit_hist, uint64_t units,
-                     const huff_codebook_t *__restrict__ cb, uint32_t *__restrict__ unit_bits,
+    k_unit_bits_hist(const uint16_t *unit_hist, uint64_t units,
+                     const huff_codebook_t *cb, uint32_t *unit_bits,
                      const int32_t *status)
 {
     __shared__ uint32_t len[256];
+    chain_wait();
+    chain_next();
     if (chain_failed(status))
         return;
     len[threadIdx.x] = cb->len[threadIdx.x];
@@ -49,12 +51,14 @@ __global__ void __launch_bounds__(kDotBlock)
 }
 
 __global__ void __launch_bounds__(kCountBlock)
-    k_unit_bits_input(const uint8_t *__restrict__ in, uint64_t n,
-                      const huff_codebook_t *__restrict__ cb, uint32_t *__restrict__ unit_bits,
+    k_unit_bits_input(const uint8_t *in, uint64_t n,
+                      const huff_codebook_t *cb, uint32_t *unit_bits,
                       const int32_t *status)
 {
     __shared__ uint32_t len[256 * 32];  // [byte][lane]
     __shared__ uint32_t s_warp[kCountBlock / 32];
+    chain_wait();
+    chain_next();
     if (chain_failed(status))
         return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -105,13 +109,16 @@ __global__ void __launch_bounds__(kCountBlock)
 // The exclusive scan of the unit counts in two launches over tiles of
 // kScanTile units (one CTA per tile, each thread kScanPer consecutive counts
 // loaded with 16-byte loads that are all in flight at once):
-//  - k_scan_tile_sums: every tile's total;
+//  - k_scan_tile_sums: every tile's total (not for few tiles, see kScanDirect);
 //  - k_scan_apply: every tile adds up the totals of the tiles before it (a
 //    few dozen at 1 GiB), scans its own counts and writes the u64 offsets;
 //    the last tile also writes the grand total at index `units`.
 constexpr int kScanThreads = 256;
 constexpr int kScanPer = 8;
 constexpr uint32_t kScanTile = kScanThreads * kScanPer;  // 2048 units
+// Up to this many tiles (256 MiB) the last tile's 14 loads per thread of the
+// counts before it cost less than a launch for the totals.
+constexpr uint32_t kScanDirect = 8;
 
 __device__ __forceinline__ void load_counts(const uint32_t *unit_bits, uint64_t units, uint64_t i,
                                             uint32_t (&v)[kScanPer])
@@ -156,10 +163,12 @@ __device__ __forceinline__ unsigned long long block_scan_u64(unsigned long long 
 }
 
 __global__ void __launch_bounds__(kScanThreads)
-    k_scan_tile_sums(const uint32_t *__restrict__ unit_bits, uint64_t units,
-                     unsigned long long *__restrict__ tile_sum, const int32_t *status)
+    k_scan_tile_sums(const uint32_t *unit_bits, uint64_t units,
+                     unsigned long long *tile_sum, const int32_t *status)
 {
     __shared__ unsigned long long s_warp[kScanThreads / 32];
+    chain_wait();
+    chain_next();
     if (chain_failed(status))
         return;
     uint32_t v[kScanPer];
@@ -176,18 +185,29 @@ __global__ void __launch_bounds__(kScanThreads)
 }
 
 __global__ void __launch_bounds__(kScanThreads)
-    k_scan_apply(const uint32_t *__restrict__ unit_bits, uint64_t units,
-                 const unsigned long long *__restrict__ tile_sum,
-                 unsigned long long *__restrict__ unit_off, const int32_t *status)
+    k_scan_apply(const uint32_t *unit_bits, uint64_t units,
+                 const unsigned long long *tile_sum,
+                 unsigned long long *unit_off, const int32_t *status)
 {
     __shared__ unsigned long long s_warp[kScanThreads / 32];
     __shared__ unsigned long long s_base;
+    chain_wait();
+    chain_next();
     if (chain_failed(status))
         return;
-    // the totals of the tiles before this one
+    // the units before this tile: the tiles' totals, or the counts themselves
     unsigned long long b = 0;
-    for (uint32_t t = threadIdx.x; t < blockIdx.x; t += kScanThreads)
-        b += tile_sum[t];
+    if (tile_sum) {
+        for (uint32_t t = threadIdx.x; t < blockIdx.x; t += kScanThreads)
+            b += tile_sum[t];
+    } else {
+        const uint4 *q = reinterpret_cast<const uint4 *>(unit_bits);
+#pragma unroll 8
+        for (uint32_t t = threadIdx.x; t < blockIdx.x * (kScanTile / 4); t += kScanThreads) {
+            const uint4 v = q[t];
+            b += (unsigned long long)v.x + v.y + v.z + v.w;
+        }
+    }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1)
         b += __shfl_xor_sync(0xffffffffu, b, d);
@@ -239,32 +259,37 @@ cudaError_t launch_unit_offsets(const uint8_t *d_in, uint64_t n, const uint16_t 
     const int sms = device_sm_count();
     if (sms < 1)
         return cudaErrorInvalidDevice;
+    cudaError_t err;
     if (d_unit_hist) {
         uint64_t grid = (units + (kDotBlock / 32) - 1) / (kDotBlock / 32);
         if (grid > (uint64_t)sms * 8)
             grid = (uint64_t)sms * 8;
-        k_unit_bits_hist<<<(unsigned)grid, kDotBlock, 0, s>>>(d_unit_hist, units, d_cb, d_unit_bits,
-                                                              d_status);
+        err = launch_chained(k_unit_bits_hist, grid, kDotBlock, 0, s, d_unit_hist, units, d_cb,
+                             d_unit_bits, d_status);
     } else {
         static KernelSetup setup;
         int per_sm = 0;
-        const cudaError_t err =
-            kernel_setup(setup, (const void *)k_unit_bits_input, kCountBlock, 0, &per_sm);
+        err = kernel_setup(setup, (const void *)k_unit_bits_input, kCountBlock, 0, &per_sm);
         if (err != cudaSuccess)
             return err;
-        uint64_t grid = units < (uint64_t)sms * per_sm ? units : (uint64_t)sms * per_sm;
-        k_unit_bits_input<<<(unsigned)grid, kCountBlock, 0, s>>>(d_in, n, d_cb, d_unit_bits,
-                                                                 d_status);
+        const uint64_t grid = units < (uint64_t)sms * per_sm ? units : (uint64_t)sms * per_sm;
+        err = launch_chained(k_unit_bits_input, grid, kCountBlock, 0, s, d_in, n, d_cb, d_unit_bits,
+                             d_status);
     }
-    cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess)
         return err;
     static_assert(kScanTile == 2048, "unit_scan_tiles assumes 2048-unit tiles");
     const uint32_t tiles = (uint32_t)unit_scan_tiles(units);
-    k_scan_tile_sums<<<tiles, kScanThreads, 0, s>>>(d_unit_bits, units, d_tile_sum, d_status);
-    k_scan_apply<<<tiles, kScanThreads, 0, s>>>(d_unit_bits, units, d_tile_sum, d_unit_off,
-                                                d_status);
-    return cudaGetLastError();
+    if (tiles <= kScanDirect) {
+        d_tile_sum = nullptr;
+    } else {
+        err = launch_chained(k_scan_tile_sums, tiles, kScanThreads, 0, s, d_unit_bits, units,
+                             d_tile_sum, d_status);
+        if (err != cudaSuccess)
+            return err;
+    }
+    return launch_chained(k_scan_apply, tiles, kScanThreads, 0, s, d_unit_bits, units, d_tile_sum,
+                          d_unit_off, d_status);
 }
 
 }  // namespace huff

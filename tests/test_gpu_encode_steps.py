@@ -90,3 +90,35 @@ def test_bytes_without_a_code_add_no_bits(longest):
         head = 272 + 8 * -(-n // CHUNK)
         assert (st, nbytes) == (0, head + words.size), n
         assert np.array_equal(out[head : head + words.size], words), n
+
+
+@pytest.mark.parametrize("n", [0, 5, 70000, 5 << 20])
+def test_chained_launches_under_capture_and_back_to_back(n):
+    rng = np.random.default_rng(n)
+    xs = [np.minimum(rng.geometric(0.3, n) * k % 256, 255).astype(np.uint8) for k in (1, 3, 7)]
+    refs = [oracle.compress(x)[1] for x in xs]
+    d = torch.zeros(max(n, 1), dtype=torch.uint8, device="cuda")
+    cap = hg.huff_max_stream_size(n)
+    out = torch.zeros(cap, dtype=torch.uint8, device="cuda")
+    nbytes = torch.zeros(1, dtype=torch.int64, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(hg.huff_workspace_size(n), dtype=torch.uint8, device="cuda")
+
+    def run():
+        hg.huff_compress(d[:n], d_out=out, d_out_bytes=nbytes, d_ws=ws, d_status=status)
+
+    run()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run()
+    for go in (graph.replay, run):
+        got = []
+        for x in xs:  # one workspace, no synchronisation in between
+            d[:n].copy_(torch.from_numpy(x))
+            go()
+            got.append((out.clone(), nbytes.clone(), status.clone()))
+        torch.cuda.synchronize()
+        for (o, b, s), ref in zip(got, refs):
+            assert int(s) == 0 and int(b) == ref.size
+            assert np.array_equal(o[: ref.size].cpu().numpy(), ref)
