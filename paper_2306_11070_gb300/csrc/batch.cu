@@ -185,6 +185,38 @@ __device__ __forceinline__ unsigned int half_broadcast(unsigned int t, HalfSync 
 }
 
 // ------------------------------------------------------------------ compress
+// The code table of both halves starts at this address of the shared window (a
+// constant, so that it is part of the table loads), a little above the end of
+// the static shared memory.
+constexpr uint32_t kTblAt = 6144;
+constexpr uint32_t kTblSlack = 1024;
+
+// One function per way of grouping: inlined together they spill.
+template <int G, int kFirst, int S>
+__device__ __noinline__ bool unit_by(const enc::Job J, uint64_t u, const uint32_t *tbl, uint32_t *wob)
+{
+    return enc::encode_unit_mad<G, kFirst, S, kTblAt>(J, u, tbl, wob);
+}
+
+__device__ __noinline__ bool unit_long(const enc::Job J, uint64_t u, const uint32_t *tbl, uint32_t *wob)
+{
+    return enc::encode_unit_long(J, u, tbl, wob);
+}
+
+__device__ __forceinline__ bool encode_unit(const enc::Job &J, uint64_t u, const uint32_t *tbl, int plan,
+                                            uint32_t *wob)
+{
+    switch (plan) {
+    case enc::kFit16: return unit_by<16, 16, 16>(J, u, tbl, wob);
+    case enc::kFit8: return unit_by<8, 8, 8>(J, u, tbl, wob);
+    case enc::kFit4: return unit_by<4, 4, 4>(J, u, tbl, wob);
+    case enc::kFit3: return unit_by<3, 3, 3>(J, u, tbl, wob);
+    case enc::kTry4: return unit_by<4, 1, 1>(J, u, tbl, wob);
+    case enc::kTry3: return unit_by<3, 1, 1>(J, u, tbl, wob);
+    default: return unit_long(J, u, tbl, wob);
+    }
+}
+
 __global__ void __launch_bounds__(kBatchBlock, 2) k_batch_compress(BatchArgs a)
 {
     extern __shared__ uint4 smem_raw[];
@@ -359,11 +391,16 @@ __global__ void __launch_bounds__(kBatchBlock, 2) k_batch_compress(BatchArgs a)
     {
         const int half = warp / kHalfWarps, htid = tid & (kHalf - 1), hwarp = warp % kHalfWarps;
         const HalfSync hs{half};
-        uint32_t *tbl = reinterpret_cast<uint32_t *>(smem_raw) + half * enc::kTblWords;
-        uint32_t *wob = reinterpret_cast<uint32_t *>(smem_raw) + 2 * enc::kTblWords + warp * enc::kWarpObuf;
+        const uint32_t pad = kTblAt - smem_u32(smem_raw);
+        if (pad > kTblSlack) {  // not where the table's address is encoded
+            fail_all(a.bufs, a.count);
+            return;
+        }
+        uint32_t *tbl = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned char *>(smem_raw) + pad);
+        uint32_t *wob = tbl + enc::kTblWords + warp * enc::kWarpObuf;
+        tbl += half * (enc::kTblRow / 2);
         uint32_t have = 0xffffffffu;  // buffer whose table is loaded
-        bool fast = true;
-        int group = 1;
+        int plan = enc::kLong;
         const unsigned int t0 = htid == 0 ? atomicAdd(a.ctl + kCtlTicket0 + 1, 1u) : 0u;
         for (unsigned int it = half_broadcast(t0, hs); it < total_items;) {
             const unsigned int nxt =
@@ -374,21 +411,20 @@ __global__ void __launch_bounds__(kBatchBlock, 2) k_batch_compress(BatchArgs a)
             const bool failed =  // this buffer's codebook failed
                 half_broadcast(htid == 0 ? (unsigned int)chain_failed(B.status) : 0u, hs) != 0;
             if (!failed) {
-                if (b != have) {
-                    const uint32_t max_len = a.cbs[b].max_len;
-                    fast = max_len <= (uint32_t)enc::kFastMaxLen;
-                    group = enc::emit_group(max_len);
-                    enc::build_table(a.cbs + b, tbl, fast, htid, kHalf);
-                    hs();
-                    have = b;
-                }
                 const uint64_t u0 = ow.z | ((uint64_t)ow.w << 32);
                 const enc::Job J =
                     enc::make_job(B.in, B.in_bytes, a.cs, a.unit_off + u0 + b, B.out, B.out_cap);
+                if (b != have) {
+                    const uint32_t max_len = a.cbs[b].max_len;
+                    plan = enc::plan_of(J, max_len);
+                    enc::build_table(a.cbs + b, tbl, plan != enc::kLong, htid, kHalf);
+                    hs();
+                    have = b;
+                }
                 const uint64_t u = (uint64_t)ow.y * kUnitsPerItem + hwarp;
                 bool overflow = false;
                 if (u < J.units)
-                    overflow = enc::encode_unit(J, u, tbl, fast, group, wob);
+                    overflow = encode_unit(J, u, tbl, plan, wob);
                 if (overflow)
                     set_status(B.status, HUFF_ERR_CAPACITY);
             }
@@ -560,11 +596,10 @@ __global__ void __launch_bounds__(kBatchBlock, 2) k_batch_decompress(BatchArgs a
     }
 }
 
-// phase 1's two sets of histogram columns, or phase 3's two code tables and
-// word buffers, whichever is larger
-constexpr int kCompressSmem = (2 * enc::kTblWords + kBatchWarps * enc::kWarpObuf) * 4 > 2 * 256 * 32 * 4
-                                  ? (2 * enc::kTblWords + kBatchWarps * enc::kWarpObuf) * 4
-                                  : 2 * 256 * 32 * 4;
+// phase 3's code tables and word buffers (phase 1's two sets of histogram
+// columns take less)
+constexpr int kCompressSmem = (int)kTblSlack + (enc::kTblWords + kBatchWarps * enc::kWarpObuf) * 4;
+static_assert(kCompressSmem >= 2 * 256 * 32 * 4, "phase 1's columns");
 
 }  // namespace
 

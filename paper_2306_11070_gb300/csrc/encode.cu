@@ -35,8 +35,8 @@ using namespace enc;
 constexpr int kEncBlock = 512;
 constexpr int kEncWarps = kEncBlock / 32;
 // the table, the padding before it, and the buffers if the gap is too small
-constexpr int kEncObufBytes = kEncWarps * kMadObuf * 4;
-constexpr int kEncSmemBytes = 65536 + kTbl2Words * 4 + kEncObufBytes;
+constexpr int kEncObufBytes = kEncWarps * kWarpObuf * 4;
+constexpr int kEncSmemBytes = 65536 + kTblWords * 4 + kEncObufBytes;
 
 struct EncodeArgs {
     const uint8_t *in;
@@ -50,8 +50,7 @@ struct EncodeArgs {
     int32_t *status;
 };
 
-// This warp's part of the CTA's dynamic shared memory, and the code table:
-// [256][32] (code, 2^len) pairs, or 2 x [256][16] for 32-bit codes.  The table
+// This warp's part of the CTA's dynamic shared memory, and the code table, which
 // lies at a 64 KiB boundary of the shared window, so that the address of a
 // byte's entry is one byte permutation of the data word and the lane's column
 // (a multiply-add per symbol fewer); the warps' buffers take the gap before
@@ -66,8 +65,8 @@ __device__ __forceinline__ Smem carve(uint4 *smem_raw)
     unsigned char *raw = reinterpret_cast<unsigned char *>(smem_raw);
     Smem m;
     m.tbl = reinterpret_cast<uint32_t *>(raw + pad);
-    m.wob = reinterpret_cast<uint32_t *>(raw + (pad >= (uint32_t)kEncObufBytes ? 0u : pad + kTbl2Words * 4)) +
-            (threadIdx.x >> 5) * kMadObuf;
+    m.wob = reinterpret_cast<uint32_t *>(raw + (pad >= (uint32_t)kEncObufBytes ? 0u : pad + kTblWords * 4)) +
+            (threadIdx.x >> 5) * kWarpObuf;
     return m;
 }
 
@@ -79,9 +78,7 @@ __device__ __forceinline__ Smem carve(uint4 *smem_raw)
     for (uint64_t u = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; u < (J).units; \
          u += (uint64_t)gridDim.x * kEncWarps)
 
-// Codes of 11 to 31 bits, in groups of G that nearly always fit.  Functions of
-// their own, as is encode_long: inlined into the kernel they would make it
-// spill (1 GiB of text: the call takes 1010 us instead of 839).
+// Codes of 11 to 31 bits, in groups of G that nearly always fit.
 template <int G>
 __device__ __noinline__ void encode_try(const EncodeArgs &a)
 {
@@ -90,7 +87,7 @@ __device__ __noinline__ void encode_try(const EncodeArgs &a)
     const Job J = make_job(a.in, a.n, a.cs, a.unit_off, a.out, a.out_cap);
     bool overflow = false;
     FOR_UNITS(u, J)
-        overflow |= encode_unit_mad<G, 1, 1>(J, u, m.tbl, m.wob);
+        overflow |= encode_unit_mad<G, 1, 1, 0>(J, u, m.tbl, m.wob);
     if (overflow)
         set_status(a.status, HUFF_ERR_CAPACITY);
 }
@@ -107,6 +104,21 @@ __device__ __noinline__ void encode_long(const EncodeArgs &a)
         set_status(a.status, HUFF_ERR_CAPACITY);
 }
 
+// A function, called once per unit, and the rarer plans in functions of their
+// own: inlined into the kernel, all or each by itself, they spill or are
+// scheduled worse (1 GiB of text: the call takes 810 to 1010 us instead of
+// 795).
+__device__ __noinline__ bool encode_unit_fit(const Job J, uint64_t u, const uint32_t *tbl, int plan,
+                                                uint32_t *wob)
+{
+    switch (plan) {
+    case kFit16: return encode_unit_mad<16, 16, 16, 0>(J, u, tbl, wob);
+    case kFit8: return encode_unit_mad<8, 8, 8, 0>(J, u, tbl, wob);
+    case kFit4: return encode_unit_mad<4, 4, 4, 0>(J, u, tbl, wob);
+    default: return encode_unit_mad<3, 3, 3, 0>(J, u, tbl, wob);
+    }
+}
+
 // One kernel for all code lengths: the host does not know them, and a second
 // launch that only finds out that it does not apply costs 2 us or more.
 __global__ void __launch_bounds__(kEncBlock, 1) k_encode(const __grid_constant__ EncodeArgs a)
@@ -117,11 +129,7 @@ __global__ void __launch_bounds__(kEncBlock, 1) k_encode(const __grid_constant__
     // table is built while the scan runs
     const Smem m = carve(smem_raw);
     const uint32_t max_len = a.cb->max_len;
-    const int group = max_len <= kMadMaxLen ? mad_group(max_len) : 0;
-    if (group)
-        build_table2(a.cb, m.tbl);
-    else
-        build_table(a.cb, m.tbl, false);
+    build_table(a.cb, m.tbl, max_len <= kMadMaxLen, threadIdx.x, kEncBlock);
     chain_wait();
     if (chain_failed(a.status))
         return;
@@ -129,18 +137,19 @@ __global__ void __launch_bounds__(kEncBlock, 1) k_encode(const __grid_constant__
     if (blockIdx.x == 0)
         write_header(J, a.cb, a.out_bytes, a.status);
     __syncthreads();  // the only CTA barrier: the table is ready
-    if (group < 3) {
-        if (!group)
+    bool overflow = false;
+    const int plan = plan_of(J, max_len);
+    if (plan < kFit3) {
+        if (plan == kLong)
             encode_long(a);
-        else if (few_bits(J))
+        else if (plan == kTry4)
             encode_try<4>(a);
         else
             encode_try<3>(a);
         return;
     }
-    bool overflow = false;
     FOR_UNITS(u, J)
-        overflow |= encode_unit_mad_g(J, u, m.tbl, group, m.wob);
+        overflow |= encode_unit_fit(J, u, m.tbl, plan, m.wob);
     if (overflow)
         set_status(a.status, HUFF_ERR_CAPACITY);
 }

@@ -7,24 +7,23 @@
 namespace huff {
 namespace enc {
 
-constexpr int kTblWords = 256 * 32;  // [byte][lane] table, 32 KiB
-// fast path (codes of at most kFastMaxLen bits): 32 symbols per lane and
-// step, 1024 per warp step, 16 steps per unit
-constexpr int kFastSyms = 32;
-constexpr int kFastStep = 32 * kFastSyms;
-constexpr int kFastSteps = kUnitSymbols / kFastStep;
-// the low 10 bits of a sum of 32 entries are the sum of their lengths while
-// every length is at most 22 (the code sits above bit 9 of its entry)
-constexpr uint32_t kFastMaxLen = 22;
-constexpr uint32_t kSumMask = 1023;
-// long codes (23..32 bits): 16 symbols per lane and step
+// 32 symbols per lane and step, 1024 per warp step, 16 steps per unit
+constexpr int kStepSyms = 32;
+constexpr int kStep = 32 * kStepSyms;
+constexpr int kSteps = kUnitSymbols / kStep;
+// 32-bit codes: 16 symbols per lane and step
 constexpr int kLongSyms = 16;
 constexpr int kLongStep = 32 * kLongSyms;
 constexpr int kLongSteps = kUnitSymbols / kLongStep;
-// warp buffer: a guard word, then the words of one step (a fast step writes
-// at most 1024 x 22 / 32 = 704 words after the < 32 carried bits, a long one
-// 512 x 32 / 32 = 512), rounded up
-constexpr int kWarpObuf = 1 + kFastStep * (int)kFastMaxLen / 32 + 15;  // 720 words
+constexpr uint32_t kMadMaxLen = 31;  // a group's marker takes a bit
+// warp buffer: a guard word, then a step of 1024 codes after < 32 carried bits
+constexpr int kWarpObuf = 1 + kStep * (int)kMadMaxLen / 32 + 15;
+// Code table: 256 rows of 64 words, of which a stream uses one half (16
+// columns of two words: lanes l and l + 16 share a column, and still no lookup
+// collides, because a warp's 64-bit loads are made for 16 lanes at a time).
+// The two halves of a row belong to two streams where two are written at once.
+constexpr int kTblRow = 64;
+constexpr int kTblWords = 256 * kTblRow;  // 64 KiB
 
 // One stream being written: input, unit offsets, output layout.
 struct Job {
@@ -59,13 +58,6 @@ __device__ __forceinline__ Job make_job(const uint8_t *in, uint64_t n, uint32_t 
     return j;
 }
 
-// Codes per emit check in the fast path: floor(32 / longest), as a template.
-__device__ __forceinline__ int emit_group(uint32_t max_len)
-{
-    const uint32_t gq = max_len ? 32u / max_len : 16u;
-    return gq >= 16 ? 16 : gq >= 8 ? 8 : gq >= 4 ? 4 : gq >= 3 ? 3 : gq >= 2 ? 2 : 1;
-}
-
 // Header (threads 0..255 of the calling CTA) and the stream size.
 __device__ __forceinline__ void write_header(const Job &J, const huff_codebook_t *cb,
                                              unsigned long long *out_bytes, int32_t *status)
@@ -88,50 +80,11 @@ __device__ __forceinline__ void write_header(const Job &J, const huff_codebook_t
     }
 }
 
-// Entry of the fast table at shared address a (the table is read-only
-// while units are encoded).
-__device__ __forceinline__ uint32_t tbl_at(uint32_t a)
-{
-    uint32_t v;
-    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-    return v;
-}
-
-// Per-lane replicated code table (16-byte aligned), built by threads tid =
-// 0..nt-1 (by default all threads of the CTA).  Fast entry = (code << (32 -
-// len)) | len: the code left-aligned, its length in the low bits, zeros
-// between them (len <= 22 leaves bits 5..9 clear).  A thread per byte reads
-// its length and code once and fills the byte's 32 lane copies with eight
-// 16-byte stores, rotated by the byte so that the stores of a warp spread
-// over all eight 16-byte bank groups.
-__device__ __forceinline__ void build_table(const huff_codebook_t *cb, uint32_t *tbl, bool fast,
-                                            int tid = threadIdx.x, int nt = blockDim.x)
-{
-    if (fast) {
-        for (int b = tid; b < 256; b += nt) {
-            const uint32_t L = cb->len[b];
-            const uint32_t e = L ? (cb->code[b] << (32 - L)) | L : 0u;
-            const uint4 v = make_uint4(e, e, e, e);
-            uint4 *row = reinterpret_cast<uint4 *>(tbl + b * 32);
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                row[(j + b) & 7] = v;
-        }
-    } else {
-        for (int i = tid; i < 256 * 16; i += nt) {
-            const int b = i >> 4;
-            tbl[i] = cb->code[b];
-            tbl[256 * 16 + i] = cb->len[b];
-        }
-    }
-}
-
 // Zero this warp's buffer (kWarpObuf words at wob); every step leaves the
 // words it used zero again, so this runs once per unit.
-template <int kWords = kWarpObuf>
 __device__ __forceinline__ void clear_buffer(uint32_t *wob, int lane)
 {
-    for (int j = lane; j < kWords; j += 32)
+    for (int j = lane; j < kWarpObuf; j += 32)
         wob[j] = 0u;
     __syncwarp();
 }
@@ -147,73 +100,6 @@ __device__ __forceinline__ void red_or(uint32_t a, uint32_t v)
     asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
-// Pack the 32 codes of one lane (fast entries e, sums sc at every emit
-// check) into the warp's word buffer, the lane's bits starting at bit p0.
-// hi:lo holds the lane's last 64 bits.  With G = floor(32 / longest) codes
-// between checks, at most one word boundary is crossed per check; each check
-// writes the last completed word (its bits of this lane: bits of this lane
-// that were not yet shifted in are zero), so a word is written once or, with
-// the same bits, again.  A check before the lane's first word is complete
-// writes zeros to the word before it (the guard word for lane 0).
-//  - kSts (a full step: every lane has 32 codes, so at least 32 bits):
-//    plain stores.  Such a zero word can only land on the previous lane's
-//    last complete word, and only at a check before the last one, while
-//    that lane writes the word again at its last check; so every complete
-//    word ends with its owner's value, with no atomics and no clearing.
-//  - otherwise a lane may have no bits at all: OR into a zeroed buffer.
-// Returns the end of the lane's bits and its last partial word (zero bits
-// when there is none), high-aligned.
-template <int G, bool kSts>
-__device__ __forceinline__ uint32_t pack32(const uint32_t (&e)[kFastSyms],
-                                           const uint32_t (&sc)[(kFastSyms + G - 1) / G], uint32_t p0,
-                                           uint32_t wob_s, uint32_t &part)
-{
-    uint32_t hi = 0u, lo = 0u, E = p0;
-#pragma unroll
-    for (int k = 0; k < kFastSyms; ++k) {
-        const uint32_t x = e[k];
-        hi = __funnelshift_l(lo, hi, x);  // (hi:lo) <<= len
-        lo = __funnelshift_l(x, lo, x);   //   ... | code
-        if ((k + 1) % G == 0 || k == kFastSyms - 1) {
-            E = p0 + (sc[k / G] & kSumMask);  // end of the lane's bits so far
-            const uint32_t a = imad(E >> 5, kc[kFour], wob_s - 4), v = __funnelshift_r(lo, hi, E);
-            if (kSts)
-                sts(a, v);
-            else
-                red_or(a, v);
-        }
-    }
-    part = __funnelshift_lc(0u, lo, 32u - (E & 31u));
-    return E;
-}
-
-// The last r (< 32) bits of the code stream before symbol `base` (> 0), as the
-// high bits of a word: lane l re-codes byte base-1-l.  Warp-uniform result.
-__device__ __forceinline__ uint32_t seam_word(const uint8_t *in, uint64_t base, uint32_t r,
-                                              const uint32_t *tbl, bool fast, int lane)
-{
-    const uint32_t b = in[base - 1 - lane];
-    uint32_t L, code;
-    if (fast) {
-        const uint32_t x = tbl[(b << 5) | lane];
-        L = x & 31u;
-        code = L ? x >> (32 - L) : 0u;
-    } else {
-        code = tbl[(b << 4) | (lane & 15)];
-        L = tbl[256 * 16 + ((b << 4) | (lane & 15))];
-    }
-    uint32_t sfx = L;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, sfx, d);
-        if (lane >= d)
-            sfx += v;
-    }
-    const uint32_t before = sfx - L;  // bits between this code's end and base
-    const uint32_t part = (L && before < r) ? code << (32 - r + before) : 0u;
-    return __reduce_or_sync(0xffffffffu, part);
-}
-
 // Shared per-unit state of the encoders below.
 struct UnitState {
     uint64_t base;   // first symbol of the unit
@@ -222,21 +108,6 @@ struct UnitState {
     uint32_t lead;   // distance from the step start to the next chunk start
     uint64_t next_chunk;  // index of that chunk
 };
-
-__device__ __forceinline__ UnitState unit_start(const Job &J, uint64_t u, const uint32_t *tbl,
-                                                bool fast, int lane)
-{
-    UnitState st;
-    st.base = u * kUnitSymbols;
-    st.gbit = J.unit_off[u];
-    st.carry = (st.base > 0 && (st.gbit & 31))
-                   ? seam_word(J.in, st.base, (uint32_t)(st.gbit & 31), tbl, fast, lane)
-                   : 0u;
-    const uint32_t umod = (uint32_t)(st.base % J.cs);
-    st.lead = umod ? J.cs - umod : 0u;
-    st.next_chunk = (st.base + st.lead) / J.cs;
-    return st;
-}
 
 // This lane's SPT input bytes of the step starting at symbol sb (m of them
 // real, the rest zero), read straight from the input (partial steps only).
@@ -347,80 +218,6 @@ __device__ __forceinline__ bool step_output(const Job &J, UnitState &st, bool la
     return overflow;
 }
 
-// One 1024-symbol step of the fast encoder (codes of at most 22 bits, G =
-// floor(32 / longest)).  kInner: the step lies inside the input and the
-// unit's words fit the output, so the step needs none of the bound checks; its
-// 32 input bytes per lane (w) were loaded ahead.  It returns true, with
-// nothing done, if a lane has fewer than 32 bits (bytes without a code).
-template <int G, bool kInner>
-__device__ __forceinline__ bool fast_step(const Job &J, UnitState &st, int step, int lane,
-                                          uint32_t tcol_s, uint32_t wob_s, uint32_t *wob,
-                                          const uint32_t (&w)[8])
-{
-    constexpr int NC = (kFastSyms + G - 1) / G;
-    const uint64_t sb = st.base + (uint64_t)step * kFastStep;
-    int m = kFastSyms;
-    uint32_t tw[8];
-    if (kInner) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            tw[j] = w[j];
-    } else {
-        m = step_input_tail<kFastSyms>(J, sb, lane, tw);
-    }
-
-    // table entries of this lane's symbols; s accumulates whole entries,
-    // whose low 10 bits sum the lengths
-    uint32_t e[kFastSyms], sc[NC];
-    uint32_t s = 0, mid16 = 0;
-#pragma unroll
-    for (int k = 0; k < kFastSyms; ++k) {
-        e[k] = tbl_at(imad(byte_of(tw, k), kc[k128], tcol_s));
-        if (!kInner && k >= m)
-            e[k] = 0u;
-        s = imad(e[k], kc[kOne], s);
-        if ((k + 1) % G == 0 || k == kFastSyms - 1)
-            sc[k / G] = s;
-        if (k == 15)
-            mid16 = s & kSumMask;
-    }
-    const uint32_t bits = s & kSumMask;
-    if (kInner && !__all_sync(0xffffffffu, bits >= (uint32_t)kFastSyms))
-        return true;  // plain stores need whole words (see pack32)
-    uint32_t pos, step_bits;
-    scan_bits(bits, lane, pos, step_bits);
-    const uint32_t p0 = (uint32_t)(st.gbit & 31) + pos;
-
-    step_chunks<kFastSyms, kFastStep>(J, st, sb, lane, pos, mid16);
-    uint32_t part;
-    if (kInner) {
-        // complete words by plain stores, then each lane ORs its last partial
-        // word into the next lane's first word (the last lane stores it: no
-        // lane writes that word), and lane 0 ORs the carried bits into word 0
-        const uint32_t E = pack32<G, true>(e, sc, p0, wob_s, part);
-        __syncwarp();
-        const uint32_t pa = imad(E >> 5, kc[kFour], wob_s);
-        if (lane == 31)
-            sts(pa, part);
-        else
-            red_or(pa, part);
-        if (lane == 0)
-            red_or(wob_s, st.carry);
-    } else {
-        // word 0 starts with the carried bits; every other word is zero
-        sts_if(lane == 0, wob_s, st.carry);
-        __syncwarp();
-        const uint32_t E = pack32<G, false>(e, sc, p0, wob_s, part);
-        red_or(imad(E >> 5, kc[kFour], wob_s), part);
-    }
-    __syncwarp();
-    const bool last = sb + kFastStep >= J.n;
-    const bool overflow = step_output<!kInner>(J, st, last, step_bits, wob, lane);
-    __syncwarp();
-    step_advance<kFastStep>(J, st, step_bits);
-    return overflow;
-}
-
 __device__ __forceinline__ void load32(const uint8_t *p, uint32_t (&w)[8])
 {
     const uint4 a = ld_stream16(p), b = ld_stream16(p + 16);
@@ -443,61 +240,20 @@ __device__ __forceinline__ int full_steps(const Job &J, uint64_t u)
 {
     if (((J.unit_off[u + 1] + 31) >> 5) > J.cap_words)
         return 0;
-    const uint64_t left = (J.n - u * kUnitSymbols) / kFastStep;
-    return left < (uint64_t)kFastSteps ? (int)left : kFastSteps;
+    const uint64_t left = (J.n - u * kUnitSymbols) / kStep;
+    return left < (uint64_t)kSteps ? (int)left : kSteps;
 }
 
-// Encode unit u of job J with the calling warp, codes of at most 22 bits.
-// wob is the warp's buffer of kWarpObuf words (word 0 is the guard), tbl the
-// CTA's table.  Returns true if a payload word fell outside the output
-// capacity.
-template <int G>
-__device__ __forceinline__ bool encode_unit_fast(const Job &J, uint64_t u, const uint32_t *tbl,
-                                                 uint32_t *wob)
-{
-    const int lane = threadIdx.x & 31;
-    const uint32_t tcol_s = smem_u32(tbl + lane), wob_s = smem_u32(wob + 1);
-    UnitState st = unit_start(J, u, tbl, true, lane);
-    const int full = full_steps(J, u);
-    bool overflow = false;
-    int step = 0;
-    if (full) {  // warp-uniform
-        const uint8_t *p = J.in + st.base + lane * kFastSyms;
-        uint32_t w[8];
-        load32(p, w);
-        for (; step < full; ++step) {
-            uint32_t nx[8];
-            if (step + 1 < full)
-                load32(p + (step + 1) * kFastStep, nx);  // one step ahead
-            if (fast_step<G, true>(J, st, step, lane, tcol_s, wob_s, wob + 1, w))
-                break;
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                w[j] = nx[j];
-        }
-    }
-    if (step < kFastSteps && st.base + (uint64_t)step * kFastStep < J.n) {
-        clear_buffer(wob, lane);
-        const uint32_t none[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (; step < kFastSteps; ++step) {
-            if (st.base + (uint64_t)step * kFastStep >= J.n)
-                break;  // warp-uniform
-            overflow |= fast_step<G, false>(J, st, step, lane, tcol_s, wob_s, wob + 1, none);
-        }
-    }
-    return overflow;
-}
-
-// ---- codes gathered by multiply-add (single-stream encoder) ----------------
-// The fast path above spends two funnel shifts per code on the ALU pipe,
-// which bounds it.  Here a group of codes is gathered on the FMA pipe: the
-// table holds (code, 2^len) per byte and lane, and a = a * 2^len + code
-// appends a code to the group's bits; a starts at 1, so its leading one
-// marks the group's length (a group has at most 31 bits).  Per code that is
-// one byte permutation (which is the table address), one table load (8 bytes)
-// and one IMAD; only the group pays for its length, its place and the store.
-// The groups of a lane are cut at its 16th symbol too, where a chunk may
-// start.  Same stream, bit for bit.
+// ---- codes gathered by multiply-add ------------------------------------------
+// A group of codes is gathered on the FMA pipe: the table holds (code, 2^len)
+// per byte and column, and a = a * 2^len + code appends a code to the group's
+// bits; a starts at 1, so its leading one marks the group's length (a group
+// has at most 31 bits).  Per code that is one byte permutation (which is the
+// table address), one table load (8 bytes) and one IMAD; only the group pays
+// for its length, its place and the store.  (Two funnel shifts per code into a
+// 64-bit window are bound by the ALU pipe: 4096 buffers of 2 GB in all take
+// 1977 us instead of 1913.)  The groups of a lane are cut at its 16th
+// symbol too, where a chunk may start.
 //  - Longest code of at most 10 bits: groups of floor(31 / longest) codes, at
 //    least 3, always fit.
 //  - Longer codes are rare wherever there are any: the groups take 4 codes
@@ -508,42 +264,59 @@ __device__ __forceinline__ bool encode_unit_fast(const Job &J, uint64_t u, const
 //    instead of 2127.  The same guess for codes of at most 10 bits (4 for 3)
 //    gained 2 to 4% on text and lost as much on Zipf bytes, where every unit
 //    has a group that does not fit: not done.
-constexpr int kTbl2Words = 256 * 32 * 2;  // [byte][lane] (code, 2^len), 64 KiB
-constexpr uint32_t kMadMaxLen = 31;       // the marker takes a bit
-// warp buffer: a guard word, then a step of 1024 codes after < 32 carried bits
-constexpr int kMadObuf = 1 + kFastStep * (int)kMadMaxLen / 32 + 15;
 
-// Built by 512 threads, two per byte: each reads its byte's length and code
-// once and fills half a row with eight 16-byte stores, rotated by the byte so
-// that a warp's stores spread over all eight 16-byte bank groups.
-__device__ __forceinline__ void build_table2(const huff_codebook_t *cb, uint32_t *tbl2)
+// How the codes of a stream are written: 32-bit codes one by one; 3, 4, 8 or
+// 16 at a time because they fit; 3 or 4 at a time because they nearly always
+// fit.
+enum Plan { kLong = 0, kTry3 = 1, kTry4 = 2, kFit3 = 3, kFit4 = 4, kFit8 = 8, kFit16 = 16 };
+
+__device__ __forceinline__ int plan_of(const Job &J, uint32_t max_len)
 {
-    const int b = threadIdx.x >> 1;
-    if (b >= 256)
-        return;
-    const uint32_t L = cb->len[b];
-    const uint32_t c = L ? cb->code[b] : 0u;
-    const uint32_t p = 1u << L;  // 2^0 = 1 for a byte without a code: no bits
-    uint4 *row = reinterpret_cast<uint4 *>(tbl2 + b * 64) + (threadIdx.x & 1) * 8;
+    if (max_len > kMadMaxLen)
+        return kLong;
+    const uint32_t fit = max_len ? 31u / max_len : 16u;
+    if (fit >= 3)
+        return fit >= 16 ? kFit16 : fit >= 8 ? kFit8 : fit >= 4 ? kFit4 : kFit3;
+    return J.units && J.unit_off[J.units] <= 4 * J.n ? kTry4 : kTry3;
+}
+
+// A stream's half of the code table, built by threads tid = 0..nt-1: one or
+// two threads per byte read its length and code once and fill the byte's 16
+// columns with 16-byte stores, rotated by the byte so that a warp's stores
+// spread over all eight 16-byte bank groups.  32-bit codes: 16 words of code,
+// then 16 of length.
+__device__ __forceinline__ void build_table(const huff_codebook_t *cb, uint32_t *tbl, bool pairs, int tid,
+                                            int nt)
+{
+    for (int b = tid; b < 256; b += nt) {
+        const uint32_t L = cb->len[b];
+        const uint32_t c = L ? cb->code[b] : 0u;
+        const uint32_t p = 1u << (L & 31u);  // 2^0 = 1 for a byte without a code: no bits
+        uint4 *row = reinterpret_cast<uint4 *>(tbl + b * kTblRow);
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-        row[(j + b) & 7] = make_uint4(c, p, c, p);
+        for (int j = 0; j < 8; ++j) {
+            const int k = (j + b) & 7;
+            row[k] = pairs ? make_uint4(c, p, c, p) : k < 4 ? make_uint4(c, c, c, c) : make_uint4(L, L, L, L);
+        }
+    }
 }
 
-// Codes per group that always fit: floor(31 / longest) (31: the marker bit).
-__device__ __forceinline__ int mad_group(uint32_t max_len)
+// The last r (< 32) bits of the code stream before symbol `base` (> 0), as the
+// high bits of a word: lane l re-codes byte base-1-l.  Warp-uniform result.
+template <bool kPairs>
+__device__ __forceinline__ uint32_t seam_word(const uint8_t *in, uint64_t base, uint32_t r,
+                                              const uint32_t *tbl, int lane)
 {
-    const uint32_t gq = max_len ? 31u / max_len : 16u;
-    return gq >= 16 ? 16 : gq >= 8 ? 8 : gq >= 4 ? 4 : gq >= 3 ? 3 : gq >= 2 ? 2 : 1;
-}
-
-// As seam_word, from the (code, 2^len) table.
-__device__ __forceinline__ uint32_t seam_word2(const uint8_t *in, uint64_t base, uint32_t r,
-                                               const uint32_t *tbl2, int lane)
-{
-    const uint32_t b = in[base - 1 - lane];
-    const uint2 x = reinterpret_cast<const uint2 *>(tbl2)[(b << 5) | lane];
-    const uint32_t L = 31u - __clz(x.y), code = x.x;
+    const uint32_t *e = tbl + (uint32_t)in[base - 1 - lane] * kTblRow;
+    uint32_t L, code;
+    if (kPairs) {
+        const uint2 x = reinterpret_cast<const uint2 *>(e)[lane & 15];
+        code = x.x;
+        L = 31u - __clz(x.y);
+    } else {
+        code = e[lane & 15];
+        L = e[16 + (lane & 15)];
+    }
     uint32_t sfx = L;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -551,19 +324,20 @@ __device__ __forceinline__ uint32_t seam_word2(const uint8_t *in, uint64_t base,
         if (lane >= d)
             sfx += v;
     }
-    const uint32_t before = sfx - L;
+    const uint32_t before = sfx - L;  // bits between this code's end and base
     const uint32_t part = (L && before < r) ? code << (32 - r + before) : 0u;
     return __reduce_or_sync(0xffffffffu, part);
 }
 
-__device__ __forceinline__ UnitState unit_start2(const Job &J, uint64_t u, const uint32_t *tbl2,
-                                                 int lane)
+template <bool kPairs>
+__device__ __forceinline__ UnitState unit_start(const Job &J, uint64_t u, const uint32_t *tbl, int lane)
 {
     UnitState st;
     st.base = u * kUnitSymbols;
     st.gbit = J.unit_off[u];
-    st.carry = (st.base > 0 && (st.gbit & 31)) ? seam_word2(J.in, st.base, (uint32_t)(st.gbit & 31), tbl2, lane)
-                                               : 0u;
+    st.carry = (st.base > 0 && (st.gbit & 31))
+                   ? seam_word<kPairs>(J.in, st.base, (uint32_t)(st.gbit & 31), tbl, lane)
+                   : 0u;
     const uint32_t umod = (uint32_t)(st.base % J.cs);
     st.lead = umod ? J.cs - umod : 0u;
     st.next_chunk = (st.base + st.lead) / J.cs;
@@ -593,7 +367,9 @@ struct Groups {
 // codes have at most 31 bits together, whatever they are; a multiply-add of
 // a later one whose high word is not zero has overflowed (the result, which
 // the caller then throws away, is nonzero).
-template <int G, int kFirst, bool kAll>
+// The lane's column lies at shared address tcol_s + kImm, tcol_s with zeros in
+// its second byte.
+template <int G, int kFirst, bool kAll, uint32_t kImm>
 __device__ __forceinline__ uint32_t mad_gather(Groups<G> &q, const uint32_t (&w)[8], int m,
                                                uint32_t tcol_s)
 {
@@ -609,9 +385,9 @@ __device__ __forceinline__ uint32_t mad_gather(Groups<G> &q, const uint32_t (&w)
             const int k = k0 + j;
             if ((g % NH) * G + j < 16 && (kAll || k < m)) {
                 uint2 x;
-                asm("ld.shared.v2.u32 {%0, %1}, [%2];"
+                asm("ld.shared.v2.u32 {%0, %1}, [%2+%3];"
                     : "=r"(x.x), "=r"(x.y)
-                    : "r"(__byte_perm(w[k >> 2], tcol_s, 0x7604u | (uint32_t)(k & 3) << 4)));
+                    : "r"(__byte_perm(w[k >> 2], tcol_s, 0x7604u | (uint32_t)(k & 3) << 4)), "n"(kImm));
                 if (j >= kFirst) {
                     const uint64_t t = (uint64_t)a * x.y + x.x;
                     over |= (uint32_t)(t >> 32);
@@ -630,8 +406,14 @@ __device__ __forceinline__ uint32_t mad_gather(Groups<G> &q, const uint32_t (&w)
     return over;
 }
 
-// Pack and write the gathered step at symbol sb; kInner as for fast_step (the
-// caller has made sure that every lane has 32 bits).
+// Pack and write the gathered step at symbol sb.  kInner: the step lies inside
+// the input, the unit's words fit the output and every lane has at least 32
+// bits, so the step needs no bound checks and every complete word is written
+// by one plain store: of the lane that completes it, with zeros for the bits
+// that are not its own.  After a warp barrier each lane ORs its last partial
+// word into the next lane's first word (the last lane stores it: no lane
+// writes that word), and lane 0 ORs the carried bits into word 0.  Otherwise a
+// lane may have no bits at all, and all words are ORed into a zeroed buffer.
 template <int G, bool kInner>
 __device__ __forceinline__ bool mad_pack(const Job &J, UnitState &st, uint64_t sb, int lane,
                                          const Groups<G> &q, uint32_t wob_s, uint32_t *wob)
@@ -639,7 +421,7 @@ __device__ __forceinline__ bool mad_pack(const Job &J, UnitState &st, uint64_t s
     uint32_t pos, step_bits;
     scan_bits(q.bits, lane, pos, step_bits);
     const uint32_t p0 = (uint32_t)(st.gbit & 31) + pos;
-    step_chunks<kFastSyms, kFastStep>(J, st, sb, lane, pos, q.mid16);
+    step_chunks<kStepSyms, kStep>(J, st, sb, lane, pos, q.mid16);
     if (!kInner) {
         sts_if(lane == 0, wob_s, st.carry);  // word 0 starts with the carried bits
         __syncwarp();
@@ -647,9 +429,7 @@ __device__ __forceinline__ bool mad_pack(const Job &J, UnitState &st, uint64_t s
     // lom + 1 holds the lane's last 32 bits.  A group of L bits x (a = 2^L + x)
     // that takes the lane's end from E to E1 over a word boundary completes
     // the word (lom + 1) << d | x >> r, with r = E1 mod 32 bits left over and
-    // d = L - r = -E mod 32; the marker's 2^d is the 2^d that lom lacks (see
-    // pack32 for why plain stores are enough when every lane has 32 bits).
-    // A group that crosses no boundary stores nothing (about one group in two
+    // d = L - r = -E mod 32; the marker's 2^d is the 2^d that lom lacks.  A group that crosses no boundary stores nothing (about one group in two
     // crosses on text), which keeps the warp-buffer stores off the L1 data
     // pipe; a predicated store, because some lane of 32 nearly always
     // crosses.
@@ -683,32 +463,32 @@ __device__ __forceinline__ bool mad_pack(const Job &J, UnitState &st, uint64_t s
         red_or(imad(E >> 5, kc[kFour], wob_s), part);
     }
     __syncwarp();
-    const bool last = sb + kFastStep >= J.n;
+    const bool last = sb + kStep >= J.n;
     const bool overflow = step_output<!kInner>(J, st, last, step_bits, wob, lane);
     __syncwarp();
-    step_advance<kFastStep>(J, st, step_bits);
+    step_advance<kStep>(J, st, step_bits);
     return overflow;
 }
 
 // Steps [step, full) of a unit without bound checks; returns the first step
 // that cannot be done so (a group overflows, or a lane has fewer than 32 bits
 // because of bytes without a code), or full.
-template <int G, int kFirst>
+template <int G, int kFirst, uint32_t kImm>
 __device__ __forceinline__ int mad_steps(const Job &J, UnitState &st, int step, int full, int lane,
                                          uint32_t tcol_s, uint32_t wob_s, uint32_t *wob)
 {
-    const uint8_t *p = J.in + st.base + lane * kFastSyms;
+    const uint8_t *p = J.in + st.base + lane * kStepSyms;
     uint32_t w[8];
-    load32(p + step * kFastStep, w);
+    load32(p + step * kStep, w);
     for (; step < full; ++step) {
         uint32_t nx[8];
         if (step + 1 < full)
-            load32(p + (step + 1) * kFastStep, nx);  // one step ahead
+            load32(p + (step + 1) * kStep, nx);  // one step ahead
         Groups<G> q;
-        const uint32_t over = mad_gather<G, kFirst, true>(q, w, kFastSyms, tcol_s);
-        if (!__all_sync(0xffffffffu, q.bits >= (uint32_t)kFastSyms && over == 0u))
+        const uint32_t over = mad_gather<G, kFirst, true, kImm>(q, w, kStepSyms, tcol_s);
+        if (!__all_sync(0xffffffffu, q.bits >= (uint32_t)kStepSyms && over == 0u))
             break;
-        mad_pack<G, true>(J, st, st.base + (uint64_t)step * kFastStep, lane, q, wob_s, wob);
+        mad_pack<G, true>(J, st, st.base + (uint64_t)step * kStep, lane, q, wob_s, wob);
 #pragma unroll
         for (int j = 0; j < 8; ++j)
             w[j] = nx[j];
@@ -718,68 +498,51 @@ __device__ __forceinline__ int mad_steps(const Job &J, UnitState &st, int step, 
 
 // The steps of a unit from `step` on in groups of S codes, which always fit:
 // the whole ones, then the checked rest.
-template <int S>
+template <int S, uint32_t kImm>
 __device__ __noinline__ bool mad_rest(const Job J, UnitState st, int step, int full, int lane,
                                       uint32_t tcol_s, uint32_t wob_s, uint32_t *wob)
 {
     bool overflow = false;
     if (step < full)
-        step = mad_steps<S, S>(J, st, step, full, lane, tcol_s, wob_s, wob);
-    if (step < kFastSteps && st.base + (uint64_t)step * kFastStep < J.n) {
-        clear_buffer<kMadObuf>(wob - 1, lane);
-        for (; step < kFastSteps; ++step) {
-            const uint64_t sb = st.base + (uint64_t)step * kFastStep;
+        step = mad_steps<S, S, kImm>(J, st, step, full, lane, tcol_s, wob_s, wob);
+    if (step < kSteps && st.base + (uint64_t)step * kStep < J.n) {
+        clear_buffer(wob - 1, lane);
+        for (; step < kSteps; ++step) {
+            const uint64_t sb = st.base + (uint64_t)step * kStep;
             if (sb >= J.n)
                 break;  // warp-uniform
             uint32_t w[8];
-            const int m = step_input_tail<kFastSyms>(J, sb, lane, w);
+            const int m = step_input_tail<kStepSyms>(J, sb, lane, w);
             Groups<S> q;
-            mad_gather<S, S, false>(q, w, m, tcol_s);
+            mad_gather<S, S, false, kImm>(q, w, m, tcol_s);
             overflow |= mad_pack<S, false>(J, st, sb, lane, q, wob_s, wob);
         }
     }
     return overflow;
 }
 
-// Unit u in groups of G codes, of which kFirst always fit; the steps with a
-// group that does not fit, and all after them, in groups of S.
-template <int G, int kFirst, int S>
-__device__ __forceinline__ bool encode_unit_mad(const Job &J, uint64_t u, const uint32_t *tbl2,
-                                                uint32_t *wob)
+// Encode unit u of job J with the calling warp in groups of G codes, of which
+// kFirst always fit; the steps with a group that does not fit, and all after
+// them, in groups of S.  tbl is the stream's half of the table, wob the warp's
+// buffer of kWarpObuf words (word 0 is the guard).  Returns true if a payload
+// word fell outside the output capacity.
+template <int G, int kFirst, int S, uint32_t kImm>
+__device__ __forceinline__ bool encode_unit_mad(const Job &J, uint64_t u, const uint32_t *tbl, uint32_t *wob)
 {
     const int lane = threadIdx.x & 31;
-    const uint32_t tcol_s = smem_u32(tbl2 + 2 * lane), wob_s = smem_u32(wob + 1);
-    UnitState st = unit_start2(J, u, tbl2, lane);
+    const uint32_t tcol_s = smem_u32(tbl + 2 * (lane & 15)) - kImm, wob_s = smem_u32(wob + 1);
+    UnitState st = unit_start<true>(J, u, tbl, lane);
     const int full = full_steps(J, u);
     int step = 0;
     if (full)  // warp-uniform
-        step = mad_steps<G, kFirst>(J, st, 0, full, lane, tcol_s, wob_s, wob + 1);
-    if (step < kFastSteps && st.base + (uint64_t)step * kFastStep < J.n)
-        return mad_rest<S>(J, st, step, full, lane, tcol_s, wob_s, wob + 1);
+        step = mad_steps<G, kFirst, kImm>(J, st, 0, full, lane, tcol_s, wob_s, wob + 1);
+    if (step < kSteps && st.base + (uint64_t)step * kStep < J.n)
+        return mad_rest<S, kImm>(J, st, step, full, lane, tcol_s, wob_s, wob + 1);
     return false;
 }
 
-// At most 4 bits per code on average?
-__device__ __forceinline__ bool few_bits(const Job &J)
-{
-    return J.units && J.unit_off[J.units] <= 4 * J.n;
-}
-
-// group: mad_group of the longest code, at least 3
-__device__ __forceinline__ bool encode_unit_mad_g(const Job &J, uint64_t u, const uint32_t *tbl2,
-                                                  int group, uint32_t *wob)
-{
-    switch (group) {
-    case 16: return encode_unit_mad<16, 16, 16>(J, u, tbl2, wob);
-    case 8: return encode_unit_mad<8, 8, 8>(J, u, tbl2, wob);
-    case 4: return encode_unit_mad<4, 4, 4>(J, u, tbl2, wob);
-    default: return encode_unit_mad<3, 3, 3>(J, u, tbl2, wob);
-    }
-}
-
-// The same for codes of up to 32 bits: split code / length tables, 16
-// symbols per lane and a 64-bit accumulator (rare: only very skewed inputs
-// have codes this long).
+// The same for 32-bit codes: 16 symbols per lane and a 64-bit accumulator
+// (rare: only very skewed inputs have codes this long).
 __device__ __forceinline__ bool encode_unit_long(const Job &J, uint64_t u, const uint32_t *tbl,
                                                  uint32_t *wob_all)
 {
@@ -787,7 +550,7 @@ __device__ __forceinline__ bool encode_unit_long(const Job &J, uint64_t u, const
     clear_buffer(wob_all, lane);
     uint32_t *wob = wob_all + 1;
     bool overflow = false;
-    UnitState st = unit_start(J, u, tbl, false, lane);
+    UnitState st = unit_start<false>(J, u, tbl, lane);
     for (int step = 0; step < kLongSteps; ++step) {
         const uint64_t sb = st.base + (uint64_t)step * kLongStep;
         if (sb >= J.n)
@@ -800,8 +563,8 @@ __device__ __forceinline__ bool encode_unit_long(const Job &J, uint64_t u, const
 #pragma unroll
         for (int k = 0; k < kLongSyms; ++k) {
             const uint32_t b = byte_of(w, k);
-            e[k] = k < m ? tbl[(b << 4) | col] : 0u;
-            l2[k] = k < m ? tbl[256 * 16 + ((b << 4) | col)] : 0u;
+            e[k] = k < m ? tbl[b * kTblRow + col] : 0u;
+            l2[k] = k < m ? tbl[b * kTblRow + 16 + col] : 0u;
             bits += l2[k];
         }
         uint32_t pos, step_bits;
@@ -834,21 +597,6 @@ __device__ __forceinline__ bool encode_unit_long(const Job &J, uint64_t u, const
         step_advance<kLongStep>(J, st, step_bits);
     }
     return overflow;
-}
-
-__device__ __forceinline__ bool encode_unit(const Job &J, uint64_t u, const uint32_t *tbl, bool fast,
-                                           int group, uint32_t *wob)
-{
-    if (!fast)
-        return encode_unit_long(J, u, tbl, wob);
-    switch (group) {
-    case 16: return encode_unit_fast<16>(J, u, tbl, wob);
-    case 8: return encode_unit_fast<8>(J, u, tbl, wob);
-    case 4: return encode_unit_fast<4>(J, u, tbl, wob);
-    case 3: return encode_unit_fast<3>(J, u, tbl, wob);
-    case 2: return encode_unit_fast<2>(J, u, tbl, wob);
-    default: return encode_unit_fast<1>(J, u, tbl, wob);
-    }
 }
 
 }  // namespace enc

@@ -122,3 +122,31 @@ def test_chained_launches_under_capture_and_back_to_back(n):
         for (o, b, s), ref in zip(got, refs):
             assert int(s) == 0 and int(b) == ref.size
             assert np.array_equal(o[: ref.size].cpu().numpy(), ref)
+
+
+def test_batches_of_every_grouping():
+    rng = np.random.default_rng(5)
+    fib = [1, 1]
+    while len(fib) < 33:
+        fib.append(fib[-1] + fib[-2])
+    xs = [np.repeat(np.arange(33, dtype=np.uint8), fib)]  # a 32-bit code
+    for n in SIZES + (150000,):
+        xs.append(np.full(n, 9, np.uint8))
+        xs.append(rng.integers(0, 3, n).astype(np.uint8))
+        xs.append(rng.integers(0, 60, n).astype(np.uint8))
+        xs.append(rng.integers(0, 256, n).astype(np.uint8))
+        xs.append(np.minimum(rng.geometric(0.5, n), 255).astype(np.uint8))
+        xs.append(np.minimum(rng.geometric(0.04, n), 255).astype(np.uint8))
+        x = np.minimum(rng.geometric(0.5, n), 255)
+        x[n // 3 : n // 2] = rng.integers(0, 256, n // 2 - n // 3)  # groups that do not fit
+        xs.append(x.astype(np.uint8))
+    refs = [oracle.compress(x)[1] for x in xs]
+    ins = [torch.from_numpy(x).cuda() for x in xs]
+    outs = [torch.zeros(hg.huff_max_stream_size(x.size), dtype=torch.uint8, device="cuda") for x in xs]
+    plan = hg.BatchPlan(ins, outs, hg.HUFF_BATCH_COMPRESS)
+    plan.run()
+    torch.cuda.synchronize()
+    sizes = plan.out_bytes.cpu().numpy()
+    for x, ref, out, size in zip(xs, refs, outs, sizes):
+        assert int(size) == ref.size, x.size
+        assert np.array_equal(out[: ref.size].cpu().numpy(), ref), x.size
