@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kBatchBlock, 2) k_batch_compress(BatchArgs a)
             o0 = o1;
             if (gn + G < total_units)
                 o1 = a.unit_owner[gn + G];
-            hst::count_unit(unit_ptr(co), co.z, 0, cur, col0 + set * (256 * 32 * 4));
+            hst::count_unit(unit_ptr(co), co.z, 0, cur, col0 + set * (256 * 32 * 4), 1u);
             __syncthreads();
             const uint32_t s = hst::fold_bin(cnt + set * (256 * 32), tid);
             a.unit_hist[g * 256 + tid] = (uint16_t)(s - (set ? prev1 : prev0));

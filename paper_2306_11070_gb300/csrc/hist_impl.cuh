@@ -13,25 +13,26 @@ constexpr int kVecPerThread = kUnitSymbols / 16 / kThreads;  // 4
 
 // One count: a shared-memory reduction at the 32-bit shared address of
 // (byte, lane); byte * 128 is the row offset of the [byte][lane] layout.
-__device__ __forceinline__ void count_at(uint32_t col, uint32_t byte)
+// `one` is 1 or, where a column holds two counts, 1 << 16 for the upper one.
+__device__ __forceinline__ void count_at(uint32_t col, uint32_t byte, uint32_t one)
 {
-    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(col + (byte << 7)) : "memory");
+    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(col + (byte << 7)), "r"(one) : "memory");
 }
 
-__device__ __forceinline__ void count_word(uint32_t col, uint32_t w)
+__device__ __forceinline__ void count_word(uint32_t col, uint32_t w, uint32_t one)
 {
-    count_at(col, __byte_perm(w, 0u, 0x4440u));
-    count_at(col, __byte_perm(w, 0u, 0x4441u));
-    count_at(col, __byte_perm(w, 0u, 0x4442u));
-    count_at(col, __byte_perm(w, 0u, 0x4443u));
+    count_at(col, __byte_perm(w, 0u, 0x4440u), one);
+    count_at(col, __byte_perm(w, 0u, 0x4441u), one);
+    count_at(col, __byte_perm(w, 0u, 0x4442u), one);
+    count_at(col, __byte_perm(w, 0u, 0x4443u), one);
 }
 
-__device__ __forceinline__ void count16(uint32_t col, uint4 v)
+__device__ __forceinline__ void count16(uint32_t col, uint4 v, uint32_t one)
 {
-    count_word(col, v.x);
-    count_word(col, v.y);
-    count_word(col, v.z);
-    count_word(col, v.w);
+    count_word(col, v.x, one);
+    count_word(col, v.y, one);
+    count_word(col, v.z, one);
+    count_word(col, v.w, one);
 }
 
 // Sum of bin `tid` over its 32 columns, in eight 16-byte loads.  The
@@ -66,7 +67,7 @@ __device__ __forceinline__ void load_unit(const uint8_t *in, uint64_t n, uint64_
 // Count the loaded pieces of unit u (and, for the last unit, the < 16-byte
 // tail) into the lane's column.
 __device__ __forceinline__ void count_unit(const uint8_t *in, uint64_t n, uint64_t u,
-                                           const uint4 (&a)[kVecPerThread], uint32_t col)
+                                           const uint4 (&a)[kVecPerThread], uint32_t col, uint32_t one)
 {
     const uint64_t units = (n + kUnitSymbols - 1) / kUnitSymbols;
     const uint64_t nvec = n >> 4;
@@ -74,10 +75,10 @@ __device__ __forceinline__ void count_unit(const uint8_t *in, uint64_t n, uint64
     for (int j = 0; j < kVecPerThread; ++j) {
         const uint64_t q = u * (kUnitSymbols / 16) + j * kThreads + threadIdx.x;
         if (q < nvec)
-            count16(col, a[j]);
+            count16(col, a[j], one);
     }
     if (u == units - 1 && threadIdx.x < (n & 15u))
-        count_at(col, in[(nvec << 4) + threadIdx.x]);
+        count_at(col, in[(nvec << 4) + threadIdx.x], one);
 }
 
 }  // namespace hst

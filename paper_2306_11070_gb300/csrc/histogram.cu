@@ -12,8 +12,13 @@
 // Optionally the kernel also writes every unit's own histogram (u16[256],
 // 512 bytes per 16 KiB): the encoder turns these into the bit offset of each
 // unit with a dot product against the code lengths, so it never has to wait
-// on another CTA.  A unit's counts are the difference of two folds of the
-// running columns, so the columns are never cleared.
+// on another CTA.  The shared-memory pipe bounds it (86% busy): 512 wavefronts
+// count a unit, 256 fold its columns.  So two units share a fold: the first
+// counts in the low, the second in the high half of the columns.  Folds are sums
+// modulo 2^32 of columns that are never cleared, and their difference is the
+// first unit's count plus 2^16 times the second's, both at most 16384.
+// A compress call
+// of 1 GiB takes 773 us instead of 786.
 #include "hist_impl.cuh"
 
 namespace huff {
@@ -45,31 +50,44 @@ __global__ void __launch_bounds__(kHistBlock)
         cnt[i] = 0;
     const uint32_t col = smem_u32(cnt) + 4u * lane;  // this lane's column
     const uint64_t units = (n + kUnitSymbols - 1) / kUnitSymbols;
-    uint32_t prev = 0;  // fold of this thread's bin at the previous unit end
+    uint32_t prev = 0, total = 0;  // this thread's bin: last fold, count so far
+    const uint32_t one2 = unit_hist ? 1u << 16 : 1u;
     uint4 a[kVecPerThread];
+    const uint64_t G = gridDim.x;
     uint64_t u = blockIdx.x;
     load_unit(in, n, u, a);
     __syncthreads();
-    for (; u < units; u += gridDim.x) {
+    for (; u < units; u += 2 * G) {
         uint4 cur[kVecPerThread];
 #pragma unroll
         for (int j = 0; j < kVecPerThread; ++j)
             cur[j] = a[j];
-        load_unit(in, n, u + gridDim.x, a);  // in flight while this unit is counted
-        count_unit(in, n, u, cur, col);
+        load_unit(in, n, u + G, a);  // in flight while this unit is counted
+        count_unit(in, n, u, cur, col, 1u);
+        if (u + G < units) {
+#pragma unroll
+            for (int j = 0; j < kVecPerThread; ++j)
+                cur[j] = a[j];
+            load_unit(in, n, u + 2 * G, a);
+            count_unit(in, n, u + G, cur, col, one2);
+        }
         if (unit_hist) {
-            __syncthreads();  // all counts of unit u are in
-            const uint32_t s = fold_bin(cnt, tid);
-            unit_hist[u * 256 + tid] = (uint16_t)(s - prev);
+            __syncthreads();  // all counts of both units are in
+            const uint32_t s = fold_bin(cnt, tid), d = s - prev;
             prev = s;
+            unit_hist[u * 256 + tid] = (uint16_t)d;
+            if (u + G < units)
+                unit_hist[(u + G) * 256 + tid] = (uint16_t)(d >> 16);
+            total += (d & 0xffffu) + (d >> 16);
             __syncthreads();  // folds read before the next unit's counts
         }
     }
     __syncthreads();
-    const uint32_t s = fold_bin(cnt, tid);
+    if (!unit_hist)
+        total = fold_bin(cnt, tid);
     chain_wait();  // the totals are cleared
-    if (s)
-        atomicAdd(hist + tid, (unsigned long long)s);
+    if (total)
+        atomicAdd(hist + tid, (unsigned long long)total);
 }
 
 }  // namespace

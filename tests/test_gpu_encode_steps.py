@@ -150,3 +150,22 @@ def test_batches_of_every_grouping():
     for x, ref, out, size in zip(xs, refs, outs, sizes):
         assert int(size) == ref.size, x.size
         assert np.array_equal(out[: ref.size].cpu().numpy(), ref), x.size
+
+
+@pytest.mark.parametrize("units", [1, 2, 3, 607, 608, 609, 1216, 1217, 1825])
+def test_unit_histograms_counted_in_pairs(units):
+    rng = np.random.default_rng(units)
+    for n in (units * 16384 - 16383, units * 16384):
+        x = rng.integers(0, 256, n, dtype=np.uint8)
+        x[: 2 * 16384] = 255  # 16384 of one byte in both of a pair
+        d = torch.from_numpy(x).cuda()
+        hist = torch.zeros(256, dtype=torch.int64, device="cuda")
+        uh = torch.zeros(hg.huff_unit_hist_size(n), dtype=torch.uint8, device="cuda")
+        hg.huff_histogram_units(d, hist, uh)
+        got = uh.cpu().numpy().view("<u2").reshape(units, 256)
+        pad = np.zeros(units * 16384, np.int64)
+        pad[:n] = x.astype(np.int64) + 1
+        at = np.arange(units * 16384) // 16384 * 257 + pad
+        ref = np.bincount(at, minlength=units * 257).reshape(units, 257)[:, 1:]
+        assert np.array_equal(got, ref)
+        assert np.array_equal(hist.cpu().numpy(), ref.sum(0))
