@@ -86,16 +86,23 @@ __device__ __forceinline__ void block_span(uint32_t i, uint32_t block, uint32_t 
 struct FirstKey {
     uint32_t q, sigma;
     uint32_t bits;      // of the digits' number
+    bool by_block;      // the blocks are sorted each by itself
+    uint64_t top;       // sigma^(q - 1), the first digit's weight
     uint8_t code[256];  // a byte value's digit
 };
 constexpr uint32_t kInitTile = 2048;
 constexpr uint32_t kMaxFirst = 16;  // most bytes in a first key
 
-// round 0 keys: (block id, the digits of the rotation's first q bytes)
+// Round 0 keys: (block id, the digits of the rotation's first q bytes).  A
+// thread makes the keys of eight consecutive rotations, each from the one
+// before (less its first digit, and one more), and the keys leave through
+// shared memory in order: 64 MiB of text take 204 us, digit by digit 421.
+// The rotations' indices need no array: the first radix pass makes them.
 __global__ void __launch_bounds__(kEw) k_bwt_init(const uint8_t *x, uint32_t n, uint32_t block,
-                                                  const __grid_constant__ FirstKey f, uint64_t *key,
-                                                  uint32_t *val)
+                                                  const __grid_constant__ FirstKey f, uint64_t *key)
 {
+    constexpr uint32_t kPer = kInitTile / kEw;  // 8
+    __shared__ uint64_t out[kInitTile + kInitTile / kPer];  // a gap per thread: no bank conflicts
     __shared__ uint8_t code[256], tile[kInitTile + kMaxFirst];
     static_assert(kEw == 256, "a thread per byte value");
     code[threadIdx.x] = f.code[threadIdx.x];
@@ -104,21 +111,37 @@ __global__ void __launch_bounds__(kEw) k_bwt_init(const uint8_t *x, uint32_t n, 
         for (uint32_t j = threadIdx.x; j < kInitTile + kMaxFirst; j += kEw)
             tile[j] = t0 + j < n ? code[x[t0 + j]] : 0;
         __syncthreads();
-        for (uint32_t j = threadIdx.x; j < kInitTile && t0 + j < n; j += kEw) {
-            const uint32_t i = (uint32_t)t0 + j;
+        const uint32_t j0 = threadIdx.x * kPer;
+        uint64_t *const o = out + threadIdx.x * (kPer + 1);
+        if (t0 + j0 < n) {
+            const uint32_t i0 = (uint32_t)t0 + j0;
             uint32_t s, m;
-            block_span(i, block, n, s, m);
-            uint64_t k = 0;
-            if (i - s + f.q <= m) {
+            block_span(i0, block, n, s, m);
+            if ((uint64_t)(i0 - s) + kPer + f.q <= m) {
+                const uint64_t id = f.bits < 64 ? (uint64_t)(i0 / block) << f.bits : 0;
+                uint64_t k = 0;
                 for (uint32_t t = 0; t < f.q; ++t)
-                    k = k * f.sigma + tile[j + t];
-            } else {  // the rotation goes on at the block's start
-                for (uint32_t t = 0; t < f.q; ++t)
-                    k = k * f.sigma + code[x[s + (uint32_t)(((uint64_t)(i - s) + t) % m)]];
+                    k = k * f.sigma + tile[j0 + t];
+                o[0] = id | k;
+#pragma unroll
+                for (uint32_t j = 1; j < kPer; ++j) {
+                    k = (k - tile[j0 + j - 1] * f.top) * f.sigma + tile[j0 + j + f.q - 1];
+                    o[j] = id | k;
+                }
+            } else {  // a rotation goes on at its block's start, or blocks end here
+                for (uint32_t j = 0; j < kPer && t0 + j0 + j < n; ++j) {
+                    const uint32_t i = i0 + j;
+                    block_span(i, block, n, s, m);
+                    uint64_t k = 0;
+                    for (uint32_t t = 0; t < f.q; ++t)
+                        k = k * f.sigma + code[x[s + (uint32_t)(((uint64_t)(i - s) + t) % m)]];
+                    o[j] = f.bits < 64 ? ((uint64_t)(i / block) << f.bits) | k : k;
+                }
             }
-            key[i] = f.bits < 64 ? ((uint64_t)(i / block) << f.bits) | k : k;
-            val[i] = i;
         }
+        __syncthreads();
+        for (uint32_t j = threadIdx.x; j < kInitTile && t0 + j < n; j += kEw)
+            key[t0 + j] = out[j + j / kPer];
     }
 }
 
@@ -747,7 +770,8 @@ cudaError_t refine(FwdWs &w, const uint64_t *ks, const uint32_t *vs, uint32_t co
 // bytes close to random differ after 1.5 log2 m.  Forward transform of 64 MiB
 // in 1 MiB blocks against keys of four bytes always (and a radix pass that
 // ranked with match.any): text 13.1 -> 8.2 ms, Zipf bytes 8.8 -> 7.0, uniform
-// bytes 7.0 -> 4.9, the bitstream stand-in 47.3 -> 45.5.
+// bytes 7.0 -> 4.9, the bitstream stand-in 47.3 -> 45.5; with blocks sorted each
+// by itself and rolling keys 7.6, 6.3, 4.4 and 46.
 FirstKey first_key(const unsigned long long *hist, uint64_t n, uint64_t blocks, uint64_t m)
 {
     FirstKey f;
@@ -763,6 +787,12 @@ FirstKey first_key(const unsigned long long *hist, uint64_t n, uint64_t blocks, 
     }
     if (f.sigma < 2)
         f.sigma = 2;
+    // The block id need not be sorted by where the passes can take each block by
+    // itself: blocks that fill their tiles, so that a pass costs no more (64 MiB
+    // of text in 1 MiB blocks: 7 passes instead of 8, each 0.55 ms).  The pass
+    // counters then lie in the ranks, which the first refinement writes.
+    const uint64_t per = div_up(m, kRadixTile), tiles = blocks * per;
+    const bool can = blocks > 1 && per * kRadixTile <= m + m / 8 && radix_tiles_bytes(tiles) <= 4 * n;
     const uint32_t room = 64 - bit_width(blocks - 1);
     const double want = (entropy > 7.5 ? 1.5 : 2.4) * bit_width(m - 1);
     f.q = f.bits = 0;
@@ -773,12 +803,16 @@ FirstKey first_key(const unsigned long long *hist, uint64_t n, uint64_t blocks, 
         const uint32_t bits = bit_width(v - 1);
         if (bits > room)
             break;
-        const uint32_t used = 64 - room;
+        const uint32_t used = can ? 0 : 64 - room;
         if (f.q >= 4 && f.q * entropy >= want && (bits + used + 7) / 8 > (f.bits + used + 7) / 8)
             break;  // enough, and one more byte would take another pass
         ++f.q;
         f.bits = bits;
     }
+    f.top = 1;
+    for (uint32_t t = 1; t < f.q; ++t)
+        f.top *= f.sigma;
+    f.by_block = can && (f.bits + 7) / 8 < (f.bits + (64 - room) + 7) / 8;
     return f;
 }
 
@@ -1376,11 +1410,13 @@ huff_status_t huff_bwt_forward(const uint8_t *d_in, uint64_t n, uint32_t block, 
         cudaStreamSynchronize(s) != cudaSuccess)
         return HUFF_ERR_CUDA;
     const FirstKey f = first_key(h_hist, n, blocks, mmax);
-    k_bwt_init<<<ew_grid((n + 7) / 8), kEw, 0, s>>>(d_in, N, block, f, w.k0, w.v0);
-    uint64_t *ks;
-    uint32_t *vs;
-    if (sort_keys(w, N, f.bits + bit_width(blocks - 1), s, ks, vs) != cudaSuccess)
+    k_bwt_init<<<ew_grid((n + 7) / 8), kEw, 0, s>>>(d_in, N, block, f, w.k0);
+    bool flip = false;
+    if (radix_sort_bits(w.k0, w.v0, w.k1, w.v1, N, 0, f.by_block ? f.bits : f.bits + bit_width(blocks - 1),
+                        f.by_block ? w.rk : w.radix, s, flip, f.by_block ? block : 0, true) != cudaSuccess)
         return HUFF_ERR_CUDA;
+    uint64_t *ks = flip ? w.k1 : w.k0;
+    uint32_t *vs = flip ? w.v1 : w.v0;
     uint32_t n_act = 0, groups = 0;
     if (refine(w, ks, vs, N, 64, s, n_act, groups) != cudaSuccess)
         return HUFF_ERR_CUDA;

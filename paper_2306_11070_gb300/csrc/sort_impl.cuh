@@ -173,21 +173,40 @@ __device__ __forceinline__ uint32_t same_digit(uint32_t d, bool ok)
     return mask;
 }
 
-__global__ void __launch_bounds__(kRadixThreads) k_radix_count(const uint64_t *keys, uint32_t count,
-                                                               uint32_t shift, uint32_t *hist,
-                                                               uint32_t tiles)
+// The elements of a sort: all of them, or blocks of `block` elements that are
+// sorted each by itself, with `per` tiles (the last one ragged) to a block.
+// Digit d of tile t of block b is counted at [(b * 256 + d) * per + t]: the
+// exclusive sum of these counts is its first place in the output.
+struct RadixSpan {
+    uint32_t count, block, per;
+    // this CTA's tile: its elements [lo, hi), and its first counter
+    __device__ __forceinline__ void tile(uint64_t &lo, uint64_t &hi, uint64_t &first) const
+    {
+        const uint32_t b = blockIdx.x / per, t = blockIdx.x - b * per;
+        const uint64_t s = (uint64_t)b * block, end = s + block < count ? s + block : count;
+        lo = s + (uint64_t)t * kRadixTile;
+        hi = lo + kRadixTile < end ? lo + kRadixTile : end;
+        if (hi < lo)
+            hi = lo;
+        first = (uint64_t)b * 256 * per + t;
+    }
+};
+
+__global__ void __launch_bounds__(kRadixThreads) k_radix_count(const uint64_t *keys, RadixSpan sp,
+                                                               uint32_t shift, uint32_t *hist)
 {
     __shared__ uint32_t c[256];
     if (threadIdx.x < 256)
         c[threadIdx.x] = 0;
     __syncthreads();
-    const uint64_t base = (uint64_t)blockIdx.x * kRadixTile;
+    uint64_t base, end, first;
+    sp.tile(base, end, first);
     const int lane = threadIdx.x & 31;
     uint32_t dig[kRadixItems];
 #pragma unroll
     for (int j = 0; j < kRadixItems; ++j) {  // every load in flight before the first use
         const uint64_t e = base + (uint64_t)j * kRadixThreads + threadIdx.x;
-        dig[j] = e < count ? (uint32_t)(keys[e] >> shift) & 255u : 256u;
+        dig[j] = e < end ? (uint32_t)(keys[e] >> shift) & 255u : 256u;
     }
 #pragma unroll
     for (int j = 0; j < kRadixItems; ++j) {
@@ -203,7 +222,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_count(const uint64_t *k
     }
     __syncthreads();
     if (threadIdx.x < 256)
-        hist[(uint64_t)threadIdx.x * tiles + blockIdx.x] = c[threadIdx.x];
+        hist[first + (uint64_t)threadIdx.x * sp.per] = c[threadIdx.x];
 }
 
 // shared memory of the scatter: the tile in sorted order, the digits' counts
@@ -217,23 +236,25 @@ struct RadixShared {
 };
 
 __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
-    const uint64_t *kin, const uint32_t *vin, uint64_t *kout, uint32_t *vout, uint32_t count,
-    uint32_t shift, const uint32_t *offs, uint32_t tiles)
+    const uint64_t *kin, const uint32_t *vin, uint64_t *kout, uint32_t *vout, RadixSpan sp,
+    uint32_t shift, const uint32_t *offs)
 {
     extern __shared__ __align__(16) unsigned char radix_sm[];
     RadixShared &sh = *reinterpret_cast<RadixShared *>(radix_sm);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     // warp w owns the tile's elements [w * 256, (w + 1) * 256), taken 32 at
     // a time in order, so ranks follow element order
-    const uint64_t base = (uint64_t)blockIdx.x * kRadixTile + (uint64_t)w * (kRadixItems * 32);
+    uint64_t tb, end, first;
+    sp.tile(tb, end, first);
+    const uint64_t base = tb + (uint64_t)w * (kRadixItems * 32);
     uint64_t key[kRadixItems];
     uint32_t val[kRadixItems], rank[kRadixItems];
 #pragma unroll
     for (int j = 0; j < kRadixItems; ++j) {  // every load in flight before the first use
         const uint64_t e = base + (uint64_t)j * 32 + lane;
-        const bool ok = e < count;
+        const bool ok = e < end;
         key[j] = ok ? kin[e] : 0ull;
-        val[j] = ok ? vin[e] : 0u;
+        val[j] = !ok ? 0u : vin ? vin[e] : (uint32_t)e;
     }
     uint32_t *const cnt = sh.cnt[w];
 #pragma unroll
@@ -242,7 +263,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
     __syncwarp();
 #pragma unroll
     for (int j = 0; j < kRadixItems; ++j) {
-        const bool ok = base + (uint64_t)j * 32 + lane < count;
+        const bool ok = base + (uint64_t)j * 32 + lane < end;
         const uint32_t d = (uint32_t)(key[j] >> shift) & 255u;
         const uint32_t mask = same_digit(d, ok);
         rank[j] = ok ? cnt[d] + __popc(mask & lanemask_lt()) : 0u;
@@ -271,7 +292,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
         }
         if (lane == 31)
             sh.ws[w] = x;
-        sh.gbase[tid] = offs[(uint64_t)tid * tiles + blockIdx.x];
+        sh.gbase[tid] = offs[first + (uint64_t)tid * sp.per];
     }
     __syncthreads();
     if (tid < 256) {
@@ -283,7 +304,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < kRadixItems; ++j) {
-        if (base + (uint64_t)j * 32 + lane < count) {
+        if (base + (uint64_t)j * 32 + lane < end) {
             const uint32_t d = (uint32_t)(key[j] >> shift) & 255u;
             const uint32_t q = sh.dstart[d] + cnt[d] + rank[j];
             sh.key[q] = key[j];
@@ -291,8 +312,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
         }
     }
     __syncthreads();
-    const uint64_t tb = (uint64_t)blockIdx.x * kRadixTile;
-    const uint32_t n_here = (uint32_t)(count - tb < kRadixTile ? count - tb : kRadixTile);
+    const uint32_t n_here = (uint32_t)(end - tb);
 #pragma unroll 4
     for (uint32_t q = tid; q < n_here; q += kRadixThreads) {
         const uint64_t k = sh.key[q];
@@ -303,31 +323,37 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
     }
 }
 
-// scratch of one radix pass: the digit counts (scanned in place) and the
-// scan's tile sums
-inline uint64_t radix_scratch_bytes(uint64_t count)
+// scratch of one radix pass over so many tiles: the digit counts (scanned in
+// place) and the scan's tile sums
+inline uint64_t radix_tiles_bytes(uint64_t tiles)
 {
-    const uint64_t hist = 256ull * div_up(count, kRadixTile);
+    const uint64_t hist = 256ull * tiles;
     return ((4 * hist + 255) & ~255ull) + scan_parts_bytes(hist);
 }
+inline uint64_t radix_scratch_bytes(uint64_t count) { return radix_tiles_bytes(div_up(count, kRadixTile)); }
 
 // Stable sort of (k, v)[0, count) by the key bits [lo, hi) in passes of 8
-// bits, ping-ponging between (k0, v0) and (k1, v1).  Returns in `flip`
+// bits, ping-ponging between (k0, v0) and (k1, v1); with a block size, of each
+// block by itself (div_up(count, block) * div_up(block, kRadixTile) tiles).
+// `indices`: v0 holds nothing yet, element i's value is i.  Returns in `flip`
 // whether the result ended in (k1, v1).
 inline cudaError_t radix_sort_bits(uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1,
                                    uint32_t count, uint32_t lo, uint32_t hi, void *scratch,
-                                   cudaStream_t s, bool &flip)
+                                   cudaStream_t s, bool &flip, uint32_t block = 0, bool indices = false)
 {
     flip = false;
     if (count <= 1)
-        return cudaSuccess;
+        return indices && count ? cudaMemsetAsync(v0, 0, sizeof(uint32_t), s) : cudaSuccess;
     static KernelSetup setup;
     int per_sm = 0;
     const cudaError_t err = kernel_setup(setup, (const void *)k_radix_scatter, kRadixThreads,
                                          sizeof(RadixShared), &per_sm);
     if (err != cudaSuccess)
         return err;
-    const uint32_t tiles = div_up(count, kRadixTile);
+    if (block == 0)
+        block = count;
+    const RadixSpan sp = {count, block, div_up(block, kRadixTile)};
+    const uint32_t tiles = div_up(count, block) * sp.per;
     uint32_t *hist = static_cast<uint32_t *>(scratch);
     const uint64_t hist_n = 256ull * tiles;
     uint32_t *part = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(scratch) +
@@ -337,11 +363,12 @@ inline cudaError_t radix_sort_bits(uint64_t *k0, uint32_t *v0, uint64_t *k1, uin
         uint32_t *vi = flip ? v1 : v0;
         uint64_t *ko = flip ? k0 : k1;
         uint32_t *vo = flip ? v0 : v1;
-        k_radix_count<<<tiles, kRadixThreads, 0, s>>>(ki, count, sh, hist, tiles);
+        k_radix_count<<<tiles, kRadixThreads, 0, s>>>(ki, sp, sh, hist);
         cudaError_t e = scan_u32(hist, hist, (uint32_t)hist_n, false, part, nullptr, s);
         if (e != cudaSuccess)
             return e;
-        k_radix_scatter<<<tiles, kRadixThreads, sizeof(RadixShared), s>>>(ki, vi, ko, vo, count, sh, hist, tiles);
+        k_radix_scatter<<<tiles, kRadixThreads, sizeof(RadixShared), s>>>(
+            ki, indices && sh == lo ? nullptr : vi, ko, vo, sp, sh, hist);
         flip = !flip;
     }
     return cudaGetLastError();

@@ -41,6 +41,20 @@ def test_first_keys_against_oracle(sigma, block):
         assert np.array_equal(prim.cpu().numpy().astype(np.uint32), ref_prim), (n, off)
 
 
+# blocks sorted each by itself (from tiles 8/9 full) and all together, with a
+# last block of any length
+@pytest.mark.parametrize("sigma", [2, 34, 256])
+@pytest.mark.parametrize("block", [3640, 3641, 4096, 4097, 8192, 8193, 14564, 65536])
+def test_blocks_sorted_by_themselves(sigma, block):
+    for n in (2 * block, 2 * block + 1, 9 * block - 1):
+        x = _input(sigma, n)
+        last, prim, st = hg.huff_bwt_forward(torch.from_numpy(x).cuda(), block)
+        ref_last, ref_prim = oracle.bwt(x, block)
+        assert int(st.item()) == 0
+        assert np.array_equal(last.cpu().numpy(), ref_last), n
+        assert np.array_equal(prim.cpu().numpy().astype(np.uint32), ref_prim), n
+
+
 # LF by tiles (blocks from 4 KiB) and by sorting (below), samples every 32 rows
 # ranked in shared memory (4 KiB..1 MiB) or every 64 by global jumps, walks of
 # a few rows to a whole block (periodic and constant blocks), blocks that do
