@@ -9,7 +9,8 @@
 //     second one.  Merged weights never decrease and merged ids grow in
 //     creation order, so the second queue is sorted by (weight, id) too; a
 //     leaf wins a weight tie because every byte id < 256 <= any merged id.
-//     This pops exactly the sequence of a (weight, id) min-heap.  (thread 0)
+//     This pops exactly the sequence of a (weight, id) min-heap, many pairs at
+//     once where the weights allow.                      (mostly parallel)
 //  3. depths by pointer jumping over the parent links          (parallel)
 //  4. the 32-bit limit check, then canonical codes with the RFC 1951
 //     next_code recurrence and a per-length rank by byte value  (parallel)

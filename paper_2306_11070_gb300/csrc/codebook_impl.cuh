@@ -10,7 +10,7 @@ namespace cbk {
 
 struct CodebookShared {
     unsigned long long w[256];
-    unsigned long long key[256];               // weight * 256 + byte, all ones if absent
+    alignas(16) unsigned long long key[256];   // weight * 256 + byte, all ones if absent
     unsigned long long pm[2][512];             // package-merge: the previous and current list
     uint16_t pos[kMaxCodeLen + 1][256];        // package-merge: position of each leaf per list
     int pm_take[kMaxCodeLen + 1];              // package-merge: leaves taken from each list
@@ -23,6 +23,7 @@ struct CodebookShared {
     uint32_t bl[kMaxCodeLen + 1];
     uint32_t next_code[kMaxCodeLen + 1];
     int s_max;
+    int q[3];  // the queues' heads and the next node, from a single thread's steps
 };
 
 // Code lengths of at most `limit` bits for the m leaves nw[0..m) (sorted by
@@ -132,8 +133,10 @@ __device__ __forceinline__ void build_codebook(const unsigned long long *__restr
         int rank = 0;
         if (!huge) {
 #pragma unroll 8
-            for (int j = 0; j < 256; ++j)
-                rank += sh.key[j] < kt;
+            for (int j = 0; j < 128; ++j) {
+                const ulonglong2 k2 = reinterpret_cast<const ulonglong2 *>(sh.key)[j];
+                rank += (k2.x < kt) + (k2.y < kt);
+            }
         } else {
             for (int j = 0; j < 256; ++j) {
                 const unsigned long long wj = sh.w[j];
@@ -146,48 +149,127 @@ __device__ __forceinline__ void build_codebook(const unsigned long long *__restr
     __syncthreads();
 
     if (m >= 2) {
-        // 2. two-queue merge
-        if (t == 0) {
-            // the first two entries of each queue are kept in registers (all
-            // ones past a queue's end), so that a take never waits for a
-            // shared load: a leaf's weight is loaded two takes before it can
-            // be needed, and a merged node's weight usually never is.  A tie
-            // takes the leaf (the smaller id).
-            constexpr unsigned long long kNone = ~0ull;
-            int li = 0, ii = m, ni = m;
-            unsigned long long l0 = sh.nw[0], l1 = sh.nw[1], i0 = kNone, i1 = kNone;  // m >= 2
-            for (int step = 0; step < m - 1; ++step) {
-                int ab[2];
-                unsigned long long wab[2];
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    // branch free: both refills are loaded (at in-range
-                    // indices) and the take selects
-                    const bool lf = l0 <= i0;
-                    const unsigned long long nl = sh.nw[li + 2 < 510 ? li + 2 : 510];
-                    const unsigned long long nq = sh.nw[ii + 2 < 510 ? ii + 2 : 510];
-                    ab[k] = lf ? li : ii;
-                    wab[k] = lf ? l0 : i0;
-                    const unsigned long long l1n = li + 2 < m ? nl : kNone;
-                    const unsigned long long i1n = ii + 2 < ni ? nq : kNone;
-                    l0 = lf ? l1 : l0;
-                    l1 = lf ? l1n : l1;
-                    i0 = lf ? i0 : i1;
-                    i1 = lf ? i1 : i1n;
-                    li += lf;
-                    ii += !lf;
-                }
-                const unsigned long long w2 = wab[0] + wab[1];
-                sh.nw[ni] = w2;
-                sh.par[ab[0]] = (int16_t)ni;
-                sh.par[ab[1]] = (int16_t)ni;
-                // the new node joins the merged queue at ni
-                i0 = ii == ni ? w2 : i0;
-                i1 = ii + 1 == ni ? w2 : i1;
-                ++ni;
+        // 2. two-queue merge, in rounds: every node not heavier than the sum
+        // T of the two lightest comes before the first new node (whose weight
+        // is T and whose id is larger), so all of them are taken in pairs at
+        // once, in (weight, id) order; one left over stays.  Rounds of fewer
+        // than six pairs (weights that grow like powers of two) give way to 32
+        // steps of one thread, a pair each; up to 64 byte values, and weights
+        // that a sum could overflow, take no rounds at all.  The codebook of
+        // 256 equally frequent bytes takes 7.2 us in rounds and 22 us step by
+        // step, that of text (34 values) 8.3 and 6.5 us.
+        constexpr unsigned long long kNone = ~0ull;
+        uint16_t *const seq = sh.pos[0];  // 512 places
+        const bool rounds = m > 64 && !huge;
+        int li = 0, ii = m, ni = m;
+        while (ni < 2 * m - 1) {  // (the same in every thread)
+            int leaves = 0, merged = 0;
+            bool leaf_in = false, merged_in = false;
+            if (rounds) {
+                const unsigned long long a0 = li < m ? sh.nw[li] : kNone;
+                const unsigned long long a1 = li + 1 < m ? sh.nw[li + 1] : kNone;
+                const unsigned long long b0 = ii < ni ? sh.nw[ii] : kNone;
+                const unsigned long long b1 = ii + 1 < ni ? sh.nw[ii + 1] : kNone;
+                const unsigned long long T = a0 <= b0 ? a0 + (a1 <= b0 ? a1 : b0) : b0 + (a0 <= b1 ? a0 : b1);
+                leaf_in = li + t < m && sh.nw[li + t] <= T;
+                merged_in = ii + t < ni && sh.nw[ii + t] <= T;
+                leaves = __syncthreads_count(leaf_in);
+                merged = __syncthreads_count(merged_in);
             }
-            sh.par[2 * m - 2] = (int16_t)(2 * m - 2);  // the root points at itself
+            const int pairs = (leaves + merged) >> 1;
+            if (pairs >= 6) {
+                if (leaf_in) {  // after the merged nodes lighter than it
+                    const unsigned long long w = sh.nw[li + t];
+                    int lo = 0, hi = merged;
+                    while (lo < hi) {
+                        const int mid = (lo + hi) >> 1;
+                        if (sh.nw[ii + mid] < w)
+                            lo = mid + 1;
+                        else
+                            hi = mid;
+                    }
+                    seq[t + lo] = (uint16_t)(li + t);
+                }
+                if (merged_in) {  // after the leaves not heavier than it
+                    const unsigned long long w = sh.nw[ii + t];
+                    int lo = 0, hi = leaves;
+                    while (lo < hi) {
+                        const int mid = (lo + hi) >> 1;
+                        if (sh.nw[li + mid] <= w)
+                            lo = mid + 1;
+                        else
+                            hi = mid;
+                    }
+                    seq[t + lo] = (uint16_t)(ii + t);
+                }
+                __syncthreads();
+                if (t < pairs) {
+                    const int a = seq[2 * t], b = seq[2 * t + 1];
+                    sh.nw[ni + t] = sh.nw[a] + sh.nw[b];
+                    sh.par[a] = sh.par[b] = (int16_t)(ni + t);
+                }
+                if ((leaves + merged) & 1) {
+                    if (seq[leaves + merged - 1] < m)
+                        --leaves;
+                    else
+                        --merged;
+                }
+                li += leaves;
+                ii += merged;
+                ni += pairs;
+                __syncthreads();
+                continue;
+            }
+            const int left = 2 * m - 1 - ni, steps = rounds && left > 32 ? 32 : left;
+            if (t == 0) {
+                // the first two entries of each queue are kept in registers (all
+                // ones past a queue's end), so that a take never waits for a
+                // shared load: a leaf's weight is loaded two takes before it can
+                // be needed, and a merged node's weight usually never is.  A tie
+                // takes the leaf (the smaller id).
+                unsigned long long l0 = li < m ? sh.nw[li] : kNone, l1 = li + 1 < m ? sh.nw[li + 1] : kNone;
+                unsigned long long i0 = ii < ni ? sh.nw[ii] : kNone, i1 = ii + 1 < ni ? sh.nw[ii + 1] : kNone;
+                for (int step = 0; step < steps; ++step) {
+                    int ab[2];
+                    unsigned long long wab[2];
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        // branch free: both refills are loaded (at in-range
+                        // indices) and the take selects
+                        const bool lf = l0 <= i0;
+                        const unsigned long long nl = sh.nw[li + 2 < 510 ? li + 2 : 510];
+                        const unsigned long long nq = sh.nw[ii + 2 < 510 ? ii + 2 : 510];
+                        ab[k] = lf ? li : ii;
+                        wab[k] = lf ? l0 : i0;
+                        const unsigned long long l1n = li + 2 < m ? nl : kNone;
+                        const unsigned long long i1n = ii + 2 < ni ? nq : kNone;
+                        l0 = lf ? l1 : l0;
+                        l1 = lf ? l1n : l1;
+                        i0 = lf ? i0 : i1;
+                        i1 = lf ? i1 : i1n;
+                        li += lf;
+                        ii += !lf;
+                    }
+                    const unsigned long long w2 = wab[0] + wab[1];
+                    sh.nw[ni] = w2;
+                    sh.par[ab[0]] = (int16_t)ni;
+                    sh.par[ab[1]] = (int16_t)ni;
+                    // the new node joins the merged queue at ni
+                    i0 = ii == ni ? w2 : i0;
+                    i1 = ii + 1 == ni ? w2 : i1;
+                    ++ni;
+                }
+                sh.q[0] = li;
+                sh.q[1] = ii;
+                sh.q[2] = ni;
+            }
+            __syncthreads();
+            li = sh.q[0];
+            ii = sh.q[1];
+            ni = sh.q[2];
         }
+        if (t == 0)
+            sh.par[2 * m - 2] = (int16_t)(2 * m - 2);  // the root points at itself
         __syncthreads();
         // 3. depth = distance to the root, by pointer jumping (9 rounds cover
         //    511 nodes; done early once every ancestor is the root)
@@ -259,20 +341,31 @@ __device__ __forceinline__ void build_codebook(const unsigned long long *__restr
     if (L)
         atomicAdd(&sh.bl[L], 1u);
     __syncthreads();
-    if (t == 0) {
+    // next_code[b] = (next_code[b - 1] + bl[b - 1]) << 1, that is the sum of
+    // bl[k] << (b - k) over the shorter lengths k, a length per thread; and the
+    // bytes of each length per warp
+    if (t >= 1 && t <= (int)kMaxCodeLen) {
         uint32_t code = 0;
-        sh.next_code[0] = 0;
-        for (int bits = 1; bits <= (int)kMaxCodeLen; ++bits) {
-            code = (code + (bits == 1 ? 0u : sh.bl[bits - 1])) << 1;
-            sh.next_code[bits] = code;
-        }
+        for (int k = 1; k < t; ++k)
+            code = (code + sh.bl[k]) << 1;
+        sh.next_code[t] = code;
     }
+    const int lane = t & 31, warp = t >> 5;
+    const uint32_t same = __match_any_sync(0xffffffffu, L);
+    uint16_t *const of_len = sh.pos[0];  // [warp][length]
+    if (t < 8 * (int)(kMaxCodeLen + 1))
+        of_len[t] = 0;
+    if (t + 256 < 8 * (int)(kMaxCodeLen + 1))
+        of_len[t + 256] = 0;
+    __syncthreads();
+    if (lane == __ffs(same) - 1)
+        of_len[warp * (kMaxCodeLen + 1) + L] = (uint16_t)__popc(same);
     __syncthreads();
     uint32_t code = 0;
     if (L) {
-        uint32_t r = 0;
-        for (int j = 0; j < t; ++j)
-            r += (sh.len_s[j] == L);
+        uint32_t r = __popc(same & ((1u << lane) - 1u));
+        for (int w = 0; w < warp; ++w)
+            r += of_len[w * (kMaxCodeLen + 1) + L];
         code = sh.next_code[L] + r;
     }
     cb->len[t] = (uint8_t)L;
