@@ -529,9 +529,10 @@ uint64_t huff_lzss_max_size(uint64_t n, uint64_t segment_bytes, const huff_lzss_
 uint64_t huff_lzss_workspace_size(uint64_t n, uint64_t segment_bytes,
                                   const huff_lzss_params_t *params);
 /* Compress d_in[0, n) into the container at d_out.  Asynchronous on the
- * stream, no host synchronisation and no allocation: one warp per segment
- * codes into a worst-case slot of d_ws, one CTA lays out the header and
- * table, a gather moves the codes into place.  *d_status is cleared first;
+ * stream, no host synchronisation and no allocation: one warp per segment,
+ * or several where there are few segments, codes into a worst-case slot of
+ * d_ws, one CTA lays out the header and table, a gather moves the codes into
+ * place.  *d_status is cleared first;
  * *d_out_bytes receives the container size; HUFF_ERR_CAPACITY in *d_status
  * when it exceeds out_cap.  d_in, d_out, d_ws 16-byte aligned (the caller's
  * buffers).  Host errors: HUFF_ERR_INVALID_ARG, HUFF_ERR_CUDA. */

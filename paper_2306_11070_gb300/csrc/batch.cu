@@ -11,9 +11,10 @@
 //                  build the codebook, dot each unit's histogram with the
 //                  code lengths, scan them into unit bit offsets, write the
 //                  stream header and size;
-//               3. encode items of up to 8 units of one buffer (one unit per
-//                  warp, dynamic tickets), the CTA's code table rebuilt only
-//                  when the item's buffer changes.
+//               3. encode items of up to 4 units of one buffer, each half of
+//                  the CTA its own (one unit per warp, dynamic tickets), the
+//                  half's code table rebuilt only when the item's buffer
+//                  changes.
 //   decompress: 1. per buffer: read n and the chunk size from the header and
 //                  size its work (chunks split across lanes so that even a
 //                  one-chunk buffer fills a warp);
@@ -189,7 +190,7 @@ __device__ __forceinline__ unsigned int half_broadcast(unsigned int t, HalfSync 
 // constant, so that it is part of the table loads), a little above the end of
 // the static shared memory.
 constexpr uint32_t kTblAt = 6144;
-constexpr uint32_t kTblSlack = 1024;
+constexpr uint32_t kTblSlack = 4096;
 
 // One function per way of grouping: inlined together they spill.
 template <int G, int kFirst, int S>

@@ -26,7 +26,7 @@
 // plus the rank of row p among the block's rows with that byte: counted per
 // tile and scanned, so LF is written in row order.  The block is the walk
 // p -> LF[p] from the primary row, emitted backwards.  The walk is cut at
-// sample rows (every 64th row and the primary rows): each sample walks to the
+// sample rows (every 32nd or 64th row and the primary rows): each sample walks to the
 // next sample, keeping the bytes it passes, list ranking by pointer jumping
 // over the samples gives each sample's distance from the primary row, and its
 // bytes are copied to their place.  A periodic block's walk returns to the

@@ -46,16 +46,15 @@
 // A code longer than the table has an all-zero entry, which consumes and
 // emits nothing: the lane waits on it until the next window resolves it.
 // Between windows each lane tops up its input ring in shared memory with
-// 16-byte cp.async copies that bypass L1 (sixteen 16-byte cells per lane
-// here, eight in the batched kernel) and
-// stores every completed group of its 128-byte output ring (laid out
-// [word][lane], so a warp's accesses never share a bank) with one global
-// store: 32-byte groups and 256-bit stores where the chunk's output is
-// 32-byte aligned (each lane's write a whole sector), else 16-byte groups.
-// The ring holds < 32 unflushed bytes, a window's <= 65 and 3 pending.  The next input word is always preloaded, so the ring's
-// latency stays off the per-codeword dependency chain.  The decoded codeword
-// sequence is exactly the sequential one, so the stream checks are those of
-// a sequential decoder.
+// 16-byte cp.async copies that bypass L1 (sixteen 16-byte cells per lane here,
+// eight in the batched kernel) and stores every completed group of its 128-byte
+// output ring (laid out [word][lane], so a warp's accesses never share a bank)
+// with one global store: 32-byte groups and 256-bit stores where the chunk's
+// output is 32-byte aligned (each lane's write a whole sector), else 16-byte
+// groups. The ring holds < 32 unflushed bytes, a window's <= 65 and 3 pending.
+// The next input word is always preloaded, so the ring's latency stays off the
+// per-codeword dependency chain.  The decoded codeword sequence is exactly the
+// sequential one, so the stream checks are those of a sequential decoder.
 #include "decode_impl.cuh"
 
 namespace huff {

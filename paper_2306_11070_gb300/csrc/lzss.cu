@@ -20,8 +20,9 @@
 //    segment's code packed MSB first into bytes from a 16-byte boundary,
 //    zero padded to the next one.
 //
-// Compression: one warp per segment.  For each token the 32 lanes search the
-// window together: for windows of 64 to 16384 bits all distances bit-parallel
+// Compression: one warp per segment, or per part of a segment where there are
+// few (see k_lzss_parts).  For each token the 32 lanes search the window
+// together: for windows of 64 to 16384 bits all distances bit-parallel
 // (a lane's 32-bit mask holds 32 sources) from a ring in shared memory, other
 // windows a distance at a time through L1.  Every lane keeps the same 64-bit
 // output accumulator and lane 0 stores the completed words into the
@@ -219,8 +220,6 @@ __host__ __device__ __forceinline__ bool ring_ok(const LzParams &P)
     return P.W >= 64 && P.W <= kRingMaxWindow;
 }
 
-// The longest match of lo..maxlen bits over 1024 distances at once, the
-// smallest distance among equally long ones.  Lane j holds 32 sources, the
 // The longest match of lo..maxlen bits over 1024 distances at once, the
 // smallest distance among equally long ones.  Lane j holds 32 sources, the
 // bits a:b (64 bits of the window from bit P - 32 j - 32 of position P); bit
@@ -509,18 +508,18 @@ __global__ void __launch_bounds__(32)
 
 // Few segments leave most of the chip idle, so a segment is coded in `parts` by
 // a warp each.  A part begins at its cut whether or not a token does; since a
-// token depends on its position alone, its code is right from the first of
-// its tokens that begins where one of the segment's tokens does (chains of
-// tokens from two starts meet after some tens of them, not counting runs).
+// token depends on its position alone, its code is right from the first of its
+// tokens that begins where one of the segment's tokens does (chains of tokens
+// from two starts meet after some tens of them, not counting runs).
 // k_lzss_parts codes the parts, noting kMarks places where a token begins, the
-// first kDense and then one in kSparse; k_lzss_join,
-// a warp per segment, takes the parts in order: from where the one before
-// ended it codes on until it meets a noted token (or, if it meets none, to the
-// part's end); k_lzss_gather_parts puts the pieces together bit by bit.
-// In a segment's slot, part k from byte k * stride on: {end, code bits, marks,
-// 0}, the code, the bits before the meeting point, the marks
-// {position, code bits before}.  Part 0 is right as it is; its marks' place
-// holds the pieces {first bit in the slot, bits}, 2 per part.
+// first kDense and then one in kSparse; k_lzss_join, a warp per segment, takes
+// the parts in order: from where the one before ended it codes on until it
+// meets a noted token (or, if it meets none, to the part's end);
+// k_lzss_gather_parts puts the pieces together bit by bit. In a segment's slot,
+// part k from byte k * stride on: {end, code bits, marks, 0}, the code, the
+// bits before the meeting point, the marks {position, code bits before}.  Part
+// 0 is right as it is; its marks' place holds the pieces {first bit in the
+// slot, bits}, 2 per part.
 constexpr uint32_t kMarks = 128, kDense = 96, kSparse = 16, kMaxParts = 8;
 constexpr uint32_t kMinPart = 4096;  // bytes
 struct PartsLayout {

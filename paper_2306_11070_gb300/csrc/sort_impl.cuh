@@ -6,7 +6,7 @@
 //    its offset), tiles of 4096 elements.
 //  - radix pass: stable scatter of (u64 key, u32 value) pairs by the 8-bit
 //    digit (key >> shift) & 255, in three launches: per-tile digit counts
-//    stored digit-major (count[d * tiles + t]), their exclusive scan (which
+//    stored digit-major (see RadixSpan), their exclusive scan (which
 //    is then each tile's first output slot per digit, tiles in order within
 //    a digit: stability across tiles), and the scatter.  The scatter ranks
 //    equal digits inside a tile in element order with a ballot per digit bit
