@@ -15,9 +15,9 @@
 //    lanes pack their groups into the warp's word buffer in shared memory,
 //    and the warp writes the whole words with coalesced stores.  The partial
 //    last word is carried in a register into the next step.
-//  - What bounds it: on text the shared-memory data pipe is 73% busy while a
+//  - What bounds it: on text the shared-memory data pipe is 66% busy while a
 //    unit runs (two wavefronts per 32 lookups, about 1.5 for the packed
-//    words) and 59% of the issue slots are taken.
+//    words) and 57% of the issue slots are taken (64 MiB).
 //  - The word a unit shares with the unit before it is completed by the later
 //    unit: it re-codes the last <= 31 bits of its predecessor from the 32
 //    input bytes before it, so no warp waits for another's output and the
