@@ -158,6 +158,8 @@ __global__ void k_bwt_round_keys(const uint32_t *sa, const uint32_t *rk, const u
                                  const uint32_t *grp, uint32_t count, uint32_t n, uint32_t block,
                                  uint64_t h, uint32_t lo_bits, uint64_t *key, uint32_t *val)
 {
+    chain_wait();
+    chain_next();
     for (uint32_t k = blockIdx.x * kEw + threadIdx.x; k < count; k += gridDim.x * kEw) {
         const uint32_t i = sa[act[k]];
         uint32_t s, m;
@@ -196,6 +198,8 @@ constexpr size_t kSegSmem = (5 * (size_t)kSegCap + (size_t)kSegWarps * 256 + 256
 __global__ void __launch_bounds__(kSegThreads) k_seg_sort(uint64_t *key, uint32_t *val, uint32_t count,
                                                           uint32_t lo_bits, uint32_t *cov)
 {
+    chain_wait();
+    chain_next();
     extern __shared__ __align__(16) uint32_t seg_sm[];
     uint32_t *sk = seg_sm;                      // [2][kSegCap] range keys
     uint32_t *sv = sk + 2 * kSegCap;            // [2][kSegCap] values
@@ -359,6 +363,8 @@ __global__ void __launch_bounds__(kSegThreads) k_seg_sort(uint64_t *key, uint32_
 // flags[k] = 1 - cov[k]: the members of groups left to the global passes
 __global__ void k_uncovered(uint32_t *cov, uint32_t count)
 {
+    chain_wait();
+    chain_next();
     for (uint32_t k = blockIdx.x * kEw + threadIdx.x; k < count; k += gridDim.x * kEw)
         cov[k] = 1u - cov[k];
 }
@@ -511,6 +517,8 @@ __global__ void __launch_bounds__(kRfThreads) k_refine_tiles(const uint64_t *key
                                                              uint32_t count, uint32_t gbits,
                                                              uint32_t *ph, uint32_t *pf, uint32_t *pm)
 {
+    chain_wait();
+    chain_next();
     extern __shared__ __align__(16) uint64_t rf_sm[];
     uint64_t *skey = rf_sm;
     uint32_t *sact = reinterpret_cast<uint32_t *>(rf_sm + kRfKeyWords);
@@ -541,6 +549,8 @@ __global__ void __launch_bounds__(kRfThreads) k_refine_tiles(const uint64_t *key
 __global__ void __launch_bounds__(kRfThreads) k_refine_parts(uint32_t *ph, uint32_t *pf, uint32_t *pm,
                                                              uint32_t tiles, uint32_t *tot)
 {
+    chain_wait();
+    chain_next();
     __shared__ uint32_t ws[kRfThreads / 32];
     constexpr int kPer = 8;  // tiles per thread and step: a step is three scans (103 -> 54 us at 1)
     uint32_t ch = 0, cf = 0, cm = 0;
@@ -592,6 +602,8 @@ __global__ void __launch_bounds__(kRfThreads) k_refine_apply(
     const uint32_t *ph, const uint32_t *pf, const uint32_t *pm, uint32_t *sa, uint32_t *rk,
     uint32_t *act2, uint32_t *grp2)
 {
+    chain_wait();
+    chain_next();
     extern __shared__ __align__(16) uint64_t rf_sm[];
     uint64_t *skey = rf_sm;
     uint32_t *sact = reinterpret_cast<uint32_t *>(rf_sm + kRfKeyWords);
@@ -644,6 +656,8 @@ __global__ void __launch_bounds__(kRfThreads) k_refine_apply(
 __global__ void k_bwt_output(const uint8_t *x, const uint32_t *sa, uint32_t n, uint32_t block,
                              uint8_t *last, uint32_t *primary)
 {
+    chain_wait();
+    chain_next();
     for (uint32_t p = blockIdx.x * kEw + threadIdx.x; p < n; p += gridDim.x * kEw) {
         const uint32_t i = sa[p];
         uint32_t s, m;
@@ -719,8 +733,10 @@ cudaError_t sort_groups(FwdWs &w, uint32_t count, uint32_t lo_bits, uint32_t bit
     uint32_t *cov = w.grp2, *idx = w.act2;
     if ((e = cudaMemsetAsync(cov, 0, 4ull * count, s)) != cudaSuccess)
         return e;
-    k_seg_sort<<<div_up(count, kSegWin), kSegThreads, kSegSmem, s>>>(w.k0, w.v0, count, lo_bits, cov);
-    k_uncovered<<<ew_grid(count), kEw, 0, s>>>(cov, count);
+    if ((e = launch_chained(k_seg_sort, div_up(count, kSegWin), kSegThreads, kSegSmem, s, w.k0, w.v0, count,
+                            lo_bits, cov)) != cudaSuccess ||
+        (e = launch_chained(k_uncovered, ew_grid(count), kEw, 0, s, cov, count)) != cudaSuccess)
+        return e;
     if ((e = scan_u32(cov, cov, count, true, w.part, w.scal + 2, s)) != cudaSuccess)
         return e;
     uint32_t big = 0;
@@ -760,13 +776,14 @@ cudaError_t refine(FwdWs &w, const uint64_t *ks, const uint32_t *vs, uint32_t co
         return e;
     // the first list is every slot in order
     const uint32_t *act = gbits < 64 ? w.act : nullptr;
-    k_refine_tiles<<<tiles, kRfThreads, kRfTilesSmem, s>>>(ks, act, count, gbits, ph, pf, pm);
-    k_refine_parts<<<1, kRfThreads, 0, s>>>(ph, pf, pm, tiles, w.scal);
-    k_refine_apply<<<tiles, kRfThreads, kRfApplySmem, s>>>(ks, vs, act, count, gbits, ph, pf, pm,
-                                                           w.sa, w.rk, w.act2, w.grp2);
+    if ((e = launch_chained(k_refine_tiles, tiles, kRfThreads, kRfTilesSmem, s, ks, act, count, gbits, ph, pf,
+                            pm)) != cudaSuccess ||
+        (e = launch_chained(k_refine_parts, 1, kRfThreads, 0, s, ph, pf, pm, tiles, w.scal)) != cudaSuccess ||
+        (e = launch_chained(k_refine_apply, tiles, kRfThreads, kRfApplySmem, s, ks, vs, act, count, gbits, ph,
+                            pf, pm, w.sa, w.rk, w.act2, w.grp2)) != cudaSuccess)
+        return e;
     uint32_t h[2];
-    if ((e = cudaGetLastError()) != cudaSuccess ||
-        (e = cudaMemcpyAsync(h, w.scal, sizeof(h), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+    if ((e = cudaMemcpyAsync(h, w.scal, sizeof(h), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
         return e;
     groups = h[0];
@@ -1444,14 +1461,17 @@ huff_status_t huff_bwt_forward(const uint8_t *d_in, uint64_t n, uint32_t block, 
         return HUFF_ERR_CUDA;
     for (uint64_t h = f.q; n_act > 0 && h < mmax; h *= 2) {
         const uint32_t lo_bits = bit_width(mmax - 1);
-        k_bwt_round_keys<<<ew_grid(n_act), kEw, 0, s>>>(w.sa, w.rk, w.act, w.grp, n_act, N, block, h,
-                                                        lo_bits, w.k0, w.v0);
+        if (launch_chained(k_bwt_round_keys, ew_grid(n_act), kEw, 0, s, w.sa, w.rk, w.act, w.grp, n_act, N,
+                           block, h, lo_bits, w.k0, w.v0) != cudaSuccess)
+            return HUFF_ERR_CUDA;
         if (sort_groups(w, n_act, lo_bits, lo_bits + bit_width(groups - 1), s, ks, vs) != cudaSuccess)
             return HUFF_ERR_CUDA;
         if (refine(w, ks, vs, n_act, lo_bits, s, n_act, groups) != cudaSuccess)
             return HUFF_ERR_CUDA;
     }
-    k_bwt_output<<<ew_grid(n), kEw, 0, s>>>(d_in, w.sa, N, block, d_last, d_primary);
+    if (launch_chained(k_bwt_output, ew_grid(n), kEw, 0, s, d_in, w.sa, N, block, d_last, d_primary) !=
+        cudaSuccess)
+        return HUFF_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? HUFF_OK : HUFF_ERR_CUDA;
 }
 

@@ -13,7 +13,8 @@
 //    and per-warp running counts, sorts the tile in shared memory and writes
 //    it out digit run by digit run, so consecutive threads write consecutive
 //    slots.
-// All loops are bounded by the element count; nothing waits on another CTA.
+// The kernels are launched behind one another (see launch_chained).  All loops
+// are bounded by the element count; nothing waits on another CTA.
 #pragma once
 
 #include "huff_internal.cuh"
@@ -68,6 +69,8 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t *warp_s
 __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(const uint32_t *in, uint32_t count,
                                                              uint32_t *part)
 {
+    chain_wait();
+    chain_next();
     __shared__ uint32_t ws[kScanThreads / 32];
     const uint64_t base = (uint64_t)blockIdx.x * kScanTile + (uint64_t)threadIdx.x * kScanItems;
     uint32_t s = 0;
@@ -85,6 +88,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(const uint32_t *in,
 __global__ void __launch_bounds__(kScanThreads) k_scan_parts(uint32_t *part, uint32_t tiles,
                                                              uint32_t *total)
 {
+    chain_wait();
+    chain_next();
     __shared__ uint32_t ws[kScanThreads / 32];
     uint32_t carry = 0;
     for (uint32_t b = 0; b < tiles; b += kScanThreads) {
@@ -104,6 +109,8 @@ template <bool kInclusive>
 __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const uint32_t *in, uint32_t count,
                                                              const uint32_t *part, uint32_t *out)
 {
+    chain_wait();
+    chain_next();
     __shared__ uint32_t ws[kScanThreads / 32];
     const uint64_t base = (uint64_t)blockIdx.x * kScanTile + (uint64_t)threadIdx.x * kScanItems;
     uint32_t v[kScanItems];
@@ -131,17 +138,15 @@ inline cudaError_t scan_u32(const uint32_t *in, uint32_t *out, uint32_t count, b
                             uint32_t *part, uint32_t *d_total, cudaStream_t s)
 {
     const uint32_t tiles = div_up(count, kScanTile);
-    if (tiles > 0) {
-        k_scan_tiles<<<tiles, kScanThreads, 0, s>>>(in, count, part);
-    }
-    k_scan_parts<<<1, kScanThreads, 0, s>>>(part, tiles, d_total);
-    if (tiles > 0) {
-        if (inclusive)
-            k_scan_apply<true><<<tiles, kScanThreads, 0, s>>>(in, count, part, out);
-        else
-            k_scan_apply<false><<<tiles, kScanThreads, 0, s>>>(in, count, part, out);
-    }
-    return cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    if (tiles > 0)
+        e = launch_chained(k_scan_tiles, tiles, kScanThreads, 0, s, in, count, part);
+    if (e == cudaSuccess)
+        e = launch_chained(k_scan_parts, 1, kScanThreads, 0, s, part, tiles, d_total);
+    if (e == cudaSuccess && tiles > 0)
+        e = launch_chained(inclusive ? k_scan_apply<true> : k_scan_apply<false>, tiles, kScanThreads, 0, s,
+                           in, count, part, out);
+    return e;
 }
 
 // ---- radix pass -----------------------------------------------------------
@@ -195,6 +200,8 @@ struct RadixSpan {
 __global__ void __launch_bounds__(kRadixThreads) k_radix_count(const uint64_t *keys, RadixSpan sp,
                                                                uint32_t shift, uint32_t *hist)
 {
+    chain_wait();
+    chain_next();
     __shared__ uint32_t c[256];
     if (threadIdx.x < 256)
         c[threadIdx.x] = 0;
@@ -246,6 +253,8 @@ __global__ void __launch_bounds__(kRadixThreads) k_radix_scatter(
     const uint64_t *kin, const uint32_t *vin, uint64_t *kout, uint32_t *vout, RadixSpan sp,
     uint32_t shift, const uint32_t *offs)
 {
+    chain_wait();
+    chain_next();
     extern __shared__ __align__(16) unsigned char radix_sm[];
     RadixShared &sh = *reinterpret_cast<RadixShared *>(radix_sm);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -373,15 +382,19 @@ inline cudaError_t radix_sort_bits(uint64_t *k0, uint32_t *v0, uint64_t *k1, uin
         uint32_t *vi = flip ? v1 : v0;
         uint64_t *ko = flip ? k0 : k1;
         uint32_t *vo = flip ? v0 : v1;
-        k_radix_count<<<tiles, kRadixThreads, 0, s>>>(ki, sp, sh, hist);
-        cudaError_t e = scan_u32(hist, hist, (uint32_t)hist_n, false, part, nullptr, s);
+        cudaError_t e = launch_chained(k_radix_count, tiles, kRadixThreads, 0, s, ki, sp, sh, hist);
         if (e != cudaSuccess)
             return e;
-        k_radix_scatter<<<tiles, kRadixThreads, sizeof(RadixShared), s>>>(
-            ki, indices && sh == lo ? nullptr : vi, ko, vo, sp, sh, hist);
+        e = scan_u32(hist, hist, (uint32_t)hist_n, false, part, nullptr, s);
+        if (e != cudaSuccess)
+            return e;
+        e = launch_chained(k_radix_scatter, tiles, kRadixThreads, sizeof(RadixShared), s, ki,
+                           indices && sh == lo ? nullptr : vi, ko, vo, sp, sh, hist);
+        if (e != cudaSuccess)
+            return e;
         flip = !flip;
     }
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 }  // namespace srt
