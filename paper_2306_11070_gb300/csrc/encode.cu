@@ -124,15 +124,12 @@ __device__ __noinline__ bool encode_unit_fit(const Job J, uint64_t u, const uint
 __global__ void __launch_bounds__(kEncBlock, 1) k_encode(const __grid_constant__ EncodeArgs a)
 {
     extern __shared__ uint4 smem_raw[];
-    // the offsets' scan is the kernel before this one and lets it start once
-    // the kernels before the scan are complete, the codebook's among them: the
-    // table is built while the scan runs
-    const Smem m = carve(smem_raw);
-    const uint32_t max_len = a.cb->max_len;
-    build_table(a.cb, m.tbl, max_len <= kMadMaxLen, threadIdx.x, kEncBlock);
     chain_wait();
     if (chain_failed(a.status))
         return;
+    const Smem m = carve(smem_raw);
+    const uint32_t max_len = a.cb->max_len;
+    build_table(a.cb, m.tbl, max_len <= kMadMaxLen, threadIdx.x, kEncBlock);
     const Job J = make_job(a.in, a.n, a.cs, a.unit_off, a.out, a.out_cap);
     if (blockIdx.x == 0)
         write_header(J, a.cb, a.out_bytes, a.status);

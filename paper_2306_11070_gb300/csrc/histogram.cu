@@ -29,8 +29,7 @@ using namespace hst;
 constexpr int kHistBlock = kThreads;
 
 // Clears the totals (and the chain's status).  A kernel instead of memory sets,
-// because the histogram can be launched behind it and needs the totals only
-// at its end.
+// because the histogram can be launched behind it.
 __global__ void __launch_bounds__(256) k_clear(unsigned long long *hist, int32_t *status)
 {
     chain_next();
@@ -40,14 +39,14 @@ __global__ void __launch_bounds__(256) k_clear(unsigned long long *hist, int32_t
 }
 
 __global__ void __launch_bounds__(kHistBlock)
-    k_histogram(const uint8_t *__restrict__ in, uint64_t n, unsigned long long *__restrict__ hist,
-                uint16_t *__restrict__ unit_hist)
+    k_histogram(const uint8_t *in, uint64_t n, unsigned long long *hist, uint16_t *unit_hist)
 {
     __shared__ __align__(16) uint32_t cnt[256 * 32];
     chain_next();
     const int tid = threadIdx.x, lane = tid & 31;
     for (int i = tid; i < 256 * 32; i += kHistBlock)
         cnt[i] = 0;
+    chain_wait();
     const uint32_t col = smem_u32(cnt) + 4u * lane;  // this lane's column
     const uint64_t units = (n + kUnitSymbols - 1) / kUnitSymbols;
     uint32_t prev = 0, total = 0;  // this thread's bin: last fold, count so far
@@ -85,7 +84,6 @@ __global__ void __launch_bounds__(kHistBlock)
     __syncthreads();
     if (!unit_hist)
         total = fold_bin(cnt, tid);
-    chain_wait();  // the totals are cleared
     if (total)
         atomicAdd(hist + tid, (unsigned long long)total);
 }

@@ -150,12 +150,14 @@ cudaError_t kernel_setup(KernelSetup &ks, const void *func, int block, size_t dy
 // chain_wait(), so that a launch's latency (1 to 2 us) passes beside the work
 // instead of after it (64 MiB compress, six kernels: 89 -> 75 us, with the two
 // memory sets and the scan's first kernel gone).  Every thread of a kernel
-// launched so calls chain_wait() on every path, before it touches what an
-// earlier kernel writes or reads; therefore, once a kernel is past its own
-// wait, all kernels before its predecessor are complete too.  chain_next() lets
-// the next kernel start.  What such a kernel reads of its predecessors has no
-// __restrict__: a load through the read-only path could be moved above the
-// wait.
+// launched so calls chain_wait() on every path before it touches any global
+// memory: the wait is what makes writes visible, those of the kernel before
+// it, which has waited itself, and so those of all kernels before that one.
+// (A kernel that started behind one past its wait would find everything
+// older complete, but nothing says that it would see it.)  Before the wait a
+// kernel may set up shared memory.  chain_next() lets the next kernel start.
+// What such a kernel reads has no __restrict__: a load through the read-only
+// path could be moved above the wait.
 __device__ __forceinline__ void chain_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
