@@ -104,10 +104,9 @@ __device__ __forceinline__ void package_merge(int m, int limit, CodebookShared &
 // longer than `limit` (1..32) bits: without `limited` that is an error (*cb
 // cleared, HUFF_ERR_CODE_TOO_LONG); with it the lengths are recomputed by
 // package-merge (the error only if the bytes present exceed 2^limit).
-__device__ __forceinline__ void build_codebook(const unsigned long long *__restrict__ hist,
-                                               huff_codebook_t *__restrict__ cb, int32_t *status,
-                                               CodebookShared &sh, int limit = (int)kMaxCodeLen,
-                                               bool limited = false)
+__device__ __forceinline__ void build_codebook(const unsigned long long *hist, huff_codebook_t *cb,
+                                               int32_t *status, CodebookShared &sh,
+                                               int limit = (int)kMaxCodeLen, bool limited = false)
 {
     if (chain_failed(status))
         return;

@@ -58,3 +58,9 @@ def test_waits_before_it_touches_memory(where):
         name = re.search(r"(\w+)\s*$", p).group(1)
         assert not re.search(rf"\b{name}\b", head), f"{name} is used before the wait"
     assert "__restrict__" not in params
+
+
+def test_their_routines_have_no_read_only_pointers():
+    """The device routines that chained kernels pass their pointers to."""
+    for name in ("codebook_impl.cuh", "hist_impl.cuh", "encode_impl.cuh", "sort_impl.cuh"):
+        assert "__restrict__" not in _text(os.path.join(CSRC, name)), name
