@@ -243,9 +243,10 @@ typedef struct huff_batch_params {
     uint32_t decode_lanes;  /* decompress: lanes to spread a buffer over
                                (1..65536): its chunks are split into the
                                smallest power of two S <= 32 of sub-segments
-                               with chunks x S >= decode_lanes.  A batch with
-                               chunks for half the launch's lanes splits a
-                               buffer only as far as that saves idle lanes  */
+                               with chunks x S >= decode_lanes.  With the
+                               default (HUFF_DEFAULT_DECODE_LANES), a batch
+                               with chunks for half the launch's lanes splits
+                               a buffer only as far as that saves idle lanes */
     uint32_t use_graph;     /* capture the launch in a CUDA graph (1) or not  */
     uint32_t barrier_extra; /* test hook, 0 in use: nonzero makes the launch's
                                grid barriers wait for that many CTAs more than
@@ -257,6 +258,7 @@ typedef struct huff_batch_params {
 typedef struct huff_batch_plan huff_batch_plan_t; /* opaque */
 
 /* Defaults: 16384-symbol chunks, full occupancy, 128 decode lanes, graph on. */
+#define HUFF_DEFAULT_DECODE_LANES 128u
 void huff_batch_default_params(huff_batch_params_t *params);
 
 /* Plan a batch of `count` buffers for `op` (params may be NULL for the
@@ -448,7 +450,10 @@ typedef struct huff_server_cfg {
     uint32_t decode_lanes;   /* lanes to spread a decompress request over, at
                                 least (128; 1..65536): a round of few
                                 requests spreads each over more, so that
-                                the round fills about one wave of decoders */
+                                the round fills about one wave of decoders.
+                                With the default, a round with chunks for
+                                half its lanes spreads a request only as far
+                                as that saves idle lanes                     */
 } huff_server_cfg_t;
 
 typedef struct huff_request {

@@ -520,8 +520,10 @@ __global__ void __launch_bounds__(kBatchBlock, 2) k_batch_decompress(BatchArgs a
             chunks += s_part[t];
         __syncthreads();
         // a batch with chunks for half the lanes the chip decodes in needs no
-        // splitting to keep it busy (the single-stream rule)
-        const uint32_t lanes = 2 * chunks >= (uint64_t)gridDim.x * kBatchBlock ? 0u : a.min_lanes;
+        // splitting to keep it busy (the single-stream rule); a caller's own
+        // number of lanes holds all the same
+        const bool fills = 2 * chunks >= (uint64_t)gridDim.x * kBatchBlock;
+        const uint32_t lanes = fills && !a.own_lanes ? 0u : a.min_lanes;
         auto items = [&](uint64_t c) -> uint64_t {
             if (c == kNoChunks || c == 0)
                 return 1;
@@ -679,7 +681,7 @@ void batch_layout(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op, 
     L.upload_bytes = L.o_di;
 }
 
-BatchArgs batch_args(const BatchLayout &L, void *d_block, uint32_t cs, uint32_t lanes,
+BatchArgs batch_args(const BatchLayout &L, void *d_block, uint32_t cs, uint32_t lanes, bool own_lanes,
                      uint32_t barrier_extra)
 {
     uint8_t *blk = static_cast<uint8_t *>(d_block);
@@ -697,6 +699,7 @@ BatchArgs batch_args(const BatchLayout &L, void *d_block, uint32_t cs, uint32_t 
     a.unit_owner = c ? reinterpret_cast<uint4 *>(blk + L.o_uw) : nullptr;
     a.item_owner = c ? reinterpret_cast<uint4 *>(blk + L.o_iw) : nullptr;
     a.min_lanes = lanes;
+    a.own_lanes = own_lanes;
     a.ctl = reinterpret_cast<unsigned int *>(blk + L.o_ctl);
     a.fail = reinterpret_cast<int32_t *>(blk + L.o_ctl + sizeof(unsigned int) * kCtlWords);
     a.barrier_extra = barrier_extra;
@@ -792,7 +795,7 @@ huff_status_t batch_once(const huff_batch_desc_t *descs, uint32_t count, huff_op
     host.resize(L.upload_bytes);
     if (batch_upload(L, scratch, host.data(), s) != cudaSuccess)
         return HUFF_ERR_CUDA;
-    const BatchArgs args = batch_args(L, scratch, prm.chunk_symbols, prm.decode_lanes);
+    const BatchArgs args = batch_args(L, scratch, prm.chunk_symbols, prm.decode_lanes, false);
     if (batch_launch(op, args, (unsigned)(device_sm_count() * per_sm), s) != cudaSuccess)
         return HUFF_ERR_CUDA;
     ran = true;
@@ -831,31 +834,12 @@ void free_plan(huff_batch_plan_t *p)
 
 }  // namespace
 
-extern "C" {
+namespace huff {
 
-void huff_batch_default_params(huff_batch_params_t *params)
+huff_status_t batch_plan(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
+                         const huff_batch_params_t &prm, bool own_lanes, huff_batch_plan_t **out_plan)
 {
-    if (!params)
-        return;
-    params->chunk_symbols = HUFF_DEFAULT_CHUNK_SYMBOLS;
-    params->ctas_per_sm = 0;  // as many as fit
-    params->decode_lanes = 128;
-    params->use_graph = 1;
-    params->barrier_extra = 0;
-}
-
-huff_status_t huff_batch_plan(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
-                              const huff_batch_params_t *params, huff_batch_plan_t **out_plan)
-{
-    HUFF_API_RANGE("huff_batch_plan");
-    if (!out_plan)
-        return HUFF_ERR_INVALID_ARG;
-    *out_plan = nullptr;
-    huff_batch_params_t prm;
-    huff_batch_default_params(&prm);
-    if (params)
-        prm = *params;
-    huff_status_t st = batch_check(descs, count, op, prm);
+    const huff_status_t st = batch_check(descs, count, op, prm);
     if (st != HUFF_OK)
         return st;
 
@@ -887,7 +871,8 @@ huff_status_t huff_batch_plan(const huff_batch_desc_t *descs, uint32_t count, hu
         free_plan(p);
         return HUFF_ERR_CUDA;
     }
-    p->args = batch_args(L, p->d_block, prm.chunk_symbols, prm.decode_lanes, prm.barrier_extra);
+    p->args = batch_args(L, p->d_block, prm.chunk_symbols, prm.decode_lanes, own_lanes,
+                         prm.barrier_extra);
     int per_sm = batch_occupancy(op);
     if (per_sm < 1) {
         free_plan(p);
@@ -924,6 +909,35 @@ huff_status_t huff_batch_plan(const huff_batch_desc_t *descs, uint32_t count, hu
     }
     *out_plan = p;
     return HUFF_OK;
+}
+
+}  // namespace huff
+
+extern "C" {
+
+void huff_batch_default_params(huff_batch_params_t *params)
+{
+    if (!params)
+        return;
+    params->chunk_symbols = HUFF_DEFAULT_CHUNK_SYMBOLS;
+    params->ctas_per_sm = 0;  // as many as fit
+    params->decode_lanes = HUFF_DEFAULT_DECODE_LANES;
+    params->use_graph = 1;
+    params->barrier_extra = 0;
+}
+
+huff_status_t huff_batch_plan(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
+                              const huff_batch_params_t *params, huff_batch_plan_t **out_plan)
+{
+    HUFF_API_RANGE("huff_batch_plan");
+    if (!out_plan)
+        return HUFF_ERR_INVALID_ARG;
+    *out_plan = nullptr;
+    huff_batch_params_t prm;
+    huff_batch_default_params(&prm);
+    if (params)
+        prm = *params;
+    return batch_plan(descs, count, op, prm, prm.decode_lanes != HUFF_DEFAULT_DECODE_LANES, out_plan);
 }
 
 huff_status_t huff_batch_run(huff_batch_plan_t *plan, huff_stream_t stream)

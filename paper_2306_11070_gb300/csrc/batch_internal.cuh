@@ -45,7 +45,8 @@ struct BatchArgs {
     uint4 *item_owner;              // compress: [items] (buffer, item within it, its first
                                     //   unit's index in unit_base order, low and high words)
     uint64_t *dec_items;            // decompress: [count + 1] items, then their prefix
-    uint32_t min_lanes;             // decompress: lanes per buffer to aim for
+    uint32_t min_lanes;             // decompress: lanes per buffer to aim for,
+    uint32_t own_lanes;             //   whatever the batch's size (the caller's own number)
     unsigned int *ctl;              // kCtlWords
     int32_t *fail;                  // whole-batch failure (barrier timeout)
     uint32_t barrier_extra;         // test hook: CTAs the barriers wait for beyond the grid
@@ -63,14 +64,17 @@ struct BatchLayout {
 };
 
 void batch_layout(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op, BatchLayout &L);
-BatchArgs batch_args(const BatchLayout &L, void *d_block, uint32_t cs, uint32_t lanes,
+BatchArgs batch_args(const BatchLayout &L, void *d_block, uint32_t cs, uint32_t lanes, bool own_lanes,
                      uint32_t barrier_extra = 0);
 cudaError_t batch_upload(const BatchLayout &L, void *d_block, uint8_t *host, cudaStream_t s);
 int batch_occupancy(huff_op_t op);
 cudaError_t batch_launch(huff_op_t op, const BatchArgs &args, unsigned grid, cudaStream_t s);
+// huff_batch_plan, with the lanes of prm the caller's own or not.
+huff_status_t batch_plan(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
+                         const huff_batch_params_t &prm, bool own_lanes, huff_batch_plan_t **out_plan);
 // Run a batch once without a plan, its device block in `scratch` (16-byte
-// aligned); `ran` is false when the block does not fit there.  `host` is read
-// by the upload until the stream has passed it.
+// aligned) and its lanes not a caller's own; `ran` is false when the block does
+// not fit there.  `host` is read by the upload until the stream has passed it.
 huff_status_t batch_once(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
                          const huff_batch_params_t &prm, void *scratch, uint64_t scratch_bytes,
                          std::vector<uint8_t> &host, cudaStream_t s, bool &ran);

@@ -209,7 +209,7 @@ huff_status_t segmented_compress(const uint8_t *d_in, uint64_t n, uint64_t segme
         huff_status_t st = batch_once(descs.data(), (uint32_t)L.count, HUFF_BATCH_COMPRESS, prm,
                                       scratch, scratch_bytes, host, s, ran);
         if (st == HUFF_OK && !ran) {
-            st = huff_batch_plan(descs.data(), (uint32_t)L.count, HUFF_BATCH_COMPRESS, &prm, &plan);
+            st = batch_plan(descs.data(), (uint32_t)L.count, HUFF_BATCH_COMPRESS, prm, false, &plan);
             if (st == HUFF_OK)
                 st = huff_batch_run(plan, reinterpret_cast<huff_stream_t>(s));
         }
@@ -301,7 +301,7 @@ huff_status_t segmented_decompress(const uint8_t *d_in, uint64_t in_bytes, uint8
     // coded) against 64 lanes
     {
         const uint64_t want = ((uint64_t)device_sm_count() * 256 + count - 1) / count;
-        uint32_t lanes = 128;
+        uint32_t lanes = HUFF_DEFAULT_DECODE_LANES;
         while (lanes < want && lanes < 65536)
             lanes <<= 1;
         prm.decode_lanes = lanes;
@@ -313,7 +313,7 @@ huff_status_t segmented_decompress(const uint8_t *d_in, uint64_t in_bytes, uint8
                                   spare ? mem + words : nullptr, spare ? scratch_bytes - words : 0,
                                   host, s, ran);
     if (st == HUFF_OK && !ran) {
-        st = huff_batch_plan(descs.data(), (uint32_t)count, HUFF_BATCH_DECOMPRESS, &prm, &plan);
+        st = batch_plan(descs.data(), (uint32_t)count, HUFF_BATCH_DECOMPRESS, prm, false, &plan);
         if (st == HUFF_OK)
             st = huff_batch_run(plan, reinterpret_cast<huff_stream_t>(s));
     }

@@ -232,7 +232,9 @@ bool start_round(huff_server_t *S, Round &r, huff_op_t op)
             while (lanes < want && lanes < 65536)
                 lanes <<= 1;
         }
-        const huff::BatchArgs args = huff::batch_args(L, blk, S->cfg.chunk_symbols, lanes);
+        const huff::BatchArgs args =
+            huff::batch_args(L, blk, S->cfg.chunk_symbols, lanes,
+                             S->cfg.decode_lanes != HUFF_DEFAULT_DECODE_LANES);
         ok = huff::batch_launch(op, args, S->grid, r.s) == cudaSuccess;
     }
     ok = ok && cudaMemcpyAsync(r.h_stage, d_meta, 16ull * count, cudaMemcpyDeviceToHost, r.s) ==
@@ -369,7 +371,7 @@ void huff_server_default_config(huff_server_cfg_t *cfg)
     cfg->max_rounds = 3;
     cfg->max_batch = 256;
     cfg->chunk_symbols = HUFF_DEFAULT_CHUNK_SYMBOLS;
-    cfg->decode_lanes = 128;
+    cfg->decode_lanes = HUFF_DEFAULT_DECODE_LANES;
 }
 
 huff_status_t huff_server_create(const huff_server_cfg_t *cfg, huff_server_t **out)
