@@ -777,31 +777,6 @@ huff_status_t batch_check(const huff_batch_desc_t *descs, uint32_t count, huff_o
     return HUFF_OK;
 }
 
-huff_status_t batch_once(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
-                         const huff_batch_params_t &prm, void *scratch, uint64_t scratch_bytes,
-                         std::vector<uint8_t> &host, cudaStream_t s, bool &ran)
-{
-    ran = false;
-    const huff_status_t st = batch_check(descs, count, op, prm);
-    if (st != HUFF_OK)
-        return st;
-    BatchLayout L;
-    batch_layout(descs, count, op, L);
-    if (!scratch || L.bytes > scratch_bytes)
-        return HUFF_OK;
-    const int per_sm = batch_occupancy(op);
-    if (per_sm < 1)
-        return HUFF_ERR_CUDA;
-    host.resize(L.upload_bytes);
-    if (batch_upload(L, scratch, host.data(), s) != cudaSuccess)
-        return HUFF_ERR_CUDA;
-    const BatchArgs args = batch_args(L, scratch, prm.chunk_symbols, prm.decode_lanes, false);
-    if (batch_launch(op, args, (unsigned)(device_sm_count() * per_sm), s) != cudaSuccess)
-        return HUFF_ERR_CUDA;
-    ran = true;
-    return HUFF_OK;
-}
-
 }  // namespace huff
 
 using namespace huff;
@@ -836,22 +811,19 @@ void free_plan(huff_batch_plan_t *p)
 
 namespace huff {
 
-huff_status_t batch_plan(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
-                         const huff_batch_params_t &prm, bool own_lanes, huff_batch_plan_t **out_plan)
-{
-    const huff_status_t st = batch_check(descs, count, op, prm);
-    if (st != HUFF_OK)
-        return st;
+namespace {
 
+// A plan of the laid-out batch L (see huff_batch_plan).
+huff_status_t make_plan(const BatchLayout &L, const huff_batch_params_t &prm, bool own_lanes,
+                        huff_batch_plan_t **out_plan)
+{
     huff_batch_plan_t *p = new (std::nothrow) huff_batch_plan_t();
     if (!p)
         return HUFF_ERR_CUDA;
     std::memset(p, 0, sizeof(*p));
-    p->op = op;
+    p->op = L.op;
     p->params = prm;
-    p->count = count;
-    BatchLayout L;
-    batch_layout(descs, count, op, L);
+    p->count = L.count;
     if (cudaMalloc(&p->d_block, L.bytes) != cudaSuccess) {
         free_plan(p);
         return HUFF_ERR_CUDA;
@@ -873,7 +845,7 @@ huff_status_t batch_plan(const huff_batch_desc_t *descs, uint32_t count, huff_op
     }
     p->args = batch_args(L, p->d_block, prm.chunk_symbols, prm.decode_lanes, own_lanes,
                          prm.barrier_extra);
-    int per_sm = batch_occupancy(op);
+    int per_sm = batch_occupancy(L.op);
     if (per_sm < 1) {
         free_plan(p);
         return HUFF_ERR_CUDA;
@@ -890,7 +862,7 @@ huff_status_t batch_plan(const huff_batch_desc_t *descs, uint32_t count, huff_op
         }
         bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
         if (ok) {
-            const cudaError_t le = batch_launch(op, p->args, p->grid, cs);
+            const cudaError_t le = batch_launch(L.op, p->args, p->grid, cs);
             ok = cudaStreamEndCapture(cs, &p->graph) == cudaSuccess && le == cudaSuccess;
         }
         if (ok)
@@ -909,6 +881,33 @@ huff_status_t batch_plan(const huff_batch_desc_t *descs, uint32_t count, huff_op
     }
     *out_plan = p;
     return HUFF_OK;
+}
+
+}  // namespace
+
+huff_status_t batch_once(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
+                         const huff_batch_params_t &prm, void *scratch, uint64_t scratch_bytes,
+                         std::vector<uint8_t> &host, cudaStream_t s, huff_batch_plan_t **plan)
+{
+    *plan = nullptr;
+    huff_status_t st = batch_check(descs, count, op, prm);
+    if (st != HUFF_OK)
+        return st;
+    BatchLayout L;
+    batch_layout(descs, count, op, L);
+    if (!scratch || L.bytes > scratch_bytes) {
+        st = make_plan(L, prm, false, plan);
+        return st == HUFF_OK ? huff_batch_run(*plan, reinterpret_cast<huff_stream_t>(s)) : st;
+    }
+    const int per_sm = batch_occupancy(op);
+    if (per_sm < 1)
+        return HUFF_ERR_CUDA;
+    host.resize(L.upload_bytes);
+    if (batch_upload(L, scratch, host.data(), s) != cudaSuccess)
+        return HUFF_ERR_CUDA;
+    const BatchArgs args = batch_args(L, scratch, prm.chunk_symbols, prm.decode_lanes, false);
+    return batch_launch(op, args, (unsigned)(device_sm_count() * per_sm), s) == cudaSuccess ? HUFF_OK
+                                                                                            : HUFF_ERR_CUDA;
 }
 
 }  // namespace huff
@@ -937,7 +936,12 @@ huff_status_t huff_batch_plan(const huff_batch_desc_t *descs, uint32_t count, hu
     huff_batch_default_params(&prm);
     if (params)
         prm = *params;
-    return batch_plan(descs, count, op, prm, prm.decode_lanes != HUFF_DEFAULT_DECODE_LANES, out_plan);
+    const huff_status_t st = batch_check(descs, count, op, prm);
+    if (st != HUFF_OK)
+        return st;
+    BatchLayout L;
+    batch_layout(descs, count, op, L);
+    return make_plan(L, prm, prm.decode_lanes != HUFF_DEFAULT_DECODE_LANES, out_plan);
 }
 
 huff_status_t huff_batch_run(huff_batch_plan_t *plan, huff_stream_t stream)

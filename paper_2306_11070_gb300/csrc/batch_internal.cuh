@@ -69,15 +69,13 @@ BatchArgs batch_args(const BatchLayout &L, void *d_block, uint32_t cs, uint32_t 
 cudaError_t batch_upload(const BatchLayout &L, void *d_block, uint8_t *host, cudaStream_t s);
 int batch_occupancy(huff_op_t op);
 cudaError_t batch_launch(huff_op_t op, const BatchArgs &args, unsigned grid, cudaStream_t s);
-// huff_batch_plan, with the lanes of prm the caller's own or not.
-huff_status_t batch_plan(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
-                         const huff_batch_params_t &prm, bool own_lanes, huff_batch_plan_t **out_plan);
-// Run a batch once without a plan, its device block in `scratch` (16-byte
-// aligned) and its lanes not a caller's own; `ran` is false when the block does
-// not fit there.  `host` is read by the upload until the stream has passed it.
+// Run a batch once, its lanes not a caller's own: with its device block in
+// `scratch` (16-byte aligned) where it fits, else by a plan, which the caller
+// destroys once the stream has passed it.  `host` is read by the upload until
+// then too.
 huff_status_t batch_once(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
                          const huff_batch_params_t &prm, void *scratch, uint64_t scratch_bytes,
-                         std::vector<uint8_t> &host, cudaStream_t s, bool &ran);
+                         std::vector<uint8_t> &host, cudaStream_t s, huff_batch_plan_t **plan);
 huff_status_t batch_check(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
                           const huff_batch_params_t &prm);
 

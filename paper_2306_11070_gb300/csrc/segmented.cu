@@ -203,16 +203,10 @@ huff_status_t segmented_compress(const uint8_t *d_in, uint64_t n, uint64_t segme
         prm.use_graph = 0;  // one run
         if (L.count > 0xffffffffull)
             return HUFF_ERR_INVALID_ARG;
-        bool ran = false;
         std::vector<uint8_t> host;
         huff_batch_plan_t *plan = nullptr;
         huff_status_t st = batch_once(descs.data(), (uint32_t)L.count, HUFF_BATCH_COMPRESS, prm,
-                                      scratch, scratch_bytes, host, s, ran);
-        if (st == HUFF_OK && !ran) {
-            st = batch_plan(descs.data(), (uint32_t)L.count, HUFF_BATCH_COMPRESS, prm, false, &plan);
-            if (st == HUFF_OK)
-                st = huff_batch_run(plan, reinterpret_cast<huff_stream_t>(s));
-        }
+                                      scratch, scratch_bytes, host, s, &plan);
         if (cudaStreamSynchronize(s) != cudaSuccess && st == HUFF_OK)
             st = HUFF_ERR_CUDA;
         huff_batch_destroy(plan);
@@ -307,16 +301,10 @@ huff_status_t segmented_decompress(const uint8_t *d_in, uint64_t in_bytes, uint8
         prm.decode_lanes = lanes;
     }
     huff_batch_plan_t *plan = nullptr;
-    bool ran = false;
     std::vector<uint8_t> host;
     huff_status_t st = batch_once(descs.data(), (uint32_t)count, HUFF_BATCH_DECOMPRESS, prm,
                                   spare ? mem + words : nullptr, spare ? scratch_bytes - words : 0,
-                                  host, s, ran);
-    if (st == HUFF_OK && !ran) {
-        st = batch_plan(descs.data(), (uint32_t)count, HUFF_BATCH_DECOMPRESS, prm, false, &plan);
-        if (st == HUFF_OK)
-            st = huff_batch_run(plan, reinterpret_cast<huff_stream_t>(s));
-    }
+                                  host, s, &plan);
     if (st == HUFF_ERR_INVALID_ARG) {  // descriptors taken from a malformed table
         cudaFree(own);
         return put_status(d_status, HUFF_ERR_CORRUPT_STREAM, s);
