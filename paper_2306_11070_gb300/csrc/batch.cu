@@ -212,6 +212,8 @@ __device__ __forceinline__ bool encode_unit(const enc::Job &J, uint64_t u, const
     case enc::kFit8: return unit_by<8, 8, 8>(J, u, tbl, wob);
     case enc::kFit4: return unit_by<4, 4, 4>(J, u, tbl, wob);
     case enc::kFit3: return unit_by<3, 3, 3>(J, u, tbl, wob);
+    case enc::kPairs4: return unit_by<4, 2, 2>(J, u, tbl, wob);
+    case enc::kPairs3: return unit_by<3, 2, 2>(J, u, tbl, wob);
     case enc::kTry4: return unit_by<4, 1, 1>(J, u, tbl, wob);
     case enc::kTry3: return unit_by<3, 1, 1>(J, u, tbl, wob);
     default: return unit_long(J, u, tbl, wob);

@@ -78,8 +78,8 @@ __device__ __forceinline__ Smem carve(uint4 *smem_raw)
     for (uint64_t u = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; u < (J).units; \
          u += (uint64_t)gridDim.x * kEncWarps)
 
-// Codes of 11 to 31 bits, in groups of G that nearly always fit.
-template <int G>
+// Codes of 11 to 31 bits, in groups of G that nearly always fit, else of S.
+template <int G, int S>
 __device__ __noinline__ void encode_try(const EncodeArgs &a)
 {
     extern __shared__ uint4 smem_raw[];
@@ -87,7 +87,7 @@ __device__ __noinline__ void encode_try(const EncodeArgs &a)
     const Job J = make_job(a.in, a.n, a.cs, a.unit_off, a.out, a.out_cap);
     bool overflow = false;
     FOR_UNITS(u, J)
-        overflow |= encode_unit_mad<G, 1, 1, 0>(J, u, m.tbl, m.wob);
+        overflow |= encode_unit_mad<G, S, S, 0>(J, u, m.tbl, m.wob);
     if (overflow)
         set_status(a.status, HUFF_ERR_CAPACITY);
 }
@@ -137,12 +137,13 @@ __global__ void __launch_bounds__(kEncBlock, 1) k_encode(const __grid_constant__
     bool overflow = false;
     const int plan = plan_of(J, max_len);
     if (plan < kFit3) {
-        if (plan == kLong)
-            encode_long(a);
-        else if (plan == kTry4)
-            encode_try<4>(a);
-        else
-            encode_try<3>(a);
+        switch (plan) {
+        case kPairs4: encode_try<4, 2>(a); break;
+        case kPairs3: encode_try<3, 2>(a); break;
+        case kTry4: encode_try<4, 1>(a); break;
+        case kTry3: encode_try<3, 1>(a); break;
+        default: encode_long(a);
+        }
         return;
     }
     FOR_UNITS(u, J)

@@ -259,16 +259,17 @@ __device__ __forceinline__ int full_steps(const Job &J, uint64_t u)
 //  - Longer codes are rare wherever there are any: the groups take 4 codes
 //    where the average is at most 4 bits, else 3, and a multiply-add whose
 //    high word is not zero shows the group that does not fit; its step and the
-//    rest of the unit then go code by code.  On geometric bytes (longest 25 to
-//    29 bits, average 2) 64 MiB take 114 us instead of 211 and 1 GiB 911
-//    instead of 2127.  The same guess for codes of at most 10 bits (4 for 3)
-//    gained 2 to 4% on text and lost as much on Zipf bytes, where every unit
-//    has a group that does not fit: not done.
+//    rest of the unit then go in pairs, if two codes always fit (at most 15
+//    bits), else code by code.  On geometric bytes (longest 25 to 29 bits,
+//    average 2) 64 MiB take 114 us instead of 211 and 1 GiB 911 instead of
+//    2127.  The same guess for codes of at most 10 bits (4 for 3) gained 2 to
+//    4% on text and lost as much on Zipf bytes, where every unit has a group
+//    that does not fit: not done.
 
-// How the codes of a stream are written: 32-bit codes one by one; 3, 4, 8 or
-// 16 at a time because they fit; 3 or 4 at a time because they nearly always
-// fit.
-enum Plan { kLong = 0, kTry3 = 1, kTry4 = 2, kFit3 = 3, kFit4 = 4, kFit8 = 8, kFit16 = 16 };
+// How the codes of a stream are written: 32-bit codes one by one; 3 or 4 at a
+// time because they nearly always fit, else one by one or in pairs; 3, 4, 8 or
+// 16 at a time because they fit.
+enum Plan { kLong, kTry3, kTry4, kPairs3, kPairs4, kFit3, kFit4, kFit8, kFit16 };
 
 __device__ __forceinline__ int plan_of(const Job &J, uint32_t max_len)
 {
@@ -277,7 +278,8 @@ __device__ __forceinline__ int plan_of(const Job &J, uint32_t max_len)
     const uint32_t fit = max_len ? 31u / max_len : 16u;
     if (fit >= 3)
         return fit >= 16 ? kFit16 : fit >= 8 ? kFit8 : fit >= 4 ? kFit4 : kFit3;
-    return J.units && J.unit_off[J.units] <= 4 * J.n ? kTry4 : kTry3;
+    const bool four = J.units && J.unit_off[J.units] <= 4 * J.n;
+    return fit == 2 ? (four ? kPairs4 : kPairs3) : four ? kTry4 : kTry3;
 }
 
 // A stream's half of the code table, built by threads tid = 0..nt-1: one or
