@@ -1237,17 +1237,30 @@ __global__ void k_emit(const T *lf, Samples S, uint32_t count, uint32_t cap, con
     }
 }
 
-// a block whose walk closed after c < m rows repeats its last c bytes
-__global__ void k_periodic_fill(uint8_t *out, uint32_t n, uint32_t block, uint32_t blocks,
+// A block whose walk closed after c < m rows repeats its last c bytes: a warp per
+// piece of a block, `per` of them to one (a CTA per block took 158 us for one
+// of 1 MiB, and as much longer as the block).
+constexpr uint32_t kFillPiece = 4096;
+__global__ void k_periodic_fill(uint8_t *out, uint32_t n, uint32_t block, uint32_t blocks, uint32_t per,
                                 uint32_t regular, const uint32_t *sum, const int32_t *status)
 {
     if (chain_failed(status))
         return;
-    for (uint32_t b = blockIdx.x; b < blocks; b += gridDim.x) {
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t pieces = (uint64_t)blocks * per, warps = (uint64_t)gridDim.x * (kEw / 32);
+    for (uint64_t i = (uint64_t)blockIdx.x * (kEw / 32) + (threadIdx.x >> 5); i < pieces; i += warps) {
+        const uint32_t b = (uint32_t)(i / per), t0 = (uint32_t)(i - (uint64_t)b * per) * kFillPiece;
         const uint32_t s = b * block, m = n - s < block ? n - s : block;
         const uint32_t c = sum[regular + b];
-        for (uint32_t t = c + threadIdx.x; t < m; t += kEw)  // walk steps past the cycle
-            out[s + m - 1 - t] = out[s + m - 1 - t % c];
+        const uint32_t end = m < t0 || m - t0 < kFillPiece ? m : t0 + kFillPiece;
+        uint32_t t = (t0 > c ? t0 : c) + lane;  // walk steps past the cycle
+        uint32_t r = t % c;
+        const uint32_t step = 32 % c;
+        for (; t < end; t += 32) {
+            out[s + m - 1 - t] = out[s + m - 1 - r];
+            r += step;
+            r = r >= c ? r - c : r;
+        }
     }
 }
 
@@ -1361,8 +1374,9 @@ bool invert(InvWs &w, const uint8_t *last, uint32_t n, uint32_t block, uint32_t 
         }
     }
     k_emit<T><<<ew_grid(count), kEw, 0, s>>>(lf, S, count, cap, w.len, nx, sm, kept, d_out, d_status);
-    k_periodic_fill<<<ew_grid((uint64_t)blocks * kEw), kEw, 0, s>>>(d_out, n, block, blocks, S.regular,
-                                                                    sm, d_status);
+    const uint32_t per = div_up(most, kFillPiece);
+    k_periodic_fill<<<ew_grid((uint64_t)blocks * per * 32), kEw, 0, s>>>(d_out, n, block, blocks, per,
+                                                                         S.regular, sm, d_status);
     return true;
 }
 
