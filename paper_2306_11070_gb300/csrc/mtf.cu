@@ -371,6 +371,17 @@ __device__ __forceinline__ void map_bytes(const uint8_t *x, uint8_t *y, uint32_t
             *reinterpret_cast<uint4 *>(y + i) = make_uint4(q[0], q[1], q[2], q[3]);
         }
     }
+    // else eight at a time: straight-line code for several bytes overlaps their
+    // steps, a byte's turn by itself takes half as long again
+    for (; i + 8 <= L; i += 8) {
+        uint32_t q[8];
+#pragma unroll
+        for (int b = 0; b < 8; ++b)
+            q[b] = x[i + b];
+#pragma unroll
+        for (int b = 0; b < 8; ++b)
+            y[i + b] = (uint8_t)f(q[b]);
+    }
     for (; i < L; ++i)
         y[i] = (uint8_t)f(x[i]);
 }
