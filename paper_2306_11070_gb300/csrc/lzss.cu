@@ -912,18 +912,34 @@ __global__ void k_lzss_gather(uint64_t n, uint64_t seg, LzParams P, const uint8_
 
 // ---------------------------------------------------------------- decompress
 // Whether a thread per segment decodes faster than a CTA of two warps per
-// segment: its tokens cost a quarter of the instructions (32 segments share
-// each one), but every segment is one chain of ~700 cycles a token, so it
-// takes very many segments to fill the chip.  1024/12/24/8, stored prefix, the
-// bitstream stand-in, threads against warps: 16384 segments 1.10 / 0.67 ms
-// (64 MiB), 65536 segments 0.74 / 0.79 (64 MiB), 2.28 / 2.52 (256 MiB), 7.1 /
-// 9.3 (1 GiB), 262144 segments 0.96 / 1.34 (64 MiB); so from 320 segments per
-// SM (48640) on.  Its branch-free step wants the stored prefix, a window that
-// fits the thread's ring and literals that fit a token's first word.
-__device__ __forceinline__ bool threads_better(uint64_t count, uint32_t W, uint32_t blk,
-                                               uint32_t dict, uint32_t sms)
+// segment.  A thread's tokens cost a fraction of the instructions (32 segments
+// share each one), but every segment is one chain of some hundreds of cycles a
+// token, so it takes very many segments to fill the chip; a CTA spends about 3
+// ns of it on a segment however short, and on short tokens (Lmin up to 6 bits)
+// as much per bit as the threads.  Measured thread / CTA times, bitstream
+// stand-in:
+//  - stored prefix, windows of 32..2048 bits, literals up to 31 bits (the
+//    branch-free step of decode_fast): 1024/12/24/8 in 1 KiB segments 1.72 from
+//    16384 segments, 1.05 from 49152, 0.76 from 131072; 64/4/11/8 0.86, 0.57
+//    and 0.41.  From 320 segments per SM on, short tokens from 100.
+//  - all others, token by token.  Short tokens: 64/4/11/8 and the counting
+//    dictionary in 256 B segments 1.68 from 8192 segments, 0.76 from 32768, 0.62
+//    from 262144, in 1 KiB segments 2.25, 0.88 and 0.70 (131072).  Longer ones
+//    only where a segment is short: 1024/12/24/8 from 16384, 49152 and 262144
+//    segments of 16 B 0.66, 0.46 and 0.34, 64 B 1.04, 0.66 and 0.53, 128 B 1.46,
+//    0.87 and 0.74, 256 B 2.12, 1.29 and 1.03, 1 KiB 3.07, 1.85 and (131072) 1.43.
+__device__ __forceinline__ bool threads_better(uint64_t count, uint64_t seg, const LzParams &P,
+                                               uint32_t sms)
 {
-    return count >= 320ull * sms && W >= 32 && W <= kThrMaxWindow && dict == 2 && blk <= 31;
+    const bool brief = P.lmin <= 6 && P.W <= kThrMaxWindow;
+    uint32_t per_sm;  // from so many segments on
+    if (P.dict == 2 && P.W >= 32 && P.W <= kThrMaxWindow && P.blk <= 31)
+        per_sm = brief ? 100 : 320;
+    else if (brief)
+        per_sm = seg <= 64 ? 100 : 200;
+    else
+        per_sm = seg <= 32 ? 100 : seg <= 64 ? 200 : seg <= 128 ? 320 : seg <= 256 ? 1000 : ~0u;
+    return per_sm != ~0u && count >= (uint64_t)per_sm * sms;
 }
 
 // Header and table checks, segment starts (scan), *d_n; statuses as the
@@ -979,7 +995,9 @@ __global__ void __launch_bounds__(kScanBlock)
             if (n > cap)
                 set_status(status, HUFF_ERR_CAPACITY);
             else
-                *path = threads_better(count, f[0], f[3], f[4], sms) ? kPathThreads : kPathWarps;
+                *path = threads_better(count, seg, make_params(f[0], f[1], f[2], f[3], f[4]), sms)
+                            ? kPathThreads
+                            : kPathWarps;
         }
     }
 }
@@ -1456,24 +1474,35 @@ struct CodeReader {
     }
 };
 
-// The bits a thread has produced so far, read back from the thread's ring of
-// recent words in shared memory; the word being filled is in a register.
-// Completed words are written out four at a time with one 16-byte store.
+// The bits a thread has produced so far, read back: with kRing from the
+// thread's ring of recent words in shared memory, else from the output; the
+// word being filled is in a register, and bits before the segment are the
+// dictionary's.  With the ring, completed words are written out four at a time
+// with one 16-byte store.
+template <bool kRing>
 struct OutBits {
     uint8_t *y;      // the segment's output (16-byte aligned)
     uint32_t m;      // its bytes (at most 16 MiB)
+    uint32_t W;
     uint32_t *ring;  // kThrRing words, word q at q mod kThrRing
     uint32_t pend;   // bits of the word being filled, left-aligned
     uint32_t npend;  // their count
     uint32_t pos;    // bits produced (< 2^27)
-    __device__ __forceinline__ uint32_t word_at(uint32_t q) const
+    __device__ __forceinline__ uint32_t word_at(int32_t q) const
     {
-        return q == (pos >> 5) ? pend : q > (pos >> 5) ? 0u : ring[q & (kThrRing - 1)];
+        const int32_t cur = (int32_t)(pos >> 5);
+        if (q < 0)
+            return W >= 32 ? dict_word((uint32_t)(q + (int32_t)(W / 32))) : dict_word(0) >> (32 - W);
+        if (q >= cur)
+            return q == cur ? pend : 0u;
+        return kRing ? ring[(uint32_t)q & (kThrRing - 1)]
+                     : bswap32(__ldcg(reinterpret_cast<const uint32_t *>(y) + q));
     }
-    // the 32 bits at output bit s
-    __device__ __forceinline__ uint32_t bits_at(uint32_t s) const
+    // the 32 bits at output bit s (at most W bits before the segment)
+    __device__ __forceinline__ uint32_t bits_at(int32_t s) const
     {
-        return __funnelshift_l(word_at((s >> 5) + 1), word_at(s >> 5), s & 31u);
+        const int32_t q = s >> 5;  // floor
+        return __funnelshift_l(word_at(q + 1), word_at(q), (uint32_t)s & 31u);
     }
     // append the top k (1..32) bits of v
     __device__ __forceinline__ void put(uint32_t v, uint32_t k)
@@ -1493,6 +1522,10 @@ struct OutBits {
     }
     __device__ __forceinline__ void complete(uint32_t q, uint32_t w) const
     {
+        if (!kRing) {
+            store_out_word(y, m, q, w);
+            return;
+        }
         ring[q & (kThrRing - 1)] = w;
         if ((q & 3) == 3) {  // a whole 16-byte group
             const uint32_t g = q >> 2;
@@ -1510,8 +1543,9 @@ struct OutBits {
     __device__ __forceinline__ void finish() const
     {
         const uint32_t q = pos >> 5;  // the word being filled
-        for (uint32_t j = q & ~3u; j < q; ++j)  // completed words of the last, unfinished group
-            store_out_word(y, m, j, ring[j & (kThrRing - 1)]);
+        if (kRing)  // completed words of the last, unfinished group
+            for (uint32_t j = q & ~3u; j < q; ++j)
+                store_out_word(y, m, j, ring[j & (kThrRing - 1)]);
         if (npend)
             store_out_word(y, m, q, pend);
     }
@@ -1571,7 +1605,7 @@ struct CodeRing {
 // diverge: both the match and the literal are formed and the token
 // selects.  False (and the caller's status) only for a length field above
 // the longest match.
-__device__ __forceinline__ bool decode_fast(CodeReader &rd, OutBits &ob, const LzParams &P,
+__device__ __forceinline__ bool decode_fast(CodeReader &rd, OutBits<true> &ob, const LzParams &P,
                                             uint32_t nbits, uint32_t in_col)
 {
     CodeRing rg;
@@ -1631,18 +1665,21 @@ __device__ __forceinline__ bool decode_fast(CodeReader &rd, OutBits &ob, const L
 }
 
 // Decode one segment's tokens; false if the code is corrupt.
-__device__ __forceinline__ bool decode_segment(CodeReader &rd, OutBits &ob, const LzParams &P,
+template <bool kRing>
+__device__ __forceinline__ bool decode_segment(CodeReader &rd, OutBits<kRing> &ob, const LzParams &P,
                                                uint32_t nbits, uint32_t in_col)
 {
-    const uint32_t raw = nbits < P.W ? nbits : P.W;
+    const uint32_t raw = P.dict != 2 ? 0u : nbits < P.W ? nbits : P.W;
     while (ob.pos < raw) {
         const uint32_t k = raw - ob.pos < 32 ? raw - ob.pos : 32u;
         if (rd.pos + k > rd.nbits)
             return false;
         ob.put(rd.get(k) << (32 - k), k);
     }
-    if (!decode_fast(rd, ob, P, nbits, in_col))
-        return false;
+    if constexpr (kRing) {
+        if (P.dict == 2 && P.blk <= 31 && !decode_fast(rd, ob, P, nbits, in_col))
+            return false;
+    }
     while (ob.pos < nbits) {
         if (rd.pos >= rd.nbits)
             return false;
@@ -1652,9 +1689,9 @@ __device__ __forceinline__ bool decode_segment(CodeReader &rd, OutBits &ob, cons
                 return false;
             const uint32_t d = rd.get(P.ob) + 1;
             const uint32_t len = rd.get(P.lb) + P.lmin;
-            if (len > P.lmax || len > r || d > ob.pos)
+            if (len > P.lmax || len > r || (P.dict == 2 && d > ob.pos))
                 return false;
-            uint32_t v = ob.bits_at(ob.pos - d);
+            uint32_t v = ob.bits_at((int32_t)ob.pos - (int32_t)d);
             if (d < len) {  // the source runs into these bits: period d
                 v &= ~(0xffffffffu >> d);
                 for (uint32_t sh = d; sh < len; sh <<= 1)
@@ -1679,30 +1716,33 @@ __global__ void __launch_bounds__(kThrBlock)
     // ring of thread t at t * (kThrRing + 1): the odd stride spreads the
     // threads' equal ring positions over the banks
     __shared__ uint32_t rings[kThrBlock * (kThrRing + 1)];
-    __shared__ __align__(16) uint4 in_ring[kLzInCells * kThrBlock];  // [cell][thread]
+    __shared__ __align__(16) uint4 cells[kLzInCells * kThrBlock];  // [cell][thread]
     if (*path != kPathThreads)
         return;
-    const uint32_t in_col = smem_u32(in_ring) + threadIdx.x * 16;
+    const uint32_t in_col = smem_u32(cells) + threadIdx.x * 16;
     const uint64_t n = *reinterpret_cast<const uint64_t *>(c);
     const uint64_t seg = *reinterpret_cast<const uint64_t *>(c + 8);
     const uint32_t *f = reinterpret_cast<const uint32_t *>(c + 16);
     const LzParams P = make_params(f[0], f[1], f[2], f[3], f[4]);
     const uint64_t count = *reinterpret_cast<const uint64_t *>(c + 40);
+    const bool in_ring = P.W >= 32 && P.W <= kThrMaxWindow;
     for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s < count;
          s += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t m = s + 1 < count ? seg : n - s * seg;
+        const uint32_t m = (uint32_t)(s + 1 < count ? seg : n - s * seg);
         CodeReader rd;
         rd.init(c + start[s], *reinterpret_cast<const uint32_t *>(c + kLzHead + 4 * s));
-        OutBits ob;
-        ob.y = out + s * seg;
-        ob.m = (uint32_t)m;
-        ob.ring = rings + threadIdx.x * (kThrRing + 1);
-        ob.pend = 0;
-        ob.npend = 0;
-        ob.pos = 0;
-        if (decode_segment(rd, ob, P, (uint32_t)(8 * m), in_col))
-            ob.finish();
-        else
+        auto decode = [&](auto ob) {
+            ob.y = out + s * seg;
+            ob.m = m;
+            ob.W = P.W;
+            ob.ring = rings + threadIdx.x * (kThrRing + 1);
+            ob.pend = ob.npend = ob.pos = 0;
+            const bool good = decode_segment(rd, ob, P, 8 * m, in_col);
+            if (good)
+                ob.finish();
+            return good;
+        };
+        if (!(in_ring ? decode(OutBits<true>()) : decode(OutBits<false>())))
             set_status(status, HUFF_ERR_CORRUPT_STREAM);
     }
 }
