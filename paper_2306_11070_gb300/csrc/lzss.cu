@@ -22,9 +22,9 @@
 //
 // Compression: one warp per segment, or per part of a segment where there are
 // few (see k_lzss_parts).  For each token the 32 lanes search the window
-// together: for windows of 64 to 16384 bits all distances bit-parallel
-// (a lane's 32-bit mask holds 32 sources) from a ring in shared memory, other
-// windows a distance at a time through L1.  Every lane keeps the same 64-bit
+// together: for windows of 64 to 16384 bits from a ring in shared memory, all
+// distances bit-parallel (a lane's 32-bit mask holds 32 sources) or, in narrow
+// windows, a distance at a time; other windows so through L1.  Every lane keeps the same 64-bit
 // output accumulator and lane 0 stores the completed words into the
 // segment's worst-case slot of the workspace; a one-CTA scan then lays out
 // the header and length table and a gather moves every code into place.
@@ -220,6 +220,25 @@ __host__ __device__ __forceinline__ bool ring_ok(const LzParams &P)
     return P.W >= 64 && P.W <= kRingMaxWindow;
 }
 
+// Whether the search takes a distance at a time instead of 1024 at once: about
+// 8 instructions per 32 bits of window against 4 or 5 per bit of the longest
+// match, of Lmin bits at least.  `many`: segments to fill the chip, so that
+// instructions count and not a chain's length.  16 MiB of random bytes, ms by
+// distances / at once (with one candidate a lane and step in all windows, before,
+// 3.4 in 1 KiB segments of 64/4/11/8):
+//               1 KiB segments  64 KiB segments
+//   64/4/11/8     2.22 / 4.69     20.3 / 30.1
+//   64/12/24/8    1.72 / 2.25     16.8 / 17.5
+//   128/4/11/8    2.39 / 4.12     21.8 / 26.6
+//   128/12/24/8   2.08 / 2.24     21.2 / 18.3
+//   256/4/11/8    2.86 / 3.61     26.4 / 23.6
+//   256/8/16/8    2.64 / 2.67     24.8 / 19.5
+//   512/4/11/8    3.84 / 3.17     36.6 / 21.3
+bool by_distance(const LzParams &P, bool many)
+{
+    return P.W <= (P.lmin < 8 ? 128u : 64u) << (many ? 1 : 0);
+}
+
 // The longest match of lo..maxlen bits over 1024 distances at once, the
 // smallest distance among equally long ones.  Lane j holds 32 sources, the
 // bits a:b (64 bits of the window from bit P - 32 j - 32 of position P); bit
@@ -229,7 +248,7 @@ __host__ __device__ __forceinline__ bool ring_ok(const LzParams &P)
 // where X's bit is 0.  About four instructions a step for 1024 candidates,
 // against six for 32 when each candidate is shifted into place and compared
 // by itself.  One vote after the first 4 G0 steps (G0 = Lmin / 4, straight-line)
-// ends most searches; else every lane finishes its steps and a warp maximum
+// ends most searches, with Lmin below 8 one after 12; else every lane finishes its steps and a warp maximum
 // picks the match.  Returns its length << 10 | (1023 - (d - 1)) with d counted
 // within the 1024, 0 for none of lo..maxlen bits.
 __device__ __forceinline__ uint32_t sign_byte3(uint32_t v)  // the top bit, 32 times
@@ -282,6 +301,8 @@ __device__ __forceinline__ uint32_t search_masks(uint32_t a, uint32_t b, uint32_
     for (int t = 4 * G0; t < 32; ++t) {
         if ((t & 3) == 0 && (uint32_t)t >= maxlen)
             break;
+        if (G0 < 2 && (t == 12 || t == 20) && !__any_sync(0xffffffffu, m != 0))
+            break;  // (from so short a start few searches go on)
         m = step(t, m);
         if (m && (uint32_t)t < maxlen) {
             best = m;
@@ -291,6 +312,30 @@ __device__ __forceinline__ uint32_t search_masks(uint32_t a, uint32_t b, uint32_
     const uint32_t key =
         len >= lo && len <= maxlen ? len << 10 | (1024u - 32u * lane - __ffs(best)) : 0u;
     return __reduce_max_sync(0xffffffffu, key);
+}
+
+// The same a distance at a time, lane's distances lane + 1, lane + 33, ... up to
+// 32 * count: its sources start at bit `at` of the ring and every 32 bits before.
+// Returns the length << 16 | (65535 - (d - 1)), whatever the length.
+__device__ __forceinline__ uint32_t search_distances(const uint32_t *ring, uint32_t R, uint32_t at,
+                                                     uint32_t count, uint32_t X, uint32_t maxlen,
+                                                     int lane)
+{
+    const uint32_t sh = at & 31u;
+    uint32_t i = (at >> 5) & (R - 1), best = 0, tag = 65535u - lane;
+    uint32_t after = ring[i + 1];
+#pragma unroll 2
+    for (uint32_t k = 0; k < count; ++k) {
+        const uint32_t w = ring[i];
+        uint32_t len = __clz(__funnelshift_l(after, w, sh) ^ X);
+        len = len < maxlen ? len : maxlen;
+        const uint32_t key = (len << 16) + tag;
+        best = key > best ? key : best;
+        after = w;
+        i = (i - 1) & (R - 1);
+        tag -= 32;
+    }
+    return __reduce_max_sync(0xffffffffu, best);
 }
 
 // Output bits of one warp, the same in every lane: the pending n < 32 bits
@@ -427,7 +472,14 @@ struct Coder {
             }
             const uint32_t maxlen = r < P.lmax ? r : P.lmax;
             uint32_t len = 0, dm1 = 0;
-            if (maxlen >= P.lmin) {
+            if constexpr (G0 < 0) {
+                const uint32_t key =
+                    search_distances(ring, R, v - lane - 1, dwords, X, maxlen, lane);
+                if (key >> 16 >= P.lmin) {
+                    len = key >> 16;
+                    dm1 = 65535u - (key & 65535u);
+                }
+            } else if (maxlen >= P.lmin) {
                 uint32_t key = search_masks<G0>(__funnelshift_l(w1, w0, sh),
                                                 __funnelshift_l(w2, w1, sh),
                                                 lane < (int)dwords ? 0xffffffffu : 0u, X, P.lmin,
@@ -1873,7 +1925,9 @@ huff_status_t huff_lzss_compress(const uint8_t *d_in, uint64_t n, uint64_t segme
                                                                            slots, bits, d_status);
                 }
             };
-            switch (P.lmin / 4) {
+            const bool many = count >= 50 * (uint64_t)sms;
+            switch (by_distance(P, many) ? -1 : (int)(P.lmin / 4)) {
+            case -1: run(std::integral_constant<int, -1>()); break;
             case 0: run(std::integral_constant<int, 0>()); break;
             case 1: run(std::integral_constant<int, 1>()); break;
             case 2: run(std::integral_constant<int, 2>()); break;
