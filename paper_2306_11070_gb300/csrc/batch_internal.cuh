@@ -63,13 +63,15 @@ struct BatchLayout {
     uint64_t upload_bytes;  // leading part filled from the host
 };
 
-void batch_layout(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op, BatchLayout &L);
+// even: buffers of one size but for the last, kept in their order.
+void batch_layout(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op, BatchLayout &L,
+                  bool even = false);
 BatchArgs batch_args(const BatchLayout &L, void *d_block, uint32_t cs, uint32_t lanes, bool own_lanes,
                      uint32_t barrier_extra = 0);
 cudaError_t batch_upload(const BatchLayout &L, void *d_block, uint8_t *host, cudaStream_t s);
 int batch_occupancy(huff_op_t op);
 cudaError_t batch_launch(huff_op_t op, const BatchArgs &args, unsigned grid, cudaStream_t s);
-// Run a batch once, its lanes not a caller's own: with its device block in
+// Run an even batch once, its lanes not a caller's own: with its device block in
 // `scratch` (16-byte aligned) where it fits, else by a plan, which the caller
 // destroys once the stream has passed it.  `host` is read by the upload until
 // then too.
