@@ -267,7 +267,8 @@ void huff_batch_default_params(huff_batch_params_t *params);
  * 520 bytes per 16 KiB of input for compression) and captures the launch in
  * a CUDA graph; runs then allocate nothing.  Buffers are 16-byte aligned;
  * compress outputs need out_cap >= header + offset table (use
- * huff_max_stream_size).  Errors: HUFF_ERR_INVALID_ARG, HUFF_ERR_CUDA. */
+ * huff_max_stream_size).  Errors: HUFF_ERR_INVALID_ARG, HUFF_ERR_CUDA,
+ * HUFF_ERR_UNSUPPORTED (a build whose compress kernel cannot run). */
 huff_status_t huff_batch_plan(const huff_batch_desc_t *descs, uint32_t count, huff_op_t op,
                               const huff_batch_params_t *params, huff_batch_plan_t **plan);
 

@@ -73,14 +73,13 @@ __device__ bool grid_barrier(unsigned int *ctl, int32_t *fail, uint32_t extra)
     return s_ok != 0;
 }
 
-// After a barrier gave up: every buffer reports the timeout.
-__device__ void fail_all(const BatchBuf *bufs, uint32_t count)
+// Every buffer reports the error, after a barrier that gave up a timeout.
+__device__ void fail_all(const BatchBuf *bufs, uint32_t count, int32_t error = HUFF_ERR_TIMEOUT)
 {
     if (threadIdx.x == 0)
         for (uint32_t b = 0; b < count; ++b)
-            set_status(bufs[b].status, HUFF_ERR_TIMEOUT);
+            set_status(bufs[b].status, error);
 }
-
 
 // Largest b with base[b] <= x, for x < base[count].
 __device__ __forceinline__ uint32_t find_owner(const uint64_t *base, uint32_t count, uint64_t x)
@@ -188,8 +187,12 @@ __device__ __forceinline__ unsigned int half_broadcast(unsigned int t, HalfSync 
 // ------------------------------------------------------------------ compress
 // The code table of both halves starts at this address of the shared window (a
 // constant, so that it is part of the table loads), a little above the end of
-// the static shared memory.
-constexpr uint32_t kTblAt = 6144;
+// the static shared memory: at most kTblSlack bytes, which the launch adds.  How
+// much that memory is is up to the compiler, so batch_occupancy checks it.
+#ifndef HUFF_BATCH_TABLE_AT
+#define HUFF_BATCH_TABLE_AT 6144
+#endif
+constexpr uint32_t kTblAt = HUFF_BATCH_TABLE_AT;
 constexpr uint32_t kTblSlack = 4096;
 
 // One function per way of grouping: inlined together they spill.
@@ -396,7 +399,7 @@ __global__ void __launch_bounds__(kBatchBlock, 2) k_batch_compress(BatchArgs a)
         const HalfSync hs{half};
         const uint32_t pad = kTblAt - smem_u32(smem_raw);
         if (pad > kTblSlack) {  // not where the table's address is encoded
-            fail_all(a.bufs, a.count);
+            fail_all(a.bufs, a.count, HUFF_ERR_UNSUPPORTED);
             return;
         }
         uint32_t *tbl = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned char *>(smem_raw) + pad);
@@ -730,10 +733,30 @@ cudaError_t batch_upload(const BatchLayout &L, void *d_block, uint8_t *host, cud
 
 KernelSetup g_compress_setup, g_decompress_setup;
 
-// Resident CTAs per SM of the batch kernel for `op` on the current device
-// (0 on error).
+// Whether the compress kernel's code table can lie at kTblAt.
+bool table_fits()
+{
+    static std::atomic<bool> known{false};
+    if (known.load(std::memory_order_relaxed))
+        return true;
+    cudaFuncAttributes attr;
+    int reserved = 0;
+    if (cudaFuncGetAttributes(&attr, k_batch_compress) != cudaSuccess ||
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, current_device()) !=
+            cudaSuccess)
+        return false;
+    const uint64_t start = (uint64_t)reserved + attr.sharedSizeBytes;  // of the dynamic part
+    const bool fits = start <= kTblAt && kTblAt - start <= kTblSlack;
+    known.store(fits, std::memory_order_relaxed);
+    return fits;
+}
+
+// Resident CTAs per SM of the batch kernel for `op` on the current device (0 on
+// error, -1 where this build's kernel cannot run).
 int batch_occupancy(huff_op_t op)
 {
+    if (op == HUFF_BATCH_COMPRESS && current_device() >= 0 && !table_fits())
+        return -1;
     int per_sm = 0;
     const cudaError_t err =
         op == HUFF_BATCH_COMPRESS
@@ -859,7 +882,7 @@ huff_status_t make_plan(const BatchLayout &L, const huff_batch_params_t &prm, bo
     int per_sm = batch_occupancy(L.op);
     if (per_sm < 1) {
         free_plan(p);
-        return HUFF_ERR_CUDA;
+        return batch_occupancy_error(per_sm);
     }
     if (prm.ctas_per_sm && (int)prm.ctas_per_sm < per_sm)
         per_sm = (int)prm.ctas_per_sm;
@@ -912,7 +935,7 @@ huff_status_t batch_once(const huff_batch_desc_t *descs, uint32_t count, huff_op
     }
     const int per_sm = batch_occupancy(op);
     if (per_sm < 1)
-        return HUFF_ERR_CUDA;
+        return batch_occupancy_error(per_sm);
     host.resize(L.upload_bytes);
     if (batch_upload(L, scratch, host.data(), s) != cudaSuccess)
         return HUFF_ERR_CUDA;

@@ -70,6 +70,10 @@ BatchArgs batch_args(const BatchLayout &L, void *d_block, uint32_t cs, uint32_t 
                      uint32_t barrier_extra = 0);
 cudaError_t batch_upload(const BatchLayout &L, void *d_block, uint8_t *host, cudaStream_t s);
 int batch_occupancy(huff_op_t op);
+inline huff_status_t batch_occupancy_error(int per_sm)
+{
+    return per_sm < 0 ? HUFF_ERR_UNSUPPORTED : HUFF_ERR_CUDA;
+}
 cudaError_t batch_launch(huff_op_t op, const BatchArgs &args, unsigned grid, cudaStream_t s);
 // Run an even batch once, its lanes not a caller's own: with its device block in
 // `scratch` (16-byte aligned) where it fits, else by a plan, which the caller

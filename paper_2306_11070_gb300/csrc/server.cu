@@ -408,7 +408,7 @@ huff_status_t huff_server_create(const huff_server_cfg_t *cfg, huff_server_t **o
                              huff::batch_occupancy(HUFF_BATCH_DECOMPRESS));
     if (occ < 1) {
         destroy_server(S);
-        return HUFF_ERR_CUDA;
+        return huff::batch_occupancy_error(occ);
     }
     S->grid = std::max(1u, (unsigned)(huff::device_sm_count() * occ) / c.max_rounds);
     S->rounds.resize(c.max_rounds);
