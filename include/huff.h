@@ -554,7 +554,7 @@ uint64_t huff_lzss_decompress_workspace_size(uint64_t in_bytes);
  * segment whose tokens do not end exactly at its recorded length is
  * HUFF_ERR_CORRUPT_STREAM in *d_status (the output is then unspecified);
  * n > out_cap is HUFF_ERR_CAPACITY.  Two warps decode each segment (a thread
- * each where there are tens of thousands of segments).
+ * each where there are very many, or many short ones).
  * d_in, d_out, d_ws 16-byte aligned.  Host errors: HUFF_ERR_INVALID_ARG,
  * HUFF_ERR_CUDA. */
 huff_status_t huff_lzss_decompress(const uint8_t *d_in, uint64_t in_bytes, uint8_t *d_out,

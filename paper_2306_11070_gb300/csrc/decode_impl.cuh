@@ -54,7 +54,6 @@ template <int C>
 struct DecodeShared {
     uint32_t lut[kLutSize * C];
     uint8_t len0[kLutSize];
-    uint8_t len_s[256];
     uint8_t sorted[256];
     uint32_t count[kMaxCodeLen + 1];
     uint32_t first[kMaxCodeLen + 1];

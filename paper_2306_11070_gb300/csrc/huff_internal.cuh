@@ -67,9 +67,8 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p)
 // shifts, logic ops and compares, at half a warp per cycle) to the work only
 // it can do.  The values are not visible to the compiler, so it cannot turn
 // the multiplies back into shifts and adds.
-enum { kOne, kMinus1, kFour, kEight, k32, kMinus32, k128, kMinusTop8, k16, kNumConst };
-static __constant__ uint32_t kc[kNumConst] = {1u, 0xffffffffu, 4u, 8u, 32u, 0xffffffe0u,
-                                              128u, 0xff000000u, 16u};
+enum { kOne, kMinus1, kFour, kEight, k32, k16, kNumConst };
+static __constant__ uint32_t kc[kNumConst] = {1u, 0xffffffffu, 4u, 8u, 32u, 16u};
 __device__ __forceinline__ uint32_t imad(uint32_t a, uint32_t b, uint32_t c) { return a * b + c; }
 
 // Shared-memory accesses by 32-bit shared address.  The rings are accessed
