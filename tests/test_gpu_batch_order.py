@@ -74,13 +74,12 @@ def test_segments_need_no_second_plan():
         L.huff_batch_destroy(h)
         return r
 
-    times = {}
-    for f in (container, planned):
-        t = []
-        for _ in range(25):
+    times = {f.__name__: [] for f in (container, planned)}
+    for _ in range(40):  # in turn, and the least of each: the host's own noise
+        for f in (container, planned):
             t0 = time.perf_counter()
             assert f() == 0
             torch.cuda.synchronize()
-            t.append(time.perf_counter() - t0)
-        times[f.__name__] = sorted(t)[12]
-    assert times["container"] < 1.2 * times["planned"], times
+            times[f.__name__].append(time.perf_counter() - t0)
+    least = {k: min(v) for k, v in times.items()}
+    assert least["container"] < 1.2 * least["planned"], least
